@@ -111,8 +111,9 @@ class ClockSampler:
 
 
 PROFILED = {  # the committed ncu summary of each timed kernel, and the sources that define it
-    "plain": ("pair_sym_kahan_production_n524288.md", ["pair_fp32.cuh", "pair_sym.cuh"]),
-    "surrogate": ("pair_sym_surr_kahan_production_n524288.md", ["pair_fp32.cuh", "surrogate_pair.cuh", "pair_sym.cuh"]),
+    "plain": ("pair_sym_kahan_production_n524288.md", ["pair_fp32.cuh", "pair2.cuh", "pair_sym.cuh"]),
+    "surrogate": ("pair_sym_surr_kahan_production_n524288.md",
+                  ["pair_fp32.cuh", "pair2.cuh", "surrogate_pair.cuh", "pair_sym.cuh"]),
 }
 
 
@@ -253,6 +254,28 @@ def measured_peaks():
             return json.load(fh)
     except (OSError, ValueError):
         return None
+
+
+LINE_MIN_NCUT = 12      # windows from this n_cut on take the far images in closed form (csrc/pair2.cuh)
+LINE_FP32_OPS = 130     # FP32 lane operations per pair of that form without softened images: the separation
+                        # and the sums of both sides 32, seven near images 43, the rest of the line 55
+FP32_PER_SM_CLK = 128
+
+
+def plain_roofline(n_sm, sm_mhz, n_cut, pairs, kernel_s):
+    """Roofline of the plain window's pair kernel (pairs: the pairs it evaluated).
+    Narrow windows are walked image by image: one MUFU rsqrt per pair-image. From
+    LINE_MIN_NCUT on the far images are in closed form, and the FP32 operations of a
+    pair bind (its 10 MUFU operations take 0.6 of their time)."""
+    if n_cut < LINE_MIN_NCUT:
+        peak = n_sm * MUFU_RSQRT_PER_SM_CLK * sm_mhz * 1e6 / (2.0 * n_cut)
+        basis = f"{n_sm} SMs x {MUFU_RSQRT_PER_SM_CLK} MUFU rsqrt/SM/clk x {sm_mhz:.0f} MHz / {2 * n_cut} images"
+    else:
+        peak = n_sm * FP32_PER_SM_CLK * sm_mhz * 1e6 / LINE_FP32_OPS
+        basis = f"{n_sm} SMs x {FP32_PER_SM_CLK} FP32 ops/SM/clk x {sm_mhz:.0f} MHz / {LINE_FP32_OPS} ops per pair"
+    achieved = pairs / kernel_s
+    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "pair interactions evaluated/s",
+            "frac": achieved / peak, "peak_basis": basis}
 
 
 def surrogate_roofline(n_sm, sm_mhz, n0, pairs, kernel_s, symmetric=False, headline=True):
@@ -484,12 +507,9 @@ def run(args):
     ev_s = sc.steps_cyl_last_eval(ctx)  # the pairs the kernel evaluated (each unordered pair once if symmetric)
     roof = surrogate_roofline(props.multi_processor_count, sm_mhz, w.n0, ev_s["pairs_evaluated"], kernel_s,
                               ev_s["symmetric"])
-    peak_plain = props.multi_processor_count * MUFU_RSQRT_PER_SM_CLK * sm_mhz * 1e6
     if not accepted:  # the plain sum ran: its own roofline
-        done = ev_s["pairs_evaluated"] * 2.0 * w.n_cut
-        roof = {"bound": "alu", "achieved": done / kernel_s, "peak": peak_plain, "unit": "pair-images evaluated/s",
-                "frac": done / kernel_s / peak_plain, "traffic": recorded_traffic("plain"),
-                "symmetric": ev_s["symmetric"]}
+        roof = {**plain_roofline(props.multi_processor_count, sm_mhz, w.n_cut, ev_s["pairs_evaluated"], kernel_s),
+                "traffic": recorded_traffic("plain"), "symmetric": ev_s["symmetric"]}
     # reorders and surrogate checks that fell in the timed region add launches
     timed = range(steps_before + 1, steps_before + args.steps + 1)
     reorders = sum(1 for s in timed if s % REORDER_EVERY == 0)
@@ -506,7 +526,6 @@ def run(args):
     plain_kernel_s = statistics.mean(plain_pair_ms) / 1e3
     plain_step_s = statistics.mean(plain_ms) / 1e3
     ev_p = sc.steps_cyl_last_eval(ctx)
-    plain_done = ev_p["pairs_evaluated"] * 2.0 * w.n_cut
     sc.steps_cyl_set_tail(ctx, sc.STEPS_TAIL_SURROGATE if accepted else sc.STEPS_TAIL_FULL)
     sc.steps_cyl_kdk_step(ctx, dt, 1)  # the switch marks the forces stale: refresh them untimed
 
@@ -560,11 +579,9 @@ def run(args):
         "plain": {"steps": plain_steps, "kdk_step_ms": 1e3 * plain_step_s, "pair_kernel_ms": 1e3 * plain_kernel_s,
                   "pair_images_per_s": images_per_step / plain_step_s,
                   "error_vs_fp64": errs["plain"],
-                  "roofline": {"bound": "alu", "achieved": plain_done / plain_kernel_s, "peak": peak_plain,
-                               "unit": "pair-images evaluated/s", "frac": plain_done / plain_kernel_s / peak_plain,
-                               "traffic": recorded_traffic("plain"), "symmetric": ev_p["symmetric"],
-                               "peak_basis": f"{props.multi_processor_count} SMs x {MUFU_RSQRT_PER_SM_CLK} MUFU "
-                                             f"rsqrt/SM/clk x {sm_mhz:.0f} MHz; 1 rsqrt per pair-image"}},
+                  "roofline": {**plain_roofline(props.multi_processor_count, sm_mhz, w.n_cut,
+                                                ev_p["pairs_evaluated"], plain_kernel_s),
+                               "traffic": recorded_traffic("plain"), "symmetric": ev_p["symmetric"]}},
         "error_reference": "library FP64 form on 4096 particles (seed 12345), pinned to the FP64 oracle in the tests",
         "roofline": roof,
         "clocks": {"sm_mhz": clk["sm_mhz"], "sm_max_mhz": clk["sm_max_mhz"], "reasons": clk["reasons"]},
@@ -773,7 +790,6 @@ def run_table1(args):
     n, n_cut = d["pos"].shape[0], 16
     pairs = n * (n - 1.0)
     props = torch.cuda.get_device_properties(0)
-    peak = props.multi_processor_count * MUFU_RSQRT_PER_SM_CLK * 2070e6
     a0 = ics.TABLE1_A_INIT
     t0 = ics.lcdm_time_of_a(a0, ics.TABLE1_OMEGA_M, ics.TABLE1_OMEGA_L)
     R = ics.TABLE1_GEOMETRY["R_sim"]
@@ -793,11 +809,12 @@ def run_table1(args):
     ev1.record()
     torch.cuda.synchronize()
     rate = pairs * 2 * n_cut / (ms * 1e-3)
-    done = evl["pairs_evaluated"] * 2 * n_cut / (ms * 1e-3)   # pair-images the kernel evaluated per second
     line = {"workload": "table1_n65536", "n": n, "n_cut": n_cut, "core_rings": d["rings"].n_in,
             "outer_rings": d["rings"].n_out, "cells_per_ring": [64, 64],
             "mass_range": float(d["m"].max() / d["m"].min()),
-            "fp32_kahan": {"pair_ms": ms, "pair_images_per_s": rate, "roofline_frac": done / peak,
+            "fp32_kahan": {"pair_ms": ms, "pair_images_per_s": rate,
+                           "roofline": plain_roofline(props.multi_processor_count, 2070.0, n_cut,
+                                                      evl["pairs_evaluated"], ms * 1e-3),
                            "symmetric": evl["symmetric"],
                            "kdk_step_ms": ev0.elapsed_time(ev1) / 10, "error_vs_fp64": _err(a32[idx], a64)}}
     sim.close()
@@ -1146,8 +1163,7 @@ def run_workload(args):
     n = w.n
     pairs = n * (n - 1.0)
     props = torch.cuda.get_device_properties(0)
-    peak = props.multi_processor_count * MUFU_RSQRT_PER_SM_CLK * 2070e6
-    line = {"workload": w.name, "n": n, "n_cut": w.n_cut, "roofline_peak_pair_images_per_s": peak}
+    line = {"workload": w.name, "n": n, "n_cut": w.n_cut}
     idx = ics.subsample(n, 4096 if w.name.startswith("precision") else 256, seed=12345)
     reps = 1 if n > 300000 else 2
     sim = _ctx_for(sc, torch, w, d, sc.STEPS_FP32_KAHAN, check_particles=1024,
@@ -1156,7 +1172,8 @@ def run_workload(args):
     ev32 = sc.steps_cyl_last_eval(sim.ctx)
     line["fp32_kahan"] = {"pair_ms": ms32, "pair_images_per_s": pairs * 2 * w.n_cut / (ms32 * 1e-3),
                           "symmetric": ev32["symmetric"],
-                          "roofline_frac": ev32["pairs_evaluated"] * 2 * w.n_cut / (ms32 * 1e-3) / peak}
+                          "roofline": plain_roofline(props.multi_processor_count, 2070.0, w.n_cut,
+                                                     ev32["pairs_evaluated"], ms32 * 1e-3)}
     sc.steps_cyl_set_precision(sim.ctx, sc.STEPS_FP64)
     a64 = sim.forces_subset(idx)
     ms64 = sc.steps_cyl_last_timing(sim.ctx)[1]

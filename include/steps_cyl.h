@@ -51,7 +51,9 @@ extern "C" {
 #define STEPS_FP32_KAHAN 1  /* FP32 pair math on hi/lo split positions, Kahan-compensated j sum */
 #define STEPS_FP32_PLAIN 2  /* FP32 pair math on hi/lo split positions, plain j sum */
 
-#define STEPS_TAIL_FULL 0       /* every image of the window summed directly */
+#define STEPS_TAIL_FULL 0       /* every image of the window: one by one in FP64 and for n_cut < 12; else the near
+                                 * images (and the softened ones) one by one and the others, a smooth function of
+                                 * the image number, in closed form to below FP32 rounding */
 #define STEPS_TAIL_SURROGATE 1  /* images |k| <= n0 direct, far tail from the learned surrogate */
 #define STEPS_TAIL_TABLE 2      /* images |k| <= n0 direct, far tail from the correction table */
 
@@ -180,9 +182,9 @@ int steps_cyl_last_timing(steps_cyl_ctx* ctx, double* pair_images, double* pair_
  * out[0] = pair-images delivered (as steps_cyl_last_timing), out[1] = pairs the
  * pair kernel evaluated, out[2] = its device time in ms, out[3] = 1 when it was
  * a symmetric kernel, 2 when that symmetric kernel was a modelled tail's
- * straight-run form (learned tail or residual table of a finite window with
- * near range n0 = 4 and every h_i + h_j below L / 2; same values as the tiered
- * form). The FP32 direct forms of an S1xR2 context whose rows are
+ * straight-run form (learned tail or residual table of a finite window of
+ * n_cut >= 24 with near range n0 = 4 and every h_i + h_j below L / 2; same values
+ * as the tiered form). The FP32 direct forms of an S1xR2 context whose rows are
  * not shared with other ranks evaluate each unordered pair of particles once
  * and add it to both (Newton's third law; the window of eq. ForceCylindrical is
  * symmetric in i and j), so out[1] is n (n - 1) / 2 plus the pairs inside each
@@ -512,7 +514,8 @@ int steps_cyl_tree_set_radial(steps_cyl_ctx* ctx, const double* table, int32_t n
  * infinite window (no plain image sum exists). */
 int steps_cyl_check_tail(steps_cyl_ctx* ctx, int32_t tail, int32_t check_particles, double* report);
 
-/* Compare the surrogate form with the plain image sum now on check_particles
+/* Compare the surrogate form with the plain image sum (in every check: each image
+ * one by one, whatever n_cut) now on check_particles
  * particles (deterministic sample): report (4 doubles) = median and 99.9th
  * percentile of the relative total-force error, and the two forms' pair-kernel
  * times in ms on that sample. */

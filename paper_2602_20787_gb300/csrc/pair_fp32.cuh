@@ -1,6 +1,9 @@
-// FP32 pair kernel of the S1xR2 direct force (arXiv 2602.20787, eqs.
+// FP32 pair arithmetic of the S1xR2 direct force (arXiv 2602.20787, eqs.
 // Force_spline_kernel and ForceCylindrical; pair term of eq.
-// ComovingEquationsOfMotionCylindrical).
+// ComovingEquationsOfMotionCylindrical), one pair at a time. The force kernels take two
+// pairs per thread (pair2.cuh); what is here are their primitives, the image-by-image
+// walk of the acceptance checks and the near images of the row kernels of the modelled
+// tails.
 //
 // Layout. Positions are pre-divided by L and split into FP32 hi/lo words, so a
 // pair separation keeps ~48 bits: d = (hi_i - hi_j) + (lo_i - lo_j). The period
@@ -12,15 +15,13 @@
 // |dz + k| < Ncut: k in [-(Ncut-1), Ncut-1] plus one edge image at
 // dz - sign(dz) Ncut when dz != 0, i.e. 2 Ncut images (2 Ncut - 1 at dz = 0).
 //
-// Inner loop. Images are walked outward in symmetric pairs (dz + k, dz - k) held
-// in one 64-bit register and processed with packed FP32x2 instructions
+// Image walk (pair_images_fp32). Images are walked outward in symmetric pairs (dz + k,
+// dz - k) held in one 64-bit register and processed with packed FP32x2 instructions
 // (add/fma/mul .f32x2), so each image costs ~3 issue slots plus one MUFU
 // rsqrt: the loop is bound by the MUFU pipe (16 rsqrt/SM/clk on sm_103).
 // Walking outward keeps the offsets' relative rounding at the ulp level.
 //
-// Softening. With the softening law of these workloads most pairs have
-// dR < h_i + h_j, so the spline of eq. Force_spline_kernel is on the main path.
-// Per j the warp takes the largest number kw of image pairs that any of its
+// Softening. Per j the warp takes the largest number kw of image pairs that any of its
 // lanes may have inside the support (|k| < h + 1/2). Of those, the few that
 // may reach the inner core (u < 1/2) on some lane use a branch-free packed
 // evaluation of all three spline branches; the others lie in the outer shell
@@ -28,18 +29,15 @@
 // remaining images a lean packed Newtonian loop. Each costs one rsqrt per
 // image, and all loop bounds are warp-uniform, so no lane diverges.
 //
-// Per-pair overhead. Everything outside the image loop is issue slots taken
-// from the FP32 pipes the MUFU leaves free, and the MUFU itself takes only the
-// image rsqrts and one rcp: the wrap of dz and the softening bound are
-// integer-valued roundings done with a 2^23 magic constant on the FMA pipe
-// (no F2I/FRND), x and y go through packed FP32x2, and the j-tile is padded to
-// kBJ with massless far particles so the j loop has a constant trip count and
-// no guard. The self pair needs no test: it has dx = dy = 0, a finite spline
+// Per-pair overhead. The wrap of dz and the softening bound are integer-valued
+// roundings done with a 2^23 magic constant on the FMA pipe (no F2I/FRND), and the
+// j-tile is padded to kBJ with massless far particles so the j loop has a constant trip
+// count and no guard. The self pair needs no test: it has dx = dy = 0, a finite spline
 // centre and an image walk symmetric in +-k, so it adds exact zeros.
 //
-// Work split (stream-K). The (i-block, j-tile) units are laid out i-block-major
-// and every CTA takes an equal contiguous range of them, so all SMs get the same
-// work for any N. A CTA writes one partial per i-block it touches into slot
+// Work split (stream-K) of the row kernels. The (i-block, j-tile) units are laid out
+// i-block-major and every CTA takes an equal contiguous range of them, so all SMs get
+// the same work for any N. A CTA writes one partial per i-block it touches into slot
 // (i-block + CTA) of a scratch array; the finalize kernel adds the partials of
 // each i in CTA order, so results are deterministic and bit-reproducible.
 #pragma once
@@ -47,7 +45,7 @@
 
 namespace steps {
 
-constexpr int kBI = 128;  // i per CTA (one per thread)
+constexpr int kBI = 128;  // i per block of rows
 constexpr int kBJ = 128;  // j per shared-memory tile
 
 // Tuning knobs (build-time; the defaults are the measured best on GB300).
@@ -58,13 +56,6 @@ constexpr int kBJ = 128;  // j per shared-memory tile
 #define STEPS_SPLINE_UNROLL 2 // unroll of the spline-capable image loop
 #endif
 constexpr int kSplineUnroll = STEPS_SPLINE_UNROLL;
-#ifndef STEPS_NCUT_FIXED
-#define STEPS_NCUT_FIXED 1    // compile the windows N_cut = 16 and 64 unrolled beside the general one
-#endif
-#ifndef STEPS_PLAIN_MIN_BLOCKS
-#define STEPS_PLAIN_MIN_BLOCKS 8  // resident CTAs per SM the plain kernels are compiled for (registers)
-#endif
-
 typedef unsigned long long u64;
 
 __device__ __forceinline__ u64 pk(float a, float b) {
@@ -341,6 +332,102 @@ __device__ __forceinline__ void pair_images_fp32(float dR2, float dz, float hh, 
   sz = (z0 + z1) + (d0 + d1);
 }
 
+// F/r of one image from its r^2: the scalar form of spline_value_r2 (all three
+// branches, core selected per lane) or, with FULL false, of the outer-shell
+// form spline_outer_value (exactly r^-3 for u >= 1). ih = 1 / hh.
+template <bool FULL>
+__device__ __forceinline__ float spline_scalar(float r2, float ih, float ih3) {
+  const float ri = rsq(fmaxf(r2, 1e-30f));
+  const float rr = r2 * ri;
+  const float n3 = ri * ri * ri;
+  const float v = fmaxf(fmaf(rr, -ih, 1.0f), 0.0f);
+  const float v2 = v * v;
+  const float nr = fmaf(fmaf(v, -10.6666666667f, 25.6f), v, -16.0f);
+  const float outer = n3 * fmaf(v2 * v2, nr, 1.0f);
+  if (!FULL) return outer;
+  const float u = rr * ih;
+  const float inner = fmaf(u * u, fmaf(u, 32.0f, -38.4f), 10.6666666667f) * ih3;
+  return u < 0.5f ? inner : outer;
+}
+
+// Near images |k| <= n0 of a pair for the modelled-tail forms: the centre
+// image k = 0 on its own (no edge image rides along), then the pairs +-k
+// walked outward packed, with the warp-uniform spline tiers of
+// pair_images_fp32.
+template <int N0 = 0>  // N0 > 0: the near range fixed at compile time (n0 is then N0)
+__device__ __forceinline__ void near_images_fp32(float dR2, float dz, float hh, int n0_rt, int kw, float& sr,
+                                                 float& sz) {
+  const int n0 = N0 > 0 ? N0 : n0_rt;
+  const u64 DR2 = pk(dR2, dR2);
+  const u64 STEP = pk(1.0f, -1.0f);
+  u64 O = pk(dz, dz);
+  u64 SR = pk(0.0f, 0.0f), SZ = pk(0.0f, 0.0f);
+  float cr;  // the centre image's F/r
+  const float c2 = fmaf(dz, dz, dR2);
+  int k = 1;
+  if (kw >= 0) {
+    const float ih = rcp_approx(hh);
+    const u64 NIH = pk(-ih, -ih);
+    const bool core = 4.0f * dR2 < hh * hh;
+    if (__any_sync(0xffffffffu, core)) {
+      const int kl = core ? __float_as_int(__fadd_rn(0.5f * hh, kTwo23)) : kTwo23Bits;
+      const int k1 = min(__reduce_max_sync(0xffffffffu, kl) - kTwo23Bits, n0);
+      const float ih3 = ih * ih * ih;
+      const u64 IH = pk(ih, ih), IH3 = pk(ih3, ih3);
+      cr = spline_scalar<true>(c2, ih, ih3);
+      for (; k <= k1; ++k) {
+        O = add2(O, STEP);
+        const u64 F = spline_over_r2(O, DR2, IH, NIH, IH3);
+        SR = add2(SR, F);
+        SZ = fma2(O, F, SZ);
+      }
+    } else {
+      cr = spline_scalar<false>(c2, ih, 0.0f);
+    }
+    const int kg = min(kw, n0);
+    for (; k <= kg; ++k) {
+      O = add2(O, STEP);
+      const u64 F = spline_outer_over_r2(O, DR2, NIH);
+      SR = add2(SR, F);
+      SZ = fma2(O, F, SZ);
+    }
+  } else {
+    const float ri = rsq(c2);
+    cr = ri * ri * ri;
+  }
+  // Newtonian pairs k .. n0: the first (count mod 4) enter a straight run
+  // part-way, the rest go in fours
+  const int cnt = n0 + 1 - k;
+  if (N0 > 0 && k == 1) {  // no softened pair: the whole fixed range, unrolled
+#pragma unroll
+    for (int q = 0; q < N0; ++q) newton_pair(O, STEP, DR2, SR, SZ);
+    float s0, s1, z0, z1;
+    upk(SR, s0, s1);
+    upk(SZ, z0, z1);
+    sr = (s0 + s1) + cr;
+    sz = (z0 + z1) + dz * cr;
+    return;
+  }
+  switch (cnt & 3) {
+    case 3: newton_pair(O, STEP, DR2, SR, SZ);  // fall through
+    case 2: newton_pair(O, STEP, DR2, SR, SZ);  // fall through
+    case 1: newton_pair(O, STEP, DR2, SR, SZ);  // fall through
+    default: break;
+  }
+#pragma unroll 1
+  for (int q = cnt >> 2; q > 0; --q) {
+    newton_pair(O, STEP, DR2, SR, SZ);
+    newton_pair(O, STEP, DR2, SR, SZ);
+    newton_pair(O, STEP, DR2, SR, SZ);
+    newton_pair(O, STEP, DR2, SR, SZ);
+  }
+  float s0, s1, z0, z1;
+  upk(SR, s0, s1);
+  upk(SZ, z0, z1);
+  sr = (s0 + s1) + cr;
+  sz = (z0 + z1) + dz * cr;
+}
+
 template <bool KAHAN>
 __device__ __forceinline__ void acc(float& s, float& c, float v) {
   if (KAHAN) {
@@ -350,80 +437,6 @@ __device__ __forceinline__ void acc(float& s, float& c, float v) {
     s = t;
   } else {
     s += v;
-  }
-}
-
-#ifndef STEPS_J_UNROLL
-#define STEPS_J_UNROLL 2      // unroll of the j loop inside a Kahan group
-#endif
-constexpr int kJUnroll = STEPS_J_UNROLL;
-static_assert(kBJ % STEPS_KAHAN_GROUP == 0, "a j-tile holds whole Kahan groups");
-
-// All pairs of i with the kBJ j of a (padded) shared-memory tile: pair forces
-// are summed plainly over groups of STEPS_KAHAN_GROUP j, and each group sum
-// enters the compensated per-i sum.
-template <bool KAHAN>
-__device__ __forceinline__ void pair_tile_fp32(const IParticle& I, const float4* sA, const float4* sB, int n_cut,
-                                               float fnc, float& sx, float& sy, float& sz, float& cx, float& cy,
-                                               float& cz) {
-#pragma unroll 1
-  for (int k0 = 0; k0 < kBJ; k0 += STEPS_KAHAN_GROUP) {
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll(kJUnroll)
-    for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; ++k) {
-      const float4 A = sA[k];
-      const float4 B = sB[k];
-      float dx, dy, dz, dR2, hh;
-      int kw;
-      pair_geometry(I, A, B, dx, dy, dz, dR2, hh, kw);
-      float sr, szz;
-      pair_images_fp32(dR2, dz, hh, n_cut, fnc, kw, sr, szz);
-      const float msr = A.w * sr;
-      gx = fmaf(dx, msr, gx);
-      gy = fmaf(dy, msr, gy);
-      gz = fmaf(A.w, szz, gz);
-    }
-    acc<KAHAN>(sx, cx, gx);
-    acc<KAHAN>(sy, cy, gy);
-    acc<KAHAN>(sz, cz, gz);
-  }
-}
-
-// part layout: [slot][3][kBI] doubles, slot = i-block + CTA. The units cover
-// the i-blocks [b0, b0 + U / NT) (all of them unless the rows are sharded), and
-// slots count i-blocks from b0.
-template <bool KAHAN>
-__global__ void __launch_bounds__(kBI, 8)
-pair_fp32_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut,
-                 long long U, int NT, int C, double* __restrict__ part, int b0 = 0) {
-  __shared__ float4 sA[kBJ];
-  __shared__ float4 sB[kBJ];
-  const int c = blockIdx.x;
-  const long long u0 = (long long)c * U / C;
-  const long long u1 = (long long)(c + 1) * U / C;
-  const float fnc = (float)n_cut;
-  long long u = u0;
-  while (u < u1) {
-    const int lb = (int)(u / NT);  // i-block of the evaluated range [b0, b0 + U / NT)
-    const int b = b0 + lb;
-    const int t0 = (int)(u % NT);
-    const long long rem = u1 - u;
-    const int t1 = (int)min((long long)NT, (long long)t0 + rem);
-    const int i = b * kBI + threadIdx.x;
-    const IParticle I = load_i(jA, jB, min(i, n - 1));
-    float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
-    for (int t = t0; t < t1; ++t) {
-      __syncthreads();
-      load_tile(jA, jB, n, t, sA, sB);
-      __syncthreads();
-      pair_tile_fp32<KAHAN>(I, sA, sB, n_cut, fnc, sx, sy, sz, cx, cy, cz);
-    }
-    const long long slot = (long long)lb + c;
-    double* dst = part + slot * 3 * kBI;
-    dst[threadIdx.x] = (double)sx + (double)cx * (KAHAN ? -1.0 : 0.0);
-    dst[kBI + threadIdx.x] = (double)sy + (double)cy * (KAHAN ? -1.0 : 0.0);
-    dst[2 * kBI + threadIdx.x] = (double)sz + (double)cz * (KAHAN ? -1.0 : 0.0);
-    u += t1 - t0;
   }
 }
 

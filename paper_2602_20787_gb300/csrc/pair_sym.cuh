@@ -8,21 +8,20 @@
 // where S is the sum that the FP32 pair kernels produce per particle (scaled by
 // -G / L^2 in the finalize step).
 //
-// Work split. The (i-block b, j-tile t) units with t >= b (the upper triangle of
-// the block grid, NB (NB + 1) / 2 units) are laid out b-major, and every CTA
-// takes an equal contiguous range, as in the stream-K split of pair_fp32.cuh.
-// A diagonal unit (t == b) evaluates all ordered pairs of its block for the i
-// side only (the self pair adds exact zeros); an off-diagonal unit evaluates
-// its 128 x 128 pairs once and adds each to both sides.
+// Work split. The (i-block b, j-tile t) units of the upper triangle of the block
+// grid are laid out b-major, and every CTA takes an equal contiguous range, as in the
+// stream-K split of the row kernels. A block is 128 rows, two per thread (pair2.cuh),
+// so a CTA is two warps. A tile is a block's 128 rows, or a quarter of them when there
+// are too few blocks to fill the GPU: at N = 2,048 the 136 whole units leave most SMs one
+// CTA (134 us), the 544 quarter units take 55 us. A unit of the diagonal block evaluates
+// all ordered pairs for the i side only (the self pair adds exact zeros); the others
+// evaluate their pairs once and add each to both sides.
 //
-// The j side. In each group of 32 j-slots of a tile, lane l pairs its i with
+// The j side. In each group of 32 j-slots of a tile, lane l pairs its two i with
 // slot (l + s) mod 32 at step s, so every slot meets every lane once in 32
 // steps. A lane keeps the running sum of m_i v for the slot it holds and passes
-// it to lane l - 1 after each step (JRing: one shuffle per component and step);
-// after the group lane l holds the warp's whole sum of slot (l + 31) mod 32 and
-// writes it to the warp's row of a shared array. (STEPS_SYM_RING = 0 keeps all
-// lanes on one slot and reduces each slot over the warp with shuffles instead.)
-// After the tile, thread q adds the four warps' sums of j-slot q in warp order.
+// it to lane l - 1 after each step (JRing: one shuffle per component and step).
+// After the tile, thread q adds the two warps' sums of j-slot q.
 //
 // Accumulation. The i-side sum of a CTA's range (FP32, Kahan-compensated as in
 // the row kernels) and the j-side sum of a unit are converted to 64-bit fixed
@@ -35,7 +34,7 @@
 #pragma once
 #include <cstdint>
 
-#include "pair_fp32.cuh"
+#include "pair2.cuh"
 #include "surrogate_pair.cuh"
 #include "tail_table.cuh"
 
@@ -69,6 +68,24 @@ __device__ __forceinline__ long long checked_index(long long v, long long size) 
   return v;
 }
 constexpr int kJRow = 3 * kBJ;    // floats of one warp's j-side row: [kBJ][3]
+constexpr int kSymThreads = kPairThreads;
+
+// Resident CTAs (of two warps) per SM the kernels are compiled for, i.e. their
+// registers. Measured at N = 65,536, N_cut = 64 (1:8 / literal law): plain 9.62 / 16.4 ms at
+// 8, 9.67 / 15.9 at 10, 9.76 / 15.9 at 12, so the straight run takes 8 and the tiered form
+// 10; table 11.7 / 17.6, 11.8 / 17.5, 11.4 / 17.5; network 23.3 / 30.7 at 6, 23.4 / 29.6 at 7 and 8.
+#ifndef STEPS_SYM_FAR_MIN_BLOCKS
+#define STEPS_SYM_FAR_MIN_BLOCKS 8
+#endif
+#ifndef STEPS_SYM_MIN_BLOCKS
+#define STEPS_SYM_MIN_BLOCKS 10
+#endif
+#ifndef STEPS_SYM_SURR_MIN_BLOCKS
+#define STEPS_SYM_SURR_MIN_BLOCKS 7
+#endif
+#ifndef STEPS_SYM_TABLE_MIN_BLOCKS
+#define STEPS_SYM_TABLE_MIN_BLOCKS 12
+#endif
 
 // Fixed-point accumulators (two's complement in unsigned words, unit
 // 1 / scale) and the error word. Unsharded (world == 0): acc[3][n]. When the
@@ -117,425 +134,337 @@ __device__ __forceinline__ int tri_row(long long u, int NB) {
   return b;
 }
 
-// Warp sums of the j-side vectors of two j (w0 for j-slot k, w1 for k + 1)
-// into the warp's shared row (lanes 0 and 16 write).
-__device__ __forceinline__ void jside_pair(const float (&w0)[3], const float (&w1)[3], float* row, int k) {
-  const int lane = threadIdx.x & 31;
-  const bool hi = (lane & 16) != 0;
-  float r[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const float send = hi ? w0[c] : w1[c];
-    float keep = hi ? w1[c] : w0[c];
-    keep += __shfl_xor_sync(0xffffffffu, send, 16);
-    keep += __shfl_xor_sync(0xffffffffu, keep, 8);
-    keep += __shfl_xor_sync(0xffffffffu, keep, 4);
-    keep += __shfl_xor_sync(0xffffffffu, keep, 2);
-    keep += __shfl_xor_sync(0xffffffffu, keep, 1);
-    r[c] = keep;
-  }
-  if ((lane & 15) == 0) {
-    float* d = row + 3 * checked_index(k + (hi ? 1 : 0), kBJ);
-    d[0] = r[0];
-    d[1] = r[1];
-    d[2] = r[2];
-  }
-}
-
-// The j-side vector m_i v of one pair.
-__device__ __forceinline__ void jside_vec(float mi, float dx, float dy, float sr, float sz, float (&w)[3]) {
-  const float misr = mi * sr;
-  w[0] = dx * misr;
-  w[1] = dy * misr;
-  w[2] = mi * sz;
-}
-
-#ifndef STEPS_SYM_RING
-#define STEPS_SYM_RING 1  // 1: the j side is carried around the warp (JRing); 0: reduced per two j (jside_pair)
-#endif
-
-// The j-slot that this lane pairs with at step k of a tile. With the ring, in
-// each group of 32 slots lane l takes slot (l + k) mod 32 at step k, so every
-// slot meets every lane once in 32 steps; otherwise all lanes take slot k.
+// The j-slot that this lane pairs with at step k of a tile: in each group of 32
+// slots lane l takes slot (l + k) mod 32, so every slot meets every lane once.
 __device__ __forceinline__ int jslot(int k) {
-#if STEPS_SYM_RING
   return (int)checked_index((k & ~31) | ((k + (int)threadIdx.x) & 31), kBJ);
-#else
-  return (int)checked_index(k, kBJ);
-#endif
 }
 
-// The j side carried around the warp: a lane keeps the running sum of the slot
-// it holds, adds its pair's vector, and takes over the sum of lane l + 1 (the
-// slot it holds at the next step). After the last step of a group no shift is
-// made: lane l then holds the whole warp's sum of slot (l + 31) mod 32, one
-// shuffle per component and step instead of a 32-lane reduction per slot.
+// The j side carried around the warp: a lane keeps the running sum of the slot it
+// holds, adds both its pairs' vectors, and takes over the sum of lane l + 1 (the
+// slot it holds at the next step): one shuffle per component and step for 64 pairs.
+// After each group of STEPS_KAHAN_GROUP steps the sums (of 2 x 8 terms) are added
+// to the slots' sums in the warp's shared row, so that no FP32 running sum is
+// longer than those groups.
 struct JRing {
   float a[3] = {0.f, 0.f, 0.f};
-  __device__ __forceinline__ void take(const float (&w)[3], bool shift) {
+  // a += m_i v of both pairs: X = m_i sr (packed), Z = m_i sz
+  __device__ __forceinline__ void take(u64 DX, u64 DY, u64 X, u64 Z, bool shift) {
+    float x0, x1, d0, d1, z0, z1;
+    upk(X, x0, x1);
+    upk(DX, d0, d1);
+    a[0] = fmaf(d1, x1, fmaf(d0, x0, a[0]));
+    upk(DY, d0, d1);
+    a[1] = fmaf(d1, x1, fmaf(d0, x0, a[1]));
+    upk(Z, z0, z1);
+    a[2] += z0 + z1;
+    if (shift) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      a[c] += w[c];
-      if (shift) a[c] = __shfl_sync(0xffffffffu, a[c], (threadIdx.x + 1) & 31);
+      for (int c = 0; c < 3; ++c) a[c] = __shfl_sync(0xffffffffu, a[c], (threadIdx.x + 1) & 31);
     }
   }
-  // k: the group's last step
-  __device__ __forceinline__ void flush(float* row, int k) {
+  // k: the group's last step; first: the first group of its 32 slots
+  __device__ __forceinline__ void flush(float* row, int k, bool first) {
     float* d = row + 3 * jslot(k);
+    __syncwarp();  // the slots' last sums were written by other lanes
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      d[c] = a[c];
+      d[c] = first ? a[c] : d[c] + a[c];
       a[c] = 0.f;
     }
   }
 };
+static_assert(32 % STEPS_KAHAN_GROUP == 0, "a round of 32 slots holds whole groups");
 
-// The j side of the two steps k, k + 1 (k even) into the warp's row.
-__device__ __forceinline__ void jside_two(JRing& ring, const float (&w0)[3], const float (&w1)[3], float* row,
-                                          int k) {
-#if STEPS_SYM_RING
-  const bool last = ((k + 2) & 31) == 0;
-  ring.take(w0, true);
-  ring.take(w1, !last);
-  if (last) ring.flush(row, k + 1);
-#else
-  (void)ring;
-  jside_pair(w0, w1, row, k);
-#endif
+// ---- pair forms ------------------------------------------------------------------
+// A form gives the image sums (SR, SZ) of a thread's two pairs.
+
+// The plain window (pair2.cuh).
+template <bool LINE, bool FAR>
+struct PlainForm {
+  int n_cut;
+  float fnc;
+  __device__ __forceinline__ void operator()(const Sep2& P, u64& SR, u64& SZ) const {
+    window2<LINE, FAR>(P, n_cut, fnc, SR, SZ);
+  }
+};
+
+// How the modelled tails' near images and base are taken:
+//   kModelWide4, kModelInf4: n0 = 4 in closed form (line_far2), the window's far ends
+//     expanded about n_cut (n_cut >= kWideNcut) or at infinity;
+//   kModelExact, kModelInf: any n0, near images walked, the base of tail_base_fp32
+//     side by side with each far end on its own, or at infinity.
+enum Model { kModelWide4, kModelInf4, kModelExact, kModelInf };
+// From this n_cut on the expansion's error in the base is below 2e-9 (its first
+// dropped term is 60 / n_cut^6 times at most 0.0052).
+constexpr int kWideNcut = 24;
+__host__ __device__ constexpr bool model_inf(int m) { return m == kModelInf4 || m == kModelInf; }
+__host__ __device__ constexpr bool model_poly(int m) { return m == kModelWide4 || m == kModelInf4; }
+
+// One side of the base of tail_base_fp32, x = LO: the sums with the first
+// Euler-Maclaurin term of the near end. The integral of f ends at the far end with
+// s, e = SE, EE there and NUM the difference of the squared ends (INF: at infinity).
+template <bool INF>
+__device__ __forceinline__ void base_side2(u64 LO, u64 DR2, u64 SE, u64 EE, u64 NUM, u64& R, u64& Z) {
+  const u64 IL = rsq2(fma2(LO, LO, DR2));
+  const u64 E = mul2(IL, IL), S = mul2(LO, IL);
+  u64 I = mul2(E, rcp2(add2(S, SE)));
+  if (!INF) I = mul2(I, mul2(EE, NUM));
+  R = fma2(mul2(mul2(E, E), S), dup(-0.125f), I);
+  Z = fma2(mul2(IL, E), fma2(mul2(S, S), dup(-0.125f), dup(1.0f / 24.0f)), IL);
 }
 
-// ---- tile functions: all pairs of one i with the kBJ j of a shared tile -------
-// They add m_j v to the i-side Kahan sums and, when sym is set (an
-// off-diagonal unit), write the warp's j-side sums of every j-slot to row.
+// The base for any n0 and each far end on its own, added to (SR, SZ).
+template <bool INF>
+__device__ __forceinline__ void base2(u64 DR2, u64 ADZ, const SurrConst& S, u64& SR, u64& SZ) {
+  const u64 LA = add2(ADZ, dup(S.A)), LB = sub2(dup(S.A), ADZ);
+  u64 RA, ZA, RB, ZB;
+  if (INF) {
+    base_side2<INF>(LA, DR2, dup(1.0f), 0, 0, RA, ZA);
+    base_side2<INF>(LB, DR2, dup(1.0f), 0, 0, RB, ZB);
+  } else {
+    // + side: n_cut - 1/2 + |dz|; - side: n_cut + 1/2 - |dz| when dz != 0 (the edge image belongs to it)
+    const u64 HA = add2(ADZ, dup(S.fnh));
+    const u64 HB = sub2(add2(dup(S.fnh), flag_nonzero2(ADZ)), ADZ);
+    const u64 IA = rsq2(fma2(HA, HA, DR2)), IB = rsq2(fma2(HB, HB, DR2));
+    const u64 EA = mul2(IA, IA), EB = mul2(IB, IB), TA = mul2(HA, IA), TB = mul2(HB, IB);
+    base_side2<INF>(LA, DR2, TA, EA, mul2(sub2(HA, LA), add2(HA, LA)), RA, ZA);
+    base_side2<INF>(LB, DR2, TB, EB, mul2(sub2(HB, LB), add2(HB, LB)), RB, ZB);
+    SR = fma2(add2(mul2(mul2(EA, EA), TA), mul2(mul2(EB, EB), TB)), dup(0.125f), SR);
+    const u64 FA = fma2(mul2(IA, EA), fma2(mul2(TA, TA), dup(-0.125f), dup(1.0f / 24.0f)), IA);
+    const u64 FB = fma2(mul2(IB, EB), fma2(mul2(TB, TB), dup(-0.125f), dup(1.0f / 24.0f)), IB);
+    SZ = add2(SZ, sub2(FB, FA));
+  }
+  SR = add2(SR, add2(RA, RB));
+  SZ = add2(SZ, sub2(ZA, ZB));
+}
 
-#ifndef STEPS_PLAIN_JUNROLL
-#define STEPS_PLAIN_JUNROLL 1  // unroll of the two-j steps of a Kahan group (plain image sum)
-#endif
-constexpr int kPlainJUnroll = STEPS_PLAIN_JUNROLL;
+// State of a modelled tail's pair across the network or the table read: the image
+// sums are a0 + b0 y0 and a1 + b1 y1 in the model's outputs; u: its inputs.
+struct Model2 {
+  u64 a0, b0, a1, b1;
+  u64 u[3];
+};
 
-// Plain image sum (pair_fp32.cuh), two j per step.
-template <bool KAHAN>
-__device__ __forceinline__ void sym_tile_plain(const IParticle& I, float mi, const float4* sA, const float4* sB,
-                                               bool sym, float* row, int n_cut, float fnc, float& sx, float& sy,
-                                               float& sz, float& cx, float& cy, float& cz) {
-  JRing ring;
-#pragma unroll 1
-  for (int k0 = 0; k0 < kBJ; k0 += STEPS_KAHAN_GROUP) {
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll(kPlainJUnroll)
-    for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; k += 2) {
-      float w[2][3];
-#pragma unroll
-      for (int jj = 0; jj < 2; ++jj) {
-        const int q = jslot(k + jj);
-        const float4 A = sA[q];
-        const float4 B = sB[q];
-        float dx, dy, dz, dR2, hh;
-        int kw;
-        pair_geometry(I, A, B, dx, dy, dz, dR2, hh, kw);
-        float sr, szz;
-#if STEPS_NCUT_FIXED
-        if (n_cut == 16)
-          pair_images_fp32<true, 16>(dR2, dz, hh, 16, fnc, kw, sr, szz);
-        else if (n_cut == 64)
-          pair_images_fp32<true, 64>(dR2, dz, hh, 64, fnc, kw, sr, szz);
-        else
-#endif
-          pair_images_fp32(dR2, dz, hh, n_cut, fnc, kw, sr, szz);
-        const float msr = A.w * sr;
-        gx = fmaf(dx, msr, gx);
-        gy = fmaf(dy, msr, gy);
-        gz = fmaf(A.w, szz, gz);
-        jside_vec(mi, dx, dy, sr, szz, w[jj]);
-      }
-      if (sym) jside_two(ring, w[0], w[1], row, k);
+// Near images, base, envelope and inputs of a modelled tail (see surr_stage_a), with
+// the exact spline in place of softened images of the tail. RAW: no base and unit
+// envelope (the nearest-image table).
+template <int MODEL, bool RAW, bool FAR>
+__device__ __forceinline__ void model_stage2(const Sep2& P, u64 ADZ, int n_cut, const SurrConst& S, Model2& M) {
+  constexpr bool POLY = model_poly(MODEL), INF = model_inf(MODEL);
+  static_assert(!FAR || POLY, "the straight run belongs to the closed near part");
+  const u64 dR = mul2(P.dr2, rsq2(max2(P.dr2, 1e-30f)));
+  M.u[0] = fma2(min2(dR, S.dR_max), dup(S.two_inv_dR_max), dup(-1.0f));
+  M.u[1] = fma2(ADZ, dup(4.0f), dup(-1.0f));
+  M.u[2] = fma2(min2(P.hh, S.A), dup(S.two_over_A), dup(-1.0f));
+  const int m = POLY ? kPolyNear : S.n0;
+  const u64 R2C = fma2(ADZ, ADZ, P.dr2);
+  u64 CR, SR, SZ;
+  const u64 H2 = mul2(P.hh, P.hh);
+  const bool soft = any_less2(R2C, H2);
+  if (FAR || (POLY && !soft)) near_far2<kPolyNear>(R2C, P.dr2, ADZ, CR, SR, SZ);
+  if (soft) {
+    const Soft2 s = soft2(P.hh);
+    if (FAR) {
+      CR = spline2<true, true>(R2C, s);
+    } else {
+      const int kw = soft_bound2(H2, P.dr2, ADZ), k1 = soft_bound2(mul2(H2, dup(0.25f)), P.dr2, ADZ);
+      CR = spline_centre2(R2C, H2, s);
+      if (POLY)
+        near_soft2<kPolyNear>(P.dr2, s, ADZ, kw, k1, SR, SZ);
+      else
+        near_soft_walk2(P.dr2, s, ADZ, m, kw, k1, SR, SZ);
+      if (kw > m) far_soft2(P.dr2, s, ADZ, m, kw, INF ? 0 : n_cut, SR, SZ);
     }
-    acc<KAHAN>(sx, cx, gx);
-    acc<KAHAN>(sy, cy, gy);
-    acc<KAHAN>(sz, cz, gz);
+  } else if (!POLY) {
+    near_newton2(R2C, P.dr2, ADZ, m, CR, SR, SZ);
   }
+  SR = add2(SR, CR);
+  SZ = fma2(ADZ, CR, SZ);
+  if (RAW) {
+    M.a0 = SR;
+    M.a1 = SZ;
+    M.b0 = M.b1 = dup(1.0f);
+    return;
+  }
+  if (POLY)
+    line_far2<INF, true>(P.dr2, ADZ, (float)n_cut, SR, SZ);
+  else
+    base2<INF>(P.dr2, ADZ, S, SR, SZ);
+  const u64 LA = add2(ADZ, dup(S.A));
+  const u64 IL = rsq2(fma2(LA, LA, P.dr2));
+  const u64 E = mul2(IL, IL), E2 = mul2(E, E);
+  const u64 ER = mul2(E2, E), EZ = mul2(E2, IL);
+  M.a0 = fma2(ER, dup(S.mu0), SR);
+  M.b0 = mul2(ER, dup(S.sc0));
+  M.a1 = fma2(EZ, dup(S.mu1), SZ);
+  M.b1 = mul2(EZ, dup(S.sc1));
 }
 
-// One network call of the learned tail for the NJ steps k .. k + NJ - 1 (slots
-// jslot(k + jj)): the i-side group sums and the j-side vectors w. FAR4 (near
-// range n0 = 4): stage A of every pair is first taken as if no lane's pair were
-// inside its softening support (surr_stage_a_far4, no branch), so that the
-// geometry, stage A and the network form one straight run in which the
-// scheduler interleaves the tensor-core chain with the FP32 and MUFU work. A
-// step where some lane's pair is inside its support (kw >= 0, warp-uniform)
-// redoes stage A of that pair with the spline tiers after the network, from
-// the same separation, which gives the tiered call's values bit for bit.
-template <int NJ, bool INF, bool FAR4>
-__device__ __forceinline__ void surr_call(const IParticle& I, float mi, const float4* sA, const float4* sB, int k,
-                                          int self, int n_cut, const SurrW& W, uint32_t* ibuf, const SurrConst& S,
-                                          float& gx, float& gy, float& gz, float (*w)[3]) {
-  float dx[NJ], dy[NJ], mj[NJ];
-  int kw[NJ];
-  SurrPair P[NJ];
-  float u[NJ][3], y[NJ][2];
-  int q[NJ];
-#pragma unroll
-  for (int jj = 0; jj < NJ; ++jj) {
-    q[jj] = jslot(k + jj);
-    const float4 A = sA[q[jj]];
-    const float4 B = sB[q[jj]];
-    float dz, dR2, hh;
-    pair_geometry(I, A, B, dx[jj], dy[jj], dz, dR2, hh, kw[jj]);
-    mj[jj] = (q[jj] == self) ? 0.0f : A.w;
-    if (FAR4)
-      surr_stage_a_far4<INF>(dR2, dz, hh, S, P[jj]);
-    else
-      surr_stage_a<INF>(dR2, dz, hh, n_cut, kw[jj], S, P[jj]);
-    u[jj][0] = P[jj].u[0];
-    u[jj][1] = P[jj].u[1];
-    u[jj][2] = P[jj].u[2];
-  }
-  mlp_warp<NJ>(W, ibuf, u, y);
-  if (FAR4) {
-#pragma unroll
-    for (int jj = 0; jj < NJ; ++jj) {
-      if (kw[jj] >= 0) {
-        float ddx, ddy, dz, dR2, hh;
-        pair_separation(I, sA[q[jj]], sB[q[jj]], ddx, ddy, dz, dR2, hh);
-        surr_stage_a<INF>(dR2, dz, hh, n_cut, kw[jj], S, P[jj]);
-      }
-    }
-  }
-#pragma unroll
-  for (int jj = 0; jj < NJ; ++jj) {
-    float sr, szz;
-    surr_stage_c<INF>(I, sA[q[jj]], sB[q[jj]], n_cut, kw[jj], S, P[jj], y[jj][0], y[jj][1], sr, szz);
-    const float msr = mj[jj] * sr;
-    gx = fmaf(dx[jj], msr, gx);
-    gy = fmaf(dy[jj], msr, gy);
-    gz = fmaf(mj[jj], szz, gz);
-    jside_vec(mi, dx[jj], dy[jj], sr, szz, w[jj]);
-  }
+// The sums from the model's outputs.
+template <int MODEL, bool RAW>
+__device__ __forceinline__ void model_finish2(const Sep2& P, u64 ADZ, int n_cut, const Model2& M, u64 Y0, u64 Y1,
+                                              u64& SR, u64& SZ) {
+  SR = fma2(M.b0, Y0, M.a0);
+  SZ = fma2(M.b1, Y1, M.a1);
+  fix_dz0<MODEL == kModelWide4 && !RAW>(ADZ, P.dr2, (float)n_cut, SR, SZ);
+  SZ = mulsign2(SZ, P.dz);
 }
 
-#ifndef STEPS_SURR_UNROLL
-#define STEPS_SURR_UNROLL 1  // unroll of the two-j steps of a Kahan group (learned tail)
-#endif
-constexpr int kSurrUnroll = STEPS_SURR_UNROLL;
-
-// Learned tail (surrogate_pair.cuh): STEPS_SURR_NJ j per network call, the
-// j side reduced two j at a time. FAR4: the straight-run calls (near range
-// n0 = 4), which the host takes when every softening support lies within half
-// a period (h_i + h_j < L / 2): only the centre image of a pair can then be
-// softened, and the steps that redo a pair stay rare. Loads with wider
-// supports take the tiered calls throughout.
-template <bool KAHAN, bool INF, bool FAR4>
-__device__ __forceinline__ void sym_tile_surr(const IParticle& I, float mi, const float4* sA, const float4* sB,
-                                              bool sym, float* row, int self, int n_cut, const SurrW& W,
-                                              uint32_t* ibuf, const SurrConst& S, float& sx, float& sy, float& sz,
-                                              float& cx, float& cy, float& cz) {
-  static_assert(STEPS_SURR_NJ == 1 || STEPS_SURR_NJ == 2, "one or two j per network call");
-  JRing ring;
-#pragma unroll 1
-  for (int k0 = 0; k0 < kBJ; k0 += STEPS_KAHAN_GROUP) {
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll(kSurrUnroll)
-    for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; k += 2) {
-      float w[2][3];
-      if (STEPS_SURR_NJ == 2) {
-        surr_call<2, INF, FAR4>(I, mi, sA, sB, k, self, n_cut, W, ibuf, S, gx, gy, gz, w);
-      } else {
-        surr_call<1, INF, FAR4>(I, mi, sA, sB, k, self, n_cut, W, ibuf, S, gx, gy, gz, w);
-        surr_call<1, INF, FAR4>(I, mi, sA, sB, k + 1, self, n_cut, W, ibuf, S, gx, gy, gz, w + 1);
-      }
-      if (sym) jside_two(ring, w[0], w[1], row, k);
-    }
-    acc<KAHAN>(sx, cx, gx);
-    acc<KAHAN>(sy, cy, gy);
-    acc<KAHAN>(sz, cz, gz);
+// Learned tail: one network call for the warp's 64 pairs (mlp_warp's two values of
+// j are here the thread's two i).
+template <int MODEL, bool FAR>
+struct SurrForm {
+  int n_cut;
+  SurrW W;
+  uint32_t* ibuf;
+  const SurrConst& S;
+  __device__ __forceinline__ void operator()(const Sep2& P, u64& SR, u64& SZ) const {
+    const u64 ADZ = abs2(P.dz);
+    Model2 M;
+    model_stage2<MODEL, false, FAR>(P, ADZ, n_cut, S, M);
+    float u[2][3], y[2][2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) upk(M.u[c], u[0][c], u[1][c]);
+    mlp_warp<2>(W, ibuf, u, y);
+    model_finish2<MODEL, false>(P, ADZ, n_cut, M, pk(y[0][0], y[1][0]), pk(y[0][1], y[1][1]), SR, SZ);
   }
-}
+};
 
-// Correction-table tail (tail_table.cuh), two j per step; READ: the table read
-// (the exact reads belong to the nearest-image table, n0 = 0, stored raw).
-// FAR4: as for the learned tail, the straight-run stage A of both pairs and
-// their table reads form one run (the fetches are issued as soon as the inputs
-// exist and return while the near images and the base are computed); a pair
-// whose step is softened is redone with the spline tiers after the reads.
-template <bool KAHAN, bool INF, int READ, bool FAR4>
-__device__ __forceinline__ void sym_tile_table(const IParticle& I, float mi, const float4* sA, const float4* sB,
-                                               bool sym, float* row, int self, int n_cut, const SurrConst& S,
-                                               const TableTail& T, float& sx, float& sy, float& sz, float& cx,
-                                               float& cy, float& cz) {
-  constexpr int RAW = READ >= kReadCicExact ? 1 : 0;
-  static_assert(!(FAR4 && RAW), "the straight run belongs to the residual tables (n0 = 4)");
-  JRing ring;
-#pragma unroll 1
-  for (int k0 = 0; k0 < kBJ; k0 += STEPS_KAHAN_GROUP) {
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll 1
-    for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; k += 2) {
-      float w[2][3];
-      if (FAR4) {
-        int q[2], kw[2];
-        float dx[2], dy[2];
-        SurrPair P[2];
-        float2 r[2];
-#pragma unroll
-        for (int jj = 0; jj < 2; ++jj) {
-          q[jj] = jslot(k + jj);
-          float dz, dR2, hh;
-          pair_geometry(I, sA[q[jj]], sB[q[jj]], dx[jj], dy[jj], dz, dR2, hh, kw[jj]);
-          surr_stage_a_far4<INF>(dR2, dz, hh, S, P[jj]);
-          r[jj] = table_read<READ>(T, P[jj].u[0], P[jj].u[1]);
-        }
-#pragma unroll
-        for (int jj = 0; jj < 2; ++jj) {
-          const float4 A = sA[q[jj]];
-          const float4 B = sB[q[jj]];
-          if (kw[jj] >= 0) {
-            float ddx, ddy, dz, dR2, hh;
-            pair_separation(I, A, B, ddx, ddy, dz, dR2, hh);
-            surr_stage_a<INF>(dR2, dz, hh, n_cut, kw[jj], S, P[jj]);
-          }
-          float sr, szz;
-          surr_stage_c<INF>(I, A, B, n_cut, kw[jj], S, P[jj], r[jj].x, r[jj].y, sr, szz);
-          const float mj = (q[jj] == self) ? 0.0f : A.w;
-          const float msr = mj * sr;
-          gx = fmaf(dx[jj], msr, gx);
-          gy = fmaf(dy[jj], msr, gy);
-          gz = fmaf(mj, szz, gz);
-          jside_vec(mi, dx[jj], dy[jj], sr, szz, w[jj]);
-        }
-      } else {
-#pragma unroll
-        for (int jj = 0; jj < 2; ++jj) {
-          const int q = jslot(k + jj);
-          const float4 A = sA[q];
-          const float4 B = sB[q];
-          float dx, dy, dz, dR2, hh;
-          int kw;
-          pair_geometry(I, A, B, dx, dy, dz, dR2, hh, kw);
-          SurrPair P;
-          surr_stage_a<INF, RAW>(dR2, dz, hh, n_cut, kw, S, P);
-          const float2 r = table_read<READ>(T, P.u[0], P.u[1]);
-          float sr, szz;
-          surr_stage_c<INF>(I, A, B, n_cut, kw, S, P, r.x, r.y, sr, szz);
-          const float mj = (q == self) ? 0.0f : A.w;
-          const float msr = mj * sr;
-          gx = fmaf(dx, msr, gx);
-          gy = fmaf(dy, msr, gy);
-          gz = fmaf(mj, szz, gz);
-          jside_vec(mi, dx, dy, sr, szz, w[jj]);
-        }
-      }
-      if (sym) jside_two(ring, w[0], w[1], row, k);
-    }
-    acc<KAHAN>(sx, cx, gx);
-    acc<KAHAN>(sy, cy, gy);
-    acc<KAHAN>(sz, cz, gz);
+// Correction-table tail (tail_table.cuh); READ: the table read (the exact reads
+// belong to the nearest-image table, n0 = 0, stored raw).
+template <int MODEL, int READ, bool FAR>
+struct TableForm {
+  static constexpr bool RAW = READ >= kReadCicExact;
+  static_assert(!(RAW && model_poly(MODEL)), "the raw tables have no base");
+  int n_cut;
+  const SurrConst& S;
+  const TableTail& Tab;
+  __device__ __forceinline__ void operator()(const Sep2& P, u64& SR, u64& SZ) const {
+    const u64 ADZ = abs2(P.dz);
+    Model2 M;
+    model_stage2<MODEL, RAW, FAR>(P, ADZ, n_cut, S, M);
+    float u0, v0, u1, v1;
+    upk(M.u[0], u0, v0);
+    upk(M.u[1], u1, v1);
+    const float2 r = table_read<READ>(Tab, u0, u1), s = table_read<READ>(Tab, v0, v1);
+    model_finish2<MODEL, RAW>(P, ADZ, n_cut, M, pk(r.x, s.x), pk(r.y, s.y), SR, SZ);
   }
-}
+};
 
 // ---- the stream-K driver over the upper triangle -----------------------------
-// tile(I, mi, sym, self, row, sx .. cz) evaluates one staged tile. sJ: the
-// warps' j-side rows, [kBI / 32][kJRow] floats.
-template <bool KAHAN, class Tile>
+// The tile width is kBJ / tpb: whole blocks (tpb = 1), or quarters (tpb = 4) when
+// there are too few blocks to fill the GPU.
+struct SymShared {
+  JTile2 T;
+  float J[kSymThreads / 32 * kJRow];
+};
+
+template <bool KAHAN, class Form>
 __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, const float4* __restrict__ jB, int n,
-                                             int NB, long long Ua, long long U, int C, float4* sA, float4* sB,
-                                             float* sJ, const FixAcc& F, Tile tile) {
+                                             int NB, int tpb, long long Ua, long long U, int C, SymShared& sh,
+                                             const FixAcc& F, const Form& form) {
   // the units [Ua, Ua + U) (all of them, or a rank's share), split over C CTAs
   const int c = blockIdx.x;
   const long long u0 = Ua + (long long)c * U / C;
   const long long u1 = Ua + (long long)(c + 1) * U / C;
-  float* row = sJ + (threadIdx.x >> 5) * kJRow;
+  const int jt = kBJ / tpb;
+  float* row = sh.J + (threadIdx.x >> 5) * kJRow;
   long long u = u0;
   while (u < u1) {
-    const int b = (int)checked_index(tri_row(u, NB), NB);
-    const int t0 = (int)checked_index(b + (u - tri_off(b, NB)), NB);
-    const int t1 = (int)min((long long)NB, (long long)t0 + (u1 - u));
-    const int i = b * kBI + threadIdx.x;
-    const IParticle I = load_i(jA, jB, min(i, n - 1));
-    const float mi = i < n ? jA[i].w : 0.0f;  // rows past n add nothing to the j side
-    float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
+    const int b = (int)checked_index(tri_row(u / tpb, NB), NB);
+    const int t0 = (int)checked_index(b * tpb + (u - tpb * tri_off(b, NB)), (long long)NB * tpb);
+    const int t1 = (int)min((long long)NB * tpb, (long long)t0 + (u1 - u));
+    const int i0 = row_i0(b), i1 = i0 + 32;
+    const I2 I = load_i2(jA, jB, i0, i1, n);
+    u64 sx = 0, sy = 0, sz = 0, cx = 0, cy = 0, cz = 0;
     for (int t = t0; t < t1; ++t) {
       __syncthreads();
-      load_tile(jA, jB, n, t, sA, sB);
+      load_tile2<kSymThreads>(jA, jB, n, t, jt, sh.T);
       __syncthreads();
-      const bool sym = t != b;
-      tile(I, mi, sA, sB, sym, i - t * kBJ, row, sx, sy, sz, cx, cy, cz);
+      const bool sym = t / tpb != b;
+      JRing ring;
+#pragma unroll 1
+      for (int k0 = 0; k0 < jt; k0 += STEPS_KAHAN_GROUP) {
+        u64 gx = 0, gy = 0, gz = 0;
+#pragma unroll 1
+        for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; ++k) {
+          const int q = jslot(k);
+          Sep2 P;
+          separation2(I, sh.T, q, P);
+          u64 SR, SZ;
+          form(P, SR, SZ);
+          const u64 m = sh.T.MH[q].x;
+          const u64 MS = mul2(m, SR);
+          gx = fma2(P.dx, MS, gx);
+          gy = fma2(P.dy, MS, gy);
+          gz = fma2(m, SZ, gz);
+          if (sym) {
+            ring.take(P.dx, P.dy, mul2(I.m, SR), mul2(I.m, SZ), k + 1 != k0 + STEPS_KAHAN_GROUP);
+          }
+        }
+        if (sym) ring.flush(row, k0 + STEPS_KAHAN_GROUP - 1, (k0 & 31) == 0);
+        acc2<KAHAN>(sx, cx, gx);
+        acc2<KAHAN>(sy, cy, gy);
+        acc2<KAHAN>(sz, cz, gz);
+      }
       if (sym) {
         __syncthreads();  // every warp's row is written
-        const int j = t * kBJ + threadIdx.x;
-        if (j < n) {
-          float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+        for (int s = threadIdx.x; s < jt; s += kSymThreads) {
+          const int j = t * jt + s;
+          if (j < n) {
 #pragma unroll
-          for (int w = 0; w < kBI / 32; ++w) {
-            const float* q = sJ + w * kJRow + 3 * threadIdx.x;
-            s0 += q[0];
-            s1 += q[1];
-            s2 += q[2];
+            for (int q = 0; q < 3; ++q) {
+              double v = 0.0;
+#pragma unroll
+              for (int w = 0; w < kSymThreads / 32; ++w) v += (double)sh.J[w * kJRow + 3 * s + q];
+              fix_add(F, q, j, -v);
+            }
           }
-          fix_add(F, 0, j, -(double)s0);
-          fix_add(F, 1, j, -(double)s1);
-          fix_add(F, 2, j, -(double)s2);
         }
       }
     }
-    if (i < n) {
-      fix_add(F, 0, i, (double)sx - (KAHAN ? (double)cx : 0.0));
-      fix_add(F, 1, i, (double)sy - (KAHAN ? (double)cy : 0.0));
-      fix_add(F, 2, i, (double)sz - (KAHAN ? (double)cz : 0.0));
+    const u64 S[3] = {sx, sy, sz}, K[3] = {cx, cy, cz};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      double s0, s1;
+      sum2<KAHAN>(S[q], K[q], s0, s1);
+      if (i0 < n) fix_add(F, q, i0, s0);
+      if (i1 < n) fix_add(F, q, i1, s1);
     }
     u += t1 - t0;
   }
 }
 
 // ---- kernels ---------------------------------------------------------------
-template <bool KAHAN>
-__global__ void __launch_bounds__(kBI, STEPS_PLAIN_MIN_BLOCKS)
-pair_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, long long Ua,
-                long long U, int C, FixAcc F) {
-  __shared__ float4 sA[kBJ];
-  __shared__ float4 sB[kBJ];
-  __shared__ float sJ[kBI / 32 * kJRow];
-  const float fnc = (float)n_cut;
-  sym_stream_k<KAHAN>(jA, jB, n, NB, Ua, U, C, sA, sB, sJ, F,
-                      [&](const IParticle& I, float mi, const float4* a, const float4* bb, bool sym, int /*self*/,
-                          float* row, float& sx, float& sy, float& sz, float& cx, float& cy, float& cz) {
-                        sym_tile_plain<KAHAN>(I, mi, a, bb, sym, row, n_cut, fnc, sx, sy, sz, cx, cy, cz);
-                      });
+template <bool KAHAN, bool LINE, bool FAR>
+__global__ void __launch_bounds__(kSymThreads, FAR ? STEPS_SYM_FAR_MIN_BLOCKS : STEPS_SYM_MIN_BLOCKS)
+pair_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
+                long long Ua, long long U, int C, FixAcc F) {
+  __shared__ SymShared sh;
+  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, Ua, U, C, sh, F, PlainForm<LINE, FAR>{n_cut, (float)n_cut});
 }
 
-template <bool KAHAN, bool INF, bool FAR4 = false>
-__global__ void __launch_bounds__(kBI, STEPS_SURR_MIN_BLOCKS)
-pair_sym_surr_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB,
+template <bool KAHAN, int MODEL, bool FAR>
+__global__ void __launch_bounds__(kSymThreads, STEPS_SYM_SURR_MIN_BLOCKS)
+pair_sym_surr_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
                      long long Ua, long long U, int C, const SurrLane* __restrict__ wl, SurrConst S, FixAcc F) {
-  __shared__ float4 sA[kBJ];
-  __shared__ float4 sB[kBJ];
-  __shared__ float sJ[kBI / 32 * kJRow];
+  __shared__ SymShared sh;
   __shared__ __align__(16) uint32_t sWT[32 * kSurrStride];
-  __shared__ __align__(16) uint32_t sIn[kBI / 32][STEPS_SURR_NJ * kInWords];
+  __shared__ __align__(16) uint32_t sIn[kSymThreads / 32][2 * kInWords];
   uint32_t* ibuf = sIn[threadIdx.x >> 5];
-  mlp_zero_inputs<STEPS_SURR_NJ>(ibuf);
+  mlp_zero_inputs<2>(ibuf);
   stage_surr_weights(wl, sWT);
-  const SurrW W{sWT + (threadIdx.x & 31) * kSurrStride};
-  sym_stream_k<KAHAN>(jA, jB, n, NB, Ua, U, C, sA, sB, sJ, F,
-                      [&](const IParticle& I, float mi, const float4* a, const float4* bb, bool sym, int self,
-                          float* row, float& sx, float& sy, float& sz, float& cx, float& cy, float& cz) {
-                        sym_tile_surr<KAHAN, INF, FAR4>(I, mi, a, bb, sym, row, self, n_cut, W, ibuf, S, sx, sy,
-                                                        sz, cx, cy, cz);
-                      });
+  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, Ua, U, C, sh, F,
+                      SurrForm<MODEL, FAR>{n_cut, SurrW{sWT + (threadIdx.x & 31) * kSurrStride}, ibuf, S});
 }
 
-template <bool KAHAN, bool INF, int READ, bool FAR4 = false>
-__global__ void __launch_bounds__(kBI, STEPS_TABLE_MIN_BLOCKS)
-pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB,
+template <bool KAHAN, int MODEL, int READ, bool FAR>
+__global__ void __launch_bounds__(kSymThreads, STEPS_SYM_TABLE_MIN_BLOCKS)
+pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
                       long long Ua, long long U, int C, TableTail T, SurrConst S, FixAcc F) {
-  __shared__ float4 sA[kBJ];
-  __shared__ float4 sB[kBJ];
-  __shared__ float sJ[kBI / 32 * kJRow];
-  sym_stream_k<KAHAN>(jA, jB, n, NB, Ua, U, C, sA, sB, sJ, F,
-                      [&](const IParticle& I, float mi, const float4* a, const float4* bb, bool sym, int self,
-                          float* row, float& sx, float& sy, float& sz, float& cx, float& cy, float& cz) {
-                        sym_tile_table<KAHAN, INF, READ, FAR4>(I, mi, a, bb, sym, row, self, n_cut, S, T, sx, sy, sz,
-                                                         cx, cy, cz);
-                      });
+  __shared__ SymShared sh;
+  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, Ua, U, C, sh, F, TableForm<MODEL, READ, FAR>{n_cut, S, T});
 }
 
 }  // namespace steps

@@ -44,6 +44,12 @@ using namespace steps;
 #define STEPS_CTA_MULT 32
 #endif
 
+// The symmetric kernels take quarter tiles (32 j) below this many 128 x 128 units
+// per SM (build-time tuning knob).
+#ifndef STEPS_SYM_SPLIT
+#define STEPS_SYM_SPLIT 64
+#endif
+
 namespace {
 
 thread_local std::string g_last_error;
@@ -255,6 +261,7 @@ struct steps_cyl_ctx {
   double h_max = 0.0;                  // the largest softening (set with fix_scale)
   bool fix_ready = false, fix_ok = false;
   long long Usym = 0;
+  int tpb = 1;                         // j-tiles per block of 128 rows of the symmetric kernels
   int SYC = 0, SYSC = 0, SYTC = 0;     // CTAs of the symmetric plain / surrogate / table kernels
   // row sharding
   bool shard = false;
@@ -1038,95 +1045,94 @@ double sym_pairs(const steps_cyl_ctx* c) {
   return 0.5 * (all - within) + within;
 }
 
-// The symmetric kernel of the form over the units [Ua, Ua + U) into F.
-// The symmetric table kernel in the context's table read (compiled per read, so
-// that the filtered CIC path carries none of the other reads' arithmetic).
+// How the symmetric kernels take a modelled tail's near images and base (pair_sym.cuh).
+Model model_kind(const steps_cyl_ctx* c) {
+  if (is_inf(c)) return c->p.n0 == 4 ? kModelInf4 : kModelInf;
+  return c->p.n0 == 4 && c->p.n_cut >= kWideNcut ? kModelWide4 : kModelExact;
+}
+
 // The straight-run calls of the learned tail and of the residual tables: a
 // finite window, near range n0 = 4, and every softening support within half a
 // period (h_i + h_j < L / 2), so that only the centre image of a pair can be
 // softened. (The infinite window keeps the tiered calls.)
 bool straight_run(const steps_cyl_ctx* c) {
-  return !is_inf(c) && c->p.n0 == 4 && 2.0 * c->h_max < 0.5 * c->p.L;
+  return model_kind(c) == kModelWide4 && 2.0 * c->h_max < 0.5 * c->p.L;
 }
 
-template <bool KAHAN, bool INF>
-void launch_sym_table(steps_cyl_ctx* c, int C, int n, int nc, int NB, long long Ua, long long U, const FixAcc& F) {
-  const TableTail& T = c->tab;
-  const bool far4 = straight_run(c);
-  switch (T.read) {
+using SymTableKernel = void (*)(const float4*, const float4*, int, int, int, int, long long, long long, int, TableTail,
+                                SurrConst, FixAcc);
+template <bool KAHAN, int MODEL>
+SymTableKernel sym_table_kernel(int read, bool far) {
+  constexpr int RAW = model_inf(MODEL) ? kModelInf : kModelExact;
+  constexpr bool FAR = MODEL == kModelWide4;
+  switch (read) {
+    case kReadCicExact: return pair_sym_table_kernel<KAHAN, RAW, kReadCicExact, false>;
+    case kReadTscExact: return pair_sym_table_kernel<KAHAN, RAW, kReadTscExact, false>;
     case kReadTsc:
-      if (far4)
-        pair_sym_table_kernel<KAHAN, INF, kReadTsc, true><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, T,
-                                                                               c->tab_const, F);
-      else
-        pair_sym_table_kernel<KAHAN, INF, kReadTsc><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, T,
-                                                                           c->tab_const, F);
-      break;
-    case kReadCicExact:
-      pair_sym_table_kernel<KAHAN, INF, kReadCicExact><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, T,
-                                                                              c->tab_const, F);
-      break;
-    case kReadTscExact:
-      pair_sym_table_kernel<KAHAN, INF, kReadTscExact><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, T,
-                                                                              c->tab_const, F);
-      break;
+      return far ? pair_sym_table_kernel<KAHAN, MODEL, kReadTsc, FAR>
+                 : pair_sym_table_kernel<KAHAN, MODEL, kReadTsc, false>;
     default:
-      if (far4)
-        pair_sym_table_kernel<KAHAN, INF, kReadCic, true><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, T,
-                                                                               c->tab_const, F);
-      else
-        pair_sym_table_kernel<KAHAN, INF, kReadCic><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, T,
-                                                                           c->tab_const, F);
+      return far ? pair_sym_table_kernel<KAHAN, MODEL, kReadCic, FAR>
+                 : pair_sym_table_kernel<KAHAN, MODEL, kReadCic, false>;
+  }
+}
+template <bool KAHAN>
+SymTableKernel sym_table_kernel(Model model, int read, bool far) {
+  switch (model) {
+    case kModelWide4: return sym_table_kernel<KAHAN, kModelWide4>(read, far);
+    case kModelInf4: return sym_table_kernel<KAHAN, kModelInf4>(read, far);
+    case kModelInf: return sym_table_kernel<KAHAN, kModelInf>(read, far);
+    default: return sym_table_kernel<KAHAN, kModelExact>(read, far);
   }
 }
 
-template <bool FAR4>
-void launch_sym_surr(steps_cyl_ctx* c, int C, int n, int nc, int NB, long long Ua, long long U, const FixAcc& F) {
-  const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
-  const SurrLane* wl = c->surr_lanes;
-  if (is_inf(c) && kahan)
-    pair_sym_surr_kernel<true, true, FAR4><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, 0, NB, Ua, U, C, wl, c->surr, F);
-  else if (is_inf(c))
-    pair_sym_surr_kernel<false, true, FAR4><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, 0, NB, Ua, U, C, wl, c->surr, F);
-  else if (kahan)
-    pair_sym_surr_kernel<true, false, FAR4><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, wl, c->surr, F);
-  else
-    pair_sym_surr_kernel<false, false, FAR4><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, wl, c->surr, F);
+using SymSurrKernel = void (*)(const float4*, const float4*, int, int, int, int, long long, long long, int,
+                               const SurrLane*, SurrConst, FixAcc);
+template <bool KAHAN>
+SymSurrKernel sym_surr_kernel(Model model, bool far) {
+  switch (model) {
+    case kModelWide4:
+      return far ? pair_sym_surr_kernel<KAHAN, kModelWide4, true> : pair_sym_surr_kernel<KAHAN, kModelWide4, false>;
+    case kModelInf4: return pair_sym_surr_kernel<KAHAN, kModelInf4, false>;
+    case kModelInf: return pair_sym_surr_kernel<KAHAN, kModelInf, false>;
+    default: return pair_sym_surr_kernel<KAHAN, kModelExact, false>;
+  }
+}
+
+using SymKernel = void (*)(const float4*, const float4*, int, int, int, int, long long, long long, int, FixAcc);
+template <bool KAHAN>
+SymKernel sym_kernel(bool line, bool far) {
+  return !line ? pair_sym_kernel<KAHAN, false, false>
+         : far ? pair_sym_kernel<KAHAN, true, true>
+               : pair_sym_kernel<KAHAN, true, false>;
 }
 
 int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const FixAcc& F) {
   const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
+  const int nc = c->p.n_cut, n = c->n, NB = c->NB, tpb = c->tpb;
+  const bool straight = straight_run(c);
   c->last_straight = (form == Form::SURROGATE || (form == Form::TABLE && (c->tab.read == kReadCic ||
                                                                           c->tab.read == kReadTsc))) &&
-                     straight_run(c);
-  const int nc = c->p.n_cut, n = c->n, NB = c->NB;
+                     straight;
   auto ctas = [&](int full) {  // the CTA count of the whole triangle, scaled to a share of it
     return (int)std::max<long long>(1, std::min<long long>(U, (long long)full * U / std::max<long long>(c->Usym, 1)));
   };
   if (form == Form::SURROGATE) {
     const int C = ctas(c->SYSC);
-    if (straight_run(c))
-      launch_sym_surr<true>(c, C, n, nc, NB, Ua, U, F);
-    else
-      launch_sym_surr<false>(c, C, n, nc, NB, Ua, U, F);
+    auto k = kahan ? sym_surr_kernel<true>(model_kind(c), straight) : sym_surr_kernel<false>(model_kind(c), straight);
+    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, Ua, U, C, c->surr_lanes, c->surr, F);
     CKLAUNCH("pair_sym_surrogate");
   } else if (form == Form::TABLE) {
     const int C = ctas(c->SYTC);
-    if (is_inf(c) && kahan)
-      launch_sym_table<true, true>(c, C, n, 0, NB, Ua, U, F);
-    else if (is_inf(c))
-      launch_sym_table<false, true>(c, C, n, 0, NB, Ua, U, F);
-    else if (kahan)
-      launch_sym_table<true, false>(c, C, n, nc, NB, Ua, U, F);
-    else
-      launch_sym_table<false, false>(c, C, n, nc, NB, Ua, U, F);
+    auto k = kahan ? sym_table_kernel<true>(model_kind(c), c->tab.read, straight)
+                   : sym_table_kernel<false>(model_kind(c), c->tab.read, straight);
+    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, Ua, U, C, c->tab, c->tab_const, F);
     CKLAUNCH("pair_sym_table");
   } else {
     const int C = ctas(c->SYC);
-    if (kahan)
-      pair_sym_kernel<true><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, F);
-    else
-      pair_sym_kernel<false><<<C, kBI, 0, c->st>>>(c->jA, c->jB, n, nc, NB, Ua, U, C, F);
+    const bool far = 2.0 * c->h_max < 0.5 * c->p.L;
+    auto k = kahan ? sym_kernel<true>(line_form(nc), far) : sym_kernel<false>(line_form(nc), far);
+    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, Ua, U, C, F);
     CKLAUNCH("pair_sym");
   }
   return STEPS_OK;
@@ -1216,14 +1222,12 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
     else
       pair_r3_kernel<false><<<c->C, kBI, 0, c->st>>>(c->jA, c->jB, c->n, c->U, c->NT, c->C, c->part, c->b0);
     CKLAUNCH("pair_fp32_r3");
-  } else if (c->p.precision == STEPS_FP32_KAHAN) {
-    pair_fp32_kernel<true><<<c->C, kBI, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, c->U, c->NT, c->C, c->part,
-                                                    c->b0);
-    CKLAUNCH("pair_fp32_kahan");
   } else {
-    pair_fp32_kernel<false><<<c->C, kBI, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, c->U, c->NT, c->C, c->part,
-                                                     c->b0);
-    CKLAUNCH("pair_fp32_plain");
+    const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
+    auto kernel = line_form(c->p.n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
+                                        : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
+    kernel<<<c->C, kPairThreads, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, c->U, c->NT, c->C, c->part, c->b0);
+    CKLAUNCH("pair_row");
   }
   CK(cudaEventRecord(c->e1, c->st));
   c->timed = true;
@@ -2141,7 +2145,7 @@ int allocate_context(steps_cyl_ctx* c) {
   // stream-K split of the FP32 pair kernel: C CTAs share U units
   int sms = 0, occ = 0;
   CKA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
-  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pair_fp32_kernel<true>, kBI, 0));
+  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pair_r3_kernel<true>, kBI, 0));
   c->NB = (c->n + kBI - 1) / kBI;
   c->NT = (c->n + kBJ - 1) / kBJ;
   c->U = (long long)c->NB * c->NT;
@@ -2154,11 +2158,12 @@ int allocate_context(steps_cyl_ctx* c) {
   c->TCcap = sms * std::max(tocc, 1) * STEPS_CTA_MULT;
   set_rows(c, 0, c->NB);
   // the symmetric kernels share the upper triangle of the block grid
-  c->Usym = (long long)c->NB * (c->NB + 1) / 2;
+  c->tpb = (long long)c->NB * (c->NB + 1) / 2 < STEPS_SYM_SPLIT * (long long)sms ? 4 : 1;
+  c->Usym = (long long)c->NB * (c->NB + 1) / 2 * c->tpb;
   int yocc = 0, ysocc = 0, ytocc = 0;
-  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&yocc, pair_sym_kernel<true>, kBI, 0));
-  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ysocc, pair_sym_surr_kernel<true, false>, kBI, 0));
-  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ytocc, pair_sym_table_kernel<true, false, kReadCic>, kBI, 0));
+  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&yocc, pair_sym_kernel<true, true, false>, kSymThreads, 0));
+  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ysocc, pair_sym_surr_kernel<true, kModelWide4, false>, kSymThreads, 0));
+  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ytocc, pair_sym_table_kernel<true, kModelWide4, kReadCic, false>, kSymThreads, 0));
   c->SYC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(yocc, 1) * STEPS_CTA_MULT);
   c->SYSC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(ysocc, 1) * STEPS_CTA_MULT);
   c->SYTC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(ytocc, 1) * STEPS_CTA_MULT);

@@ -23,6 +23,7 @@
 
 #include "steps_cyl.h"
 #include "nbody_kernels.cuh"
+#include "pair2.cuh"
 
 using namespace steps;
 
@@ -71,7 +72,7 @@ int setup_device(int dev, cudaError_t pending, DeviceScratch** out) {
       return noalloc_cuda_fail(pending, "cudaGetSymbolAddress of the scratch array failed");
     int sms = 0, occ = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pair_fp32_kernel<true>, kBI, 0) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pair_row_kernel<true, true>, kPairThreads, 0) != cudaSuccess)
       return noalloc_cuda_fail(pending, "device query failed");
     d.base = static_cast<unsigned char*>(ptr);
     d.ctas = std::max(1, std::min(kNoallocMaxCtas, sms * std::max(occ, 1)));
@@ -132,10 +133,10 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   // packed positions here, and each stream-K partial slot whole, before the
   // finalize kernel reads it
   pack_kernel<<<(nn + 255) / 256, 256, 0, st>>>(x, y, z, m, h, nn, invL, jA, jB);
-  if (precision == STEPS_FP32_KAHAN)
-    pair_fp32_kernel<true><<<C, kBI, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part);
-  else
-    pair_fp32_kernel<false><<<C, kBI, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part);
+  const bool kahan = precision == STEPS_FP32_KAHAN;
+  auto kernel = line_form(n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
+                                 : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
+  kernel<<<C, kPairThreads, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part, 0);
   BgParams off{};
   off.mode = STEPS_BG_OFF;
   finalize_kernel<<<(nn + 255) / 256, 256, 0, st>>>(part, nn, NT, U, C, -G * invL * invL, off, x, y, z, ax, ay, az,

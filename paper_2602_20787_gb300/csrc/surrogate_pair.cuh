@@ -291,102 +291,6 @@ __device__ __forceinline__ void tail_base_inf_fp32(float R2, float lo_a, float l
   bz = fmaf(t_a, 1.0f / 24.0f, il_a) - fmaf(t_b, 1.0f / 24.0f, il_b);
 }
 
-// F/r of one image from its r^2: the scalar form of spline_value_r2 (all three
-// branches, core selected per lane) or, with FULL false, of the outer-shell
-// form spline_outer_value (exactly r^-3 for u >= 1). ih = 1 / hh.
-template <bool FULL>
-__device__ __forceinline__ float spline_scalar(float r2, float ih, float ih3) {
-  const float ri = rsq(fmaxf(r2, 1e-30f));
-  const float rr = r2 * ri;
-  const float n3 = ri * ri * ri;
-  const float v = fmaxf(fmaf(rr, -ih, 1.0f), 0.0f);
-  const float v2 = v * v;
-  const float nr = fmaf(fmaf(v, -10.6666666667f, 25.6f), v, -16.0f);
-  const float outer = n3 * fmaf(v2 * v2, nr, 1.0f);
-  if (!FULL) return outer;
-  const float u = rr * ih;
-  const float inner = fmaf(u * u, fmaf(u, 32.0f, -38.4f), 10.6666666667f) * ih3;
-  return u < 0.5f ? inner : outer;
-}
-
-// Near images |k| <= n0 of a pair for the modelled-tail forms: the centre
-// image k = 0 on its own (no edge image rides along), then the pairs +-k
-// walked outward packed, with the warp-uniform spline tiers of
-// pair_images_fp32.
-template <int N0 = 0>  // N0 > 0: the near range fixed at compile time (n0 is then N0)
-__device__ __forceinline__ void near_images_fp32(float dR2, float dz, float hh, int n0_rt, int kw, float& sr,
-                                                 float& sz) {
-  const int n0 = N0 > 0 ? N0 : n0_rt;
-  const u64 DR2 = pk(dR2, dR2);
-  const u64 STEP = pk(1.0f, -1.0f);
-  u64 O = pk(dz, dz);
-  u64 SR = pk(0.0f, 0.0f), SZ = pk(0.0f, 0.0f);
-  float cr;  // the centre image's F/r
-  const float c2 = fmaf(dz, dz, dR2);
-  int k = 1;
-  if (kw >= 0) {
-    const float ih = rcp_approx(hh);
-    const u64 NIH = pk(-ih, -ih);
-    const bool core = 4.0f * dR2 < hh * hh;
-    if (__any_sync(0xffffffffu, core)) {
-      const int kl = core ? __float_as_int(__fadd_rn(0.5f * hh, kTwo23)) : kTwo23Bits;
-      const int k1 = min(__reduce_max_sync(0xffffffffu, kl) - kTwo23Bits, n0);
-      const float ih3 = ih * ih * ih;
-      const u64 IH = pk(ih, ih), IH3 = pk(ih3, ih3);
-      cr = spline_scalar<true>(c2, ih, ih3);
-      for (; k <= k1; ++k) {
-        O = add2(O, STEP);
-        const u64 F = spline_over_r2(O, DR2, IH, NIH, IH3);
-        SR = add2(SR, F);
-        SZ = fma2(O, F, SZ);
-      }
-    } else {
-      cr = spline_scalar<false>(c2, ih, 0.0f);
-    }
-    const int kg = min(kw, n0);
-    for (; k <= kg; ++k) {
-      O = add2(O, STEP);
-      const u64 F = spline_outer_over_r2(O, DR2, NIH);
-      SR = add2(SR, F);
-      SZ = fma2(O, F, SZ);
-    }
-  } else {
-    const float ri = rsq(c2);
-    cr = ri * ri * ri;
-  }
-  // Newtonian pairs k .. n0: the first (count mod 4) enter a straight run
-  // part-way, the rest go in fours
-  const int cnt = n0 + 1 - k;
-  if (N0 > 0 && k == 1) {  // no softened pair: the whole fixed range, unrolled
-#pragma unroll
-    for (int q = 0; q < N0; ++q) newton_pair(O, STEP, DR2, SR, SZ);
-    float s0, s1, z0, z1;
-    upk(SR, s0, s1);
-    upk(SZ, z0, z1);
-    sr = (s0 + s1) + cr;
-    sz = (z0 + z1) + dz * cr;
-    return;
-  }
-  switch (cnt & 3) {
-    case 3: newton_pair(O, STEP, DR2, SR, SZ);  // fall through
-    case 2: newton_pair(O, STEP, DR2, SR, SZ);  // fall through
-    case 1: newton_pair(O, STEP, DR2, SR, SZ);  // fall through
-    default: break;
-  }
-#pragma unroll 1
-  for (int q = cnt >> 2; q > 0; --q) {
-    newton_pair(O, STEP, DR2, SR, SZ);
-    newton_pair(O, STEP, DR2, SR, SZ);
-    newton_pair(O, STEP, DR2, SR, SZ);
-    newton_pair(O, STEP, DR2, SR, SZ);
-  }
-  float s0, s1, z0, z1;
-  upk(SR, s0, s1);
-  upk(SZ, z0, z1);
-  sr = (s0 + s1) + cr;
-  sz = (z0 + z1) + dz * cr;
-}
-
 #ifndef STEPS_SURR_N0_FIXED
 #define STEPS_SURR_N0_FIXED 1  // compile the n0 = 4 near range unrolled beside the general one
 #endif
