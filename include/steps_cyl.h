@@ -184,10 +184,10 @@ int steps_cyl_last_timing(steps_cyl_ctx* ctx, double* pair_images, double* pair_
  * a symmetric kernel, 2 when that symmetric kernel was a modelled tail's
  * straight-run form (learned tail or residual table of a finite window of
  * n_cut >= 24 with near range n0 = 4 and every h_i + h_j below L / 2; same values
- * as the tiered form). The FP32 direct forms of an S1xR2 context whose rows are
+ * as the tiered form). The FP32 direct forms of a context whose rows are
  * not shared with other ranks evaluate each unordered pair of particles once
- * and add it to both (Newton's third law; the window of eq. ForceCylindrical is
- * symmetric in i and j), so out[1] is n (n - 1) / 2 plus the pairs inside each
+ * and add it to both (Newton's third law; the window of eq. ForceCylindrical and
+ * the one image of R^3 are symmetric in i and j), so out[1] is n (n - 1) / 2 plus the pairs inside each
  * block of 128 rows, which are taken both ways; the row kernels evaluate
  * (rows) x (n - 1) ordered pairs. The octree reports its interactions in
  * steps_cyl_tree_stats instead. */

@@ -41,6 +41,7 @@
 namespace steps {
 
 constexpr int kErrFixRange = 32;  // a pair sum left the range of the fixed-point accumulators
+constexpr int kMaxFixExpF = 120;  // the largest scale exponent taken as a float
 constexpr int kErrIndex = 64;     // (index-checked builds) an index left its buffer
 
 // Index-checked builds (STEPS_DEBUG_INDEX=1) check every computed index of the
@@ -97,6 +98,7 @@ struct FixAcc {
   unsigned long long* acc;
   int n;
   double scale;
+  float scale_f;  // the scale when it is a normal float, else 0
   int* err;
   int world, base, extra, chunk;
 };
@@ -109,14 +111,34 @@ __device__ __forceinline__ long long fix_index(const FixAcc& F, int c, int i) {
   return ((long long)r * 3 + c) * F.chunk + (i - first);
 }
 
-__device__ __forceinline__ void fix_add(const FixAcc& F, int c, int i, double v) {
-  const double q = v * F.scale;
-  if (!(fabs(q) < 4.0e18)) {  // beyond 2^62 (or not finite): flag it, never wrap
-    atomicOr(F.err, kErrFixRange);
-    return;
+// value * scale as a 64-bit integer; one beyond 2^62 (or not finite) sets the error bit
+// and gives 0, so that nothing ever wraps. The scale is a power of two: where it is a
+// normal float (F.scale_f, else 0) the product is exact in FP32 and the conversion keeps
+// off the FP64 pipe, whose 2 lanes per SM and clock took 10 of the 40 us of an R^3
+// force at N = 5,000 (three or four FP64 operations per sum).
+__device__ __forceinline__ long long fix_value(const FixAcc& F, float v) {
+  if (F.scale_f > 0.0f) {
+    const float q = v * F.scale_f;
+    if (fabsf(q) < 4.0e18f) return __float2ll_rn(q);
+  } else {
+    const double q = (double)v * F.scale;
+    if (fabs(q) < 4.0e18) return __double2ll_rn(q);
   }
+  atomicOr(F.err, kErrFixRange);
+  return 0;
+}
+__device__ __forceinline__ void fix_add(const FixAcc& F, int c, int i, long long q) {
   const long long size = F.world == 0 ? 3LL * F.n : 3LL * F.world * F.chunk;
-  atomicAdd(F.acc + checked_index(fix_index(F, c, i), size), (unsigned long long)__double2ll_rn(q));
+  atomicAdd(F.acc + checked_index(fix_index(F, c, i), size), (unsigned long long)q);
+}
+// The sums of rows i0 and i1 (packed s, compensation k) into component c.
+template <bool KAHAN>
+__device__ __forceinline__ void fix_add_rows(const FixAcc& F, int c, int i0, int i1, u64 s, u64 k) {
+  float s0, s1, k0, k1;
+  upk(s, s0, s1);
+  upk(k, k0, k1);
+  if (i0 < F.n) fix_add(F, c, i0, fix_value(F, s0) - (KAHAN ? fix_value(F, k0) : 0));
+  if (i1 < F.n) fix_add(F, c, i1, fix_value(F, s1) - (KAHAN ? fix_value(F, k1) : 0));
 }
 
 // Offset of row b of the upper triangle (units t = b .. NB - 1 per row).
@@ -149,7 +171,7 @@ __device__ __forceinline__ int jslot(int k) {
 struct JRing {
   float a[3] = {0.f, 0.f, 0.f};
   // a += m_i v of both pairs: X = m_i sr (packed), Z = m_i sz
-  __device__ __forceinline__ void take(u64 DX, u64 DY, u64 X, u64 Z, bool shift) {
+  __device__ __forceinline__ void take(u64 DX, u64 DY, u64 X, u64 Z, bool shift_on) {
     float x0, x1, d0, d1, z0, z1;
     upk(X, x0, x1);
     upk(DX, d0, d1);
@@ -158,10 +180,20 @@ struct JRing {
     a[1] = fmaf(d1, x1, fmaf(d0, x0, a[1]));
     upk(Z, z0, z1);
     a[2] += z0 + z1;
-    if (shift) {
+    if (shift_on) shift();
+  }
+  // a += both halves of V
+  __device__ __forceinline__ void add(const u64 (&V)[3]) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) a[c] = __shfl_sync(0xffffffffu, a[c], (threadIdx.x + 1) & 31);
+    for (int c = 0; c < 3; ++c) {
+      float v0, v1;
+      upk(V[c], v0, v1);
+      a[c] += v0 + v1;
     }
+  }
+  __device__ __forceinline__ void shift() {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[c] = __shfl_sync(0xffffffffu, a[c], (threadIdx.x + 1) & 31);
   }
   // k: the group's last step; first: the first group of its 32 slots
   __device__ __forceinline__ void flush(float* row, int k, bool first) {
@@ -415,10 +447,10 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
           if (j < n) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-              double v = 0.0;
+              long long v = 0;
 #pragma unroll
-              for (int w = 0; w < kSymThreads / 32; ++w) v += (double)sh.J[w * kJRow + 3 * s + q];
-              fix_add(F, q, j, -v);
+              for (int w = 0; w < kSymThreads / 32; ++w) v -= fix_value(F, sh.J[w * kJRow + 3 * s + q]);
+              fix_add(F, q, j, v);
             }
           }
         }
@@ -426,12 +458,7 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
     }
     const u64 S[3] = {sx, sy, sz}, K[3] = {cx, cy, cz};
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      double s0, s1;
-      sum2<KAHAN>(S[q], K[q], s0, s1);
-      if (i0 < n) fix_add(F, q, i0, s0);
-      if (i1 < n) fix_add(F, q, i1, s1);
-    }
+    for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN>(F, q, i0, i1, S[q], K[q]);
     u += t1 - t0;
   }
 }
@@ -465,6 +492,132 @@ pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ 
                       long long Ua, long long U, int C, TableTail T, SurrConst S, FixAcc F) {
   __shared__ SymShared sh;
   sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, Ua, U, C, sh, F, TableForm<MODEL, READ, FAR>{n_cut, S, T});
+}
+
+// ---- R^3 -------------------------------------------------------------------
+// The R^3 pair force (eq. NewtonianForce, one image per pair) is symmetric as well. A
+// pair costs about 26 FP32 operations and one rsqrt, so what is left around it counts:
+// a lane takes four rows (two packed sets), so that the four 128-bit j loads, the
+// ring's three shuffles and the loop serve four pairs, and one warp is a CTA. With two
+// rows per lane the duplicated j words alone would keep the shared-memory pipe busier
+// than the FP32 one. The row kernel (r3_pair.cuh) evaluates every ordered pair in 31 issue
+// slots per 32 pairs: 3.33 ms per force at N = 65,536 against 2.77 here.
+#ifndef STEPS_SYM_R3_MIN_BLOCKS
+#define STEPS_SYM_R3_MIN_BLOCKS 16  // resident CTAs (warps) per SM the kernel is compiled for
+#endif
+#ifndef STEPS_SYM_R3_UNROLL
+#define STEPS_SYM_R3_UNROLL 4
+#endif
+constexpr int kSymR3Unroll = STEPS_SYM_R3_UNROLL;
+
+template <bool KAHAN>
+__global__ void __launch_bounds__(32, STEPS_SYM_R3_MIN_BLOCKS)
+pair_sym_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int NB, int tpb, long long U,
+                   int C, FixAcc F) {
+  constexpr int NS = kBI / 64;  // packed sets of two rows per lane
+  __shared__ JTile2 T;
+  __shared__ float row[kJRow];
+  const int c = blockIdx.x, lane = threadIdx.x;
+  const long long u1 = (long long)(c + 1) * U / C;
+  const int jt = kBJ / tpb;
+  long long u = (long long)c * U / C;
+  while (u < u1) {
+    const int b = (int)checked_index(tri_row(u / tpb, NB), NB);
+    const int t0 = (int)checked_index(b * tpb + (u - tpb * tri_off(b, NB)), (long long)NB * tpb);
+    const int t1 = (int)min((long long)NB * tpb, (long long)t0 + (u1 - u));
+    I2 I[NS];
+    u64 S[NS][3], K[NS][3];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i0 = b * kBI + 64 * s + lane;
+      I[s] = load_i2(jA, jB, i0, i0 + 32, n);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) S[s][q] = K[s][q] = 0;
+    }
+    for (int t = t0; t < t1; ++t) {
+      __syncwarp();
+      load_tile2<32>(jA, jB, n, t, jt, T);
+      __syncwarp();
+      const bool sym = t / tpb != b;
+      JRing ring;
+#pragma unroll 1
+      for (int k0 = 0; k0 < jt; k0 += STEPS_KAHAN_GROUP) {
+        u64 g[NS][3];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) g[s][0] = g[s][1] = g[s][2] = 0;
+#pragma unroll(kSymR3Unroll)
+        for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; ++k) {
+          const int q = jslot(k);
+          const ulonglong2 xy = T.XY[q], xyl = T.XYL[q], z = T.Z[q], mh = T.MH[q];
+          u64 D[NS][3], R2[NS], RI[NS], HH[NS], Fr[NS];
+          bool soft = false;
+#pragma unroll
+          for (int s = 0; s < NS; ++s) {
+            D[s][0] = add2(sub2(I[s].xh, xy.x), sub2(I[s].xl, xyl.x));
+            D[s][1] = add2(sub2(I[s].yh, xy.y), sub2(I[s].yl, xyl.y));
+            D[s][2] = add2(sub2(I[s].zh, z.x), sub2(I[s].zl, z.y));
+            R2[s] = fma2(D[s][0], D[s][0], fma2(D[s][1], D[s][1], mul2(D[s][2], D[s][2])));
+            HH[s] = add2(I[s].h, mh.y);
+            float ra, rb, ha, hb;
+            upk(R2[s], ra, rb);
+            upk(mul2(HH[s], HH[s]), ha, hb);
+            soft = soft || ra < ha || rb < hb;
+            RI[s] = rsq2(max2(R2[s], 1e-30f));
+            Fr[s] = mul2(mul2(RI[s], RI[s]), RI[s]);
+          }
+          if (__any_sync(0xffffffffu, soft)) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+              const Soft2 h = soft2(HH[s]);
+              Fr[s] = spline_value_r2(R2[s], RI[s], Fr[s], h.ih, h.nih, h.ih3);
+            }
+          }
+#pragma unroll
+          for (int s = 0; s < NS; ++s) {
+            const u64 MF = mul2(mh.x, Fr[s]);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) g[s][a] = fma2(D[s][a], MF, g[s][a]);
+          }
+          if (sym) {
+            // the four pairs are added up first: the running sum takes one term per step
+            u64 X[NS], V[3];
+#pragma unroll
+            for (int s = 0; s < NS; ++s) X[s] = mul2(I[s].m, Fr[s]);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              V[a] = mul2(D[0][a], X[0]);
+#pragma unroll
+              for (int s = 1; s < NS; ++s) V[a] = fma2(D[s][a], X[s], V[a]);
+            }
+            ring.add(V);
+            if (k + 1 != k0 + STEPS_KAHAN_GROUP) ring.shift();
+          }
+        }
+        if (sym) ring.flush(row, k0 + STEPS_KAHAN_GROUP - 1, (k0 & 31) == 0);
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+#pragma unroll
+          for (int a = 0; a < 3; ++a) acc2<KAHAN>(S[s][a], K[s][a], g[s][a]);
+      }
+      if (sym) {
+        __syncwarp();
+        for (int s = lane; s < jt; s += 32) {
+          const int j = t * jt + s;
+          if (j < n) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) fix_add(F, q, j, -fix_value(F, row[3 * s + q]));
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int i0 = b * kBI + 64 * s + lane;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN>(F, q, i0, i0 + 32, S[s][q], K[s][q]);
+    }
+    u += t1 - t0;
+  }
 }
 
 }  // namespace steps

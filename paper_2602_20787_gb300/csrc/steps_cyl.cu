@@ -262,7 +262,7 @@ struct steps_cyl_ctx {
   bool fix_ready = false, fix_ok = false;
   long long Usym = 0;
   int tpb = 1;                         // j-tiles per block of 128 rows of the symmetric kernels
-  int SYC = 0, SYSC = 0, SYTC = 0;     // CTAs of the symmetric plain / surrogate / table kernels
+  int SYC = 0, SYSC = 0, SYTC = 0, SYRC = 0;  // CTAs of the symmetric plain / surrogate / table / R^3 kernels
   // row sharding
   bool shard = false;
   int shard_rank = 0, shard_world = 1, chunk = 0;
@@ -1011,15 +1011,18 @@ int fix_scale(steps_cyl_ctx* c) {
   return STEPS_OK;
 }
 
+float fix_scale_f(const steps_cyl_ctx* c) {
+  return c->fix_scale <= std::ldexp(1.0, kMaxFixExpF) ? (float)c->fix_scale : 0.0f;
+}
+
 #ifndef STEPS_SYMMETRIC
 #define STEPS_SYMMETRIC 1  // evaluate each unordered pair once (build-time switch)
 #endif
 
-// The FP32 direct forms of an S1xR2 context take the symmetric kernels, unless
-// its rows are shared with other ranks (a rank has no j side for rows it does
-// not own).
+// The FP32 direct forms take the symmetric kernels, unless the context's rows are
+// shared with other ranks (a rank has no j side for rows it does not own).
 bool use_sym(const steps_cyl_ctx* c) {
-  return STEPS_SYMMETRIC && (!c->shard || c->shard_world == 1) && !is_r3(c) && c->fix_ok;
+  return STEPS_SYMMETRIC && (!c->shard || c->shard_world == 1) && c->fix_ok;
 }
 
 // The pair form of the next force evaluation: FP64, the selected modelled tail
@@ -1128,6 +1131,11 @@ int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const Fix
                    : sym_table_kernel<false>(model_kind(c), c->tab.read, straight);
     k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, Ua, U, C, c->tab, c->tab_const, F);
     CKLAUNCH("pair_sym_table");
+  } else if (is_r3(c)) {
+    const int C = ctas(c->SYRC);  // never a share of the triangle: a sharded R^3 context keeps the row step
+    auto k = kahan ? pair_sym_r3_kernel<true> : pair_sym_r3_kernel<false>;
+    k<<<C, 32, 0, c->st>>>(c->jA, c->jB, n, NB, tpb, U, C, F);
+    CKLAUNCH("pair_sym_r3");
   } else {
     const int C = ctas(c->SYC);
     const bool far = 2.0 * c->h_max < 0.5 * c->p.L;
@@ -1169,7 +1177,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
   if (form != Form::FP64 && use_sym(c)) {
     CK(cudaMemsetAsync(c->facc, 0, sizeof(unsigned long long) * 3 * (size_t)c->n, c->st));
     CK(cudaEventRecord(c->e0, c->st));
-    int rc = launch_sym(c, form, 0, c->Usym, FixAcc{c->facc, c->n, c->fix_scale, c->err, 0, 0, 0, 0});
+    int rc = launch_sym(c, form, 0, c->Usym, FixAcc{c->facc, c->n, c->fix_scale, fix_scale_f(c), c->err, 0, 0, 0, 0});
     if (rc) return rc;
     CK(cudaEventRecord(c->e1, c->st));
     c->timed = true;
@@ -2160,7 +2168,9 @@ int allocate_context(steps_cyl_ctx* c) {
   // the symmetric kernels share the upper triangle of the block grid
   c->tpb = (long long)c->NB * (c->NB + 1) / 2 < STEPS_SYM_SPLIT * (long long)sms ? 4 : 1;
   c->Usym = (long long)c->NB * (c->NB + 1) / 2 * c->tpb;
-  int yocc = 0, ysocc = 0, ytocc = 0;
+  int yocc = 0, ysocc = 0, ytocc = 0, yrocc = 0;
+  CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&yrocc, pair_sym_r3_kernel<true>, 32, 0));
+  c->SYRC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(yrocc, 1) * STEPS_CTA_MULT);
   CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&yocc, pair_sym_kernel<true, true, false>, kSymThreads, 0));
   CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ysocc, pair_sym_surr_kernel<true, kModelWide4, false>, kSymThreads, 0));
   CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ytocc, pair_sym_table_kernel<true, kModelWide4, kReadCic, false>, kSymThreads, 0));
@@ -2649,7 +2659,7 @@ int steps_cyl_shard_force(steps_cyl_ctx* c, const float* recv, int64_t* sums) {
   // this rank's equal share of the upper-triangle units, both sides of each pair
   const int W = c->shard_world, r = c->shard_rank;
   const long long Ua = (long long)r * c->Usym / W, Ub = (long long)(r + 1) * c->Usym / W;
-  const FixAcc F{reinterpret_cast<unsigned long long*>(sums), c->n, c->fix_scale, c->err, W, c->NB / W, c->NB % W,
+  const FixAcc F{reinterpret_cast<unsigned long long*>(sums), c->n, c->fix_scale, fix_scale_f(c), c->err, W, c->NB / W, c->NB % W,
                  c->chunk};
   CK(cudaEventRecord(c->e0, c->st));
   int rc = launch_sym(c, form, Ua, Ub - Ua, F);
