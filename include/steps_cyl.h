@@ -51,9 +51,9 @@ extern "C" {
 #define STEPS_FP32_KAHAN 1  /* FP32 pair math on hi/lo split positions, Kahan-compensated j sum */
 #define STEPS_FP32_PLAIN 2  /* FP32 pair math on hi/lo split positions, plain j sum */
 
-#define STEPS_TAIL_FULL 0       /* every image of the window: one by one in FP64 and for n_cut < 12; else the near
+#define STEPS_TAIL_FULL 0       /* every image of the window: one by one for n_cut < 12 (FP64: < 14); else the near
                                  * images (and the softened ones) one by one and the others, a smooth function of
-                                 * the image number, in closed form to below FP32 rounding */
+                                 * the image number, in closed form to below the precision's rounding */
 #define STEPS_TAIL_SURROGATE 1  /* images |k| <= n0 direct, far tail from the learned surrogate */
 #define STEPS_TAIL_TABLE 2      /* images |k| <= n0 direct, far tail from the correction table */
 
@@ -188,7 +188,7 @@ int steps_cyl_last_timing(steps_cyl_ctx* ctx, double* pair_images, double* pair_
  * not shared with other ranks evaluate each unordered pair of particles once
  * and add it to both (Newton's third law; the window of eq. ForceCylindrical and
  * the one image of R^3 are symmetric in i and j), so out[1] is n (n - 1) / 2 plus the pairs inside each
- * block of 128 rows, which are taken both ways; the row kernels evaluate
+ * block of 128 rows, which are taken both ways (FP64: n (n - 1) / 2 alone); the row kernels evaluate
  * (rows) x (n - 1) ordered pairs. The octree reports its interactions in
  * steps_cyl_tree_stats instead. */
 int steps_cyl_last_eval(steps_cyl_ctx* ctx, double out[4]);

@@ -31,6 +31,7 @@
 #include "nbody_kernels.cuh"
 #include "surrogate_pair.cuh"
 #include "surrogate_train.cuh"
+#include "pair_fp64.cuh"
 #include "tail_table.cuh"
 #include "octree.cuh"
 #include "r3_pair.cuh"
@@ -257,6 +258,7 @@ struct steps_cyl_ctx {
   int Ccap = 0, SCcap = 0, TCcap = 0;
   // symmetric (Newton's third law) evaluation into fixed-point accumulators
   unsigned long long* facc = nullptr;  // [3][n]
+  unsigned long long* facc_lo = nullptr;  // [3][n], the FP64 form's low words (allocated when it first runs)
   double fix_scale = 0.0;              // 2^S
   double h_max = 0.0;                  // the largest softening (set with fix_scale)
   bool fix_ready = false, fix_ok = false;
@@ -630,6 +632,13 @@ int build_background(steps_cyl_ctx* c) {
   return STEPS_OK;
 }
 
+#ifndef STEPS_FP64_MIN_STEPS
+#define STEPS_FP64_MIN_STEPS 8  // fewest steps (of 32 pairs) worth a warp of the symmetric FP64 kernel
+#endif
+#ifndef STEPS_FP64_WARPS
+#define STEPS_FP64_WARPS 64  // warps per SM it is split over
+#endif
+
 // FP64 pair sums of the listed particles (all when idx == nullptr) into
 // out[3][ni], with the j-range split across CTAs so that short lists fill the GPU.
 int launch_fp64(steps_cyl_ctx* c, const int64_t* idx, int ni, double* out) {
@@ -646,11 +655,40 @@ int launch_fp64(steps_cyl_ctx* c, const int64_t* idx, int ni, double* out) {
     CK(cudaMalloc(&c->chk, sizeof(double) * (size_t)JC * 3 * ni));
     c->chk_elems = (size_t)JC * 3 * ni;
   }
-  pair_fp64_kernel<<<dim3(gx, JC), 128, 0, c->st>>>(c->x, c->y, c->z, c->m, c->h, c->n, idx, ni, c->invL, n_cut_eff(c),
-                                                    tpc, c->chk, is_r3(c) ? 1 : 0);
+  const int nc = n_cut_eff(c);
+  auto kernel = is_r3(c) ? pair_fp64_kernel<kPair64R3>
+                : line_form64(nc) ? pair_fp64_kernel<kPair64Line>
+                                  : pair_fp64_kernel<kPair64Walk>;
+  kernel<<<dim3(gx, JC), 128, 0, c->st>>>(c->x, c->y, c->z, c->m, c->h, c->n, idx, ni, c->invL, nc, tpc, c->chk);
   CKLAUNCH("pair_fp64");
   chunk_sum_kernel<<<(ni + 255) / 256, 256, 0, c->st>>>(c->chk, ni, JC, out);
   CKLAUNCH("chunk_sum");
+  return STEPS_OK;
+}
+
+// FP64 pair sums of every particle into out[3][n], each unordered pair once.
+int launch_fp64_sym(steps_cyl_ctx* c, double* out) {
+  const long long m = 3LL * c->n;
+  if (!c->facc_lo) CK(cudaMalloc(&c->facc_lo, sizeof(unsigned long long) * (size_t)m));
+  CK(cudaMemsetAsync(c->facc, 0, sizeof(unsigned long long) * (size_t)m, c->st));
+  CK(cudaMemsetAsync(c->facc_lo, 0, sizeof(unsigned long long) * (size_t)m, c->st));
+  int sms = 0;
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
+  const int NB = (c->n + 31) / 32, nc = n_cut_eff(c);
+  const long long W = row_step64(NB, NB);
+  const long long warps = std::max(1LL, std::min((W + STEPS_FP64_MIN_STEPS - 1) / STEPS_FP64_MIN_STEPS,
+                                                 (long long)sms * STEPS_FP64_WARPS));
+  auto kernel = is_r3(c) ? pair_sym_fp64_kernel<kPair64R3>
+                : line_form64(nc) ? pair_sym_fp64_kernel<kPair64Line>
+                                  : pair_sym_fp64_kernel<kPair64Walk>;
+  const int per = kThreads64 / 32;
+  kernel<<<(unsigned)((warps + per - 1) / per), kThreads64, 0, c->st>>>(
+      c->x, c->y, c->z, c->m, c->h, c->n, c->invL, nc, NB, W, warps,
+      Fix64Acc{c->facc, c->facc_lo, c->n, c->fix_scale, c->err});
+  CKLAUNCH("pair_sym_fp64");
+  fix64_sum_kernel<<<grid_for((int)std::min(m, 1LL << 30), 256), 256, 0, c->st>>>(c->facc, c->facc_lo, m,
+                                                                                1.0 / c->fix_scale, out);
+  CKLAUNCH("fix64_sum");
   return STEPS_OK;
 }
 
@@ -1192,7 +1230,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
   }
   CK(cudaEventRecord(c->e0, c->st));
   if (form == Form::FP64) {
-    int rc = launch_fp64(c, nullptr, c->n, c->part);  // never sharded
+    int rc = use_sym(c) ? launch_fp64_sym(c, c->part) : launch_fp64(c, nullptr, c->n, c->part);  // never sharded
     if (rc) return rc;
   } else if (form == Form::SURROGATE) {
     const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
@@ -1240,8 +1278,9 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
   CK(cudaEventRecord(c->e1, c->st));
   c->timed = true;
   c->last_images = (double)(c->k1 - c->k0) * (double)(c->n - 1) * images_per_pair(c);
-  c->last_pairs = (double)(c->k1 - c->k0) * (double)(c->n - 1);
-  c->last_sym = false;
+  c->last_sym = form == Form::FP64 && use_sym(c);
+  c->last_straight = false;
+  c->last_pairs = (double)(c->k1 - c->k0) * (double)(c->n - 1) * (c->last_sym ? 0.5 : 1.0);
   const int NT = form == Form::FP64 ? 0 : c->NT;
   const int ctas = form == Form::SURROGATE ? c->SC : form == Form::TABLE ? c->TC : c->C;
   // rows [k0, k1): every row, or the rows this context owns when they are sharded
@@ -1363,6 +1402,7 @@ void release(steps_cyl_ctx* c) {
   cudaFree(c->chk);
   cudaFree(c->shard_off);
   cudaFree(c->facc);
+  cudaFree(c->facc_lo);
   {
     auto& T = c->tr;
     void* ptrs[] = {T.key[0], T.key[1], T.val[0], T.val[1], T.hist, T.offs, T.u4, T.u4s, T.zt, T.sA, T.sB,
