@@ -16,6 +16,8 @@
 #pragma once
 #include <cstdint>
 
+#include "pair_fp32.cuh"
+
 namespace steps {
 
 constexpr int kH = 32;                                   // hidden width
@@ -161,137 +163,230 @@ static __global__ void surrogate_dataset_kernel(const double* __restrict__ smp, 
   }
 }
 
-// ---------------------------------------------------------------------------
-// FP32 MLP training. One block of kTrainThreads threads takes kTrainThreads
-// samples of the minibatch; each thread runs its sample forward and backward,
-// the block forms its partial gradient from the per-sample activations and
-// deltas staged in shared memory, and writes it to gpart[block][kNW].
-// ---------------------------------------------------------------------------
-constexpr int kTrainThreads = 64;
+// Normalised FP32 targets t = (r - mu) / sc.
+static __global__ void surrogate_normalise_kernel(const double* __restrict__ r, int64_t ns, double mu0, double mu1,
+                                                  double sc0, double sc1, float* __restrict__ t) {
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
+    t[2 * s] = (float)((r[2 * s] - mu0) / sc0);
+    t[2 * s + 1] = (float)((r[2 * s + 1] - mu1) / sc1);
+  }
+}
 
-static __global__ void __launch_bounds__(kTrainThreads)
+// ---------------------------------------------------------------------------
+// FP32 MLP training. A block of kTrainCta threads takes kTrainThreads samples of the
+// minibatch and writes their summed gradient to gpart[block][kNW].
+//
+// What bounds a step is latency: 4,096 samples are 64 blocks of a few thousand cycles, 1,200
+// times in a row. Four threads share a sample (8 of 32 neurons each, two per packed
+// FP32x2 operation), the weights lie in shared memory in both orders so that either
+// direction reads the 8 it needs in two 128-bit broadcasts, and activations and deltas
+// lie unit-major, so that the gradients read four samples per 128-bit load and a thread's
+// tile of 2 x 2 weights shares them. With one thread per sample and the weights read
+// through L1 the kernel took 19.8 us, the reduction, whose loads waited for each other, 6.4.
+// Every sum keeps its order (inputs, samples, blocks ascending), so the trained weights
+// keep their bits.
+// ---------------------------------------------------------------------------
+constexpr int kTrainThreads = 64;              // samples of a block
+constexpr int kTrainCta = 4 * kTrainThreads;   // its threads
+constexpr int kTrainRow = kTrainThreads + 4;   // row stride: 128-bit reads of 8 rows hit 32 banks
+constexpr int kTrainT = kH + 4;                // row stride of the transposed W2
+
+// v[0 .. 7] += x * w[0 .. 7] as four packed FMAs
+__device__ __forceinline__ void axpy8(u64 (&v)[4], float x, const float* w) {
+  const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(w), b = *reinterpret_cast<const ulonglong2*>(w + 4);
+  const u64 X = pk(x, x);
+  v[0] = fma2(a.x, X, v[0]);
+  v[1] = fma2(a.y, X, v[1]);
+  v[2] = fma2(b.x, X, v[2]);
+  v[3] = fma2(b.y, X, v[3]);
+}
+
+static __global__ void __launch_bounds__(kTrainCta)
 mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ u, const float* __restrict__ t,
                    const int* __restrict__ order, int64_t first, int64_t count, float* __restrict__ gpart,
                    float* __restrict__ lpart) {
-  __shared__ float s_in[kTrainThreads][4];
-  __shared__ float s_a1[kTrainThreads][kH + 1];
-  __shared__ float s_d1[kTrainThreads][kH + 1];
-  __shared__ float s_a2[kTrainThreads][kH + 1];
-  __shared__ float s_d2[kTrainThreads][kH + 1];
-  __shared__ float s_e[kTrainThreads][2];
-  __shared__ float s_loss[kTrainThreads];
-  const int tid = threadIdx.x;
-  const int64_t q = (int64_t)blockIdx.x * kTrainThreads + tid;
+  static_assert(kH == 32 && kOW2 % 4 == 0, "eight neurons per thread, 128-bit reads of W2");
+  __shared__ __align__(16) float sW[kNW];
+  __shared__ __align__(16) float sT[kH * kTrainT];
+  __shared__ __align__(16) float s_in[3][kTrainRow], s_a1[kH][kTrainRow], s_d1[kH][kTrainRow], s_a2[kH][kTrainRow],
+      s_d2[kH][kTrainRow], s_e[2][kTrainRow], s_loss[kTrainThreads];
+  const int tid = threadIdx.x, s = tid % kTrainThreads, g = tid / kTrainThreads, o0 = 8 * g;
+  const int64_t q = (int64_t)blockIdx.x * kTrainThreads + s;
   const bool valid = q < count;
-  const float* W1 = w + kOW1;
-  const float* b1 = w + kOB1;
-  const float* W2 = w + kOW2;
-  const float* b2 = w + kOB2;
-  const float* W3 = w + kOW3;
-  const float* b3 = w + kOB3;
-  float in[3] = {0.f, 0.f, 0.f}, tg[2] = {0.f, 0.f};
-  if (valid) {
-    const int64_t s = order ? (int64_t)order[first + q] : first + q;
-    for (int k = 0; k < 3; ++k) in[k] = u[3 * s + k];
-    tg[0] = t[2 * s];
-    tg[1] = t[2 * s + 1];
-  }
-  // forward; ReLU'(z) is read from a = relu(z) > 0 (the same mask)
-  float a1[kH], a2[kH];
-#pragma unroll
-  for (int o = 0; o < kH; ++o) {
-    float v = b1[o];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) v = fmaf(W1[o * 3 + k], in[k], v);
-    a1[o] = fmaxf(v, 0.f);
-    s_a1[tid][o] = a1[o];
-  }
-#pragma unroll
-  for (int o = 0; o < kH; ++o) {
-    float v = b2[o];
-#pragma unroll
-    for (int k = 0; k < kH; ++k) v = fmaf(W2[o * kH + k], a1[k], v);
-    a2[o] = fmaxf(v, 0.f);
-  }
-  float y[2], e[2];
-#pragma unroll
-  for (int o = 0; o < 2; ++o) {
-    float v = b3[o];
-#pragma unroll
-    for (int k = 0; k < kH; ++k) v = fmaf(W3[o * kH + k], a2[k], v);
-    y[o] = v;
-    e[o] = valid ? (y[o] - tg[o]) : 0.f;
-  }
-  // backward: d2 = (W3^T e) * relu'(z2), d1 = (W2^T d2) * relu'(z1)
-  float d2[kH];
-#pragma unroll
-  for (int k = 0; k < kH; ++k) {
-    const float g = W3[k] * e[0] + W3[kH + k] * e[1];
-    d2[k] = a2[k] > 0.f ? g : 0.f;
-    s_a2[tid][k] = a2[k];
-    s_d2[tid][k] = d2[k];
-  }
-  for (int k = 0; k < kH; ++k) {
-    float g = 0.f;
-#pragma unroll
-    for (int o = 0; o < kH; ++o) g = fmaf(W2[o * kH + k], d2[o], g);
-    s_d1[tid][k] = s_a1[tid][k] > 0.f ? g : 0.f;
-  }
-  for (int k = 0; k < 3; ++k) s_in[tid][k] = in[k];
-  s_e[tid][0] = e[0];
-  s_e[tid][1] = e[1];
-  s_loss[tid] = 0.5f * (e[0] * e[0] + e[1] * e[1]);
-  __syncthreads();
-  // block partial gradient, one weight per thread per pass, samples in order
-  float* gp = gpart + (int64_t)blockIdx.x * kNW;
-  for (int p = tid; p < kNW; p += kTrainThreads) {
-    float g = 0.f;
-    if (p < kOB1) {
-      const int o = p / 3, k = p % 3;
-      for (int s = 0; s < kTrainThreads; ++s) g = fmaf(s_d1[s][o], s_in[s][k], g);
-    } else if (p < kOW2) {
-      const int o = p - kOB1;
-      for (int s = 0; s < kTrainThreads; ++s) g += s_d1[s][o];
-    } else if (p < kOB2) {
-      const int o = (p - kOW2) / kH, k = (p - kOW2) % kH;
-      for (int s = 0; s < kTrainThreads; ++s) g = fmaf(s_d2[s][o], s_a1[s][k], g);
-    } else if (p < kOW3) {
-      const int o = p - kOB2;
-      for (int s = 0; s < kTrainThreads; ++s) g += s_d2[s][o];
-    } else if (p < kOB3) {
-      const int o = (p - kOW3) / kH, k = (p - kOW3) % kH;
-      for (int s = 0; s < kTrainThreads; ++s) g = fmaf(s_e[s][o], s_a2[s][k], g);
-    } else {
-      const int o = p - kOB3;
-      for (int s = 0; s < kTrainThreads; ++s) g += s_e[s][o];
+  float tg = 0.f;
+  if (g < 2) {
+    float i0 = 0.f, i1 = 0.f;
+    if (valid) {
+      const int64_t k = order ? (int64_t)order[first + q] : first + q;
+      tg = t[2 * k + g];
+      i0 = u[3 * k + 2 * g];
+      if (g == 0) i1 = u[3 * k + 1];
     }
-    gp[p] = g;
+    s_in[2 * g][s] = i0;
+    if (g == 0) s_in[1][s] = i1;
   }
-  if (tid == 0) {
+#pragma unroll
+  for (int r = 0; r < (kNW + kTrainCta - 1) / kTrainCta; ++r) {
+    const int p = r * kTrainCta + tid;
+    if (p < kNW) {
+      const float v = w[p];
+      sW[p] = v;
+      if (p >= kOW2 && p < kOB2) sT[((p - kOW2) % kH) * kTrainT + (p - kOW2) / kH] = v;
+    }
+  }
+  __syncthreads();
+  // forward; ReLU'(z) is read from a = relu(z) > 0 (the same mask)
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int o = o0 + j;
+    float v = sW[kOB1 + o];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v = fmaf(sW[kOW1 + o * 3 + k], s_in[k][s], v);
+    s_a1[o][s] = fmaxf(v, 0.f);
+  }
+  __syncthreads();
+  float a2[8];
+  {
+    u64 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = pk(sW[kOB2 + o0 + 2 * j], sW[kOB2 + o0 + 2 * j + 1]);
+#pragma unroll 8
+    for (int k = 0; k < kH; ++k) axpy8(v, s_a1[k][s], sT + k * kTrainT + o0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      upk(v[j], a2[2 * j], a2[2 * j + 1]);
+      a2[2 * j] = fmaxf(a2[2 * j], 0.f);
+      a2[2 * j + 1] = fmaxf(a2[2 * j + 1], 0.f);
+      s_a2[o0 + 2 * j][s] = a2[2 * j];
+      s_a2[o0 + 2 * j + 1][s] = a2[2 * j + 1];
+    }
+  }
+  __syncthreads();
+  if (g < 2) {
+    float v = sW[kOB3 + g];
+#pragma unroll
+    for (int k = 0; k < kH; ++k) v = fmaf(sW[kOW3 + g * kH + k], s_a2[k][s], v);
+    s_e[g][s] = valid ? (v - tg) : 0.f;
+  }
+  __syncthreads();
+  // backward: d2 = (W3^T e) * relu'(z2), d1 = (W2^T d2) * relu'(z1)
+  const float e[2] = {s_e[0][s], s_e[1][s]};
+  const float* W3 = sW + kOW3;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int k = o0 + j;
+    const float d = W3[k] * e[0] + W3[kH + k] * e[1];
+    s_d2[k][s] = a2[j] > 0.f ? d : 0.f;
+  }
+  if (g == 0) s_loss[s] = 0.5f * (e[0] * e[0] + e[1] * e[1]);
+  __syncthreads();
+  {
+    u64 v[4] = {0, 0, 0, 0};
+#pragma unroll 8
+    for (int o = 0; o < kH; ++o) axpy8(v, s_d2[o][s], sW + kOW2 + o * kH + o0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float x, y;
+      upk(v[j], x, y);
+      s_d1[o0 + 2 * j][s] = s_a1[o0 + 2 * j][s] > 0.f ? x : 0.f;
+      s_d1[o0 + 2 * j + 1][s] = s_a1[o0 + 2 * j + 1][s] > 0.f ? y : 0.f;
+    }
+  }
+  __syncthreads();
+  // block partial gradient, samples in order. W2: rows o, o + 16, columns k, k + 16
+  float* gp = gpart + (int64_t)blockIdx.x * kNW;
+  {
+    const int k = tid % 16, o = tid / 16;
+    float c00 = 0.f, c01 = 0.f, c10 = 0.f, c11 = 0.f;
+#pragma unroll 4
+    for (int r = 0; r < kTrainThreads; r += 4) {
+      const float4 A0 = *reinterpret_cast<const float4*>(&s_a1[k][r]), A1 = *reinterpret_cast<const float4*>(&s_a1[k + 16][r]);
+      const float4 D0 = *reinterpret_cast<const float4*>(&s_d2[o][r]), D1 = *reinterpret_cast<const float4*>(&s_d2[o + 16][r]);
+      c00 = fmaf(D0.w, A0.w, fmaf(D0.z, A0.z, fmaf(D0.y, A0.y, fmaf(D0.x, A0.x, c00))));
+      c01 = fmaf(D0.w, A1.w, fmaf(D0.z, A1.z, fmaf(D0.y, A1.y, fmaf(D0.x, A1.x, c01))));
+      c10 = fmaf(D1.w, A0.w, fmaf(D1.z, A0.z, fmaf(D1.y, A0.y, fmaf(D1.x, A0.x, c10))));
+      c11 = fmaf(D1.w, A1.w, fmaf(D1.z, A1.z, fmaf(D1.y, A1.y, fmaf(D1.x, A1.x, c11))));
+    }
+    float* d = gp + kOW2 + o * kH + k;
+    d[0] = c00;
+    d[16] = c01;
+    d[16 * kH] = c10;
+    d[16 * kH + 16] = c11;
+  }
+  // the other weights: sums over the samples of a row product (W1, W3) or of a row (b1, b2, b3)
+  constexpr int kRest = kNW - kH * kH;
+  static_assert(kRest <= kTrainCta - 1, "one of the other weights per thread, the last thread sums the loss");
+  if (tid < kRest) {
+    const int p = tid < kOW2 ? tid : tid + kH * kH;
+    const float *A, *B = nullptr;
+    if (p < kOB1) {
+      A = s_d1[p / 3];
+      B = s_in[p % 3];
+    } else if (p < kOW2) {
+      A = s_d1[p - kOB1];
+    } else if (p < kOW3) {
+      A = s_d2[p - kOB2];
+    } else if (p < kOB3) {
+      A = s_e[(p - kOW3) / kH];
+      B = s_a2[(p - kOW3) % kH];
+    } else {
+      A = s_e[p - kOB3];
+    }
+    float c = 0.f;
+    if (B) {
+#pragma unroll 4
+      for (int r = 0; r < kTrainThreads; r += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(A + r), b = *reinterpret_cast<const float4*>(B + r);
+        c = fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
+      }
+    } else {
+#pragma unroll 4
+      for (int r = 0; r < kTrainThreads; r += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(A + r);
+        c = (((c + a.x) + a.y) + a.z) + a.w;
+      }
+    }
+    gp[p] = c;
+  } else if (tid == kTrainCta - 1) {
     float l = 0.f;
-    for (int s = 0; s < kTrainThreads; ++s) l += s_loss[s];
+    for (int r = 0; r < kTrainThreads; ++r) l += s_loss[r];
     lpart[blockIdx.x] = l;
   }
 }
 
 // Sum the block partials of each weight in block order, divide by the batch,
 // and (when adam) take an Adam step. grad_out (optional) receives the gradient.
-static __global__ void mlp_reduce_adam_kernel(const float* __restrict__ gpart, int nblocks, float inv_batch,
-                                              float* __restrict__ w, float* __restrict__ m1, float* __restrict__ m2,
-                                              float lr, float beta1, float beta2, float eps, float c1, float c2,
-                                              int adam, float* __restrict__ grad_out) {
+// One warp per CTA: the 1,250 sums spread over 40 SMs, and 32 of a sum's loads are in flight.
+constexpr int kAdamThreads = 32, kAdamLoads = 32;
+static __global__ void __launch_bounds__(kAdamThreads)
+mlp_reduce_adam_kernel(const float* __restrict__ gpart, int nblocks, float inv_batch, float* __restrict__ w,
+                       float* __restrict__ m1, float* __restrict__ m2, float lr, float beta1, float beta2, float eps,
+                       float c1, float c2, int adam, float* __restrict__ grad_out) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= kNW) return;
+  float M1 = 0.f, M2 = 0.f, W = 0.f;
+  if (adam) {
+    M1 = m1[p];
+    M2 = m2[p];
+    W = w[p];
+  }
   float g = 0.f;
-  for (int b = 0; b < nblocks; ++b) g += gpart[(int64_t)b * kNW + p];
+  for (int b = 0; b < nblocks; b += kAdamLoads) {
+    float v[kAdamLoads];
+#pragma unroll
+    for (int k = 0; k < kAdamLoads; ++k) v[k] = b + k < nblocks ? gpart[(int64_t)(b + k) * kNW + p] : 0.f;
+#pragma unroll
+    for (int k = 0; k < kAdamLoads; ++k)
+      if (b + k < nblocks) g += v[k];
+  }
   g *= inv_batch;
   if (grad_out) grad_out[p] = g;
   if (adam) {
-    const float a = beta1 * m1[p] + (1.f - beta1) * g;
-    const float v = beta2 * m2[p] + (1.f - beta2) * g * g;
+    const float a = fmaf(1.f - beta1, g, beta1 * M1);
+    const float v = fmaf((1.f - beta2) * g, g, beta2 * M2);
     m1[p] = a;
     m2[p] = v;
-    w[p] -= lr * (a / c1) / (sqrtf(v / c2) + eps);
+    w[p] = W - lr * (a / c1) / (sqrtf(v / c2) + eps);
   }
 }
 
