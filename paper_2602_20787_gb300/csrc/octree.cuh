@@ -32,6 +32,7 @@
 #pragma once
 #include <cstdint>
 
+#include "pair_sym.cuh"
 #include "tail_table.cuh"
 
 namespace steps {
@@ -403,101 +404,115 @@ __device__ __forceinline__ bool tree_opens(const float4& u, const float4& g, flo
   return clear <= __fadd_rn(u.w, hm);
 }
 
-// All lanes against the nl entries of the warp's list: the pair form of the
-// correction-table tail over the infinite window (entry `self` of a lane,
-// its own particle, has zero mass).
-template <bool KAHAN>
-__device__ __forceinline__ void tree_eval(const IParticle& I, int me, const float4* __restrict__ A_,
-                                          const float4* __restrict__ B_, const int* __restrict__ id_, int nl,
-                                          const SurrConst& S, const TableTail& T, float& sx, float& sy, float& sz,
-                                          float& cx, float& cy, float& cz) {
-#pragma unroll 1
-  for (int k0 = 0; k0 < nl; k0 += STEPS_KAHAN_GROUP) {
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-#pragma unroll 2
-    for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; ++k) {
-      const int kc = min(k, nl - 1);
-      const float4 A = A_[kc];
-      const float4 B = B_[kc];
-      float dx, dy, dz, dR2, hh;
-      int kw;
-      pair_geometry(I, A, B, dx, dy, dz, dR2, hh, kw);
-      SurrPair P;
-      surr_stage_a<true, -1>(dR2, dz, hh, 0, kw, S, P);
-      const float2 r = table_read(T, P.u[0], P.u[1]);
-      float sr, szz;
-      surr_stage_c<true>(I, A, B, 0, kw, S, P, r.x, r.y, sr, szz);
-      const float mj = (k < nl && id_[kc] != me) ? A.w : 0.0f;
-      const float msr = mj * sr;
-      gx = fmaf(dx, msr, gx);
-      gy = fmaf(dy, msr, gy);
-      gz = fmaf(mj, szz, gz);
-    }
-    acc<KAHAN>(sx, cx, gx);
-    acc<KAHAN>(sy, cy, gy);
-    acc<KAHAN>(sz, cz, gz);
+// A warp's interaction list, one array per word, so that one 64-bit load (the same address on
+// every lane) yields two entries as a packed operand of pair2.cuh's two-pair forms.
+struct TreeList {
+  float xh[kWalkList], yh[kWalkList], zh[kWalkList], m[kWalkList];
+  float xl[kWalkList], yl[kWalkList], zl[kWalkList], h[kWalkList];
+  __device__ __forceinline__ void put(int k, const float4& a, const float4& b) {
+    xh[k] = a.x;
+    yh[k] = a.y;
+    zh[k] = a.z;
+    m[k] = a.w;
+    xl[k] = b.x;
+    yl[k] = b.y;
+    zl[k] = b.z;
+    h[k] = b.w;
   }
+  __device__ __forceinline__ static u64 two(const float* v, int k) { return *reinterpret_cast<const u64*>(v + k); }
+};
+static_assert(kWalkList % 2 == 0, "an odd list is filled up by one entry");
+
+// A lane's particle against the entries k and k + 1: separations and softening sums.
+__device__ __forceinline__ void tree_separation(const I2& I, const TreeList& T, int k, bool periodic, Sep2& P) {
+  P.dx = add2(sub2(I.xh, TreeList::two(T.xh, k)), sub2(I.xl, TreeList::two(T.xl, k)));
+  P.dy = add2(sub2(I.yh, TreeList::two(T.yh, k)), sub2(I.yl, TreeList::two(T.yl, k)));
+  const u64 zl = sub2(I.zl, TreeList::two(T.zl, k));
+  const u64 d = sub2(I.zh, TreeList::two(T.zh, k)), r = dup(kRound23);
+  P.dz = add2(periodic ? sub2(d, sub2(add2(d, r), r)) : d, zl);
+  P.dr2 = fma2(P.dx, P.dx, mul2(P.dy, P.dy));
+  P.hh = add2(I.h, TreeList::two(T.h, k));
 }
 
-// The R^3 form of the list evaluation (eq. NewtonianForce, one image): two
-// entries per packed FP32x2 op, the spline only when some lane is softened.
-template <bool KAHAN>
-__device__ __forceinline__ void tree_eval_r3(const IParticle& I, int me, const float4* __restrict__ A_,
-                                             const float4* __restrict__ B_, const int* __restrict__ id_, int nl,
-                                             float& sx, float& sy, float& sz, float& cx, float& cy, float& cz) {
-  float xh, yh, xl, yl;
-  upk(I.xyh, xh, yh);
-  upk(I.xyl, xl, yl);
-  const u64 XH = pk(xh, xh), YH = pk(yh, yh), ZH = pk(I.zh, I.zh);
-  const u64 XL = pk(xl, xl), YL = pk(yl, yl), ZL = pk(I.zl, I.zl);
-  const u64 HI = pk(I.h, I.h);
-#pragma unroll 1
-  for (int k0 = 0; k0 < nl; k0 += 8) {
-    u64 GX = pk(0.f, 0.f), GY = pk(0.f, 0.f), GZ = pk(0.f, 0.f);
-#pragma unroll 1
-    for (int k = k0; k < k0 + 8; k += 2) {
-      const int ka = min(k, nl - 1), kb = min(k + 1, nl - 1);
-      const float4 A0 = A_[ka], A1 = A_[kb], B0 = B_[ka], B1 = B_[kb];
-      const float m0 = (k < nl && id_[ka] != me) ? A0.w : 0.0f;
-      const float m1 = (k + 1 < nl && id_[kb] != me) ? A1.w : 0.0f;
-      const u64 DX = add2(sub2(XH, pk(A0.x, A1.x)), sub2(XL, pk(B0.x, B1.x)));
-      const u64 DY = add2(sub2(YH, pk(A0.y, A1.y)), sub2(YL, pk(B0.y, B1.y)));
-      const u64 DZ = add2(sub2(ZH, pk(A0.z, A1.z)), sub2(ZL, pk(B0.z, B1.z)));
-      const u64 R2 = fma2(DX, DX, fma2(DY, DY, mul2(DZ, DZ)));
-      const u64 HH = add2(HI, pk(B0.w, B1.w));
-      float ra, rb, ha, hb;
-      upk(R2, ra, rb);
-      upk(HH, ha, hb);
-      const u64 RI = pk(rsq(fmaxf(ra, 1e-30f)), rsq(fmaxf(rb, 1e-30f)));
-      u64 F = mul2(mul2(RI, RI), RI);
-      if (__any_sync(0xffffffffu, ra < ha * ha || rb < hb * hb)) {
-        const float iha = rcp_approx(ha), ihb = rcp_approx(hb);
-        const u64 IH = pk(iha, ihb);
-        F = spline_value_r2(R2, RI, F, IH, pk(-iha, -ihb), mul2(mul2(IH, IH), IH));
-      }
-      const u64 MF = mul2(pk(m0, m1), F);
-      GX = fma2(DX, MF, GX);
-      GY = fma2(DY, MF, GY);
-      GZ = fma2(DZ, MF, GZ);
+// Pair forms of two list entries: image sums (SR, SZ).
+// S1xR2: the correction-table tail over the infinite window; n0 = 4 in closed form, as the
+// direct kernels take it (pair_sym.cuh), else near images and base one by one.
+// RAW: the nearest-image table (n0 = 0), which holds the tail sums themselves.
+template <int MODEL, bool RAW>
+struct TreeTableForm {
+  static constexpr bool periodic = true;
+  const SurrConst& S;
+  const TableTail& T;
+  __device__ __forceinline__ void operator()(const Sep2& P, u64& SR, u64& SZ) const {
+    const u64 ADZ = abs2(P.dz);
+    Model2 M;
+    model_stage2<MODEL, RAW, false>(P, ADZ, 0, S, M);
+    float u0, v0, u1, v1;
+    upk(M.u[0], u0, v0);
+    upk(M.u[1], u1, v1);
+    const float2 r = table_read(T, u0, u1), s = table_read(T, v0, v1);
+    model_finish2<MODEL, RAW>(P, ADZ, 0, M, pk(r.x, s.x), pk(r.y, s.y), SR, SZ);
+  }
+};
+// R^3 (eq. NewtonianForce): one image, the spline only when some lane is softened.
+struct TreeR3Form {
+  static constexpr bool periodic = false;
+  __device__ __forceinline__ void operator()(const Sep2& P, u64& SR, u64& SZ) const {
+    const u64 R2 = fma2(P.dz, P.dz, P.dr2), RI = rsq2(max2(R2, 1e-30f));
+    SR = mul2(mul2(RI, RI), RI);
+    if (any_less2(R2, mul2(P.hh, P.hh))) {
+      const Soft2 s = soft2(P.hh);
+      SR = spline_value_r2(R2, RI, SR, s.ih, s.nih, s.ih3);
     }
-    float a, b;
-    upk(GX, a, b);
-    acc<KAHAN>(sx, cx, a + b);
-    upk(GY, a, b);
-    acc<KAHAN>(sy, cy, a + b);
-    upk(GZ, a, b);
-    acc<KAHAN>(sz, cz, a + b);
+    SZ = mul2(P.dz, SR);
+  }
+};
+
+// Packed sums of a lane: the two halves hold the even and the odd entries.
+struct TreeSum {
+  u64 x = 0, y = 0, z = 0, cx = 0, cy = 0, cz = 0;
+};
+
+// All lanes against the nl entries of the warp's list, two per step. A lane's own particle is
+// among them: its separation is zero, so it adds exact zeros.
+template <bool KAHAN, class Form>
+__device__ __forceinline__ void tree_eval(const I2& I, TreeList& L, int nl, int lane, const Form& form, TreeSum& A) {
+  if (nl & 1) {  // an odd list ends with a massless entry far off the axis
+    if (lane == 0) L.put(nl, make_float4(4096.0f, 4096.0f, 0.0f, 0.0f), make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+    __syncwarp();
+  }
+#pragma unroll 1
+  for (int k0 = 0; k0 < nl; k0 += 2 * STEPS_KAHAN_GROUP) {
+    u64 gx = 0, gy = 0, gz = 0;
+    const int ke = min(nl, k0 + 2 * STEPS_KAHAN_GROUP);
+#pragma unroll 1
+    for (int k = k0; k < ke; k += 2) {
+      Sep2 P;
+      tree_separation(I, L, k, Form::periodic, P);
+      u64 SR, SZ;
+      form(P, SR, SZ);
+      const u64 m = TreeList::two(L.m, k), MS = mul2(m, SR);
+      gx = fma2(P.dx, MS, gx);
+      gy = fma2(P.dy, MS, gy);
+      gz = fma2(m, SZ, gz);
+    }
+    acc2<KAHAN>(A.x, A.cx, gx);
+    acc2<KAHAN>(A.y, A.cy, gy);
+    acc2<KAHAN>(A.z, A.cz, gz);
   }
 }
 
 #ifndef STEPS_TREE_MIN_BLOCKS
-#define STEPS_TREE_MIN_BLOCKS 4  // co-resident CTAs per SM asked of the register allocator
+#define STEPS_TREE_MIN_BLOCKS 5  // co-resident CTAs per SM asked of the register allocator
 #endif
 
 // One warp per group of 32 particles in key order (sA/sB, u4s: key order);
 // out = [3][n] pair sums in internal order (sidx maps key order to internal).
-// R3: the R^3 pair force (no images, no table).
-template <bool KAHAN, bool R3 = false>
+// FORM: S1xR2 with the near range n0 = 4, any other, or none (the nearest-image table), or the
+// R^3 pair force (no images, no table).
+enum TreeForm { kTreeInf4, kTreeInf, kTreeRaw, kTreeR3 };
+
+template <bool KAHAN, int FORM>
 __global__ void __launch_bounds__(kWalkWarps * 32, STEPS_TREE_MIN_BLOCKS)
 tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, const float4* __restrict__ u4s,
                  const int* __restrict__ sidx, int n, const int4* __restrict__ link, const float4* __restrict__ geo,
@@ -505,92 +520,72 @@ tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, c
                  TreeCrit C, TableTail T, SurrConst S, double* __restrict__ out,
                  unsigned long long* __restrict__ inter, int* __restrict__ err) {
   __shared__ int stk[kWalkWarps][kWalkStack];
-  __shared__ float4 lA[kWalkWarps][kWalkList];
-  __shared__ float4 lB[kWalkWarps][kWalkList];
-  __shared__ int lid[kWalkWarps][kWalkList];
+  __shared__ __align__(16) TreeList list[kWalkWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = blockIdx.x * kWalkWarps + w;
   if (g * 32 >= n) return;  // the whole warp leaves; the walk uses warp-level synchronisation only
   const int q = g * 32 + lane;
   const bool valid = q < n;
   const int qc = min(q, n - 1);
-  const IParticle I = load_i(sA, sB, qc);
+  const float4 a = sA[qc], b = sB[qc];
+  const I2 I{dup(a.x), dup(b.x), dup(a.y), dup(b.y), dup(a.z), dup(b.z), dup(b.w), 0};
   const float4 u = u4s[qc];
-  const int me = valid ? q : -1;
   const int nvalid = min(32, n - g * 32);
   int* st = stk[w];
-  float4* A_ = lA[w];
-  float4* B_ = lB[w];
-  int* id_ = lid[w];
-  float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
+  TreeList& L = list[w];
+  TreeSum A;
   unsigned long long count = 0;
   bool overflow = false;
+  int top = 1, nl = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    if constexpr (FORM == kTreeR3)
+      tree_eval<KAHAN>(I, L, nl, lane, TreeR3Form{}, A);
+    else
+      tree_eval<KAHAN>(I, L, nl, lane, TreeTableForm<FORM == kTreeInf4 ? kModelInf4 : kModelInf, FORM == kTreeRaw>{S, T}, A);
+    count += (unsigned long long)nl * nvalid;
+    nl = 0;
+    __syncwarp();
+  };
+  // One place evaluates: `left` holds what of an opened leaf is still to be listed, and a list
+  // without room for 32 more (or with nothing left to walk) is evaluated before the next step.
   if (lane == 0) st[0] = 0;
   __syncwarp();
-  int top = 1, nl = 0;
-  while (top > 0) {
+  int p0 = 0, p1 = 0;
+  while (true) {
+    if (nl > kWalkList - 33 || (top == 0 && p0 == p1)) {
+      if (nl > 0) flush();
+      if (top == 0 && p0 == p1) break;
+    }
+    if (p0 < p1) {
+      const int c = min(32, p1 - p0);
+      if (lane < c) L.put(nl + lane, sA[p0 + lane], sB[p0 + lane]);
+      nl += c;
+      p0 += c;
+      continue;
+    }
     const int node = st[--top];
     const float4 gm = geo[node];
     const int4 lk = link[node];
     const float hm = hmf[node];
     const bool open = __any_sync(0xffffffffu, valid && tree_opens(u, gm, hm, C));
     __syncwarp();  // every lane has read st[top] before it is reused
-    if (open && lk.y > 0) {
+    if (!open) {
+      if (lane == 0) L.put(nl, nA[node], nB[node]);
+      ++nl;
+    } else if (lk.y > 0) {
       if (top + lk.y > kWalkStack) {
         overflow = true;
-        break;
+        top = 0;
+        continue;
       }
       if (lane < lk.y) st[top + lane] = lk.x + lane;
       __syncwarp();
       top += lk.y;
-      continue;
-    }
-    if (!open) {
-      if (lane == 0) {
-        A_[nl] = nA[node];
-        B_[nl] = nB[node];
-        id_[nl] = -1;
-      }
-      ++nl;
     } else {
-      for (int b0 = lk.z; b0 < lk.w; b0 += 32) {
-        const int c = min(32, lk.w - b0);
-        if (nl + c > kWalkList) {
-          __syncwarp();
-          if (R3)
-            tree_eval_r3<KAHAN>(I, me, A_, B_, id_, nl, sx, sy, sz, cx, cy, cz);
-          else
-            tree_eval<KAHAN>(I, me, A_, B_, id_, nl, S, T, sx, sy, sz, cx, cy, cz);
-          count += (unsigned long long)nl * nvalid;
-          nl = 0;
-          __syncwarp();
-        }
-        if (lane < c) {
-          A_[nl + lane] = sA[b0 + lane];
-          B_[nl + lane] = sB[b0 + lane];
-          id_[nl + lane] = b0 + lane;
-        }
-        nl += c;
-      }
+      p0 = lk.z;
+      p1 = lk.w;
     }
-    if (nl > kWalkList - 33) {
-      __syncwarp();
-      if (R3)
-        tree_eval_r3<KAHAN>(I, me, A_, B_, id_, nl, sx, sy, sz, cx, cy, cz);
-      else
-        tree_eval<KAHAN>(I, me, A_, B_, id_, nl, S, T, sx, sy, sz, cx, cy, cz);
-      count += (unsigned long long)nl * nvalid;
-      nl = 0;
-      __syncwarp();
-    }
-  }
-  __syncwarp();
-  if (nl > 0) {
-    if (R3)
-      tree_eval_r3<KAHAN>(I, me, A_, B_, id_, nl, sx, sy, sz, cx, cy, cz);
-    else
-      tree_eval<KAHAN>(I, me, A_, B_, id_, nl, S, T, sx, sy, sz, cx, cy, cz);
-    count += (unsigned long long)nl * nvalid;
   }
   if (lane == 0) {
     atomicAdd(inter, count);
@@ -598,9 +593,13 @@ tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, c
   }
   if (valid) {
     const int i = sidx[q];
-    out[i] = (double)sx - (KAHAN ? (double)cx : 0.0);
-    out[(long long)n + i] = (double)sy - (KAHAN ? (double)cy : 0.0);
-    out[2 * (long long)n + i] = (double)sz - (KAHAN ? (double)cz : 0.0);
+    double e, o;
+    sum2<KAHAN>(A.x, A.cx, e, o);
+    out[i] = e + o;
+    sum2<KAHAN>(A.y, A.cy, e, o);
+    out[(long long)n + i] = e + o;
+    sum2<KAHAN>(A.z, A.cz, e, o);
+    out[2 * (long long)n + i] = e + o;
   }
 }
 

@@ -932,22 +932,12 @@ int tree_walk(steps_cyl_ctx* c, double* out) {
   const int blocks = (groups + kWalkWarps - 1) / kWalkWarps;
   CKT(cudaMemsetAsync(T.inter, 0, sizeof(unsigned long long), c->st));
   const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
-  if (is_r3(c) && kahan)
-    tree_walk_kernel<true, true><<<blocks, kWalkWarps * 32, 0, c->st>>>(T.sA, T.sB, T.u4s, T.val[0], c->n, T.link,
-                                                                        T.geo, T.hmf, T.nA, T.nB, C, c->tab,
-                                                                        c->tab_const, out, T.inter, c->err);
-  else if (is_r3(c))
-    tree_walk_kernel<false, true><<<blocks, kWalkWarps * 32, 0, c->st>>>(T.sA, T.sB, T.u4s, T.val[0], c->n, T.link,
-                                                                         T.geo, T.hmf, T.nA, T.nB, C, c->tab,
-                                                                         c->tab_const, out, T.inter, c->err);
-  else if (kahan)
-    tree_walk_kernel<true><<<blocks, kWalkWarps * 32, 0, c->st>>>(T.sA, T.sB, T.u4s, T.val[0], c->n, T.link, T.geo,
-                                                                  T.hmf, T.nA, T.nB, C, c->tab, c->tab_const, out,
-                                                                  T.inter, c->err);
-  else
-    tree_walk_kernel<false><<<blocks, kWalkWarps * 32, 0, c->st>>>(T.sA, T.sB, T.u4s, T.val[0], c->n, T.link, T.geo,
-                                                                   T.hmf, T.nA, T.nB, C, c->tab, c->tab_const, out,
-                                                                   T.inter, c->err);
+  auto walk = is_r3(c) ? (kahan ? tree_walk_kernel<true, kTreeR3> : tree_walk_kernel<false, kTreeR3>)
+              : c->p.n0 == 4 ? (kahan ? tree_walk_kernel<true, kTreeInf4> : tree_walk_kernel<false, kTreeInf4>)
+              : c->p.n0 > 0 ? (kahan ? tree_walk_kernel<true, kTreeInf> : tree_walk_kernel<false, kTreeInf>)
+                            : (kahan ? tree_walk_kernel<true, kTreeRaw> : tree_walk_kernel<false, kTreeRaw>);
+  walk<<<blocks, kWalkWarps * 32, 0, c->st>>>(T.sA, T.sB, T.u4s, T.val[0], c->n, T.link, T.geo, T.hmf, T.nA, T.nB, C,
+                                              c->tab, c->tab_const, out, T.inter, c->err);
   CKLAUNCH("tree_walk");
   return STEPS_OK;
 }
