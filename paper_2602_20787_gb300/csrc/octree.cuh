@@ -161,30 +161,40 @@ radix_hist_kernel(const uint64_t* __restrict__ key, int n, int shift, int ntiles
   hist[(size_t)threadIdx.x * ntiles + blockIdx.x] = hcount[threadIdx.x];
 }
 
-// Exclusive scan of m counts by one CTA of 1024 threads (each takes a
-// contiguous chunk). total (may be null) gets the sum.
+// Exclusive scan of m counts (m a multiple of 4: 256 per sort tile) by one CTA, 4,096 at a time with
+// a running sum; total (may be null) gets the sum. Every access is a coalesced 128-bit one (each
+// thread walking a chunk of its own took 56 us for 32,768 counts).
 static __global__ void __launch_bounds__(1024)
 scan_exclusive_kernel(const unsigned* __restrict__ in, unsigned* __restrict__ out, int m, unsigned* total) {
-  __shared__ unsigned part[1024];
-  const int chunk = (m + 1023) / 1024;
-  const int b = threadIdx.x * chunk, e = min(m, b + chunk);
-  unsigned s = 0;
-  for (int k = b; k < e; ++k) s += in[k];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {  // Hillis-Steele inclusive scan of the chunk sums
-    const unsigned v = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
+  __shared__ unsigned part[32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto load = [&](int k) { return k < m ? *reinterpret_cast<const uint4*>(in + k) : make_uint4(0, 0, 0, 0); };
+  auto inclusive = [&](unsigned v) {  // over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned t = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += t;
+    }
+    return v;
+  };
+  unsigned run = 0;
+  uint4 v = load(4 * threadIdx.x);
+  for (int base = 0; base < m; base += 4096) {
+    const int k = base + 4 * threadIdx.x;
+    const uint4 next = load(k + 4096);
+    const unsigned s = v.x + v.y + v.z + v.w, i = inclusive(s);
+    if (lane == 31) part[w] = i;
     __syncthreads();
-    part[threadIdx.x] += v;
+    if (w == 0) part[lane] = inclusive(part[lane]);
+    __syncthreads();
+    const unsigned e = run + (w > 0 ? part[w - 1] : 0u) + i - s;
+    if (k < m)
+      *reinterpret_cast<uint4*>(out + k) = make_uint4(e, e + v.x, e + v.x + v.y, e + v.x + v.y + v.z);
+    run += part[31];
+    v = next;
     __syncthreads();
   }
-  unsigned run = part[threadIdx.x] - s;
-  for (int k = b; k < e; ++k) {
-    const unsigned v = in[k];
-    out[k] = run;
-    run += v;
-  }
-  if (total && threadIdx.x == 1023) *total = part[1023];
+  if (total && threadIdx.x == 0) *total = run;
 }
 
 // Stable scatter: the keys of a tile are taken in order, kSortThreads per
@@ -233,99 +243,108 @@ radix_scatter_kernel(const uint64_t* __restrict__ kin, const int* __restrict__ v
 // ---- level-by-level build ---------------------------------------------------
 // Node records: link = (first child or -1, children, first, end sorted
 // positions), geo = (centre, side) in root units, pre = key prefix.
-// Thread per (active node, child digit): the child's sorted range.
-static __global__ void tree_children_kernel(const int* __restrict__ active, int n_active, int level,
-                                            const uint64_t* __restrict__ key, const int4* __restrict__ link,
-                                            const uint64_t* __restrict__ pre, int* __restrict__ cnt,
-                                            int* __restrict__ beg) {
+// Thread per (active node, child digit): the child's sorted range. blk[CTA]: how many of the
+// CTA's slots hold a child, and how many of these are active at the next level.
+constexpr int kSlotThreads = 256;
+static __global__ void __launch_bounds__(kSlotThreads)
+tree_children_kernel(const int* __restrict__ active, int n_active, int level, int leaf,
+                     const uint64_t* __restrict__ key, const int4* __restrict__ link,
+                     const uint64_t* __restrict__ pre, int* __restrict__ cnt, int* __restrict__ beg,
+                     int2* __restrict__ blk) {
   const int slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= 8 * n_active) return;
-  const int node = active[slot >> 3], c = slot & 7;
-  const int4 lk = link[node];
-  const int sh = 3 * (kTreeDepth - 1 - level);
-  const uint64_t target = (pre[node] << 3) | (uint64_t)c;
-  int lo = lk.z, hi = lk.w;  // first q with key[q] >> sh >= target
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if ((key[mid] >> sh) < target) lo = mid + 1;
-    else hi = mid;
+  int ck = 0;
+  if (slot < 8 * n_active) {
+    const int node = active[slot >> 3], c = slot & 7;
+    const int4 lk = link[node];
+    const int sh = 3 * (kTreeDepth - 1 - level);
+    const uint64_t target = (pre[node] << 3) | (uint64_t)c;
+    int lo = lk.z, hi = lk.w;  // first q with key[q] >> sh >= target
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((key[mid] >> sh) < target) lo = mid + 1;
+      else hi = mid;
+    }
+    int lo2 = lo, hi2 = lk.w;  // first q with key[q] >> sh > target
+    while (lo2 < hi2) {
+      const int mid = (lo2 + hi2) >> 1;
+      if ((key[mid] >> sh) <= target) lo2 = mid + 1;
+      else hi2 = mid;
+    }
+    ck = lo2 - lo;
+    cnt[slot] = ck;
+    beg[slot] = lo;
   }
-  int lo2 = lo, hi2 = lk.w;  // first q with key[q] >> sh > target
-  while (lo2 < hi2) {
-    const int mid = (lo2 + hi2) >> 1;
-    if ((key[mid] >> sh) <= target) lo2 = mid + 1;
-    else hi2 = mid;
-  }
-  cnt[slot] = lo2 - lo;
-  beg[slot] = lo;
+  const int c1 = __syncthreads_count(ck > 0);
+  const int c2 = __syncthreads_count(level + 1 < kTreeDepth && ck > leaf);
+  if (threadIdx.x == 0) blk[blockIdx.x] = make_int2(c1, c2);
 }
 
-// One CTA: numbers the non-empty child slots (new nodes from id `base`, in
-// slot order, so each parent's children are consecutive) and the next active
-// nodes; writes the children, links the parents, and stores the two totals.
-static __global__ void __launch_bounds__(1024)
+// Numbers the non-empty child slots (new nodes from id `base`, in slot order, so each
+// parent's children are consecutive) and the next active nodes; writes the children, links the
+// parents, and stores the two totals. Each CTA adds up the counts of the CTAs before it, a few
+// hundred words from L2 (one CTA walking all slots took 65 us at the widest level of N = 262,144).
+static __global__ void __launch_bounds__(kSlotThreads)
 tree_link_kernel(const int* __restrict__ active, int n_active, int level, int leaf, int base,
-                 const int* __restrict__ cnt, const int* __restrict__ beg, int* __restrict__ pos,
+                 const int* __restrict__ cnt, const int* __restrict__ beg, const int2* __restrict__ blk,
                  int4* __restrict__ link, float4* __restrict__ geo, uint64_t* __restrict__ pre,
                  int* __restrict__ next_active, int* __restrict__ totals) {
-  __shared__ int s1[1024], s2[1024];
-  const int m = 8 * n_active;
-  const int chunk = (m + 1023) / 1024;
-  const int b = threadIdx.x * chunk, e = min(m, b + chunk);
-  const bool deeper = level + 1 < kTreeDepth;
-  int c1 = 0, c2 = 0;
-  for (int k = b; k < e; ++k) {
-    c1 += cnt[k] > 0;
-    c2 += deeper && cnt[k] > leaf;
+  constexpr int kWarps = kSlotThreads / 32;
+  __shared__ int before1[kWarps], before2[kWarps], here1[kWarps], here2[kWarps];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+  int b1 = 0, b2 = 0;
+  for (int k = threadIdx.x; k < (int)blockIdx.x; k += kSlotThreads) {
+    const int2 c = blk[k];
+    b1 += c.x;
+    b2 += c.y;
   }
-  s1[threadIdx.x] = c1;
-  s2[threadIdx.x] = c2;
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    const int v1 = threadIdx.x >= off ? s1[threadIdx.x - off] : 0;
-    const int v2 = threadIdx.x >= off ? s2[threadIdx.x - off] : 0;
-    __syncthreads();
-    s1[threadIdx.x] += v1;
-    s2[threadIdx.x] += v2;
-    __syncthreads();
-  }
-  int p1 = s1[threadIdx.x] - c1, p2 = s2[threadIdx.x] - c2;
-  const float side = ldexpf(1.0f, -(level + 1));
-  for (int k = b; k < e; ++k) {
-    pos[k] = p1;
-    const int ck = cnt[k];
-    if (ck > 0) {
-      const int id = base + p1;
-      const uint64_t pf = (pre[active[k >> 3]] << 3) | (uint64_t)(k & 7);
-      pre[id] = pf;
-      link[id] = make_int4(-1, 0, beg[k], beg[k] + ck);
-      const uint32_t ix = compact3(pf >> 2), iy = compact3(pf >> 1), iz = compact3(pf);
-      geo[id] = make_float4(__fmul_rn((float)ix + 0.5f, side), __fmul_rn((float)iy + 0.5f, side),
-                            __fmul_rn((float)iz + 0.5f, side), side);
-      ++p1;
-      if (deeper && ck > leaf) next_active[p2++] = id;
-    }
+  b1 = __reduce_add_sync(0xffffffffu, b1);
+  b2 = __reduce_add_sync(0xffffffffu, b2);
+  const int ck = slot < 8 * n_active ? cnt[slot] : 0;
+  const bool child = ck > 0, deep = level + 1 < kTreeDepth && ck > leaf;
+  const unsigned m1 = __ballot_sync(0xffffffffu, child), m2 = __ballot_sync(0xffffffffu, deep);
+  if (lane == 0) {
+    before1[w] = b1;
+    before2[w] = b2;
+    here1[w] = __popc(m1);
+    here2[w] = __popc(m2);
   }
   __syncthreads();
-  for (int a = threadIdx.x; a < n_active; a += 1024) {
-    const int first = pos[8 * a];
-    const int last = 8 * a + 7;
-    const int nch = pos[last] + (cnt[last] > 0) - first;
-    int4 lk = link[active[a]];
-    lk.x = base + first;
-    lk.y = nch;
-    link[active[a]] = lk;
+  int p1 = __popc(m1 & ((1u << lane) - 1u)), p2 = __popc(m2 & ((1u << lane) - 1u));
+#pragma unroll
+  for (int k = 0; k < kWarps; ++k) {
+    p1 += before1[k] + (k < w ? here1[k] : 0);
+    p2 += before2[k] + (k < w ? here2[k] : 0);
   }
-  if (threadIdx.x == 1023) {
-    totals[0] = s1[1023];
-    totals[1] = s2[1023];
+  if (child) {
+    const float side = ldexpf(1.0f, -(level + 1));
+    const int id = base + p1, bk = beg[slot];
+    const uint64_t pf = (pre[active[slot >> 3]] << 3) | (uint64_t)(slot & 7);
+    pre[id] = pf;
+    link[id] = make_int4(-1, 0, bk, bk + ck);
+    const uint32_t ix = compact3(pf >> 2), iy = compact3(pf >> 1), iz = compact3(pf);
+    geo[id] = make_float4(__fmul_rn((float)ix + 0.5f, side), __fmul_rn((float)iy + 0.5f, side),
+                          __fmul_rn((float)iz + 0.5f, side), side);
+    if (deep) next_active[p2] = id;
+  }
+  if (slot < 8 * n_active && (slot & 7) == 0) {  // a node's eight slots lie in one warp
+    const int node = active[slot >> 3];
+    int4 lk = link[node];
+    lk.x = base + p1;
+    lk.y = __popc((m1 >> lane) & 0xffu);
+    link[node] = lk;
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kSlotThreads - 1) {
+    totals[0] = p1 + (child ? 1 : 0);
+    totals[1] = p2 + (deep ? 1 : 0);
   }
 }
 
-// Moments of the nodes [n0, n1) of one level, children first: a leaf sums its
-// particles (sorted order), an inner node its children (FP64). mom = (M,
+// Moments of the nodes [n0, n1): a leaf sums its particles (sorted order), all leaves in one
+// launch; then level by level from the deepest an inner node sums its children (FP64). mom = (M,
 // sum m x, sum m y, sum m z'); hmax: largest h; hmf: largest hu.
-static __global__ void tree_moments_kernel(int n0, int n1, const int4* __restrict__ link,
+template <bool LEAF>
+__global__ void tree_moments_kernel(int n0, int n1, const int4* __restrict__ link,
                                            const int* __restrict__ sidx, const double* __restrict__ x,
                                            const double* __restrict__ y, const double* __restrict__ zt,
                                            const double* __restrict__ m, const double* __restrict__ h,
@@ -334,9 +353,10 @@ static __global__ void tree_moments_kernel(int n0, int n1, const int4* __restric
   const int id = n0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= n1) return;
   const int4 lk = link[id];
+  if ((lk.y == 0) != LEAF) return;
   double M = 0.0, sx = 0.0, sy = 0.0, sz = 0.0, hm = 0.0;
   float hu = 0.0f;
-  if (lk.y == 0) {
+  if (LEAF) {
     for (int q = lk.z; q < lk.w; ++q) {
       const int i = sidx[q];
       const double mi = m[i];

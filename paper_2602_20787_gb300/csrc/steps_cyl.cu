@@ -893,10 +893,12 @@ int tree_build(steps_cyl_ctx* c, const TreeDraw& f) {
     if ((rc = tree_grow_nodes(c, nn + 8 * n_active, nn))) return rc;
     // active nodes hold > leaf particles each, so 8 n_active <= 8 (n / (leaf + 1)), the size taken above
     if (8 * n_active > T.slot_cap) return fail(STEPS_ECUDA, "octree build: child slots exceed their bound");
-    tree_children_kernel<<<(8 * n_active + 255) / 256, 256, 0, c->st>>>(T.active[cur], n_active, level, key, T.link,
-                                                                       T.pre, T.cnt, T.beg);
-    tree_link_kernel<<<1, 1024, 0, c->st>>>(T.active[cur], n_active, level, leaf, nn, T.cnt, T.beg, T.pos, T.link,
-                                            T.geo, T.pre, T.active[cur ^ 1], T.totals);
+    const int g = (8 * n_active + kSlotThreads - 1) / kSlotThreads;  // <= slot_cap / 2 counts fit pos
+    int2* blk = reinterpret_cast<int2*>(T.pos);
+    tree_children_kernel<<<g, kSlotThreads, 0, c->st>>>(T.active[cur], n_active, level, leaf, key, T.link, T.pre, T.cnt,
+                                                        T.beg, blk);
+    tree_link_kernel<<<g, kSlotThreads, 0, c->st>>>(T.active[cur], n_active, level, leaf, nn, T.cnt, T.beg, blk, T.link,
+                                                    T.geo, T.pre, T.active[cur ^ 1], T.totals);
     CKLAUNCH("tree_level");
     CKT(cudaMemcpyAsync(T.totals_h, T.totals, sizeof(int) * 2, cudaMemcpyDeviceToHost, c->st));
     CKT(cudaStreamSynchronize(c->st));
@@ -907,11 +909,13 @@ int tree_build(steps_cyl_ctx* c, const TreeDraw& f) {
   }
   T.nodes = nn;
   T.depth = (int)lstart.size() - 2;
-  for (int l = (int)lstart.size() - 2; l >= 0; --l) {
+  tree_moments_kernel<true><<<(nn + 63) / 64, 64, 0, c->st>>>(0, nn, T.link, sidx, c->x, c->y, T.zt, c->m, c->h, T.u4,
+                                                              T.mom, T.hmx, T.hmf);
+  for (int l = (int)lstart.size() - 3; l >= 0; --l) {  // the deepest level has leaves alone
     const int a = lstart[l], b = lstart[l + 1];
     if (b <= a) continue;
-    tree_moments_kernel<<<(b - a + 255) / 256, 256, 0, c->st>>>(a, b, T.link, sidx, c->x, c->y, T.zt, c->m, c->h,
-                                                               T.u4, T.mom, T.hmx, T.hmf);
+    tree_moments_kernel<false><<<(b - a + 63) / 64, 64, 0, c->st>>>(a, b, T.link, sidx, c->x, c->y, T.zt, c->m, c->h,
+                                                                   T.u4, T.mom, T.hmx, T.hmf);
   }
   tree_pack_kernel<<<grid_for(nn, 256), 256, 0, c->st>>>(nn, T.mom, T.hmx, zeta, c->p.L, c->invL, is_r3(c) ? 0 : 1,
                                                          T.nA, T.nB);
