@@ -124,6 +124,14 @@ __device__ __forceinline__ void radial_correct(const RadialCorr& R, double x, do
   if (R.sph) g2 -= D * z / rho;
 }
 
+// Accelerations a = g / a^3 written besides (x null: none), in the caller's order when perm maps
+// the internal index to it.
+struct AccelOut {
+  double *x, *y, *z;
+  double inv_a3;
+  const int* perm;
+};
+
 // The common end of a finalize: the pair sums (sx, sy, sz) scaled to the
 // comoving field g = a^3 (pair + background), the radial correction, the
 // background; g stored, optionally p += g K, optionally a = g / a^3 written.
@@ -132,9 +140,8 @@ __device__ __forceinline__ void finish_particle(int i, double sx, double sy, dou
                                                 const double* __restrict__ y, const double* __restrict__ z,
                                                 double* __restrict__ gx, double* __restrict__ gy,
                                                 double* __restrict__ gz, double K, double* __restrict__ px,
-                                                double* __restrict__ py, double* __restrict__ pz, double inv_a3,
-                                                double* __restrict__ ox, double* __restrict__ oy,
-                                                double* __restrict__ oz, int* __restrict__ err, const RadialCorr& rc) {
+                                                double* __restrict__ py, double* __restrict__ pz, const AccelOut& out,
+                                                int* __restrict__ err, const RadialCorr& rc) {
   double g0 = pair_scale * sx, g1 = pair_scale * sy, g2 = pair_scale * sz;
   radial_correct(rc, x[i], y[i], z[i], g0, g1, g2);
   add_background(bg, x[i], y[i], z[i], g0, g1, g2, err);
@@ -145,20 +152,26 @@ __device__ __forceinline__ void finish_particle(int i, double sx, double sy, dou
     py[i] += g1 * K;
     pz[i] += g2 * K;
   }
-  if (ox) {
-    ox[i] = g0 * inv_a3;
-    oy[i] = g1 * inv_a3;
-    oz[i] = g2 * inv_a3;
+  if (out.x) {
+    const int o = out.perm ? out.perm[i] : i;
+    out.x[o] = g0 * out.inv_a3;
+    out.y[o] = g1 * out.inv_a3;
+    out.z[o] = g2 * out.inv_a3;
   }
 }
+
+// Threads per CTA of the O(N) kernels with FP64 work per particle (this finalize, its
+// fixed-point form, the kick and drift). An SM's FP64 pipe takes a warp's instruction in 16 cycles, so what
+// counts is how many SMs share the particles: at N = 2,048, CTAs of 256 leave 144 of 152 SMs
+// idle (finalize 10.2 us, kick and drift 6.0).
+inline int particle_threads(int n) { return n <= 152 * 8 * 32 ? 32 : 128; }
 
 static __global__ void finalize_kernel(const double* __restrict__ part, int n, int NT, long long U, int C,
                                 double pair_scale, BgParams bg, const double* __restrict__ x,
                                 const double* __restrict__ y, const double* __restrict__ z, double* __restrict__ gx,
                                 double* __restrict__ gy, double* __restrict__ gz, double K,
                                 double* __restrict__ px, double* __restrict__ py, double* __restrict__ pz,
-                                double inv_a3, double* __restrict__ ox, double* __restrict__ oy,
-                                double* __restrict__ oz, int* __restrict__ err,
+                                AccelOut out, int* __restrict__ err,
                                 RadialCorr rc = RadialCorr{nullptr, 0, 0.0, 0}, int i0 = 0) {
   // rows [i0, n), i0 a multiple of kBI (all rows unless they are sharded); the
   // partials and direct sums are indexed from i0
@@ -182,7 +195,7 @@ static __global__ void finalize_kernel(const double* __restrict__ part, int n, i
       sz += q[2 * kBI + l];
     }
   }
-  finish_particle(i, sx, sy, sz, pair_scale, bg, x, y, z, gx, gy, gz, K, px, py, pz, inv_a3, ox, oy, oz, err, rc);
+  finish_particle(i, sx, sy, sz, pair_scale, bg, x, y, z, gx, gy, gz, K, px, py, pz, out, err, rc);
 }
 
 // Finalize from the fixed-point accumulators of the symmetric pair kernels
@@ -195,18 +208,19 @@ static __global__ void finalize_fix_kernel(const unsigned long long* __restrict_
                                            const double* __restrict__ z, double* __restrict__ gx,
                                            double* __restrict__ gy, double* __restrict__ gz, double K,
                                            double* __restrict__ px, double* __restrict__ py,
-                                           double* __restrict__ pz, int* __restrict__ err) {
+                                           double* __restrict__ pz, AccelOut out, int* __restrict__ err) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = i0 + q;
   if (i >= n) return;
   const double sx = (double)(long long)acc[q] * inv_scale;
   const double sy = (double)(long long)acc[(long long)stride + q] * inv_scale;
   const double sz = (double)(long long)acc[2 * (long long)stride + q] * inv_scale;
-  finish_particle(i, sx, sy, sz, pair_scale, bg, x, y, z, gx, gy, gz, K, px, py, pz, 1.0, nullptr, nullptr, nullptr,
-                  err, RadialCorr{nullptr, 0, 0.0, 0});
+  finish_particle(i, sx, sy, sz, pair_scale, bg, x, y, z, gx, gy, gz, K, px, py, pz, out, err,
+                  RadialCorr{nullptr, 0, 0.0, 0});
 }
 
-// First half of a KDK step: p += g K1; x += p D; z wrapped into [0, L); repack.
+// First half of a KDK step: p += g K1; x += p D; z wrapped into [0, L); repack. facc (may be
+// null): the fixed-point sums [3][n] of the force evaluation that follows, set to zero.
 static __global__ void kick_drift_pack_kernel(double* __restrict__ x, double* __restrict__ y,
                                        double* __restrict__ z, double* __restrict__ px,
                                        double* __restrict__ py, double* __restrict__ pz,
@@ -214,8 +228,13 @@ static __global__ void kick_drift_pack_kernel(double* __restrict__ x, double* __
                                        const double* __restrict__ gz, const double* __restrict__ m,
                                        const double* __restrict__ h, int n, double K1, double D, double L,
                                        double invL, float4* __restrict__ jA, float4* __restrict__ jB,
-                                       int* __restrict__ err, int wrap) {
+                                       int* __restrict__ err, int wrap, unsigned long long* __restrict__ facc) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    if (facc) {
+      facc[i] = 0;
+      facc[(size_t)n + i] = 0;
+      facc[2 * (size_t)n + i] = 0;
+    }
     const double qx = px[i] + gx[i] * K1, qy = py[i] + gy[i] * K1, qz = pz[i] + gz[i] * K1;
     px[i] = qx; py[i] = qy; pz[i] = qz;
     const double nx = x[i] + qx * D, ny = y[i] + qy * D;

@@ -464,10 +464,16 @@ __global__ void gather_kernel(const double* __restrict__ src, const int* __restr
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) dst[k] = s * src[map[k]];
 }
 
-// dst[map[k]] = s * src[k]
-__global__ void scatter_kernel(const double* __restrict__ src, const int* __restrict__ map, int n, double s,
-                               double* __restrict__ dst) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) dst[map[k]] = s * src[k];
+// dst[map[k]] = s * src[k] for three arrays (null destinations left out)
+__global__ void scatter3_kernel(const double* __restrict__ s0, const double* __restrict__ s1,
+                                const double* __restrict__ s2, const int* __restrict__ map, int n, double s,
+                                double* __restrict__ d0, double* __restrict__ d1, double* __restrict__ d2) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int o = map[k];
+    if (d0) d0[o] = s * s0[k];
+    if (d1) d1[o] = s * s1[k];
+    if (d2) d2[o] = s * s2[k];
+  }
 }
 
 // dst[map[k]] = s * src[k] for k in [k0, k1), 0 for the other k
@@ -1183,11 +1189,13 @@ int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const Fix
 }
 
 // One force evaluation at the current packed positions. Stores g = a^3 (pair +
-// background) in gx/gy/gz (internal order); kicks p by K when kick is set.
-int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
+// background) in gx/gy/gz (internal order); kicks p by K when kick is set; writes the accelerations
+// to out besides. cleared: the fixed-point sums are zero already.
+int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = AccelOut{}, bool cleared = false) {
   Range range("steps_cyl.forces");
   const double pair_scale = -c->p.G * c->invL * c->invL;
   c->forces_stale = false;
+  const int ft = particle_threads(c->n);
   if (is_tree(c)) {  // the octree: its own build and walk, then the common finalize
     CK(cudaEventRecord(c->e0, c->st));
     int rc = tree_forces(c, c->part);
@@ -1197,10 +1205,9 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
     c->last_images = c->tr.interactions;
     c->last_pairs = c->tr.interactions;
     c->last_sym = false;
-    finalize_kernel<<<(c->n + 255) / 256, 256, 0, c->st>>>(
+    finalize_kernel<<<(c->n + ft - 1) / ft, ft, 0, c->st>>>(
         c->part, c->n, 0, c->U, c->C, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K,
-        kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, 1.0, nullptr, nullptr, nullptr,
-        c->err, radial_corr(c));
+        kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, out, c->err, radial_corr(c));
     CKLAUNCH("finalize");
     return STEPS_OK;
   }
@@ -1211,7 +1218,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
     if (rc) return rc;
   }
   if (form != Form::FP64 && use_sym(c)) {
-    CK(cudaMemsetAsync(c->facc, 0, sizeof(unsigned long long) * 3 * (size_t)c->n, c->st));
+    if (!cleared) CK(cudaMemsetAsync(c->facc, 0, sizeof(unsigned long long) * 3 * (size_t)c->n, c->st));
     CK(cudaEventRecord(c->e0, c->st));
     int rc = launch_sym(c, form, 0, c->Usym, FixAcc{c->facc, c->n, c->fix_scale, fix_scale_f(c), c->err, 0, 0, 0, 0});
     if (rc) return rc;
@@ -1220,9 +1227,9 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
     c->last_images = (double)c->n * (double)(c->n - 1) * images_per_pair(c);
     c->last_pairs = sym_pairs(c);
     c->last_sym = true;
-    finalize_fix_kernel<<<(c->n + 255) / 256, 256, 0, c->st>>>(
+    finalize_fix_kernel<<<(c->n + ft - 1) / ft, ft, 0, c->st>>>(
         c->facc, c->n, 0, c->n, 1.0 / c->fix_scale, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz,
-        K, kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, c->err);
+        K, kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, out, c->err);
     CKLAUNCH("finalize_fix");
     return STEPS_OK;
   }
@@ -1282,9 +1289,9 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K) {
   const int NT = form == Form::FP64 ? 0 : c->NT;
   const int ctas = form == Form::SURROGATE ? c->SC : form == Form::TABLE ? c->TC : c->C;
   // rows [k0, k1): every row, or the rows this context owns when they are sharded
-  finalize_kernel<<<(c->k1 - c->k0 + 255) / 256, 256, 0, c->st>>>(
+  finalize_kernel<<<(c->k1 - c->k0 + ft - 1) / ft, ft, 0, c->st>>>(
       c->part, c->k1, NT, c->U, ctas, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K,
-      kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, 1.0, nullptr, nullptr, nullptr, c->err,
+      kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, out, c->err,
       RadialCorr{nullptr, 0, 0.0, 0}, c->k0);
   CKLAUNCH("finalize");
   return STEPS_OK;
@@ -1436,19 +1443,24 @@ struct DeviceGuard {
 // rows and zeros elsewhere, so a sum over the ranks assembles the whole.
 int scatter_out(steps_cyl_ctx* c, const double* const src[3], double* const dst[3], double scale) {
   bool host = false;
+  double* d[3];
   for (int q = 0; q < 3; ++q) {
-    if (!dst[q]) continue;
-    double* d = is_host_ptr(dst[q]) ? c->stage + (size_t)q * c->n : dst[q];
-    if (c->shard)
-      scatter_rows_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(src[q], c->perm, c->n, scale, c->k0, c->k1, d);
-    else
-      scatter_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(src[q], c->perm, c->n, scale, d);
-    CKLAUNCH("scatter");
-    if (d != dst[q]) {
-      CK(cudaMemcpyAsync(dst[q], d, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
-      host = true;
-    }
+    const bool h = dst[q] && is_host_ptr(dst[q]);
+    d[q] = h ? c->stage + (size_t)q * c->n : dst[q];
+    host = host || h;
   }
+  if (c->shard) {
+    for (int q = 0; q < 3; ++q)
+      if (d[q])
+        scatter_rows_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(src[q], c->perm, c->n, scale, c->k0, c->k1, d[q]);
+  } else {
+    scatter3_kernel<<<grid_for(c->n, 128), 128, 0, c->st>>>(src[0], src[1], src[2], c->perm, c->n, scale, d[0], d[1],
+                                                            d[2]);
+  }
+  CKLAUNCH("scatter");
+  for (int q = 0; q < 3; ++q)
+    if (d[q] != dst[q])
+      CK(cudaMemcpyAsync(dst[q], d[q], sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
   if (host) CK(cudaStreamSynchronize(c->st));
   return STEPS_OK;
 }
@@ -2370,11 +2382,15 @@ int steps_cyl_forces(steps_cyl_ctx* c, double* ax, double* ay, double* az) {
   if (c->drifted) return fail(STEPS_EINVAL, "a sharded step is half done: steps_cyl_shard_kick must come first");
   DeviceGuard guard(c->dev);
   int rc;
+  const double inv_a3 = 1.0 / (c->a * c->a * c->a);
+  const bool host = is_host_ptr(ax) || is_host_ptr(ay) || is_host_ptr(az);
+  if (!host && !c->shard)  // device outputs: written by the finalize kernel
+    return eval_forces(c, false, 0.0, AccelOut{ax, ay, az, inv_a3, c->perm});
   if ((rc = eval_forces(c, false, 0.0))) return rc;
   const double* src[3] = {c->gx, c->gy, c->gz};
   double* dst[3] = {ax, ay, az};
-  if ((rc = scatter_out(c, src, dst, 1.0 / (c->a * c->a * c->a)))) return rc;
-  if (is_host_ptr(ax) || is_host_ptr(ay) || is_host_ptr(az)) {
+  if ((rc = scatter_out(c, src, dst, inv_a3))) return rc;
+  if (host) {
     int e = 0;
     if ((rc = read_and_clear_err(c, &e))) return rc;
     if (e) return device_error(e);
@@ -2451,11 +2467,12 @@ int steps_cyl_kdk_step(steps_cyl_ctx* c, double dt, int32_t nsteps) {
     const Factors f = kdk_factors(c->cosmo, c->a, dt);
     if (!std::isfinite(f.K1) || !std::isfinite(f.D) || !std::isfinite(f.a_next) || !(f.a_next > 0))
       return fail(STEPS_EINVAL, "the Friedmann integration left the valid range (a = %g)", f.a_next);
-    kick_drift_pack_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(c->x, c->y, c->z, c->px, c->py, c->pz, c->gx,
-                                                                   c->gy, c->gz, c->m, c->h, c->n, f.K1, f.D, c->p.L,
-                                                                   c->invL, c->jA, c->jB, c->err, is_r3(c) ? 0 : 1);
+    const int kt = particle_threads(c->n);
+    kick_drift_pack_kernel<<<grid_for(c->n, kt), kt, 0, c->st>>>(c->x, c->y, c->z, c->px, c->py, c->pz, c->gx, c->gy,
+                                                                 c->gz, c->m, c->h, c->n, f.K1, f.D, c->p.L, c->invL,
+                                                                 c->jA, c->jB, c->err, is_r3(c) ? 0 : 1, c->facc);
     CKLAUNCH("kick_drift_pack");
-    if ((rc = eval_forces(c, true, f.K2))) return rc;
+    if ((rc = eval_forces(c, true, f.K2, AccelOut{}, true))) return rc;
     c->a = f.a_next;
     c->t += dt;
     if (c->p.reorder_every > 0 && ++c->steps_since_order >= c->p.reorder_every) {
@@ -2639,7 +2656,7 @@ int steps_cyl_shard_drift(steps_cyl_ctx* c, double dt, float* send) {
   const int k0 = c->k0, rows = c->k1 - c->k0;
   kick_drift_pack_kernel<<<grid_for(rows, 256), 256, 0, c->st>>>(
       c->x + k0, c->y + k0, c->z + k0, c->px + k0, c->py + k0, c->pz + k0, c->gx + k0, c->gy + k0, c->gz + k0,
-      c->m + k0, c->h + k0, rows, f.K1, f.D, c->p.L, c->invL, c->jA + k0, c->jB + k0, c->err, is_r3(c) ? 0 : 1);
+      c->m + k0, c->h + k0, rows, f.K1, f.D, c->p.L, c->invL, c->jA + k0, c->jB + k0, c->err, is_r3(c) ? 0 : 1, nullptr);
   CKLAUNCH("kick_drift_pack");
   shard_send_kernel<<<grid_for(c->chunk, 256), 256, 0, c->st>>>(c->jA, c->jB, k0, rows, c->chunk,
                                                                  reinterpret_cast<float4*>(send));
@@ -2738,10 +2755,11 @@ int steps_cyl_shard_finish(steps_cyl_ctx* c, const int64_t* own) {
   DeviceGuard guard(c->dev);
   Range range("steps_cyl.shard_finish");
   const int rows = c->k1 - c->k0;
-  finalize_fix_kernel<<<(rows + 255) / 256, 256, 0, c->st>>>(
+  const int ft = particle_threads(rows);
+  finalize_fix_kernel<<<(rows + ft - 1) / ft, ft, 0, c->st>>>(
       reinterpret_cast<const unsigned long long*>(own), c->k1, c->k0, c->chunk, 1.0 / c->fix_scale,
       -c->p.G * c->invL * c->invL, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, c->pend_K2, c->px, c->py,
-      c->pz, c->err);
+      c->pz, AccelOut{}, c->err);
   CKLAUNCH("finalize_fix");
   c->forces_stale = false;
   c->a = c->pend_a;

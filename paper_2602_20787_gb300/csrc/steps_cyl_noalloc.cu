@@ -139,9 +139,9 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   kernel<<<C, kPairThreads, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part, 0);
   BgParams off{};
   off.mode = STEPS_BG_OFF;
-  finalize_kernel<<<(nn + 255) / 256, 256, 0, st>>>(part, nn, NT, U, C, -G * invL * invL, off, x, y, z, ax, ay, az,
-                                                    0.0, nullptr, nullptr, nullptr, 1.0, nullptr, nullptr, nullptr,
-                                                    nullptr);
+  const int ft = particle_threads(nn);
+  finalize_kernel<<<(nn + ft - 1) / ft, ft, 0, st>>>(part, nn, NT, U, C, -G * invL * invL, off, x, y, z, ax, ay, az,
+                                                     0.0, nullptr, nullptr, nullptr, AccelOut{}, nullptr);
   // a launch failure replaces the thread's last error; one equal to the error
   // pending before the call is taken as the caller's, which stays in place
   const cudaError_t after = cudaPeekAtLastError();
