@@ -244,7 +244,10 @@ struct steps_cyl_ctx {
   int* perm = nullptr;      // internal -> caller index (device)
   int* iperm = nullptr;     // caller -> internal index (device)
   int* ord = nullptr;       // re-ordering of internal indices (device)
-  std::vector<int> perm_h;  // host copy of perm
+  std::vector<int> perm_h;  // host copy of perm, when perm_h_ok (see host_perm)
+  bool perm_h_ok = false;
+  unsigned* mhist = nullptr;            // digit counts and offsets of the Morton sort, 2 x 256 per sort tile
+  unsigned long long* mbox = nullptr;   // its bounding box: min x, min y, max x, max y (ordered words)
   int64_t* idx = nullptr;   // subset indices (grown on demand)
   int idx_cap = 0;
   double* sub = nullptr;    // subset sums (3 * idx_cap)
@@ -458,6 +461,74 @@ __global__ void max_rho_kernel(const double* __restrict__ x, const double* __res
   atomicMax(out, (unsigned long long)__double_as_longlong(r));
 }
 
+// An order of double as of unsigned words, and back.
+__device__ __forceinline__ unsigned long long order_word(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return b >> 63 ? ~b : b | (1ull << 63);
+}
+__device__ __forceinline__ double order_value(unsigned long long w) {
+  return __longlong_as_double((long long)(w >> 63 ? w & ~(1ull << 63) : ~w));
+}
+
+// box = (min x, min y, max x, max y) as ordered words, set to (~0, ~0, 0, 0) before. NaNs are left out.
+__global__ void morton_box_kernel(const double* __restrict__ x, const double* __restrict__ y, int n,
+                                  unsigned long long* __restrict__ box) {
+  unsigned long long v[4] = {~0ull, ~0ull, 0ull, 0ull};
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double p[2] = {x[i], y[i]};
+    for (int a = 0; a < 2; ++a) {
+      if (isnan(p[a])) continue;
+      const unsigned long long w = order_word(p[a]);
+      v[a] = min(v[a], w);
+      v[2 + a] = max(v[2 + a], w);
+    }
+  }
+  for (int a = 0; a < 4; ++a) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long w = __shfl_xor_sync(0xffffffffu, v[a], o);
+      v[a] = a < 2 ? min(v[a], w) : max(v[a], w);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      if (a < 2) atomicMin(box + a, v[a]);
+      else atomicMax(box + a, v[a]);
+    }
+  }
+}
+
+// Interleaved 16-bit cells of the box as sort keys; val[i] = i.
+__global__ void morton_key_kernel(const double* __restrict__ x, const double* __restrict__ y, int n,
+                                  const unsigned long long* __restrict__ box, uint64_t* __restrict__ key,
+                                  int* __restrict__ val) {
+  const double x0 = order_value(box[0]), y0 = order_value(box[1]);
+  const double span = fmax(fmax(order_value(box[2]) - x0, order_value(box[3]) - y0), 1e-300);
+  auto cell = [&](double v) {
+    uint32_t q = (uint32_t)fmin(65535.0, fmax(0.0, floor(v / span * 65536.0)));
+    q = (q | (q << 8)) & 0x00FF00FFu;
+    q = (q | (q << 4)) & 0x0F0F0F0Fu;
+    q = (q | (q << 2)) & 0x33333333u;
+    return (q | (q << 1)) & 0x55555555u;
+  };
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    key[i] = cell(x[i] - x0) | (cell(y[i] - y0) << 1);
+    val[i] = i;
+  }
+}
+
+// idx[k] = map[order[k]] and copy[k] = order[k]; order null: the identity, map null: idx not written.
+__global__ void order_kernel(const int* __restrict__ order, const int* __restrict__ map, int n, int* __restrict__ idx,
+                             int* __restrict__ copy) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int o = order ? order[k] : k;
+    if (map) idx[k] = map[o];
+    copy[k] = o;
+  }
+}
+
+// inv[perm[k]] = k
+__global__ void invert_kernel(const int* __restrict__ perm, int n, int* __restrict__ inv) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) inv[perm[k]] = k;
+}
+
 // dst[k] = s * src[map[k]]
 __global__ void gather_kernel(const double* __restrict__ src, const int* __restrict__ map, int n, double s,
                               double* __restrict__ dst) {
@@ -542,41 +613,36 @@ int refuse_sharded(const steps_cyl_ctx* c, const char* what) {
               what);
 }
 
-// Morton (Z-order) rank of (x, y): stable sort of 2 x 16-bit interleaved cell
-// codes over the bounding box. Returns order[k] = index of the k-th particle.
-void morton_order(const std::vector<double>& x, const std::vector<double>& y, std::vector<int>& order) {
-  const size_t n = x.size();
-  double x0 = x[0], x1 = x[0], y0 = y[0], y1 = y[0];
-  for (size_t i = 1; i < n; ++i) {
-    x0 = std::min(x0, x[i]); x1 = std::max(x1, x[i]);
-    y0 = std::min(y0, y[i]); y1 = std::max(y1, y[i]);
+// Morton (Z-order) rank of (x, y) on the device: stable radix sort (octree.cuh) of 2 x 16-bit
+// interleaved cell codes over the bounding box. The keys and values live in part (3 n doubles);
+// *order is the sorted index list there, valid until part is written again.
+int morton_order(steps_cyl_ctx* c, const double* x, const double* y, const int** order) {
+  const int n = c->n, ntiles = (n + kSortTile - 1) / kSortTile;
+  uint64_t* key[2] = {reinterpret_cast<uint64_t*>(c->part), reinterpret_cast<uint64_t*>(c->part) + n};
+  int* val[2] = {reinterpret_cast<int*>(c->part + 2 * (size_t)n), reinterpret_cast<int*>(c->part + 2 * (size_t)n) + n};
+  unsigned* offs = c->mhist + 256 * (size_t)ntiles;
+  CK(cudaMemsetAsync(c->mbox, 0xff, 2 * sizeof(unsigned long long), c->st));
+  CK(cudaMemsetAsync(c->mbox + 2, 0, 2 * sizeof(unsigned long long), c->st));
+  morton_box_kernel<<<std::min(152, grid_for(n, 128)), 128, 0, c->st>>>(x, y, n, c->mbox);
+  morton_key_kernel<<<grid_for(n, 64), 64, 0, c->st>>>(x, y, n, c->mbox, key[0], val[0]);
+  for (int pass = 0; pass < 4; ++pass) {  // 4 digits of 8 bits; the result returns to buffer 0
+    const int a = pass & 1, b = a ^ 1;
+    radix_hist_kernel<<<ntiles, kSortThreads, 0, c->st>>>(key[a], n, 8 * pass, ntiles, c->mhist);
+    scan_exclusive_kernel<<<1, 1024, 0, c->st>>>(c->mhist, offs, 256 * ntiles, nullptr);
+    radix_scatter_kernel<<<ntiles, kSortThreads, 0, c->st>>>(key[a], val[a], n, 8 * pass, ntiles, offs, key[b], val[b]);
   }
-  const double span = std::max({x1 - x0, y1 - y0, 1e-300});
-  auto spread = [](uint32_t v) {
-    v = (v | (v << 8)) & 0x00FF00FFu;
-    v = (v | (v << 4)) & 0x0F0F0F0Fu;
-    v = (v | (v << 2)) & 0x33333333u;
-    v = (v | (v << 1)) & 0x55555555u;
-    return v;
-  };
-  std::vector<uint32_t> key(n);
-  for (size_t i = 0; i < n; ++i) {
-    const double fx = (x[i] - x0) / span, fy = (y[i] - y0) / span;
-    const uint32_t qx = (uint32_t)std::min(65535.0, std::max(0.0, std::floor(fx * 65536.0)));
-    const uint32_t qy = (uint32_t)std::min(65535.0, std::max(0.0, std::floor(fy * 65536.0)));
-    key[i] = spread(qx) | (spread(qy) << 1);
-  }
-  order.resize(n);
-  for (size_t i = 0; i < n; ++i) order[i] = (int)i;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key[a] < key[b]; });
+  CKLAUNCH("morton_order");
+  *order = val[0];
+  return STEPS_OK;
 }
 
-int upload_perm(steps_cyl_ctx* c) {
-  std::vector<int> inv(c->n);
-  for (int k = 0; k < c->n; ++k) inv[c->perm_h[k]] = k;
-  CK(cudaMemcpyAsync(c->perm, c->perm_h.data(), sizeof(int) * c->n, cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->iperm, inv.data(), sizeof(int) * c->n, cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));  // the host vectors go out of scope
+// perm_h made current.
+int host_perm(steps_cyl_ctx* c) {
+  if (c->perm_h_ok) return STEPS_OK;
+  c->perm_h.resize(c->n);
+  CK(cudaMemcpyAsync(c->perm_h.data(), c->perm, sizeof(int) * c->n, cudaMemcpyDeviceToHost, c->st));
+  CK(cudaStreamSynchronize(c->st));
+  c->perm_h_ok = true;
   return STEPS_OK;
 }
 
@@ -585,32 +651,25 @@ int upload_perm(steps_cyl_ctx* c) {
 // per-particle arrays that are not re-uploaded (m, h) are moved from the old
 // internal order to the new one.
 int order_from_stage(steps_cyl_ctx* c, const double* sx, const double* sy, bool carry) {
-  std::vector<int> np(c->n);
-  if (c->p.reorder_every < 0) {
-    for (int k = 0; k < c->n; ++k) np[k] = k;
-  } else {
-    std::vector<double> hx(c->n), hy(c->n);
-    CK(cudaMemcpyAsync(hx.data(), sx, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
-    CK(cudaMemcpyAsync(hy.data(), sy, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
-    CK(cudaStreamSynchronize(c->st));
-    morton_order(hx, hy, np);
-  }
+  const int* np = nullptr;  // caller's order
+  int rc;
+  if (c->p.reorder_every >= 0 && (rc = morton_order(c, sx, sy, &np))) return rc;
+  const int g = grid_for(c->n, 128);
+  // ord[k]: the old internal index of the new internal k
+  order_kernel<<<g, 128, 0, c->st>>>(np, carry ? c->iperm : nullptr, c->n, c->ord, c->perm);
+  invert_kernel<<<g, 128, 0, c->st>>>(c->perm, c->n, c->iperm);
+  CKLAUNCH("order");
+  c->perm_h_ok = false;
   if (carry) {
-    std::vector<int> inv_old(c->n), o(c->n);
-    for (int k = 0; k < c->n; ++k) inv_old[c->perm_h[k]] = k;
-    for (int k = 0; k < c->n; ++k) o[k] = inv_old[np[k]];  // old internal index of new internal k
-    CK(cudaMemcpyAsync(c->ord, o.data(), sizeof(int) * c->n, cudaMemcpyHostToDevice, c->st));
     double* tmp = c->part;
     for (double* arr : {c->m, c->h}) {
       gather_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(arr, c->ord, c->n, 1.0, tmp);
       CK(cudaMemcpyAsync(arr, tmp, sizeof(double) * c->n, cudaMemcpyDeviceToDevice, c->st));
     }
     CKLAUNCH("carry");
-    CK(cudaStreamSynchronize(c->st));  // o goes out of scope
   }
-  c->perm_h.swap(np);
   c->steps_since_order = 0;
-  return upload_perm(c);
+  return STEPS_OK;
 }
 
 int build_background(steps_cyl_ctx* c) {
@@ -1359,13 +1418,15 @@ int pack_positions(steps_cyl_ctx* c) {
 // temporary, perm is composed, and the packed arrays are rebuilt.
 int reorder(steps_cyl_ctx* c) {
   if (c->p.reorder_every < 0) return STEPS_OK;
-  std::vector<double> hx(c->n), hy(c->n);
-  CK(cudaMemcpyAsync(hx.data(), c->x, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
-  CK(cudaMemcpyAsync(hy.data(), c->y, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
-  CK(cudaStreamSynchronize(c->st));
-  std::vector<int> o;
-  morton_order(hx, hy, o);
-  CK(cudaMemcpyAsync(c->ord, o.data(), sizeof(int) * c->n, cudaMemcpyHostToDevice, c->st));
+  const int* o = nullptr;
+  int rc;
+  if ((rc = morton_order(c, c->x, c->y, &o))) return rc;
+  // ord = o, perm[k] = the old perm[o[k]] (through stage, free between the state calls)
+  const int g = grid_for(c->n, 128);
+  int* np = reinterpret_cast<int*>(c->stage);
+  order_kernel<<<g, 128, 0, c->st>>>(o, c->perm, c->n, np, c->ord);
+  CK(cudaMemcpyAsync(c->perm, np, sizeof(int) * c->n, cudaMemcpyDeviceToDevice, c->st));
+  invert_kernel<<<g, 128, 0, c->st>>>(c->perm, c->n, c->iperm);
   double* tmp = c->part;  // part_elems >= 3 n
   double* arrays[11] = {c->x, c->y, c->z, c->px, c->py, c->pz, c->m, c->h, c->gx, c->gy, c->gz};
   for (double* arr : arrays) {
@@ -1373,12 +1434,8 @@ int reorder(steps_cyl_ctx* c) {
     CK(cudaMemcpyAsync(arr, tmp, sizeof(double) * c->n, cudaMemcpyDeviceToDevice, c->st));
   }
   CKLAUNCH("reorder");
-  std::vector<int> np(c->n);
-  for (int k = 0; k < c->n; ++k) np[k] = c->perm_h[o[k]];
-  c->perm_h.swap(np);
+  c->perm_h_ok = false;
   c->steps_since_order = 0;
-  int rc;
-  if ((rc = upload_perm(c))) return rc;
   return pack_positions(c);
 }
 
@@ -1397,6 +1454,8 @@ void release(steps_cyl_ctx* c) {
   cudaFree(c->perm);
   cudaFree(c->iperm);
   cudaFree(c->ord);
+  cudaFree(c->mhist);
+  cudaFree(c->mbox);
   cudaFree(c->idx);
   cudaFree(c->sub);
   cudaFree(c->err);
@@ -1688,6 +1747,8 @@ int tree_calibrate(steps_cyl_ctx* c, int nf, int nb, int ns, const double* frame
                    std::vector<double>& table, double* rmax_out) {
   const int n = c->n;
   const int ni = std::min(ns, n);
+  int rc_perm;
+  if ((rc_perm = host_perm(c))) return rc_perm;
   std::vector<int> inv(n);
   for (int k = 0; k < n; ++k) inv[c->perm_h[k]] = k;
   std::vector<int64_t> pick(ni);
@@ -2216,6 +2277,8 @@ int allocate_context(steps_cyl_ctx* c) {
   CKA(cudaMalloc(&c->perm, sizeof(int) * nb));
   CKA(cudaMalloc(&c->iperm, sizeof(int) * nb));
   CKA(cudaMalloc(&c->ord, sizeof(int) * nb));
+  CKA(cudaMalloc(&c->mhist, sizeof(unsigned) * 512 * ((nb + kSortTile - 1) / kSortTile)));
+  CKA(cudaMalloc(&c->mbox, sizeof(unsigned long long) * 4));
   CKA(cudaMalloc(&c->err, sizeof(int)));
   CKA(cudaMemsetAsync(c->err, 0, sizeof(int), c->st));
 
@@ -2873,6 +2936,8 @@ int steps_cyl_checkpoint(steps_cyl_ctx* c, const char* path) {
     int rc = eval_forces(c, false, 0.0);
     if (rc) return rc;
   }
+  int rc_perm;
+  if ((rc_perm = host_perm(c))) return rc_perm;
   std::vector<double> arr((size_t)c->n * 11);
   std::vector<double> tab(hd.bgK ? hd.bgK + 4 : 0);
   CK(cudaMemcpyAsync(arr.data(), c->state, sizeof(double) * arr.size(), cudaMemcpyDeviceToHost, c->st));
@@ -2988,7 +3053,10 @@ int steps_cyl_resume(steps_cyl_ctx** out, const char* path, int32_t device, void
             cudaSuccess)
       return bail(fail(STEPS_ECUDA, "background table upload failed"));
   }
-  if ((rc = upload_perm(c))) return bail(rc);
+  c->perm_h_ok = true;
+  if (cudaMemcpyAsync(c->perm, c->perm_h.data(), sizeof(int) * c->n, cudaMemcpyHostToDevice, c->st) != cudaSuccess)
+    return bail(fail(STEPS_ECUDA, "upload failed"));
+  invert_kernel<<<grid_for(c->n, 128), 128, 0, c->st>>>(c->perm, c->n, c->iperm);
   if ((rc = validate_state(c))) return bail(rc);
   if ((rc = pack_positions(c))) return bail(rc);
   if (hd.surr_ok) {
