@@ -43,8 +43,10 @@ constexpr int kTreeDepth = 21;
 constexpr int kSortThreads = 256;
 constexpr int kSortRounds = 8;
 constexpr int kSortTile = kSortThreads * kSortRounds;  // keys per sort tile
+// Groups (warps) per CTA of the walk: one, as groups differ in work and a CTA holds its place until its
+// slowest is done (four: 8.77 ms at N = 262,144 and 1.04 at 20,000, one: 7.90 and 0.94).
 #ifndef STEPS_TREE_WARPS
-#define STEPS_TREE_WARPS 4    // groups (warps) per CTA of the walk
+#define STEPS_TREE_WARPS 1
 #endif
 #ifndef STEPS_TREE_LIST
 #define STEPS_TREE_LIST 128   // interaction-list entries per warp (>= 64)
@@ -532,7 +534,7 @@ __device__ __forceinline__ void tree_eval(const I2& I, TreeList& L, int nl, int 
 }
 
 #ifndef STEPS_TREE_MIN_BLOCKS
-#define STEPS_TREE_MIN_BLOCKS 5  // co-resident CTAs per SM asked of the register allocator
+#define STEPS_TREE_MIN_BLOCKS (20 / STEPS_TREE_WARPS)  // co-resident CTAs per SM asked of the register allocator
 #endif
 
 // One warp per group of 32 particles in key order (sA/sB, u4s: key order);
