@@ -700,13 +700,6 @@ int build_background(steps_cyl_ctx* c) {
   return STEPS_OK;
 }
 
-#ifndef STEPS_FP64_MIN_STEPS
-#define STEPS_FP64_MIN_STEPS 8  // fewest steps (of 32 pairs) worth a warp of the symmetric FP64 kernel
-#endif
-#ifndef STEPS_FP64_WARPS
-#define STEPS_FP64_WARPS 64  // warps per SM it is split over
-#endif
-
 // FP64 pair sums of the listed particles (all when idx == nullptr) into
 // out[3][ni], with the j-range split across CTAs so that short lists fill the GPU.
 int launch_fp64(steps_cyl_ctx* c, const int64_t* idx, int ni, double* out) {
@@ -744,8 +737,11 @@ int launch_fp64_sym(steps_cyl_ctx* c, double* out) {
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
   const int NB = (c->n + 31) / 32, nc = n_cut_eff(c);
   const long long W = row_step64(NB, NB);
-  const long long warps = std::max(1LL, std::min((W + STEPS_FP64_MIN_STEPS - 1) / STEPS_FP64_MIN_STEPS,
-                                                 (long long)sms * STEPS_FP64_WARPS));
+  // One wave of 16 warps per SM (what 128 registers allow) shares the steps evenly and so keeps every SM
+  // busy to the end: 155 / 1,253 us at N = 600 / 2,048 (N_cut = 64), 182 / 1,256 with two waves. From 128 steps a
+  // warp on two waves make up for the steps' unequal work: N = 6,000, N_cut = 30 10.39 -> 10.28 ms.
+  const long long wave = 16LL * sms;
+  const long long warps = std::max(1LL, std::min(W / 2, W / wave < 128 ? wave : 2 * wave));
   auto kernel = is_r3(c) ? pair_sym_fp64_kernel<kPair64R3>
                 : line_form64(nc) ? pair_sym_fp64_kernel<kPair64Line>
                                   : pair_sym_fp64_kernel<kPair64Walk>;
