@@ -2040,9 +2040,11 @@ struct TrainBuffers {
   float *u = nullptr, *t = nullptr, *w = nullptr, *m1 = nullptr, *m2 = nullptr, *gpart = nullptr, *lpart = nullptr,
         *loss = nullptr;
   int* order = nullptr;
+  float2* corr = nullptr;     // Adam's bias corrections of an epoch's steps
+  unsigned* bar = nullptr;    // barrier arrivals, failure flag
   ~TrainBuffers() {
     for (void* p : {(void*)smp, (void*)tail, (void*)r, (void*)u, (void*)t, (void*)w, (void*)m1, (void*)m2,
-                    (void*)gpart, (void*)lpart, (void*)loss, (void*)order})
+                    (void*)gpart, (void*)lpart, (void*)loss, (void*)order, (void*)corr, (void*)bar})
       if (p) cudaFreeAsync(p, st);
     if (st) cudaStreamSynchronize(st);
   }
@@ -2145,7 +2147,18 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
   CK(cudaMemcpyAsync(B.w, w.data(), sizeof(float) * kNW, cudaMemcpyHostToDevice, c->st));
   CK(cudaMemsetAsync(B.m1, 0, sizeof(float) * kNW, c->st));
   CK(cudaMemsetAsync(B.m2, 0, sizeof(float) * kNW, c->st));
-  const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
+  AdamCfg adam{0.f, 0.9f, 0.999f, 1e-8f};
+  // one cooperative launch per epoch where all blocks of a step fit the GPU at once
+  const int64_t nsteps = (ntrain + cfg->batch - 1) / cfg->batch;
+  const int grid = (int)((std::min<int64_t>(cfg->batch, ntrain) + kTrainThreads - 1) / kTrainThreads);
+  int sms = 0, per_sm = 0;
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_epoch_kernel, kTrainCta, 0));
+  const bool whole = grid <= sms * per_sm;
+  CK(cudaMallocAsync(&B.corr, sizeof(float2) * nsteps, c->st));
+  CK(cudaMallocAsync(&B.bar, sizeof(unsigned) * 2, c->st));
+  CK(cudaMemsetAsync(B.bar, 0, sizeof(unsigned) * 2, c->st));
+  std::vector<float2> corr(nsteps);
   // The epochs' sample orders: each a Fisher-Yates shuffle of its own stretch of the generator's
   // sequence, so several are drawn ahead on host threads (one takes 0.9 ms for 245,760
   // samples, the GPU's epoch less).
@@ -2174,23 +2187,43 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
     const std::vector<int> order = orders[ep % ahead].get();
     if (ep + ahead < cfg->epochs) draw(ep + ahead);
     CK(cudaMemcpyAsync(B.order, order.data(), sizeof(int) * ntrain, cudaMemcpyHostToDevice, c->st));
-    const float lr = (float)(cfg->lr * 0.5 * (1.0 + std::cos(M_PI * ep / cfg->epochs)));
+    adam.lr = (float)(cfg->lr * 0.5 * (1.0 + std::cos(M_PI * ep / cfg->epochs)));
+    for (int64_t k = 0; k < nsteps; ++k) {
+      ++step;
+      corr[k] = make_float2((float)(1.0 - std::pow((double)adam.beta1, (double)step)),
+                            (float)(1.0 - std::pow((double)adam.beta2, (double)step)));
+    }
+    last_count = ntrain - (nsteps - 1) * cfg->batch;
+    if (whole) {
+      CK(cudaMemcpyAsync(B.corr, corr.data(), sizeof(float2) * nsteps, cudaMemcpyHostToDevice, c->st));
+      CK(cudaMemsetAsync(B.bar, 0, sizeof(unsigned), c->st));  // the arrivals; bar[1] stays
+      int64_t nt = ntrain;
+      int batch = cfg->batch;
+      unsigned* bar = B.bar;
+      int* bad = reinterpret_cast<int*>(B.bar + 1);
+      void* args[] = {&B.w,     &B.u,  &B.t,  &B.order, &nt,     &batch, &B.gpart,
+                      &B.lpart, &B.m1, &B.m2, &adam,    &B.corr, &bar,   &bad};
+      CK(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(mlp_epoch_kernel), dim3(grid), dim3(kTrainCta), args, 0,
+                                     c->st));
+      continue;
+    }
     for (int64_t first = 0; first < ntrain; first += cfg->batch) {
       const int64_t count = std::min<int64_t>(cfg->batch, ntrain - first);
       const int nblk = (int)((count + kTrainThreads - 1) / kTrainThreads);
       mlp_fwd_bwd_kernel<<<nblk, kTrainCta, 0, c->st>>>(B.w, B.u, B.t, B.order, first, count, B.gpart, B.lpart);
-      ++step;
-      const float cb1 = (float)(1.0 - std::pow((double)beta1, (double)step));
-      const float cb2 = (float)(1.0 - std::pow((double)beta2, (double)step));
-      mlp_reduce_adam_kernel<<<(kNW + kAdamThreads - 1) / kAdamThreads, kAdamThreads, 0, c->st>>>(B.gpart, nblk, 1.0f / (float)count, B.w, B.m1,
-                                                                   B.m2, lr, beta1, beta2, eps, cb1, cb2, 1, nullptr);
-      last_count = count;
+      const float2 cb = corr[first / cfg->batch];
+      mlp_reduce_adam_kernel<<<(kNW + kAdamThreads - 1) / kAdamThreads, kAdamThreads, 0, c->st>>>(
+          B.gpart, nblk, 1.0f / (float)count, B.w, B.m1, B.m2, adam, cb.x, cb.y, 1, nullptr);
     }
     CKLAUNCH("train epoch");
   }
   {
     int rc = read_loss(c->st, B.lpart, (int)((last_count + kTrainThreads - 1) / kTrainThreads), B.loss, &last_loss);
     if (rc) return rc;
+    unsigned bad = 0;
+    CK(cudaMemcpyAsync(&bad, B.bar + 1, sizeof bad, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    if (bad) return fail(STEPS_EDEVICE, "training: a barrier between the blocks of a step ran out");
   }
   // held-out loss (forward and backward over the held-out tail, no update)
   double hold_sum = 0.0;
@@ -3133,8 +3166,8 @@ int steps_cyl_mlp_loss_grad(int64_t ns, const float* w, const float* u, const fl
   CK(cudaMemcpyAsync(du, u, sizeof(float) * 3 * ns, cudaMemcpyDefault, st));
   CK(cudaMemcpyAsync(dt, t, sizeof(float) * 2 * ns, cudaMemcpyDefault, st));
   mlp_fwd_bwd_kernel<<<nblk, kTrainCta, 0, st>>>(dw, du, dt, nullptr, 0, ns, gp, lp);
-  mlp_reduce_adam_kernel<<<(kNW + kAdamThreads - 1) / kAdamThreads, kAdamThreads, 0, st>>>(gp, nblk, 1.0f / (float)ns, nullptr, nullptr, nullptr,
-                                                            0.f, 0.f, 0.f, 0.f, 1.f, 1.f, 0, dg);
+  mlp_reduce_adam_kernel<<<(kNW + kAdamThreads - 1) / kAdamThreads, kAdamThreads, 0, st>>>(
+      gp, nblk, 1.0f / (float)ns, nullptr, nullptr, nullptr, AdamCfg{}, 1.f, 1.f, 0, dg);
   sum_floats_kernel<<<1, 32, 0, st>>>(lp, nblk, 1.0f / (float)ns, dl);
   CKLAUNCH("mlp_loss_grad");
   CK(cudaMemcpyAsync(grad, dg, sizeof(float) * kNW, cudaMemcpyDefault, st));

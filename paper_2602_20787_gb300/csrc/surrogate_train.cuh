@@ -201,37 +201,50 @@ __device__ __forceinline__ void axpy8(u64 (&v)[4], float x, const float* w) {
   v[3] = fma2(b.y, X, v[3]);
 }
 
-static __global__ void __launch_bounds__(kTrainCta)
-mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ u, const float* __restrict__ t,
-                   const int* __restrict__ order, int64_t first, int64_t count, float* __restrict__ gpart,
-                   float* __restrict__ lpart) {
-  static_assert(kH == 32 && kOW2 % 4 == 0, "eight neurons per thread, 128-bit reads of W2");
-  __shared__ __align__(16) float sW[kNW];
-  __shared__ __align__(16) float sT[kH * kTrainT];
-  __shared__ __align__(16) float s_in[3][kTrainRow], s_a1[kH][kTrainRow], s_d1[kH][kTrainRow], s_a2[kH][kTrainRow],
+// The sample of a thread (threads of the first half: target g, and inputs 2 g and, g = 0, 1).
+struct TrainSample {
+  bool valid;
+  float tg, i0, i1;
+};
+__device__ __forceinline__ TrainSample load_sample(const float* __restrict__ u, const float* __restrict__ t,
+                                                   const int* __restrict__ order, int64_t first, int64_t count,
+                                                   int block) {
+  const int s = threadIdx.x % kTrainThreads, g = threadIdx.x / kTrainThreads;
+  const int64_t q = (int64_t)block * kTrainThreads + s;
+  TrainSample in{q < count, 0.f, 0.f, 0.f};
+  if (g < 2 && in.valid) {
+    const int64_t k = order ? (int64_t)order[first + q] : first + q;
+    in.tg = t[2 * k + g];
+    in.i0 = u[3 * k + 2 * g];
+    if (g == 0) in.i1 = u[3 * k + 1];
+  }
+  return in;
+}
+
+struct TrainShared {
+  __align__(16) float sW[kNW + 2];
+  __align__(16) float sT[kH * kTrainT];
+  __align__(16) float s_in[3][kTrainRow], s_a1[kH][kTrainRow], s_d1[kH][kTrainRow], s_a2[kH][kTrainRow],
       s_d2[kH][kTrainRow], s_e[2][kTrainRow], s_loss[kTrainThreads];
+};
+
+// Summed gradient and loss of a block's samples. The weights are read past L1: inside
+// mlp_epoch_kernel other SMs write them.
+__device__ __forceinline__ void fwd_bwd_block(TrainShared& sh, const float* w, const TrainSample& in, int block,
+                                              float* __restrict__ gpart, float* __restrict__ lpart) {
+  static_assert(kH == 32 && kOW2 % 4 == 0, "eight neurons per thread, 128-bit reads of W2");
   const int tid = threadIdx.x, s = tid % kTrainThreads, g = tid / kTrainThreads, o0 = 8 * g;
-  const int64_t q = (int64_t)blockIdx.x * kTrainThreads + s;
-  const bool valid = q < count;
-  float tg = 0.f;
   if (g < 2) {
-    float i0 = 0.f, i1 = 0.f;
-    if (valid) {
-      const int64_t k = order ? (int64_t)order[first + q] : first + q;
-      tg = t[2 * k + g];
-      i0 = u[3 * k + 2 * g];
-      if (g == 0) i1 = u[3 * k + 1];
-    }
-    s_in[2 * g][s] = i0;
-    if (g == 0) s_in[1][s] = i1;
+    sh.s_in[2 * g][s] = in.i0;
+    if (g == 0) sh.s_in[1][s] = in.i1;
   }
 #pragma unroll
   for (int r = 0; r < (kNW + kTrainCta - 1) / kTrainCta; ++r) {
     const int p = r * kTrainCta + tid;
     if (p < kNW) {
-      const float v = w[p];
-      sW[p] = v;
-      if (p >= kOW2 && p < kOB2) sT[((p - kOW2) % kH) * kTrainT + (p - kOW2) / kH] = v;
+      const float v = __ldcg(w + p);
+      sh.sW[p] = v;
+      if (p >= kOW2 && p < kOB2) sh.sT[((p - kOW2) % kH) * kTrainT + (p - kOW2) / kH] = v;
     }
   }
   __syncthreads();
@@ -239,69 +252,69 @@ mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ u, con
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int o = o0 + j;
-    float v = sW[kOB1 + o];
+    float v = sh.sW[kOB1 + o];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) v = fmaf(sW[kOW1 + o * 3 + k], s_in[k][s], v);
-    s_a1[o][s] = fmaxf(v, 0.f);
+    for (int k = 0; k < 3; ++k) v = fmaf(sh.sW[kOW1 + o * 3 + k], sh.s_in[k][s], v);
+    sh.s_a1[o][s] = fmaxf(v, 0.f);
   }
   __syncthreads();
   float a2[8];
   {
     u64 v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = pk(sW[kOB2 + o0 + 2 * j], sW[kOB2 + o0 + 2 * j + 1]);
+    for (int j = 0; j < 4; ++j) v[j] = pk(sh.sW[kOB2 + o0 + 2 * j], sh.sW[kOB2 + o0 + 2 * j + 1]);
 #pragma unroll 8
-    for (int k = 0; k < kH; ++k) axpy8(v, s_a1[k][s], sT + k * kTrainT + o0);
+    for (int k = 0; k < kH; ++k) axpy8(v, sh.s_a1[k][s], sh.sT + k * kTrainT + o0);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       upk(v[j], a2[2 * j], a2[2 * j + 1]);
       a2[2 * j] = fmaxf(a2[2 * j], 0.f);
       a2[2 * j + 1] = fmaxf(a2[2 * j + 1], 0.f);
-      s_a2[o0 + 2 * j][s] = a2[2 * j];
-      s_a2[o0 + 2 * j + 1][s] = a2[2 * j + 1];
+      sh.s_a2[o0 + 2 * j][s] = a2[2 * j];
+      sh.s_a2[o0 + 2 * j + 1][s] = a2[2 * j + 1];
     }
   }
   __syncthreads();
   if (g < 2) {
-    float v = sW[kOB3 + g];
+    float v = sh.sW[kOB3 + g];
 #pragma unroll
-    for (int k = 0; k < kH; ++k) v = fmaf(sW[kOW3 + g * kH + k], s_a2[k][s], v);
-    s_e[g][s] = valid ? (v - tg) : 0.f;
+    for (int k = 0; k < kH; ++k) v = fmaf(sh.sW[kOW3 + g * kH + k], sh.s_a2[k][s], v);
+    sh.s_e[g][s] = in.valid ? (v - in.tg) : 0.f;
   }
   __syncthreads();
   // backward: d2 = (W3^T e) * relu'(z2), d1 = (W2^T d2) * relu'(z1)
-  const float e[2] = {s_e[0][s], s_e[1][s]};
-  const float* W3 = sW + kOW3;
+  const float e[2] = {sh.s_e[0][s], sh.s_e[1][s]};
+  const float* W3 = sh.sW + kOW3;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int k = o0 + j;
     const float d = W3[k] * e[0] + W3[kH + k] * e[1];
-    s_d2[k][s] = a2[j] > 0.f ? d : 0.f;
+    sh.s_d2[k][s] = a2[j] > 0.f ? d : 0.f;
   }
-  if (g == 0) s_loss[s] = 0.5f * (e[0] * e[0] + e[1] * e[1]);
+  if (g == 0) sh.s_loss[s] = 0.5f * (e[0] * e[0] + e[1] * e[1]);
   __syncthreads();
   {
     u64 v[4] = {0, 0, 0, 0};
 #pragma unroll 8
-    for (int o = 0; o < kH; ++o) axpy8(v, s_d2[o][s], sW + kOW2 + o * kH + o0);
+    for (int o = 0; o < kH; ++o) axpy8(v, sh.s_d2[o][s], sh.sW + kOW2 + o * kH + o0);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       float x, y;
       upk(v[j], x, y);
-      s_d1[o0 + 2 * j][s] = s_a1[o0 + 2 * j][s] > 0.f ? x : 0.f;
-      s_d1[o0 + 2 * j + 1][s] = s_a1[o0 + 2 * j + 1][s] > 0.f ? y : 0.f;
+      sh.s_d1[o0 + 2 * j][s] = sh.s_a1[o0 + 2 * j][s] > 0.f ? x : 0.f;
+      sh.s_d1[o0 + 2 * j + 1][s] = sh.s_a1[o0 + 2 * j + 1][s] > 0.f ? y : 0.f;
     }
   }
   __syncthreads();
   // block partial gradient, samples in order. W2: rows o, o + 16, columns k, k + 16
-  float* gp = gpart + (int64_t)blockIdx.x * kNW;
+  float* gp = gpart + (int64_t)block * kNW;
   {
     const int k = tid % 16, o = tid / 16;
     float c00 = 0.f, c01 = 0.f, c10 = 0.f, c11 = 0.f;
 #pragma unroll 4
     for (int r = 0; r < kTrainThreads; r += 4) {
-      const float4 A0 = *reinterpret_cast<const float4*>(&s_a1[k][r]), A1 = *reinterpret_cast<const float4*>(&s_a1[k + 16][r]);
-      const float4 D0 = *reinterpret_cast<const float4*>(&s_d2[o][r]), D1 = *reinterpret_cast<const float4*>(&s_d2[o + 16][r]);
+      const float4 A0 = *reinterpret_cast<const float4*>(&sh.s_a1[k][r]), A1 = *reinterpret_cast<const float4*>(&sh.s_a1[k + 16][r]);
+      const float4 D0 = *reinterpret_cast<const float4*>(&sh.s_d2[o][r]), D1 = *reinterpret_cast<const float4*>(&sh.s_d2[o + 16][r]);
       c00 = fmaf(D0.w, A0.w, fmaf(D0.z, A0.z, fmaf(D0.y, A0.y, fmaf(D0.x, A0.x, c00))));
       c01 = fmaf(D0.w, A1.w, fmaf(D0.z, A1.z, fmaf(D0.y, A1.y, fmaf(D0.x, A1.x, c01))));
       c10 = fmaf(D1.w, A0.w, fmaf(D1.z, A0.z, fmaf(D1.y, A0.y, fmaf(D1.x, A0.x, c10))));
@@ -320,17 +333,17 @@ mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ u, con
     const int p = tid < kOW2 ? tid : tid + kH * kH;
     const float *A, *B = nullptr;
     if (p < kOB1) {
-      A = s_d1[p / 3];
-      B = s_in[p % 3];
+      A = sh.s_d1[p / 3];
+      B = sh.s_in[p % 3];
     } else if (p < kOW2) {
-      A = s_d1[p - kOB1];
+      A = sh.s_d1[p - kOB1];
     } else if (p < kOW3) {
-      A = s_d2[p - kOB2];
+      A = sh.s_d2[p - kOB2];
     } else if (p < kOB3) {
-      A = s_e[(p - kOW3) / kH];
-      B = s_a2[(p - kOW3) % kH];
+      A = sh.s_e[(p - kOW3) / kH];
+      B = sh.s_a2[(p - kOW3) % kH];
     } else {
-      A = s_e[p - kOB3];
+      A = sh.s_e[p - kOB3];
     }
     float c = 0.f;
     if (B) {
@@ -349,9 +362,29 @@ mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ u, con
     gp[p] = c;
   } else if (tid == kTrainCta - 1) {
     float l = 0.f;
-    for (int r = 0; r < kTrainThreads; ++r) l += s_loss[r];
-    lpart[blockIdx.x] = l;
+    for (int r = 0; r < kTrainThreads; ++r) l += sh.s_loss[r];
+    lpart[block] = l;
   }
+}
+
+static __global__ void __launch_bounds__(kTrainCta)
+mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ u, const float* __restrict__ t,
+                   const int* __restrict__ order, int64_t first, int64_t count, float* __restrict__ gpart,
+                   float* __restrict__ lpart) {
+  __shared__ TrainShared sh;
+  fwd_bwd_block(sh, w, load_sample(u, t, order, first, count, blockIdx.x), blockIdx.x, gpart, lpart);
+}
+
+struct AdamCfg {
+  float lr, beta1, beta2, eps;
+};
+__device__ __forceinline__ void adam_update(float g, const AdamCfg& A, float c1, float c2, float& w, float& m1,
+                                            float& m2) {
+  const float a = fmaf(1.f - A.beta1, g, A.beta1 * m1);
+  const float v = fmaf((1.f - A.beta2) * g, g, A.beta2 * m2);
+  m1 = a;
+  m2 = v;
+  w -= A.lr * (a / c1) / (sqrtf(v / c2) + A.eps);
 }
 
 // Sum the block partials of each weight in block order, divide by the batch,
@@ -360,8 +393,8 @@ mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ u, con
 constexpr int kAdamThreads = 32, kAdamLoads = 32;
 static __global__ void __launch_bounds__(kAdamThreads)
 mlp_reduce_adam_kernel(const float* __restrict__ gpart, int nblocks, float inv_batch, float* __restrict__ w,
-                       float* __restrict__ m1, float* __restrict__ m2, float lr, float beta1, float beta2, float eps,
-                       float c1, float c2, int adam, float* __restrict__ grad_out) {
+                       float* __restrict__ m1, float* __restrict__ m2, AdamCfg A, float c1, float c2, int adam,
+                       float* __restrict__ grad_out) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= kNW) return;
   float M1 = 0.f, M2 = 0.f, W = 0.f;
@@ -382,11 +415,84 @@ mlp_reduce_adam_kernel(const float* __restrict__ gpart, int nblocks, float inv_b
   g *= inv_batch;
   if (grad_out) grad_out[p] = g;
   if (adam) {
-    const float a = fmaf(1.f - beta1, g, beta1 * M1);
-    const float v = fmaf((1.f - beta2) * g, g, beta2 * M2);
-    m1[p] = a;
-    m2[p] = v;
-    w[p] = W - lr * (a / c1) / (sqrtf(v / c2) + eps);
+    adam_update(g, A, c1, c2, W, M1, M2);
+    m1[p] = M1;
+    m2[p] = M2;
+    w[p] = W;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// All steps of an epoch in one cooperative launch, a block of samples per CTA: between the
+// gradient of a step and its update, and between that and the next step, the CTAs meet at a
+// barrier in memory, and a CTA's next samples are fetched meanwhile. As two launches per step
+// (the kernels above) a step of 64 blocks took 14 us, most of it launch latency and cold loads.
+// ---------------------------------------------------------------------------
+constexpr unsigned kBarrierSpins = 1u << 22;  // polls (of some 0.5 us) before a barrier gives up
+
+// Every CTA of the grid arrives (target: arrivals once all have). A wait that runs out sets *fail, and
+// later waits end at once.
+__device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, int* fail) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    unsigned seen = 0;
+    for (unsigned k = 0; k < kBarrierSpins; ++k) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      if (seen >= target || ((k & 1023u) == 1023u && atomicAdd(fail, 0) != 0)) break;
+    }
+    if (seen < target) atomicExch(fail, 1);
+    __threadfence();
+  }
+  __syncthreads();
+}
+
+constexpr int kRedRow = kTrainThreads + 1;  // row stride of the gradient tile (32 weights x 64 blocks)
+static __global__ void __launch_bounds__(kTrainCta)
+mlp_epoch_kernel(float* w, const float* __restrict__ u, const float* __restrict__ t, const int* __restrict__ order,
+                 int64_t ntrain, int batch, float* gpart, float* lpart, float* m1, float* m2, AdamCfg A,
+                 const float2* __restrict__ corr, unsigned* bar, int* fail) {
+  __shared__ TrainShared sh;
+  static_assert(sizeof(sh.s_a1) >= sizeof(float) * 32 * kRedRow, "the gradient tile takes the activations' place");
+  float* red = &sh.s_a1[0][0];
+  unsigned target = 0;
+  int step = 0;
+  TrainSample in = load_sample(u, t, order, 0, min((int64_t)batch, ntrain), blockIdx.x);
+  for (int64_t first = 0; first < ntrain; first += batch, ++step) {
+    const int64_t count = min((int64_t)batch, ntrain - first), rest = ntrain - first - count;
+    const int nblk = (int)((count + kTrainThreads - 1) / kTrainThreads);
+    if ((int)blockIdx.x < nblk) fwd_bwd_block(sh, w, in, blockIdx.x, gpart, lpart);
+    in = load_sample(u, t, order, first + count, min((int64_t)batch, rest), blockIdx.x);
+    grid_barrier(bar, target += gridDim.x, fail);
+    const int lane = threadIdx.x % 32, r0 = threadIdx.x / 32;
+    for (int p0 = 32 * blockIdx.x; p0 < kNW; p0 += 32 * gridDim.x) {
+      const int p = p0 + lane;
+      float g = 0.f;
+      for (int b0 = 0; b0 < nblk; b0 += kTrainThreads) {
+        const int nb = min(kTrainThreads, nblk - b0);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kTrainThreads; r += kTrainCta / 32) {
+          const int b = r + r0;
+          if (b < nb && p < kNW) red[lane * kRedRow + b] = __ldcg(gpart + (int64_t)(b0 + b) * kNW + p);
+        }
+        __syncthreads();
+        if (r0 == 0 && p < kNW) {
+#pragma unroll 16
+          for (int b = 0; b < nb; ++b) g += red[lane * kRedRow + b];
+        }
+      }
+      if (r0 == 0 && p < kNW) {
+        const float2 c = corr[step];
+        float W = __ldcg(w + p), M1 = m1[p], M2 = m2[p];
+        adam_update(g * (1.0f / (float)count), A, c.x, c.y, W, M1, M2);
+        m1[p] = M1;
+        m2[p] = M2;
+        w[p] = W;
+      }
+    }
+    grid_barrier(bar, target += gridDim.x, fail);
   }
 }
 
