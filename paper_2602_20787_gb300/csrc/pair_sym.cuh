@@ -386,7 +386,8 @@ struct TableForm {
 
 // ---- the stream-K driver over the upper triangle -----------------------------
 // The tile width is kBJ / tpb: whole blocks (tpb = 1), or quarters (tpb = 4) when
-// there are too few blocks to fill the GPU.
+// there are too few blocks to fill the GPU. A quarter's 32 steps are split once more, over sp units of
+// 32 / sp steps (whole Kahan groups), when even the quarters leave CTAs' places empty.
 struct SymShared {
   JTile2 T;
   float J[kSymThreads / 32 * kJRow];
@@ -394,30 +395,31 @@ struct SymShared {
 
 template <bool KAHAN, class Form>
 __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, const float4* __restrict__ jB, int n,
-                                             int NB, int tpb, long long Ua, long long U, int C, SymShared& sh,
+                                             int NB, int tpb, int sp, long long Ua, long long U, int C, SymShared& sh,
                                              const FixAcc& F, const Form& form) {
   // the units [Ua, Ua + U) (all of them, or a rank's share), split over C CTAs
   const int c = blockIdx.x;
   const long long u0 = Ua + (long long)c * U / C;
   const long long u1 = Ua + (long long)(c + 1) * U / C;
-  const int jt = kBJ / tpb;
+  const int jt = kBJ / tpb, upb = tpb * sp, ks = jt / sp;  // units per block, steps per unit
   float* row = sh.J + (threadIdx.x >> 5) * kJRow;
   long long u = u0;
   while (u < u1) {
-    const int b = (int)checked_index(tri_row(u / tpb, NB), NB);
-    const int t0 = (int)checked_index(b * tpb + (u - tpb * tri_off(b, NB)), (long long)NB * tpb);
-    const int t1 = (int)min((long long)NB * tpb, (long long)t0 + (u1 - u));
+    const int b = (int)checked_index(tri_row(u / upb, NB), NB);
+    const int v0 = (int)checked_index(b * upb + (u - upb * tri_off(b, NB)), (long long)NB * upb);
+    const int v1 = (int)min((long long)NB * upb, (long long)v0 + (u1 - u));
     const int i0 = row_i0(b), i1 = i0 + 32;
     const I2 I = load_i2(jA, jB, i0, i1, n);
     u64 sx = 0, sy = 0, sz = 0, cx = 0, cy = 0, cz = 0;
-    for (int t = t0; t < t1; ++t) {
+    for (int v = v0; v < v1; ++v) {
+      const int t = v / sp, kb = (v - t * sp) * ks;
       __syncthreads();
       load_tile2<kSymThreads>(jA, jB, n, t, jt, sh.T);
       __syncthreads();
       const bool sym = t / tpb != b;
       JRing ring;
 #pragma unroll 1
-      for (int k0 = 0; k0 < jt; k0 += STEPS_KAHAN_GROUP) {
+      for (int k0 = kb; k0 < kb + ks; k0 += STEPS_KAHAN_GROUP) {
         u64 gx = 0, gy = 0, gz = 0;
 #pragma unroll 1
         for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; ++k) {
@@ -435,7 +437,7 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
             ring.take(P.dx, P.dy, mul2(I.m, SR), mul2(I.m, SZ), k + 1 != k0 + STEPS_KAHAN_GROUP);
           }
         }
-        if (sym) ring.flush(row, k0 + STEPS_KAHAN_GROUP - 1, (k0 & 31) == 0);
+        if (sym) ring.flush(row, k0 + STEPS_KAHAN_GROUP - 1, k0 == kb || (k0 & 31) == 0);
         acc2<KAHAN>(sx, cx, gx);
         acc2<KAHAN>(sy, cy, gy);
         acc2<KAHAN>(sz, cz, gz);
@@ -447,10 +449,10 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
           if (j < n) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-              long long v = 0;
+              long long f = 0;
 #pragma unroll
-              for (int w = 0; w < kSymThreads / 32; ++w) v -= fix_value(F, sh.J[w * kJRow + 3 * s + q]);
-              fix_add(F, q, j, v);
+              for (int w = 0; w < kSymThreads / 32; ++w) f -= fix_value(F, sh.J[w * kJRow + 3 * s + q]);
+              fix_add(F, q, j, f);
             }
           }
         }
@@ -459,22 +461,22 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
     const u64 S[3] = {sx, sy, sz}, K[3] = {cx, cy, cz};
 #pragma unroll
     for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN>(F, q, i0, i1, S[q], K[q]);
-    u += t1 - t0;
+    u += v1 - v0;
   }
 }
 
 // ---- kernels ---------------------------------------------------------------
 template <bool KAHAN, bool LINE, bool FAR>
 __global__ void __launch_bounds__(kSymThreads, FAR ? STEPS_SYM_FAR_MIN_BLOCKS : STEPS_SYM_MIN_BLOCKS)
-pair_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
+pair_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb, int sp,
                 long long Ua, long long U, int C, FixAcc F) {
   __shared__ SymShared sh;
-  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, Ua, U, C, sh, F, PlainForm<LINE, FAR>{n_cut, (float)n_cut});
+  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, sp, Ua, U, C, sh, F, PlainForm<LINE, FAR>{n_cut, (float)n_cut});
 }
 
 template <bool KAHAN, int MODEL, bool FAR>
 __global__ void __launch_bounds__(kSymThreads, STEPS_SYM_SURR_MIN_BLOCKS)
-pair_sym_surr_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
+pair_sym_surr_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb, int sp,
                      long long Ua, long long U, int C, const SurrLane* __restrict__ wl, SurrConst S, FixAcc F) {
   __shared__ SymShared sh;
   __shared__ __align__(16) uint32_t sWT[32 * kSurrStride];
@@ -482,16 +484,16 @@ pair_sym_surr_kernel(const float4* __restrict__ jA, const float4* __restrict__ j
   uint32_t* ibuf = sIn[threadIdx.x >> 5];
   mlp_zero_inputs<2>(ibuf);
   stage_surr_weights(wl, sWT);
-  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, Ua, U, C, sh, F,
+  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, sp, Ua, U, C, sh, F,
                       SurrForm<MODEL, FAR>{n_cut, SurrW{sWT + (threadIdx.x & 31) * kSurrStride}, ibuf, S});
 }
 
 template <bool KAHAN, int MODEL, int READ, bool FAR>
 __global__ void __launch_bounds__(kSymThreads, STEPS_SYM_TABLE_MIN_BLOCKS)
-pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
+pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb, int sp,
                       long long Ua, long long U, int C, TableTail T, SurrConst S, FixAcc F) {
   __shared__ SymShared sh;
-  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, Ua, U, C, sh, F, TableForm<MODEL, READ, FAR>{n_cut, S, T});
+  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, sp, Ua, U, C, sh, F, TableForm<MODEL, READ, FAR>{n_cut, S, T});
 }
 
 // ---- R^3 -------------------------------------------------------------------

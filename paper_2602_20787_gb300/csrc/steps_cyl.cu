@@ -54,6 +54,11 @@ using namespace steps;
 #define STEPS_SYM_SPLIT 64
 #endif
 
+// The most units that a quarter tile's steps are split over: it holds four Kahan groups.
+#ifndef STEPS_SYM_MAX_STEP_SPLIT
+#define STEPS_SYM_MAX_STEP_SPLIT 4
+#endif
+
 namespace {
 
 thread_local std::string g_last_error;
@@ -270,6 +275,7 @@ struct steps_cyl_ctx {
   bool fix_ready = false, fix_ok = false;
   long long Usym = 0;
   int tpb = 1;                         // j-tiles per block of 128 rows of the symmetric kernels
+  int sp = 1;                          // units a quarter tile's steps are split over
   int SYC = 0, SYSC = 0, SYTC = 0, SYRC = 0;  // CTAs of the symmetric plain / surrogate / table / R^3 kernels
   // row sharding
   bool shard = false;
@@ -1159,7 +1165,7 @@ bool straight_run(const steps_cyl_ctx* c) {
   return model_kind(c) == kModelWide4 && 2.0 * c->h_max < 0.5 * c->p.L;
 }
 
-using SymTableKernel = void (*)(const float4*, const float4*, int, int, int, int, long long, long long, int, TableTail,
+using SymTableKernel = void (*)(const float4*, const float4*, int, int, int, int, int, long long, long long, int, TableTail,
                                 SurrConst, FixAcc);
 template <bool KAHAN, int MODEL>
 SymTableKernel sym_table_kernel(int read, bool far) {
@@ -1186,7 +1192,7 @@ SymTableKernel sym_table_kernel(Model model, int read, bool far) {
   }
 }
 
-using SymSurrKernel = void (*)(const float4*, const float4*, int, int, int, int, long long, long long, int,
+using SymSurrKernel = void (*)(const float4*, const float4*, int, int, int, int, int, long long, long long, int,
                                const SurrLane*, SurrConst, FixAcc);
 template <bool KAHAN>
 SymSurrKernel sym_surr_kernel(Model model, bool far) {
@@ -1199,7 +1205,7 @@ SymSurrKernel sym_surr_kernel(Model model, bool far) {
   }
 }
 
-using SymKernel = void (*)(const float4*, const float4*, int, int, int, int, long long, long long, int, FixAcc);
+using SymKernel = void (*)(const float4*, const float4*, int, int, int, int, int, long long, long long, int, FixAcc);
 template <bool KAHAN>
 SymKernel sym_kernel(bool line, bool far) {
   return !line ? pair_sym_kernel<KAHAN, false, false>
@@ -1209,7 +1215,7 @@ SymKernel sym_kernel(bool line, bool far) {
 
 int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const FixAcc& F) {
   const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
-  const int nc = c->p.n_cut, n = c->n, NB = c->NB, tpb = c->tpb;
+  const int nc = c->p.n_cut, n = c->n, NB = c->NB, tpb = c->tpb, sp = c->sp;
   const bool straight = straight_run(c);
   c->last_straight = (form == Form::SURROGATE || (form == Form::TABLE && (c->tab.read == kReadCic ||
                                                                           c->tab.read == kReadTsc))) &&
@@ -1220,13 +1226,13 @@ int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const Fix
   if (form == Form::SURROGATE) {
     const int C = ctas(c->SYSC);
     auto k = kahan ? sym_surr_kernel<true>(model_kind(c), straight) : sym_surr_kernel<false>(model_kind(c), straight);
-    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, Ua, U, C, c->surr_lanes, c->surr, F);
+    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, sp, Ua, U, C, c->surr_lanes, c->surr, F);
     CKLAUNCH("pair_sym_surrogate");
   } else if (form == Form::TABLE) {
     const int C = ctas(c->SYTC);
     auto k = kahan ? sym_table_kernel<true>(model_kind(c), c->tab.read, straight)
                    : sym_table_kernel<false>(model_kind(c), c->tab.read, straight);
-    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, Ua, U, C, c->tab, c->tab_const, F);
+    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, sp, Ua, U, C, c->tab, c->tab_const, F);
     CKLAUNCH("pair_sym_table");
   } else if (is_r3(c)) {
     const int C = ctas(c->SYRC);  // never a share of the triangle: a sharded R^3 context keeps the row step
@@ -1237,7 +1243,7 @@ int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const Fix
     const int C = ctas(c->SYC);
     const bool far = 2.0 * c->h_max < 0.5 * c->p.L;
     auto k = kahan ? sym_kernel<true>(line_form(nc), far) : sym_kernel<false>(line_form(nc), far);
-    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, Ua, U, C, F);
+    k<<<C, kSymThreads, 0, c->st>>>(c->jA, c->jB, n, nc, NB, tpb, sp, Ua, U, C, F);
     CKLAUNCH("pair_sym");
   }
   return STEPS_OK;
@@ -2328,7 +2334,11 @@ int allocate_context(steps_cyl_ctx* c) {
   set_rows(c, 0, c->NB);
   // the symmetric kernels share the upper triangle of the block grid
   c->tpb = (long long)c->NB * (c->NB + 1) / 2 < STEPS_SYM_SPLIT * (long long)sms ? 4 : 1;
-  c->Usym = (long long)c->NB * (c->NB + 1) / 2 * c->tpb;
+  c->sp = 1;
+  while (!is_r3(c) && c->tpb == 4 && c->sp < STEPS_SYM_MAX_STEP_SPLIT &&
+         (long long)c->NB * (c->NB + 1) / 2 * c->tpb * c->sp * 2 <= (long long)sms * STEPS_SYM_MIN_BLOCKS)
+    c->sp *= 2;
+  c->Usym = (long long)c->NB * (c->NB + 1) / 2 * c->tpb * c->sp;
   int yocc = 0, ysocc = 0, ytocc = 0, yrocc = 0;
   CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&yrocc, pair_sym_r3_kernel<true>, 32, 0));
   c->SYRC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(yrocc, 1) * STEPS_CTA_MULT);
