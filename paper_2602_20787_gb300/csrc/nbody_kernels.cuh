@@ -166,6 +166,20 @@ __device__ __forceinline__ void finish_particle(int i, double sx, double sy, dou
 // idle (finalize 10.2 us, kick and drift 6.0).
 inline int particle_threads(int n) { return n <= 152 * 8 * 32 ? 32 : 128; }
 
+// The stream-K partials of evaluated row q, in CTA order.
+__device__ __forceinline__ void row_sums(const double* __restrict__ part, int q, int NT, long long U, int C, double& sx,
+                                         double& sy, double& sz) {
+  const int b = q / kBI, l = q % kBI;
+  const long long p_lo = (long long)b * NT, p_hi = p_lo + NT - 1;
+  const int c_lo = cta_of_unit(p_lo, U, C), c_hi = cta_of_unit(p_hi, U, C);
+  for (int c = c_lo; c <= c_hi; ++c) {
+    const double* v = part + ((long long)b + c) * 3 * kBI;
+    sx += v[l];
+    sy += v[kBI + l];
+    sz += v[2 * kBI + l];
+  }
+}
+
 static __global__ void finalize_kernel(const double* __restrict__ part, int n, int NT, long long U, int C,
                                 double pair_scale, BgParams bg, const double* __restrict__ x,
                                 const double* __restrict__ y, const double* __restrict__ z, double* __restrict__ gx,
@@ -185,15 +199,7 @@ static __global__ void finalize_kernel(const double* __restrict__ part, int n, i
     sy = part[m + q];
     sz = part[2 * m + q];
   } else {
-    const int b = (i - i0) / kBI, l = (i - i0) % kBI;
-    const long long p_lo = (long long)b * NT, p_hi = p_lo + NT - 1;
-    const int c_lo = cta_of_unit(p_lo, U, C), c_hi = cta_of_unit(p_hi, U, C);
-    for (int c = c_lo; c <= c_hi; ++c) {
-      const double* q = part + ((long long)b + c) * 3 * kBI;
-      sx += q[l];
-      sy += q[kBI + l];
-      sz += q[2 * kBI + l];
-    }
+    row_sums(part, i - i0, NT, U, C, sx, sy, sz);
   }
   finish_particle(i, sx, sy, sz, pair_scale, bg, x, y, z, gx, gy, gz, K, px, py, pz, out, err, rc);
 }

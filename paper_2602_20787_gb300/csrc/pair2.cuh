@@ -524,8 +524,9 @@ __device__ __forceinline__ void window2(const Sep2& P, int n_cut, float fnc, u64
 template <bool KAHAN, bool LINE>
 __global__ void __launch_bounds__(kPairThreads, STEPS_ROW_MIN_BLOCKS)
 pair_row_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, long long U, int NT,
-                int C, double* __restrict__ part, int b0) {
+                int C, double* __restrict__ part, int b0, const int* __restrict__ skip = nullptr) {
   __shared__ JTile2 T;
+  if (skip && *skip) return;  // the symmetric kernel has taken the pairs
   const int c = blockIdx.x;
   const long long u1 = (long long)(c + 1) * U / C;
   const float fnc = (float)n_cut;

@@ -388,6 +388,24 @@ struct TableForm {
 // The tile width is kBJ / tpb: whole blocks (tpb = 1), or quarters (tpb = 4) when
 // there are too few blocks to fill the GPU. A quarter's 32 steps are split once more, over sp units of
 // 32 / sp steps (whole Kahan groups), when even the quarters leave CTAs' places empty.
+
+// Quarter tiles are taken below this many 128 x 128 units per SM.
+#ifndef STEPS_SYM_SPLIT
+#define STEPS_SYM_SPLIT 64
+#endif
+// The most units that a quarter tile's steps are split over: it holds four Kahan groups.
+#ifndef STEPS_SYM_MAX_STEP_SPLIT
+#define STEPS_SYM_MAX_STEP_SPLIT 4
+#endif
+inline void sym_split(int NB, int sms, bool steps, int& tpb, int& sp) {
+  const long long blocks = (long long)NB * (NB + 1) / 2;
+  tpb = blocks < STEPS_SYM_SPLIT * (long long)sms ? 4 : 1;
+  sp = 1;
+  while (steps && tpb == 4 && sp < STEPS_SYM_MAX_STEP_SPLIT &&
+         blocks * tpb * sp * 2 <= (long long)sms * STEPS_SYM_MIN_BLOCKS)
+    sp *= 2;
+}
+
 struct SymShared {
   JTile2 T;
   float J[kSymThreads / 32 * kJRow];

@@ -48,17 +48,6 @@ using namespace steps;
 #define STEPS_CTA_MULT 32
 #endif
 
-// The symmetric kernels take quarter tiles (32 j) below this many 128 x 128 units
-// per SM (build-time tuning knob).
-#ifndef STEPS_SYM_SPLIT
-#define STEPS_SYM_SPLIT 64
-#endif
-
-// The most units that a quarter tile's steps are split over: it holds four Kahan groups.
-#ifndef STEPS_SYM_MAX_STEP_SPLIT
-#define STEPS_SYM_MAX_STEP_SPLIT 4
-#endif
-
 namespace {
 
 thread_local std::string g_last_error;
@@ -1338,7 +1327,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
     auto kernel = line_form(c->p.n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
                                         : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
-    kernel<<<c->C, kPairThreads, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, c->U, c->NT, c->C, c->part, c->b0);
+    kernel<<<c->C, kPairThreads, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, c->U, c->NT, c->C, c->part, c->b0, nullptr);
     CKLAUNCH("pair_row");
   }
   CK(cudaEventRecord(c->e1, c->st));
@@ -2333,11 +2322,7 @@ int allocate_context(steps_cyl_ctx* c) {
   c->TCcap = sms * std::max(tocc, 1) * STEPS_CTA_MULT;
   set_rows(c, 0, c->NB);
   // the symmetric kernels share the upper triangle of the block grid
-  c->tpb = (long long)c->NB * (c->NB + 1) / 2 < STEPS_SYM_SPLIT * (long long)sms ? 4 : 1;
-  c->sp = 1;
-  while (!is_r3(c) && c->tpb == 4 && c->sp < STEPS_SYM_MAX_STEP_SPLIT &&
-         (long long)c->NB * (c->NB + 1) / 2 * c->tpb * c->sp * 2 <= (long long)sms * STEPS_SYM_MIN_BLOCKS)
-    c->sp *= 2;
+  sym_split(c->NB, sms, !is_r3(c), c->tpb, c->sp);
   c->Usym = (long long)c->NB * (c->NB + 1) / 2 * c->tpb * c->sp;
   int yocc = 0, ysocc = 0, ytocc = 0, yrocc = 0;
   CKA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&yrocc, pair_sym_r3_kernel<true>, 32, 0));

@@ -6,9 +6,9 @@
 // arena reserved at start-up), a loop that must not take cudaMalloc's implicit
 // device-wide synchronisation, or a plug-in that is only allowed to allocate
 // during its initialisation. For them this entry point evaluates the pair term
-// with the same pack, stream-K pair and finalize kernels as a context does, but
-// keeps every intermediate (the packed FP32 positions and the stream-K partial
-// sums) in one file-scope __device__ array of fixed size. It never calls
+// with the same pair forms as a context does, but keeps every intermediate (the
+// packed FP32 positions and the pair sums) in one file-scope __device__ array of
+// fixed size. It never calls
 // cudaMalloc, cudaFree or an allocating library routine. The call stays
 // asynchronous, so it keeps no device error word: nothing would read it.
 //
@@ -23,7 +23,7 @@
 
 #include "steps_cyl.h"
 #include "nbody_kernels.cuh"
-#include "pair2.cuh"
+#include "pair_sym.cuh"
 
 using namespace steps;
 
@@ -40,9 +40,109 @@ static_assert(kScratchBytes == STEPS_NOALLOC_SCRATCH_BYTES, "scratch size must m
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
+// Each unordered pair is evaluated once where the fixed-point sums that this takes (pair_sym.cuh)
+// have a scale. Their bound needs the total mass and the smallest softening, which the
+// host cannot look at without waiting: the pack kernel reduces them on the device, the symmetric
+// kernel derives the scale, or leaves the pairs to the row kernel, whose CTAs otherwise
+// return at once. (N = 10,007, N_cut = 16, literal softening law: rows alone 730 us.)
+// The record lies in the partials' last slot, which the row kernel's split never reaches.
+constexpr int kPackThreads = 256;
+constexpr int kPackParts = (kNoallocMaxN + kPackThreads - 1) / kPackThreads;
+struct NoallocHead {
+  unsigned long long hmin;  // bits of the smallest h; 0 when some h is not > 0
+  int err, sym;             // error bits of the symmetric kernel; whether it has taken the pairs
+  double scale;             // its sums' scale
+  double mass[kPackParts];  // sums of |m| over each CTA of the pack kernel
+};
+constexpr size_t kHeadOffset = kScratchBytes - sizeof(double) * 3 * kBI;
+static_assert(sizeof(NoallocHead) <= sizeof(double) * 3 * kBI, "the record takes one partial-sum slot");
+static_assert(sizeof(unsigned long long) * 3 * kNoallocMaxN <= kPartBytes - sizeof(double) * 3 * kBI,
+              "the fixed-point sums take the partials' place");
+
+__global__ void __launch_bounds__(kPackThreads)
+noalloc_pack_kernel(const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
+                    const double* __restrict__ m, const double* __restrict__ h, int n, double invL,
+                    float4* __restrict__ jA, float4* __restrict__ jB, unsigned long long* __restrict__ acc,
+                    NoallocHead* __restrict__ head) {
+  __shared__ double warp[kPackThreads / 32];
+  const int i = blockIdx.x * kPackThreads + threadIdx.x;
+  double s = 0.0;
+  unsigned long long hb = ~0ull;
+  if (i < n) {
+    pack_one(x[i], y[i], z[i], m[i], h[i], i, invL, jA, jB);
+    acc[i] = acc[(size_t)n + i] = acc[2 * (size_t)n + i] = 0;
+    s = fabs(m[i]);
+    hb = h[i] > 0.0 ? (unsigned long long)__double_as_longlong(h[i]) : 0ull;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_down_sync(0xffffffffu, s, o);
+    hb = min(hb, __shfl_down_sync(0xffffffffu, hb, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    warp[threadIdx.x >> 5] = s;
+    atomicMin(&head->hmin, hb);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kPackThreads / 32; ++w) t += warp[w];
+    head->mass[blockIdx.x] = t;
+  }
+}
+
+// The scale as the contexts choose it (2^57 over the bound on |S_i|, at least 2^40), 0: none. By a whole warp.
+__device__ __forceinline__ double noalloc_scale(const NoallocHead* head, int parts, double L) {
+  double M = 0.0;
+  for (int k = threadIdx.x & 31; k < parts; k += 32) M += head->mass[k];
+  for (int o = 16; o > 0; o >>= 1) M += __shfl_xor_sync(0xffffffffu, M, o);
+  const double q = L / __longlong_as_double((long long)head->hmin), B = M * (q * q + 10.0);
+  if (!(B >= 1e-290 && B < 1e290)) return 0.0;
+  const int S = 57 - (((__double2hiint(B) >> 20) & 0x7ff) - 1022);  // B < 2^(exponent + 1)
+  return S >= 40 && S <= 1000 ? __hiloint2double((S + 1023) << 20, 0) : 0.0;
+}
+
+template <bool KAHAN, bool LINE>
+__global__ void __launch_bounds__(kSymThreads, STEPS_SYM_MIN_BLOCKS)
+noalloc_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
+                   int sp, long long U, int C, unsigned long long* __restrict__ acc, NoallocHead* __restrict__ head,
+                   int parts, double L) {
+  __shared__ SymShared sh;
+  const double scale = noalloc_scale(head, parts, L);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    head->sym = scale > 0.0;
+    head->scale = scale;
+  }
+  if (!(scale > 0.0)) return;
+  const float f = scale <= ldexp(1.0, kMaxFixExpF) ? (float)scale : 0.0f;
+  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, sp, 0, U, C, sh, FixAcc{acc, n, scale, f, &head->err, 0, 0, 0, 0},
+                      PlainForm<LINE, false>{n_cut, (float)n_cut});
+}
+
+// Accelerations from either kernel's sums. A sum beyond the fixed-point range can only come from a
+// position that is not finite, whose pairs with every particle give NaN.
+__global__ void noalloc_finalize_kernel(const unsigned long long* __restrict__ acc, const double* __restrict__ part,
+                                        const NoallocHead* __restrict__ head, int n, int NT, long long U, int C,
+                                        double pair_scale, double* __restrict__ ax, double* __restrict__ ay,
+                                        double* __restrict__ az) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double s[3] = {0.0, 0.0, 0.0};
+  if (head->sym) {
+    const double inv = 1.0 / head->scale;
+    for (int q = 0; q < 3; ++q)
+      s[q] = head->err ? __longlong_as_double(0x7ff8000000000000LL) : (double)(long long)acc[(size_t)q * n + i] * inv;
+  } else {
+    row_sums(part, i, NT, U, C, s[0], s[1], s[2]);
+  }
+  ax[i] = pair_scale * s[0];
+  ay[i] = pair_scale * s[1];
+  az[i] = pair_scale * s[2];
+}
+
 struct DeviceScratch {
   unsigned char* base = nullptr;  // device address of g_noalloc_scratch on this device
-  int ctas = 0;                   // co-resident CTAs of the pair kernel (capped)
+  int ctas = 0;                   // co-resident CTAs of the row kernel (capped)
+  int sms = 0, sym_ctas = 0;      // SMs; co-resident CTAs of the symmetric kernel
   bool ready = false;
 };
 
@@ -70,12 +170,16 @@ int setup_device(int dev, cudaError_t pending, DeviceScratch** out) {
     void* ptr = nullptr;
     if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess)
       return noalloc_cuda_fail(pending, "cudaGetSymbolAddress of the scratch array failed");
-    int sms = 0, occ = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+    int sms = 0, occ = 0, socc = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&socc, noalloc_sym_kernel<true, true>, kSymThreads, 0) !=
+            cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pair_row_kernel<true, true>, kPairThreads, 0) != cudaSuccess)
       return noalloc_cuda_fail(pending, "device query failed");
     d.base = static_cast<unsigned char*>(ptr);
     d.ctas = std::max(1, std::min(kNoallocMaxCtas, sms * std::max(occ, 1)));
+    d.sms = sms;
+    d.sym_ctas = sms * std::max(socc, 1);
     d.ready = true;
   }
   *out = &d;
@@ -129,19 +233,29 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   const int C = (int)std::min<long long>(U, d->ctas);
   const double invL = 1.0 / L;
 
-  // every byte of the scratch array this call reads, it writes first: the
-  // packed positions here, and each stream-K partial slot whole, before the
+  // every byte of the scratch array this call reads, it writes first: the record, the packed
+  // positions and the cleared sums here, or each stream-K partial slot whole, before the
   // finalize kernel reads it
-  pack_kernel<<<(nn + 255) / 256, 256, 0, st>>>(x, y, z, m, h, nn, invL, jA, jB);
+  NoallocHead* head = reinterpret_cast<NoallocHead*>(d->base + kHeadOffset);
+  unsigned long long* acc = reinterpret_cast<unsigned long long*>(part);
+  const int parts = (nn + kPackThreads - 1) / kPackThreads;
+  cudaMemsetAsync(&head->hmin, 0xff, sizeof head->hmin, st);
+  cudaMemsetAsync(&head->err, 0, 2 * sizeof(int), st);
+  noalloc_pack_kernel<<<parts, kPackThreads, 0, st>>>(x, y, z, m, h, nn, invL, jA, jB, acc, head);
   const bool kahan = precision == STEPS_FP32_KAHAN;
+  int tpb, sp;
+  sym_split(NB, d->sms, true, tpb, sp);
+  const long long SU = (long long)NB * (NB + 1) / 2 * tpb * sp;
+  const int SC = (int)std::min<long long>(SU, 32LL * d->sym_ctas);
+  auto sym = line_form(n_cut) ? (kahan ? noalloc_sym_kernel<true, true> : noalloc_sym_kernel<false, true>)
+                              : (kahan ? noalloc_sym_kernel<true, false> : noalloc_sym_kernel<false, false>);
+  sym<<<SC, kSymThreads, 0, st>>>(jA, jB, nn, n_cut, NB, tpb, sp, SU, SC, acc, head, parts, L);
   auto kernel = line_form(n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
                                  : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
-  kernel<<<C, kPairThreads, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part, 0);
-  BgParams off{};
-  off.mode = STEPS_BG_OFF;
+  kernel<<<C, kPairThreads, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part, 0, &head->sym);
   const int ft = particle_threads(nn);
-  finalize_kernel<<<(nn + ft - 1) / ft, ft, 0, st>>>(part, nn, NT, U, C, -G * invL * invL, off, x, y, z, ax, ay, az,
-                                                     0.0, nullptr, nullptr, nullptr, AccelOut{}, nullptr);
+  noalloc_finalize_kernel<<<(nn + ft - 1) / ft, ft, 0, st>>>(acc, part, head, nn, NT, U, C, -G * invL * invL, ax, ay,
+                                                             az);
   // a launch failure replaces the thread's last error; one equal to the error
   // pending before the call is taken as the caller's, which stays in place
   const cudaError_t after = cudaPeekAtLastError();
