@@ -193,11 +193,14 @@ static __global__ void finalize_kernel(const double* __restrict__ part, int n, i
   if (i >= n) return;
   double sx = 0.0, sy = 0.0, sz = 0.0;
   if (NT == 0) {
-    // direct sums (FP64 pair kernel): part = [3][n - i0]
+    // direct sums (FP64 pair kernel, octree): C sets [3][n - i0]
     const long long q = i - i0, m = n - i0;
-    sx = part[q];
-    sy = part[m + q];
-    sz = part[2 * m + q];
+    for (int c = 0; c < C; ++c) {
+      const double* v = part + 3 * m * c;
+      sx += v[q];
+      sy += v[m + q];
+      sz += v[2 * m + q];
+    }
   } else {
     row_sums(part, i - i0, NT, U, C, sx, sy, sz);
   }

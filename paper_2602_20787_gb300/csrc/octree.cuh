@@ -32,6 +32,7 @@
 // |k| <= n0 exact, the rest from the table), exactly as the direct kernel
 // evaluates a j-tile.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 
 #include "pair_sym.cuh"
@@ -534,27 +535,44 @@ __device__ __forceinline__ void tree_eval(const I2& I, TreeList& L, int nl, int 
 }
 
 #ifndef STEPS_TREE_MIN_BLOCKS
-#define STEPS_TREE_MIN_BLOCKS (20 / STEPS_TREE_WARPS)  // co-resident CTAs per SM asked of the register allocator
+// Co-resident CTAs per SM asked of the register allocator: 24 against 20 walk N = 262,144 in 7.48 against
+// 7.54 ms, 400,000 in 12.3 against 13.3.
+#define STEPS_TREE_MIN_BLOCKS (24 / STEPS_TREE_WARPS)
 #endif
 
 // One warp per group of 32 particles in key order (sA/sB, u4s: key order);
 // out = [3][n] pair sums in internal order (sidx maps key order to internal).
+// parts > 1: that many warps share a group's walk, each taking the subtrees of the tree's level kPartLevel
+// whose number is `part` modulo parts (and part 0 what ends above that level), with its own sums
+// out + 3 n part. A warp's walk takes milliseconds, so with a few warps per place on the GPU the last ones run
+// nearly alone; the opened nodes above the level are tested by every part.
 // FORM: S1xR2 with the near range n0 = 4, any other, or none (the nearest-image table), or the
 // R^3 pair force (no images, no table).
 enum TreeForm { kTreeInf4, kTreeInf, kTreeRaw, kTreeR3 };
+
+#ifndef STEPS_TREE_PART_LEVEL
+#define STEPS_TREE_PART_LEVEL 6
+#endif
+constexpr int kPartLevel = STEPS_TREE_PART_LEVEL, kMaxParts = 8;
+// As many parts as make two and a half warps per place of `places`. Walk at N = 20,000 / 60,000 /
+// 262,144, one part: 0.94 / 1.57 / 8.04 ms; two warps per place (8, 4, 1 parts) 0.60 / 1.36 / 7.93; four
+// (8, 7, 2 parts) 0.60 / 1.54 / 7.54. Level 5 costs the same, 7 more at small N (0.84 at 20,000).
+inline int walk_parts(int groups, int places) {
+  return std::max(1, std::min(kMaxParts, (int)((5LL * places / 2 + groups - 1) / groups)));
+}
 
 template <bool KAHAN, int FORM>
 __global__ void __launch_bounds__(kWalkWarps * 32, STEPS_TREE_MIN_BLOCKS)
 tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, const float4* __restrict__ u4s,
                  const int* __restrict__ sidx, int n, const int4* __restrict__ link, const float4* __restrict__ geo,
                  const float* __restrict__ hmf, const float4* __restrict__ nA, const float4* __restrict__ nB,
-                 TreeCrit C, TableTail T, SurrConst S, double* __restrict__ out,
+                 TreeCrit C, TableTail T, SurrConst S, int parts, double* __restrict__ out,
                  unsigned long long* __restrict__ inter, int* __restrict__ err) {
   __shared__ int stk[kWalkWarps][kWalkStack];
   __shared__ __align__(16) TreeList list[kWalkWarps];
   __shared__ float4 su[kWalkWarps][32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = blockIdx.x * kWalkWarps + w;
+  const int gp = blockIdx.x * kWalkWarps + w, g = gp / parts, part = gp - g * parts;
   if (g * 32 >= n) return;  // the whole warp leaves; the walk uses warp-level synchronisation only
   const int q = g * 32 + lane;
   const bool valid = q < n;
@@ -562,6 +580,7 @@ tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, c
   const float4 a = sA[qc], b = sB[qc];
   const I2 I{dup(a.x), dup(b.x), dup(a.y), dup(b.y), dup(a.z), dup(b.z), dup(b.w), 0};
   const int nvalid = min(32, n - g * 32);
+  const float part_side = ldexpf(1.0f, -kPartLevel);
   int* st = stk[w];
   TreeList& L = list[w];
   TreeSum A;
@@ -617,14 +636,22 @@ tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, c
     }
     top -= c;
     const unsigned lt = (1u << lane) - 1u;
-    const unsigned take = __ballot_sync(0xffffffffu, mine && !open);
-    if (mine && !open) L.put(nl + __popc(take & lt), nA[node], nB[node]);
+    // with several parts, what ends above the level of the split belongs to the first
+    const bool ours = mine && (parts == 1 || part == 0 || gm.w <= part_side);
+    const unsigned take = __ballot_sync(0xffffffffu, ours && !open);
+    if (ours && !open) L.put(nl + __popc(take & lt), nA[node], nB[node]);
     nl += __popc(take);
-    const bool leaf = mine && open && lk.y == 0;
+    const bool leaf = ours && open && lk.y == 0;
     leaves = __ballot_sync(0xffffffffu, leaf);
     lf = make_int2(lk.z, lk.w);
-    // children, those of a lane's node together
-    const int nc = mine && open ? lk.y : 0;
+    // children, those of a lane's node together; at the level of the split this part's alone
+    const bool split = parts > 1 && gm.w == 2.0f * part_side;
+    int first = lk.x, step = 1, nc = mine && open ? lk.y : 0;
+    if (split) {
+      step = parts;
+      first += (part - lk.x % parts + parts) % parts;
+      nc = mine && open ? max(0, (lk.x + lk.y - first + parts - 1) / parts) : 0;
+    }
     int at = nc;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -640,7 +667,7 @@ tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, c
       leaves = 0;
       continue;
     }
-    for (int k = 0; k < nc; ++k) st[at + k] = lk.x + k;
+    for (int k = 0; k < nc; ++k) st[at + k] = first + k * step;
     top += all;
     __syncwarp();
   }
@@ -650,6 +677,7 @@ tree_walk_kernel(const float4* __restrict__ sA, const float4* __restrict__ sB, c
   }
   if (valid) {
     const int i = sidx[q];
+    out += 3 * (long long)n * part;
     double e, o;
     sum2<KAHAN>(A.x, A.cx, e, o);
     out[i] = e + o;

@@ -318,6 +318,7 @@ struct steps_cyl_ctx {
     unsigned long long* inter = nullptr;
     int nodes = 0, depth = 0;
     double interactions = 0.0, build_ms = 0.0, walk_ms = 0.0;
+    int parts = 1;  // warps a group of the last walk was shared by
     bool ready = false;                     // every per-particle buffer above is allocated
     bool fixed = false;
     TreeDraw fd{};                          // the fixed frame
@@ -979,8 +980,8 @@ int tree_build(steps_cyl_ctx* c, const TreeDraw& f) {
   return STEPS_OK;
 }
 
-// The walk: pair sums [3][n] (internal order) into out.
-int tree_walk(steps_cyl_ctx* c, double* out) {
+// The walk: pair sums [parts][3][n] (internal order) into out.
+int tree_walk(steps_cyl_ctx* c, double* out, int parts) {
   Range range("steps_cyl.tree_walk");
   auto& T = c->tr;
   TreeCrit C;
@@ -989,7 +990,7 @@ int tree_walk(steps_cyl_ctx* c, double* out) {
   C.hLu = 0.5f * C.Lu;
   C.th2 = (float)(c->p.theta * c->p.theta);
   const int groups = (c->n + 31) / 32;
-  const int blocks = (groups + kWalkWarps - 1) / kWalkWarps;
+  const int blocks = (int)(((long long)groups * parts + kWalkWarps - 1) / kWalkWarps);
   CKT(cudaMemsetAsync(T.inter, 0, sizeof(unsigned long long), c->st));
   const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
   auto walk = is_r3(c) ? (kahan ? tree_walk_kernel<true, kTreeR3> : tree_walk_kernel<false, kTreeR3>)
@@ -997,7 +998,7 @@ int tree_walk(steps_cyl_ctx* c, double* out) {
               : c->p.n0 > 0 ? (kahan ? tree_walk_kernel<true, kTreeInf> : tree_walk_kernel<false, kTreeInf>)
                             : (kahan ? tree_walk_kernel<true, kTreeRaw> : tree_walk_kernel<false, kTreeRaw>);
   walk<<<blocks, kWalkWarps * 32, 0, c->st>>>(T.sA, T.sB, T.u4s, T.val[0], c->n, T.link, T.geo, T.hmf, T.nA, T.nB, C,
-                                              c->tab, c->tab_const, out, T.inter, c->err);
+                                              c->tab, c->tab_const, parts, out, T.inter, c->err);
   CKLAUNCH("tree_walk");
   return STEPS_OK;
 }
@@ -1049,7 +1050,11 @@ int tree_forces(steps_cyl_ctx* c, double* out) {
   CKT(cudaEventRecord(T.t0, c->st));
   if ((rc = tree_build(c, f))) return rc;
   CKT(cudaEventRecord(T.t1, c->st));
-  if ((rc = tree_walk(c, out))) return rc;
+  int sms = 0;
+  CKT(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
+  T.parts = walk_parts((c->n + 31) / 32, sms * STEPS_TREE_MIN_BLOCKS * kWalkWarps);
+  while (T.parts > 1 && 3 * (size_t)c->n * T.parts > c->part_elems) --T.parts;
+  if ((rc = tree_walk(c, out, T.parts))) return rc;
   CKT(cudaEventRecord(T.t2, c->st));
   unsigned long long inter = 0;
   CKT(cudaMemcpyAsync(&inter, T.inter, sizeof inter, cudaMemcpyDeviceToHost, c->st));
@@ -1256,7 +1261,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     c->last_pairs = c->tr.interactions;
     c->last_sym = false;
     finalize_kernel<<<(c->n + ft - 1) / ft, ft, 0, c->st>>>(
-        c->part, c->n, 0, c->U, c->C, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K,
+        c->part, c->n, 0, c->U, c->tr.parts, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K,
         kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, out, c->err, radial_corr(c));
     CKLAUNCH("finalize");
     return STEPS_OK;
@@ -1337,7 +1342,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
   c->last_straight = false;
   c->last_pairs = (double)(c->k1 - c->k0) * (double)(c->n - 1) * (c->last_sym ? 0.5 : 1.0);
   const int NT = form == Form::FP64 ? 0 : c->NT;
-  const int ctas = form == Form::SURROGATE ? c->SC : form == Form::TABLE ? c->TC : c->C;
+  const int ctas = form == Form::FP64 ? 1 : form == Form::SURROGATE ? c->SC : form == Form::TABLE ? c->TC : c->C;
   // rows [k0, k1): every row, or the rows this context owns when they are sharded
   finalize_kernel<<<(c->k1 - c->k0 + ft - 1) / ft, ft, 0, c->st>>>(
       c->part, c->k1, NT, c->U, ctas, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K,
@@ -1833,7 +1838,7 @@ int tree_calibrate(steps_cyl_ctx* c, int nf, int nb, int ns, const double* frame
       fd.phi = frames[2 * f + 1];
     }
     if ((rc = check_frame(c, fd))) break;
-    if ((rc = tree_build(c, fd)) || (rc = tree_walk(c, c->part))) break;
+    if ((rc = tree_build(c, fd)) || (rc = tree_walk(c, c->part, 1))) break;
     for (int a = 0; a < 3; ++a)
       gather_kernel<<<grid_for(ni, 256), 256, 0, c->st>>>(c->part + (size_t)a * n, dpick, ni, 1.0,
                                                          c->sub + (size_t)a * ni);
