@@ -204,6 +204,16 @@ bool is_host_ptr(const void* p) {
   return at.type != cudaMemoryTypeDevice && at.type != cudaMemoryTypeManaged;
 }
 
+// Memory that kernels on device dev may read: its own or managed.
+bool own_ptr(int dev, const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
+}
+
 int grid_for(int n, int threads) {
   long long g = ((long long)n + threads - 1) / threads;
   return (int)std::max(1LL, std::min(g, 152LL * 32));
@@ -491,23 +501,86 @@ __global__ void morton_box_kernel(const double* __restrict__ x, const double* __
   }
 }
 
-// Interleaved 16-bit cells of the box as sort keys; val[i] = i.
-__global__ void morton_key_kernel(const double* __restrict__ x, const double* __restrict__ y, int n,
-                                  const unsigned long long* __restrict__ box, uint64_t* __restrict__ key,
-                                  int* __restrict__ val) {
-  const double x0 = order_value(box[0]), y0 = order_value(box[1]);
-  const double span = fmax(fmax(order_value(box[2]) - x0, order_value(box[3]) - y0), 1e-300);
-  auto cell = [&](double v) {
+// Interleaved 16-bit cells of the box.
+struct MortonBox {
+  double x0, y0, span;
+  __device__ explicit MortonBox(const unsigned long long* box) {
+    x0 = order_value(box[0]);
+    y0 = order_value(box[1]);
+    span = fmax(fmax(order_value(box[2]) - x0, order_value(box[3]) - y0), 1e-300);
+  }
+  __device__ uint32_t cell(double v) const {
     uint32_t q = (uint32_t)fmin(65535.0, fmax(0.0, floor(v / span * 65536.0)));
     q = (q | (q << 8)) & 0x00FF00FFu;
     q = (q | (q << 4)) & 0x0F0F0F0Fu;
     q = (q | (q << 2)) & 0x33333333u;
     return (q | (q << 1)) & 0x55555555u;
-  };
+  }
+  __device__ uint32_t key(double x, double y) const { return cell(x - x0) | (cell(y - y0) << 1); }
+};
+
+// These cells as sort keys; val[i] = i.
+__global__ void morton_key_kernel(const double* __restrict__ x, const double* __restrict__ y, int n,
+                                  const unsigned long long* __restrict__ box, uint64_t* __restrict__ key,
+                                  int* __restrict__ val) {
+  const MortonBox B(box);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    key[i] = cell(x[i] - x0) | (cell(y[i] - y0) << 1);
+    key[i] = B.key(x[i], y[i]);
     val[i] = i;
   }
+}
+
+// The same order by one CTA for n <= kSmallOrder: box, keys and a bitonic sort of (key, index) words in
+// shared memory; sixteen launches less than the radix sort (of some 50 us).
+constexpr int kSmallOrder = 4096;
+__global__ void __launch_bounds__(1024)
+morton_small_kernel(const double* __restrict__ x, const double* __restrict__ y, int n, int* __restrict__ order) {
+  __shared__ unsigned long long key[kSmallOrder];
+  __shared__ unsigned long long box[4];
+  const int t = threadIdx.x;
+  if (t < 4) box[t] = t < 2 ? ~0ull : 0ull;
+  __syncthreads();
+  {
+    unsigned long long v[4] = {~0ull, ~0ull, 0ull, 0ull};
+    for (int i = t; i < n; i += 1024) {
+      const double p[2] = {x[i], y[i]};
+      for (int a = 0; a < 2; ++a) {
+        if (isnan(p[a])) continue;
+        const unsigned long long w = order_word(p[a]);
+        v[a] = min(v[a], w);
+        v[2 + a] = max(v[2 + a], w);
+      }
+    }
+    for (int a = 0; a < 4; ++a) {
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_xor_sync(0xffffffffu, v[a], o);
+        v[a] = a < 2 ? min(v[a], w) : max(v[a], w);
+      }
+      if ((t & 31) == 0) {
+        if (a < 2) atomicMin(box + a, v[a]);
+        else atomicMax(box + a, v[a]);
+      }
+    }
+  }
+  __syncthreads();
+  int P = 2;
+  while (P < n) P <<= 1;
+  const MortonBox B(box);
+  for (int i = t; i < P; i += 1024) key[i] = i < n ? (unsigned long long)B.key(x[i], y[i]) << 32 | (unsigned)i : ~0ull;
+  for (int k = 2; k <= P; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      __syncthreads();
+      for (int q = t; q < P / 2; q += 1024) {
+        const int a = 2 * q - (q & (j - 1)), b = a + j;
+        const unsigned long long u = key[a], v = key[b];
+        if ((u > v) == ((a & k) == 0)) {
+          key[a] = v;
+          key[b] = u;
+        }
+      }
+    }
+  __syncthreads();
+  for (int i = t; i < n; i += 1024) order[i] = (int)(unsigned)key[i];
 }
 
 // idx[k] = map[order[k]] and copy[k] = order[k]; order null: the identity, map null: idx not written.
@@ -529,6 +602,18 @@ __global__ void invert_kernel(const int* __restrict__ perm, int n, int* __restri
 __global__ void gather_kernel(const double* __restrict__ src, const int* __restrict__ map, int n, double s,
                               double* __restrict__ dst) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) dst[k] = s * src[map[k]];
+}
+
+// dst[k] = s * src[map[k]] for three arrays (the third may be null)
+__global__ void gather3_in_kernel(const double* __restrict__ s0, const double* __restrict__ s1,
+                                  const double* __restrict__ s2, const int* __restrict__ map, int n, double s,
+                                  double* __restrict__ d0, double* __restrict__ d1, double* __restrict__ d2) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int o = map[k];
+    d0[k] = s * s0[o];
+    d1[k] = s * s1[o];
+    if (d2) d2[k] = s * s2[o];
+  }
 }
 
 // dst[map[k]] = s * src[k] for three arrays (null destinations left out)
@@ -617,6 +702,12 @@ int morton_order(steps_cyl_ctx* c, const double* x, const double* y, const int**
   uint64_t* key[2] = {reinterpret_cast<uint64_t*>(c->part), reinterpret_cast<uint64_t*>(c->part) + n};
   int* val[2] = {reinterpret_cast<int*>(c->part + 2 * (size_t)n), reinterpret_cast<int*>(c->part + 2 * (size_t)n) + n};
   unsigned* offs = c->mhist + 256 * (size_t)ntiles;
+  *order = val[0];
+  if (n <= kSmallOrder) {
+    morton_small_kernel<<<1, 1024, 0, c->st>>>(x, y, n, val[0]);
+    CKLAUNCH("morton_small");
+    return STEPS_OK;
+  }
   CK(cudaMemsetAsync(c->mbox, 0xff, 2 * sizeof(unsigned long long), c->st));
   CK(cudaMemsetAsync(c->mbox + 2, 0, 2 * sizeof(unsigned long long), c->st));
   morton_box_kernel<<<std::min(152, grid_for(n, 128)), 128, 0, c->st>>>(x, y, n, c->mbox);
@@ -628,7 +719,6 @@ int morton_order(steps_cyl_ctx* c, const double* x, const double* y, const int**
     radix_scatter_kernel<<<ntiles, kSortThreads, 0, c->st>>>(key[a], val[a], n, 8 * pass, ntiles, offs, key[b], val[b]);
   }
   CKLAUNCH("morton_order");
-  *order = val[0];
   return STEPS_OK;
 }
 
@@ -656,12 +746,9 @@ int order_from_stage(steps_cyl_ctx* c, const double* sx, const double* sy, bool 
   invert_kernel<<<g, 128, 0, c->st>>>(c->perm, c->n, c->iperm);
   CKLAUNCH("order");
   c->perm_h_ok = false;
-  if (carry) {
-    double* tmp = c->part;
-    for (double* arr : {c->m, c->h}) {
-      gather_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(arr, c->ord, c->n, 1.0, tmp);
-      CK(cudaMemcpyAsync(arr, tmp, sizeof(double) * c->n, cudaMemcpyDeviceToDevice, c->st));
-    }
+  if (carry) {  // m and h lie one after the other
+    gather3_in_kernel<<<g, 128, 0, c->st>>>(c->m, c->h, nullptr, c->ord, c->n, 1.0, c->part, c->part + c->n, nullptr);
+    CK(cudaMemcpyAsync(c->m, c->part, sizeof(double) * 2 * c->n, cudaMemcpyDeviceToDevice, c->st));
     CKLAUNCH("carry");
   }
   c->steps_since_order = 0;
@@ -1243,10 +1330,20 @@ int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const Fix
   return STEPS_OK;
 }
 
+DriftStep drift_step(const steps_cyl_ctx* c, const Factors& f) {
+  return DriftStep{f.K1, f.D, c->p.L, c->invL, is_r3(c) ? 0 : 1};
+}
+// Whether the next force evaluation ends in the finalize that can take a kick and drift along.
+bool takes_drift(const steps_cyl_ctx* c) {
+  return !is_tree(c) && c->fix_ready && use_sym(c) && force_form(c) != Form::FP64;
+}
+
 // One force evaluation at the current packed positions. Stores g = a^3 (pair +
 // background) in gx/gy/gz (internal order); kicks p by K when kick is set; writes the accelerations
-// to out besides. cleared: the fixed-point sums are zero already.
-int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = AccelOut{}, bool cleared = false) {
+// to out besides. cleared: the fixed-point sums are zero already. next (where takes_drift, with a kick):
+// the next step's kick and drift follow, and its sums are cleared.
+int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = AccelOut{}, bool cleared = false,
+                const DriftStep* next = nullptr) {
   Range range("steps_cyl.forces");
   const double pair_scale = -c->p.G * c->invL * c->invL;
   c->forces_stale = false;
@@ -1282,6 +1379,13 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     c->last_images = (double)c->n * (double)(c->n - 1) * images_per_pair(c);
     c->last_pairs = sym_pairs(c);
     c->last_sym = true;
+    if (next) {
+      finalize_fix_drift_kernel<<<(c->n + ft - 1) / ft, ft, 0, c->st>>>(
+          c->facc, c->n, 1.0 / c->fix_scale, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K, c->px,
+          c->py, c->pz, c->m, c->h, *next, c->jA, c->jB, c->err);
+      CKLAUNCH("finalize_fix_drift");
+      return STEPS_OK;
+    }
     finalize_fix_kernel<<<(c->n + ft - 1) / ft, ft, 0, c->st>>>(
         c->facc, c->n, 0, c->n, 1.0 / c->fix_scale, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz,
         K, kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, out, c->err);
@@ -1375,15 +1479,19 @@ int gather_in(steps_cyl_ctx* c, const double* src, double* dst, double scale) {
 // Staged positions (caller order) and caller velocities -> internal state.
 int install_state(steps_cyl_ctx* c, const double* vx, const double* vy, const double* vz) {
   double* s = c->stage;
-  gather_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(s, c->perm, c->n, 1.0, c->x);
-  gather_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(s + c->n, c->perm, c->n, 1.0, c->y);
-  gather_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(s + 2 * (size_t)c->n, c->perm, c->n, 1.0, c->z);
+  const size_t n = (size_t)c->n;
+  const int g = grid_for(c->n, 128);
+  gather3_in_kernel<<<g, 128, 0, c->st>>>(s, s + n, s + 2 * n, c->perm, c->n, 1.0, c->x, c->y, c->z);
   CKLAUNCH("gather positions");
-  int rc;
   const double a2 = c->a * c->a;  // canonical momentum p = a^2 dx/dt
-  if ((rc = gather_in(c, vx, c->px, a2))) return rc;
-  if ((rc = gather_in(c, vy, c->py, a2))) return rc;
-  if ((rc = gather_in(c, vz, c->pz, a2))) return rc;
+  const double* v[3] = {vx, vy, vz};
+  if (!own_ptr(c->dev, vx) || !own_ptr(c->dev, vy) || !own_ptr(c->dev, vz))  // through stage, free by now
+    for (int q = 0; q < 3; ++q) {
+      CK(cudaMemcpyAsync(s + q * n, v[q], sizeof(double) * n, cudaMemcpyDefault, c->st));
+      v[q] = s + q * n;
+    }
+  gather3_in_kernel<<<g, 128, 0, c->st>>>(v[0], v[1], v[2], c->perm, c->n, a2, c->px, c->py, c->pz);
+  CKLAUNCH("gather velocities");
   return STEPS_OK;
 }
 
@@ -2554,17 +2662,31 @@ int steps_cyl_kdk_step(steps_cyl_ctx* c, double dt, int32_t nsteps) {
   bool rejected = false;
   char reject_msg[160] = "";
   if (nsteps > 0 && c->forces_stale && (rc = eval_forces(c, false, 0.0))) return rc;
+  auto valid = [](const Factors& f) {
+    return std::isfinite(f.K1) && std::isfinite(f.D) && std::isfinite(f.a_next) && f.a_next > 0;
+  };
+  bool drifted = false;  // the step's kick and drift are done
   for (int s = 0; s < nsteps; ++s) {
     Range range("steps_cyl.kdk_step");
     const Factors f = kdk_factors(c->cosmo, c->a, dt);
-    if (!std::isfinite(f.K1) || !std::isfinite(f.D) || !std::isfinite(f.a_next) || !(f.a_next > 0))
-      return fail(STEPS_EINVAL, "the Friedmann integration left the valid range (a = %g)", f.a_next);
-    const int kt = particle_threads(c->n);
-    kick_drift_pack_kernel<<<grid_for(c->n, kt), kt, 0, c->st>>>(c->x, c->y, c->z, c->px, c->py, c->pz, c->gx, c->gy,
-                                                                 c->gz, c->m, c->h, c->n, f.K1, f.D, c->p.L, c->invL,
-                                                                 c->jA, c->jB, c->err, is_r3(c) ? 0 : 1, c->facc);
-    CKLAUNCH("kick_drift_pack");
-    if ((rc = eval_forces(c, true, f.K2, AccelOut{}, true))) return rc;
+    if (!valid(f)) return fail(STEPS_EINVAL, "the Friedmann integration left the valid range (a = %g)", f.a_next);
+    if (!drifted) {
+      const int kt = particle_threads(c->n);
+      kick_drift_pack_kernel<<<grid_for(c->n, kt), kt, 0, c->st>>>(c->x, c->y, c->z, c->px, c->py, c->pz, c->gx, c->gy,
+                                                                   c->gz, c->m, c->h, c->n, drift_step(c, f), c->jA,
+                                                                   c->jB, c->err, c->facc);
+      CKLAUNCH("kick_drift_pack");
+    }
+    // the next step's kick and drift go with this step's finalize when nothing stands between them
+    DriftStep next{};
+    drifted = false;
+    if (s + 1 < nsteps && !(c->p.reorder_every > 0 && c->steps_since_order + 1 >= c->p.reorder_every) &&
+        !(c->p.tail != STEPS_TAIL_FULL && c->p.check_every > 0 && c->steps_since_check + 1 >= c->p.check_every)) {
+      const Factors fn = kdk_factors(c->cosmo, f.a_next, dt);
+      drifted = valid(fn) && takes_drift(c);
+      next = drift_step(c, fn);
+    }
+    if ((rc = eval_forces(c, true, f.K2, AccelOut{}, true, drifted ? &next : nullptr))) return rc;
     c->a = f.a_next;
     c->t += dt;
     if (c->p.reorder_every > 0 && ++c->steps_since_order >= c->p.reorder_every) {
@@ -2748,7 +2870,7 @@ int steps_cyl_shard_drift(steps_cyl_ctx* c, double dt, float* send) {
   const int k0 = c->k0, rows = c->k1 - c->k0;
   kick_drift_pack_kernel<<<grid_for(rows, 256), 256, 0, c->st>>>(
       c->x + k0, c->y + k0, c->z + k0, c->px + k0, c->py + k0, c->pz + k0, c->gx + k0, c->gy + k0, c->gz + k0,
-      c->m + k0, c->h + k0, rows, f.K1, f.D, c->p.L, c->invL, c->jA + k0, c->jB + k0, c->err, is_r3(c) ? 0 : 1, nullptr);
+      c->m + k0, c->h + k0, rows, drift_step(c, f), c->jA + k0, c->jB + k0, c->err, nullptr);
   CKLAUNCH("kick_drift_pack");
   shard_send_kernel<<<grid_for(c->chunk, 256), 256, 0, c->st>>>(c->jA, c->jB, k0, rows, c->chunk,
                                                                  reinterpret_cast<float4*>(send));
