@@ -168,6 +168,11 @@ __device__ __forceinline__ int jslot(int k) {
 // After each group of STEPS_KAHAN_GROUP steps the sums (of 2 x 8 terms) are added
 // to the slots' sums in the warp's shared row, so that no FP32 running sum is
 // longer than those groups.
+// COMP: the rounding of each sum of groups is kept beside it (exactly, by the two-sum), in the second half
+// of a row of 2 kJRow floats, so that only the groups themselves round. The R^3 force takes it: there
+// four rows per lane make a group of 64 terms, and its 2-norm error against FP64 at N = 20,000 was 3.38e-7 without,
+// 3.27e-7 with it (as with sums of 16 terms), for 1.5% of its time.
+template <bool COMP>
 struct JRing {
   float a[3] = {0.f, 0.f, 0.f};
   // a += m_i v of both pairs: X = m_i sr (packed), Z = m_i sz
@@ -201,7 +206,16 @@ struct JRing {
     __syncwarp();  // the slots' last sums were written by other lanes
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      d[c] = first ? a[c] : d[c] + a[c];
+      if (!COMP) {
+        d[c] = first ? a[c] : d[c] + a[c];
+      } else if (first) {
+        d[c] = a[c];
+        d[kJRow + c] = 0.f;
+      } else {
+        const float o = d[c], t = o + a[c], b = t - o;
+        d[kJRow + c] += (o - (t - b)) + (a[c] - b);
+        d[c] = t;
+      }
       a[c] = 0.f;
     }
   }
@@ -435,7 +449,7 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
       load_tile2<kSymThreads>(jA, jB, n, t, jt, sh.T);
       __syncthreads();
       const bool sym = t / tpb != b;
-      JRing ring;
+      JRing<false> ring;
 #pragma unroll 1
       for (int k0 = kb; k0 < kb + ks; k0 += STEPS_KAHAN_GROUP) {
         u64 gx = 0, gy = 0, gz = 0;
@@ -521,7 +535,7 @@ pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ 
 // ring's three shuffles and the loop serve four pairs, and one warp is a CTA. With two
 // rows per lane the duplicated j words alone would keep the shared-memory pipe busier
 // than the FP32 one. The row kernel (r3_pair.cuh) evaluates every ordered pair in 31 issue
-// slots per 32 pairs: 3.33 ms per force at N = 65,536 against 2.77 here.
+// slots per 32 pairs: 3.39 ms per force at N = 65,536 against 2.85 here.
 #ifndef STEPS_SYM_R3_MIN_BLOCKS
 #define STEPS_SYM_R3_MIN_BLOCKS 16  // resident CTAs (warps) per SM the kernel is compiled for
 #endif
@@ -536,7 +550,7 @@ pair_sym_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
                    int C, FixAcc F) {
   constexpr int NS = kBI / 64;  // packed sets of two rows per lane
   __shared__ JTile2 T;
-  __shared__ float row[kJRow];
+  __shared__ float row[2 * kJRow];
   const int c = blockIdx.x, lane = threadIdx.x;
   const long long u1 = (long long)(c + 1) * U / C;
   const int jt = kBJ / tpb;
@@ -559,7 +573,7 @@ pair_sym_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
       load_tile2<32>(jA, jB, n, t, jt, T);
       __syncwarp();
       const bool sym = t / tpb != b;
-      JRing ring;
+      JRing<true> ring;
 #pragma unroll 1
       for (int k0 = 0; k0 < jt; k0 += STEPS_KAHAN_GROUP) {
         u64 g[NS][3];
@@ -625,7 +639,7 @@ pair_sym_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
           const int j = t * jt + s;
           if (j < n) {
 #pragma unroll
-            for (int q = 0; q < 3; ++q) fix_add(F, q, j, -fix_value(F, row[3 * s + q]));
+            for (int q = 0; q < 3; ++q) fix_add(F, q, j, -fix_value(F, row[3 * s + q]) - fix_value(F, row[kJRow + 3 * s + q]));
           }
         }
       }
