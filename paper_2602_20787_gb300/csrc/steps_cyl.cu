@@ -2191,14 +2191,6 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
   CK(cudaEventCreate(&t0));
   CK(cudaEventCreate(&t1));
   CK(cudaEventRecord(t0, c->st));
-  // samples: dR with density ~ dR (pairs in a plane), |dz| and h uniform
-  SplitMix rng(cfg->seed);
-  std::vector<double> smp(3 * (size_t)ns);
-  for (int64_t s = 0; s < ns; ++s) {
-    smp[3 * s] = dR_max * std::sqrt(rng.uniform());
-    smp[3 * s + 1] = 0.5 * rng.uniform();
-    smp[3 * s + 2] = A * rng.uniform();
-  }
   TrainBuffers B;
   B.st = c->st;
   const int maxblocks = cfg->batch / kTrainThreads;
@@ -2216,7 +2208,10 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
   CK(cudaMallocAsync(&B.gpart, sizeof(float) * kNW * nb_alloc, c->st));
   CK(cudaMallocAsync(&B.lpart, sizeof(float) * nb_alloc, c->st));
   CK(cudaMallocAsync(&B.loss, sizeof(float), c->st));
-  CK(cudaMemcpyAsync(B.smp, smp.data(), sizeof(double) * 3 * ns, cudaMemcpyHostToDevice, c->st));
+  SplitMix rng(cfg->seed);
+  training_samples_kernel<<<grid_for((int)std::min<int64_t>(ns, 1 << 30), 128), 128, 0, c->st>>>(rng.s, ns, dR_max, A,
+                                                                                               B.smp);
+  rng.skip(3 * (uint64_t)ns);
   // exact FP64 targets, residual over the base, in envelope units
   tail_sums_fp64_kernel<<<grid_for((int)std::min<int64_t>(ns, 1 << 30), 128), 128, 0, c->st>>>(B.smp, ns, n_cut, n0,
                                                                                              B.tail);
@@ -2270,7 +2265,8 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
   // The epochs' sample orders: each a Fisher-Yates shuffle of its own stretch of the generator's
   // sequence, so several are drawn ahead on host threads (one takes 0.9 ms for 245,760
   // samples, the GPU's epoch less).
-  const int ahead = (int)std::max(1u, std::min({8u, std::thread::hardware_concurrency(), (unsigned)cfg->epochs}));
+  const int ahead = (int)std::max<int64_t>(1, std::min<int64_t>({8, std::thread::hardware_concurrency(), cfg->epochs,
+                                                                 (1LL << 26) / ntrain}));  // 256 MB of orders at most
   auto shuffled = [ntrain](SplitMix g) {
     std::vector<int> order(ntrain);
     for (int64_t k = 0; k < ntrain; ++k) order[k] = (int)k;

@@ -140,6 +140,23 @@ __host__ __device__ __forceinline__ void tail_base_inf_fp64(double dR, double ad
   EZ = e * e * sqrt(e);
 }
 
+// Training samples: dR with density ~ dR (pairs in a plane), |dz| and h uniform, from the draws
+// 3 s .. 3 s + 2 of the generator (SplitMix64 of state seed, a counter).
+__device__ __forceinline__ double splitmix_uniform(uint64_t seed, uint64_t draw) {
+  uint64_t z = seed + (draw + 1) * 0x9E3779B97F4A7C15ull;
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  return (double)((z ^ (z >> 31)) >> 11) * (1.0 / 9007199254740992.0);
+}
+static __global__ void training_samples_kernel(uint64_t seed, int64_t ns, double dR_max, double A,
+                                               double* __restrict__ smp) {
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
+    smp[3 * s] = dR_max * sqrt(splitmix_uniform(seed, 3 * s));
+    smp[3 * s + 1] = 0.5 * splitmix_uniform(seed, 3 * s + 1);
+    smp[3 * s + 2] = A * splitmix_uniform(seed, 3 * s + 2);
+  }
+}
+
 // Training pairs: inputs u (FP32, ns x 3) and raw targets r = (tail - B1) / E
 // (FP64, ns x 2, before the mean/scale normalisation) from exact tail sums
 // (n_cut = 0: the infinite window over its base).
