@@ -452,15 +452,14 @@ constexpr unsigned kBarrierSpins = 1u << 22;  // polls (of some 0.5 us) before a
 __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, int* fail) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(bar, 1u);
+    // release: the CTA's writes (ordered before by the block's barrier) are visible with the arrival
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     unsigned seen = 0;
     for (unsigned k = 0; k < kBarrierSpins; ++k) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
       if (seen >= target || ((k & 1023u) == 1023u && atomicAdd(fail, 0) != 0)) break;
     }
     if (seen < target) atomicExch(fail, 1);
-    __threadfence();
   }
   __syncthreads();
 }
