@@ -528,9 +528,9 @@ int steps_cyl_check_surrogate(steps_cyl_ctx* ctx, int32_t check_particles, doubl
  * loop that must not take cudaMalloc's implicit device-wide synchronisation, or
  * a plug-in that may allocate only while it initialises. Its result is what
  * steps_cyl_forces returns for a context with background STEPS_BG_OFF in static
- * space (a = 1), computed with the same kernels, and it calls no cudaMalloc,
+ * space (a = 1), computed with the same pair forms, and it calls no cudaMalloc,
  * cudaFree or allocating library routine. Its scratch (packed positions and the
- * work split's partial sums) is one file-scope device array of
+ * pair sums) is one file-scope device array of
  * STEPS_NOALLOC_SCRATCH_BYTES bytes that every device loading this library
  * holds until the process exits.
  *   - n: 2 <= n <= STEPS_NOALLOC_MAX_N, else STEPS_EINVAL (nothing is launched).

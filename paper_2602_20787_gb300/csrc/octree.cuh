@@ -18,11 +18,12 @@
 // largest softening. Each node is packed as a pseudo-particle in the layout of
 // the pair kernels (hi/lo position over L, mass, h/L).
 //
-// Walk. One warp per group of 32 consecutive particles in key order, all lanes
-// on one shared stack, up to 32 nodes a step: a lane takes a node and tests it against the
-// group's particles one by one. (All lanes on one node waited for the node's three dependent
-// loads from L2, some 3,500 times per group: 9.58 ms at N = 262,144 against 8.94, 1.28 against 1.04 at 20,000.) A node is opened for the group when any particle opens it:
-// s^2 >= theta^2 d^2, or |d| - (sqrt(3)/2) s <= hu_i + hu_max (d: offset of u
+// Walk. One warp per group of 32 consecutive particles in key order (several at small
+// N), all lanes on one shared stack, up to 32 nodes a step: a lane takes a node and tests it
+// against the group's particles one by one. (All lanes on one node waited for the node's
+// three dependent loads from L2, some 3,500 times per group: 9.58 ms at N = 262,144 against
+// 8.94, 1.28 against 1.04 at 20,000.) A node is opened for the group when any particle opens
+// it: s^2 >= theta^2 d^2, or |d| - (sqrt(3)/2) s <= hu_i + hu_max (d: offset of u
 // from the node centre with z wrapped to the nearest image, hu = h / S). The
 // test is evaluated in FP32 with exactly rounded operations in the order
 // written, so it is reproducible off the GPU. An accepted node, or the

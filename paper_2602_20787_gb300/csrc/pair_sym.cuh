@@ -13,7 +13,7 @@
 // stream-K split of the row kernels. A block is 128 rows, two per thread (pair2.cuh),
 // so a CTA is two warps. A tile is a block's 128 rows, or a quarter of them when there
 // are too few blocks to fill the GPU: at N = 2,048 the 136 whole units leave most SMs one
-// CTA (134 us), the 544 quarter units take 55 us. A unit of the diagonal block evaluates
+// CTA (134 us a force), the 544 quarter units take 55 us, their steps split in two 50. A unit of the diagonal block evaluates
 // all ordered pairs for the i side only (the self pair adds exact zeros); the others
 // evaluate their pairs once and add each to both sides.
 //
