@@ -304,23 +304,6 @@ static __global__ void kick_drift_pack_kernel(double* __restrict__ x, double* __
   }
 }
 
-// y = s x for three arrays (acceleration output = g / a^3).
-static __global__ void scale3_kernel(const double* __restrict__ ax, const double* __restrict__ ay,
-                              const double* __restrict__ az, int n, double s, double* __restrict__ ox,
-                              double* __restrict__ oy, double* __restrict__ oz) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    ox[i] = ax[i] * s; oy[i] = ay[i] * s; oz[i] = az[i] * s;
-  }
-}
-
-// p = a^2 v (and back) on three arrays.
-static __global__ void axpy_scale3_kernel(double* __restrict__ a0, double* __restrict__ a1, double* __restrict__ a2,
-                                   int n, double s) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    a0[i] *= s; a1[i] *= s; a2[i] *= s;
-  }
-}
-
 // Deterministic reductions for the diagnostics: each block writes its partial
 // sums of (m px, m py, m pz, m (x py - y px), m |p|^2 / 2, m) into part[block][6].
 constexpr int kRedThreads = 256;

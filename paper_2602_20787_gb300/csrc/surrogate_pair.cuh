@@ -350,50 +350,6 @@ __device__ __forceinline__ void surr_stage_a(float dR2, float dz, float hh, int 
   P.u[2] = fmaf(fminf(hh, A), S.two_over_A, -1.0f);
 }
 
-// Stage A of a pair that no lane of the warp has inside its softening support
-// (kw < 0), with the near range n0 = 4 fixed: the same arithmetic as
-// surr_stage_a on that path (centre image, then the four image pairs +-k
-// packed, then the tail base, envelope and inputs), written without a branch so
-// that a caller can place it in one straight run with the network.
-template <bool INF = false>
-__device__ __forceinline__ void surr_stage_a_far4(float dR2, float dz, float hh, const SurrConst& S, SurrPair& P) {
-  const float adz = fabsf(dz), A = S.A;
-  const float dR = dR2 * rsq(fmaxf(dR2, 1e-30f));
-  P.u[0] = fmaf(fminf(dR, S.dR_max), S.two_inv_dR_max, -1.0f);
-  P.u[1] = fmaf(adz, 4.0f, -1.0f);
-  P.u[2] = fmaf(fminf(hh, A), S.two_over_A, -1.0f);
-  // near images |k| <= 4, all Newtonian
-  const u64 DR2 = pk(dR2, dR2);
-  const u64 STEP = pk(1.0f, -1.0f);
-  u64 O = pk(dz, dz);
-  u64 SR = pk(0.0f, 0.0f), SZ = pk(0.0f, 0.0f);
-  const float ri = rsq(fmaf(dz, dz, dR2));
-  const float cr = ri * ri * ri;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) newton_pair(O, STEP, DR2, SR, SZ);
-  float s0, s1, z0, z1;
-  upk(SR, s0, s1);
-  upk(SZ, z0, z1);
-  const float sr = (s0 + s1) + cr;
-  const float sz = (z0 + z1) + dz * cr;
-  // tail base and envelope, as in surr_stage_a
-  float br, bz, il1;
-  if (INF) {
-    tail_base_inf_fp32(dR2, A + adz, A - adz, br, bz, il1);
-  } else {
-    const float hb = (adz > 0.0f ? S.fnh + 1.0f : S.fnh) - adz;
-    tail_base_fp32(dR2, A + adz, A - adz, S.fnh + adz, hb, br, bz, il1);
-  }
-  const float e = il1 * il1;
-  const float er = e * e * e;
-  const float sg = dz > 0.0f ? 1.0f : (dz < 0.0f ? -1.0f : 0.0f);
-  const float ez = sg * (e * e * il1);
-  P.a0 = fmaf(er, S.mu0, sr + br);
-  P.b0 = er * S.sc0;
-  P.a1 = fmaf(ez, S.mu1, fmaf(sg, bz, sz));
-  P.b1 = ez * S.sc1;
-}
-
 // Stage C: tail = base + envelope x network output, plus the exact spline
 // correction of tail images inside some lane's softening support.
 // The separation is recomputed from the tile (same arithmetic, same values)
