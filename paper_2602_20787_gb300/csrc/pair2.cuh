@@ -254,12 +254,22 @@ __device__ __forceinline__ void near_newton2(u64 R2C, u64 DR2, u64 ADZ, int m, u
   for (int k = 1; k <= m; ++k, fk += 1.0f) newton_k2(ADZ, fk, DR2, SR, SZ);
 }
 
+// The last image that a support of the warp's pairs can reach from |dz| <= 1/2: rn(h).
+__device__ __forceinline__ int soft_reach2(u64 HH) {
+  float a, b;
+  upk(add2(HH, dup(kTwo23)), a, b);  // 2^23 + rn(h)
+  return __reduce_max_sync(0xffffffffu, max(__float_as_int(a), __float_as_int(b))) - kTwo23Bits;
+}
+
 // What the softened images m < |k| <= kw add to a Newtonian far part: spline minus
-// Newtonian. n_cut > 0: the window's edge image (k = n_cut, on one side, absent at
-// dz = 0) ends them.
-__device__ __forceinline__ void far_soft2(u64 DR2, const Soft2& s, u64 ADZ, int m, int kw, int n_cut, u64& SR,
+// Newtonian. The window's edge image (k = n_cut, on one side, absent at dz = 0) ends them;
+// INF (n_cut unused): over the infinite window rn(h) does, as a position that is not a number
+// makes kw as large as an integer can be. (A template, so that the plain window's registers
+// hold no h: at run time the choice cost 2% of its literal-law force.)
+template <bool INF>
+__device__ __forceinline__ void far_soft2(u64 DR2, u64 HH, const Soft2& s, u64 ADZ, int m, int kw, int n_cut, u64& SR,
                                           u64& SZ) {
-  const int ke = n_cut > 0 ? min(kw, n_cut) : kw;
+  const int ke = min(kw, INF ? soft_reach2(HH) : n_cut);
   float fk = (float)(m + 1);
 #pragma unroll 1
   for (int k = m + 1; k <= ke; ++k, fk += 1.0f) {
@@ -267,7 +277,7 @@ __device__ __forceinline__ void far_soft2(u64 DR2, const Soft2& s, u64 ADZ, int 
     const u64 RA = fma2(OA, OA, DR2), RB = fma2(OB, OB, DR2);
     u64 DA = fma2(inv_r3(RA), dup(-1.0f), spline2<true, false>(RA, s));
     u64 DB = fma2(inv_r3(RB), dup(-1.0f), spline2<true, false>(RB, s));
-    if (k == n_cut) {
+    if (!INF && k == n_cut) {
       DA = mul2(DA, flag_nonzero2(ADZ));
       DB = 0;
     }
@@ -504,7 +514,7 @@ __device__ __forceinline__ void window2(const Sep2& P, int n_cut, float fnc, u64
       }
       CR = spline_centre2(R2C, H2, s);
       near_soft2<kPolyNear>(P.dr2, s, ADZ, kw, soft_bound2(mul2(H2, dup(0.25f)), P.dr2, ADZ), SR, SZ);
-      if (kw > kPolyNear) far_soft2(P.dr2, s, ADZ, kPolyNear, kw, n_cut, SR, SZ);
+      if (kw > kPolyNear) far_soft2<false>(P.dr2, P.hh, s, ADZ, kPolyNear, kw, n_cut, SR, SZ);
     }
   }
   SR = add2(SR, CR);

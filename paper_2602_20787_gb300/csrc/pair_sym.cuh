@@ -320,7 +320,7 @@ __device__ __forceinline__ void model_stage2(const Sep2& P, u64 ADZ, int n_cut, 
         near_soft2<kPolyNear>(P.dr2, s, ADZ, kw, k1, SR, SZ);
       else
         near_soft_walk2(P.dr2, s, ADZ, m, kw, k1, SR, SZ);
-      if (kw > m) far_soft2(P.dr2, s, ADZ, m, kw, INF ? 0 : n_cut, SR, SZ);
+      if (kw > m) far_soft2<INF>(P.dr2, P.hh, s, ADZ, m, kw, n_cut, SR, SZ);
     }
   } else if (!POLY) {
     near_newton2(R2C, P.dr2, ADZ, m, CR, SR, SZ);
