@@ -62,6 +62,7 @@ struct Soft64 {
   double hh2, ih, ih3;
 };
 constexpr double kTinyR2 = 1e-150;  // floor of r^2: keeps the seed and its cube finite
+constexpr double kHugeR2 = 1e300;   // its ceiling: keeps the seed's square normal and the series finite
 
 // F / r at r^2 = r2: y0^3 (1 + 3 e / 2 + 15 e^2 / 8) with e = 1 - r^2 y0^2 for 1 / r^3, and
 // the spline where soft and r < h.
@@ -157,11 +158,13 @@ enum Pair64 { kPair64Walk, kPair64Line, kPair64R3 };
 template <int KIND>
 __device__ __forceinline__ void window64(double dR2, double dz, double hh, int n_cut, double& SR, double& SZ) {
   const double adz = fabs(dz);
+  if (less_pos(kHugeR2, dR2)) dR2 = kHugeR2;  // a NaN stays one in dx or dy
   Soft64 h;
   h.hh2 = hh * hh;
   h.ih = h.ih3 = 0.0;
   const double c2 = fma(adz, adz, dR2);
-  const double r2c = less_pos(c2, kTinyR2) ? kTinyR2 : c2;
+  double r2c = less_pos(c2, kTinyR2) ? kTinyR2 : c2;
+  if (KIND == kPair64R3 && less_pos(kHugeR2, r2c)) r2c = kHugeR2;
   const bool soft = less_pos(c2, h.hh2);
   int m = KIND == kPair64Line ? kNear64 : n_cut - 1;
   float R2f = 0.0f;
