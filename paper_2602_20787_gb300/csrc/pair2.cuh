@@ -363,11 +363,12 @@ __device__ __forceinline__ u64 base_poly_z(u64 Q, u64 D2) {
 }
 
 // The far ends: s and e at N, and what they add to the sums to infinity (the integral
-// of f ends at N). Products of several powers of 1 / dR are taken with the reciprocal of
-// s + s_N among them, so that none leaves FP32's normal range before the sum itself does
-// (e e_N alone does from dR = 3e9 on; this order costs 0.9%: N = 65,536, N_cut = 16, literal law
-// 13.34 -> 13.46 ms); kFarFloor keeps that reciprocal finite where dR^2 is infinite, and is below
-// s_N's rounding elsewhere.
+// of f ends at N). e e_N / (s + s_N): the product of the two squares leaves FP32's normal range
+// from dR = 3e9 on. WIDE takes the reciprocal between them, so that no product does before the
+// sum itself: the row kernels, whose sums are in floating point. In the symmetric kernels all pairs
+// so far apart add up to a few units of the fixed-point sums at most, and they keep the order with the
+// shorter chain (N = 65,536, N_cut = 16, literal law: 13.35 ms, the other order 13.46). kFarFloor
+// keeps the reciprocals finite where dR^2 is infinite, and is below the rounding of what it is added to elsewhere.
 constexpr float kFarFloor = 1e-30f;
 struct FarEnd2 {
   u64 IH, SN, EN, R, Z;
@@ -405,7 +406,7 @@ __device__ __forceinline__ void fix_dz0(u64 ADZ, u64 DR2, float N, u64& SR, u64&
 
 // The images beyond the near ones |k| <= kPolyNear added to (SR, SZ), at ADZ >= 0. INF:
 // the infinite line, else the window of N. BASE: with the modelled tails' base.
-template <bool INF, bool BASE>
+template <bool INF, bool BASE, bool WIDE = false>
 __device__ __forceinline__ void line_far2(u64 DR2, u64 ADZ, float N, u64& SR, u64& SZ) {
   const u64 IL = rsq2(add2(DR2, dup(kPolyA * kPolyA)));
   const u64 S = mul2(IL, dup(kPolyA)), E = mul2(IL, IL);
@@ -417,7 +418,8 @@ __device__ __forceinline__ void line_far2(u64 DR2, u64 ADZ, float N, u64& SR, u6
     I = mul2(mul2(E, dup(2.0f)), rcp2(add2(S, dup(1.0f))));
   } else {
     const FarEnd2 f = far_end2(DR2, ADZ, N);
-    I = fma2(mul2(E, dup(2.0f * (N * N - kPolyA * kPolyA))), mul2(f.EN, rcp2(add2(S, f.SN))), f.R);
+    const u64 EC = mul2(E, dup(2.0f * (N * N - kPolyA * kPolyA))), V = rcp2(add2(S, f.SN));
+    I = WIDE ? fma2(EC, mul2(f.EN, V), f.R) : fma2(mul2(EC, f.EN), V, f.R);
     SZ = add2(SZ, f.Z);
   }
   SR = add2(SR, fma2(mul2(G, E), T, I));
@@ -431,10 +433,12 @@ __device__ __forceinline__ void line_far2(u64 DR2, u64 ADZ, float N, u64& SR, u6
 struct LineSide2 {
   u64 NR, IL, Z;
 };
+template <bool WIDE>
 __device__ __forceinline__ LineSide2 line_side2(u64 LO, u64 DR2, const FarEnd2& f, float N2) {
   const u64 IL = rsq2(fma2(LO, LO, DR2));
   const u64 S = mul2(LO, IL), E = mul2(IL, IL);
-  const u64 NI = mul2(mul2(fma2(LO, LO, dup(-N2)), E), mul2(f.EN, rcp2(add2(S, f.SN))));
+  const u64 NN = fma2(LO, LO, dup(-N2)), V = rcp2(add2(S, f.SN));
+  const u64 NI = WIDE ? mul2(mul2(NN, E), mul2(f.EN, V)) : mul2(mul2(NN, mul2(E, f.EN)), V);
   const u64 Q = mul2(S, S), W = mul2(E, Q);
   u64 PR = fma2(W, dup(0.238131417f), fma2(E, dup(-0.168406769f), dup(-0.127495596f)));
   PR = fma2(W, PR, fma2(E, dup(0.0547808694f), dup(0.125f)));
@@ -446,6 +450,7 @@ __device__ __forceinline__ LineSide2 line_side2(u64 LO, u64 DR2, const FarEnd2& 
 // ---- image sums of the plain window ------------------------------------------------
 // The images one by one up to m (softened: to the bounds kw, k1), then the far part of
 // each side in closed form from A = m + 1/2, or for m = n_cut - 1 the edge image.
+template <bool WIDE>
 __device__ __forceinline__ void window_walk2(u64 DR2, u64 HH, u64 R2C, u64 ADZ, bool soft, int m, int n_cut,
                                              float fnc, u64& SR, u64& SZ) {
   u64 CR, H2 = mul2(HH, HH);
@@ -471,19 +476,21 @@ __device__ __forceinline__ void window_walk2(u64 DR2, u64 HH, u64 R2C, u64 ADZ, 
   }
   const FarEnd2 f = far_end2(DR2, ADZ, fnc);
   const float A = (float)m + 0.5f;
-  const LineSide2 a = line_side2(add2(ADZ, dup(A)), DR2, f, fnc * fnc);
-  const LineSide2 b = line_side2(sub2(dup(A), ADZ), DR2, f, fnc * fnc);
+  const LineSide2 a = line_side2<WIDE>(add2(ADZ, dup(A)), DR2, f, fnc * fnc);
+  const LineSide2 b = line_side2<WIDE>(sub2(dup(A), ADZ), DR2, f, fnc * fnc);
   SR = add2(SR, sub2(f.R, add2(a.NR, b.NR)));
   // the integrals of z f, IL_a - IL_b, without cancellation at large dR
   const u64 P = mul2(a.IL, b.IL);
-  const u64 IZ = mul2(mul2(P, mul2(ADZ, dup(-4.0f * A))), mul2(P, rcp2(add2(a.IL, add2(b.IL, dup(kFarFloor))))));
+  const u64 AD = mul2(ADZ, dup(-4.0f * A)), V = rcp2(add2(add2(a.IL, dup(kFarFloor)), b.IL));
+  const u64 IZ = WIDE ? mul2(mul2(P, AD), mul2(P, V)) : mul2(mul2(mul2(P, P), AD), V);
   SZ = add2(SZ, add2(add2(IZ, sub2(a.Z, b.Z)), f.Z));
   fix_dz0<true>(ADZ, DR2, fnc, SR, SZ);
 }
 // The same out of line, for the rare steps of the closed form.
+template <bool WIDE>
 static __device__ __noinline__ ulonglong2 window_walk_call2(u64 DR2, u64 HH, u64 ADZ, int n_cut) {
   u64 SR, SZ;
-  window_walk2(DR2, HH, fma2(ADZ, ADZ, DR2), ADZ, true, kPolyMaxSoft, n_cut, (float)n_cut, SR, SZ);
+  window_walk2<WIDE>(DR2, HH, fma2(ADZ, ADZ, DR2), ADZ, true, kPolyMaxSoft, n_cut, (float)n_cut, SR, SZ);
   return make_ulonglong2(SR, SZ);
 }
 
@@ -491,15 +498,15 @@ static __device__ __noinline__ ulonglong2 window_walk_call2(u64 DR2, u64 HH, u64
 // the near ones in closed form (line_form(n_cut)), else every image walked.
 // FAR: every h_i + h_j below half a period, so only the centre image can be
 // softened: the near images are taken as Newtonian in one straight run and the centre
-// replaced where it is softened.
-template <bool LINE, bool FAR>
+// replaced where it is softened. WIDE: see far_end2.
+template <bool LINE, bool FAR, bool WIDE = false>
 __device__ __forceinline__ void window2(const Sep2& P, int n_cut, float fnc, u64& SR, u64& SZ) {
   static_assert(!FAR || LINE, "the straight run belongs to the closed far part");
   const u64 ADZ = abs2(P.dz);
   const u64 R2C = fma2(ADZ, ADZ, P.dr2), H2 = mul2(P.hh, P.hh);
   const bool soft = any_less2(R2C, H2);
   if (!LINE) {
-    window_walk2(P.dr2, P.hh, R2C, ADZ, soft, n_cut - 1, n_cut, fnc, SR, SZ);
+    window_walk2<WIDE>(P.dr2, P.hh, R2C, ADZ, soft, n_cut - 1, n_cut, fnc, SR, SZ);
     SZ = mulsign2(SZ, P.dz);
     return;
   }
@@ -512,7 +519,7 @@ __device__ __forceinline__ void window2(const Sep2& P, int n_cut, float fnc, u64
     } else {
       const int kw = soft_bound2(H2, P.dr2, ADZ);
       if (kw > kPolyMaxSoft) {
-        const ulonglong2 w = window_walk_call2(P.dr2, P.hh, ADZ, n_cut);
+        const ulonglong2 w = window_walk_call2<WIDE>(P.dr2, P.hh, ADZ, n_cut);
         SR = w.x;
         SZ = mulsign2(w.y, P.dz);
         return;
@@ -524,7 +531,7 @@ __device__ __forceinline__ void window2(const Sep2& P, int n_cut, float fnc, u64
   }
   SR = add2(SR, CR);
   SZ = fma2(ADZ, CR, SZ);
-  line_far2<false, false>(P.dr2, ADZ, fnc, SR, SZ);
+  line_far2<false, false, WIDE>(P.dr2, ADZ, fnc, SR, SZ);
   fix_dz0<true>(ADZ, P.dr2, fnc, SR, SZ);
   SZ = mulsign2(SZ, P.dz);
 }
@@ -565,7 +572,7 @@ pair_row_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, in
           Sep2 P;
           separation2(I, T, k, P);
           u64 SR, SZ;
-          window2<LINE, false>(P, n_cut, fnc, SR, SZ);
+          window2<LINE, false, true>(P, n_cut, fnc, SR, SZ);
           const u64 m = T.MH[k].x, MS = mul2(m, SR);
           gx = fma2(P.dx, MS, gx);
           gy = fma2(P.dy, MS, gy);

@@ -14,10 +14,12 @@ WRAP = r"""
 extern "C" void run(int kind, float d2, float adz, int n_cut, float* out) {
   const u64 DR2 = dup(d2), ADZ = dup(adz);
   u64 SR = 0, SZ = 0;
-  if (kind == 0) { line_far2<false, false>(DR2, ADZ, (float)n_cut, SR, SZ); }
+  if (kind == 0) { line_far2<false, false, true>(DR2, ADZ, (float)n_cut, SR, SZ); }
+  if (kind == 4) { line_far2<false, false>(DR2, ADZ, (float)n_cut, SR, SZ); }
   if (kind == 1) { line_far2<true, false>(DR2, ADZ, 0.0f, SR, SZ); }
   if (kind == 2) { line_far2<false, true>(DR2, ADZ, (float)n_cut, SR, SZ); }
-  if (kind == 3) window_walk2(DR2, dup(0.0f), fma2(ADZ, ADZ, DR2), ADZ, false, 8, n_cut, (float)n_cut, SR, SZ);
+  if (kind == 3) window_walk2<true>(DR2, dup(0.0f), fma2(ADZ, ADZ, DR2), ADZ, false, 8, n_cut, (float)n_cut, SR, SZ);
+  if (kind == 5) window_walk2<false>(DR2, dup(0.0f), fma2(ADZ, ADZ, DR2), ADZ, false, 8, n_cut, (float)n_cut, SR, SZ);
   float x;
   upk(SR, out[0], x);
   upk(SZ, out[1], x);
@@ -48,6 +50,21 @@ def sums(tmp_path_factory):
         lib.run(*args, out.ctypes.data)
         return out
     return run
+
+
+@pytest.mark.parametrize("n_cut", [12, 64, 4096])
+def test_window_of_the_symmetric_kernels(sums, n_cut):
+    # the other order of its products: the same to rounding up to 1e9, and finite and no larger beyond
+    for adz in (0.0, 0.25, 0.5):
+        for dR in 10.0 ** np.arange(0.5, 9.1, 0.5):
+            d2 = np.float32(dR * dR)
+            for wide, kind in ((0, 4), (3, 5)):
+                a, b = sums(wide, d2, adz, n_cut), sums(kind, d2, adz, n_cut)
+                assert abs(a[0] - b[0]) <= 4e-7 * a[0] and abs(a[1] - b[1]) <= 4e-7 * n_cut * a[0]
+        for d2 in (1e19, 1e22, 1e26, 1e30, 1e37, 3e38, np.inf):
+            for kind in (4, 5):
+                got = sums(kind, d2, adz, n_cut)
+                assert np.all(np.abs(got) <= 2 * n_cut * n_cut * min(1e-28, 1.01 * float(np.float32(d2)) ** -1.5)), (d2, got)
 
 
 @pytest.mark.parametrize("n_cut", [12, 64, 4096])
