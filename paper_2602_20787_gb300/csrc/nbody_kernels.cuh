@@ -232,10 +232,17 @@ __device__ __forceinline__ void kick_drift_one(int i, double g0, double g1, doub
   pack_one(nx, ny, nz, m[i], h[i], i, S.invL, jA, jB);
 }
 
+// A fixed-point sum as a double: hi in units of inv_scale, *lo (null: none) in units of 2^-40 of it.
+__device__ __forceinline__ double fix_sum(unsigned long long hi, const unsigned long long* lo, double inv_scale) {
+  const double s = (double)(long long)hi * inv_scale;
+  return lo ? fma((double)(long long)*lo, inv_scale * 0x1p-40, s) : s;
+}
+
 // The end of a step and the beginning of the next in one pass: the finalize from the fixed-point
-// sums [3][n], the kick K of the step that ends, then the kick and drift of the next, with the sums
+// sums [3][n] (lo: their low words or null), the kick K of the step that ends, then the kick and drift of the next, with the sums
 // cleared for its force evaluation: one launch for two (7.8 and 5.1 us of 42 at N = 2,048).
-static __global__ void finalize_fix_drift_kernel(unsigned long long* __restrict__ acc, int n, double inv_scale,
+static __global__ void finalize_fix_drift_kernel(unsigned long long* __restrict__ acc,
+                                                 unsigned long long* __restrict__ lo, int n, double inv_scale,
                                                  double pair_scale, BgParams bg, double* __restrict__ x,
                                                  double* __restrict__ y, double* __restrict__ z,
                                                  double* __restrict__ gx, double* __restrict__ gy,
@@ -249,9 +256,10 @@ static __global__ void finalize_fix_drift_kernel(unsigned long long* __restrict_
   double s[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    unsigned long long* a = acc + (size_t)c * n + i;
-    s[c] = (double)(long long)*a * inv_scale;
-    *a = 0;
+    const size_t o = (size_t)c * n + i;
+    s[c] = fix_sum(acc[o], lo ? lo + o : nullptr, inv_scale);
+    acc[o] = 0;
+    if (lo) lo[o] = 0;
   }
   double g0 = pair_scale * s[0], g1 = pair_scale * s[1], g2 = pair_scale * s[2];
   add_background(bg, x[i], y[i], z[i], g0, g1, g2, err);
@@ -267,7 +275,8 @@ static __global__ void finalize_fix_drift_kernel(unsigned long long* __restrict_
 // (pair_sym.cuh), in units of 1 / scale, for the rows [i0, n): acc[3][stride]
 // indexed from i0 (stride = n, i0 = 0 for every row; a rank's own rows of a
 // sharded step have i0 = its first row and stride = its exchange chunk).
-static __global__ void finalize_fix_kernel(const unsigned long long* __restrict__ acc, int n, int i0, int stride,
+static __global__ void finalize_fix_kernel(const unsigned long long* __restrict__ acc,
+                                           const unsigned long long* __restrict__ lo, int n, int i0, int stride,
                                            double inv_scale, double pair_scale, BgParams bg,
                                            const double* __restrict__ x, const double* __restrict__ y,
                                            const double* __restrict__ z, double* __restrict__ gx,
@@ -277,15 +286,17 @@ static __global__ void finalize_fix_kernel(const unsigned long long* __restrict_
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = i0 + q;
   if (i >= n) return;
-  const double sx = (double)(long long)acc[q] * inv_scale;
-  const double sy = (double)(long long)acc[(long long)stride + q] * inv_scale;
-  const double sz = (double)(long long)acc[2 * (long long)stride + q] * inv_scale;
+  const long long p = (long long)stride + q, r = 2 * (long long)stride + q;
+  const double sx = fix_sum(acc[q], lo ? lo + q : nullptr, inv_scale);
+  const double sy = fix_sum(acc[p], lo ? lo + p : nullptr, inv_scale);
+  const double sz = fix_sum(acc[r], lo ? lo + r : nullptr, inv_scale);
   finish_particle(i, sx, sy, sz, pair_scale, bg, x, y, z, gx, gy, gz, K, px, py, pz, out, err,
                   RadialCorr{nullptr, 0, 0.0, 0});
 }
 
 // First half of a KDK step: p += g K1; x += p D; z wrapped into [0, L); repack. facc (may be
-// null): the fixed-point sums [3][n] of the force evaluation that follows, set to zero.
+// null): the fixed-point sums [3][n] of the force evaluation that follows, set to zero (and lo,
+// their low words).
 static __global__ void kick_drift_pack_kernel(double* __restrict__ x, double* __restrict__ y,
                                        double* __restrict__ z, double* __restrict__ px,
                                        double* __restrict__ py, double* __restrict__ pz,
@@ -293,12 +304,14 @@ static __global__ void kick_drift_pack_kernel(double* __restrict__ x, double* __
                                        const double* __restrict__ gz, const double* __restrict__ m,
                                        const double* __restrict__ h, int n, DriftStep S, float4* __restrict__ jA,
                                        float4* __restrict__ jB, int* __restrict__ err,
-                                       unsigned long long* __restrict__ facc) {
+                                       unsigned long long* __restrict__ facc,
+                                       unsigned long long* __restrict__ lo) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (facc) {
       facc[i] = 0;
       facc[(size_t)n + i] = 0;
       facc[2 * (size_t)n + i] = 0;
+      if (lo) lo[i] = lo[(size_t)n + i] = lo[2 * (size_t)n + i] = 0;
     }
     kick_drift_one(i, gx[i], gy[i], gz[i], S, x, y, z, px, py, pz, m, h, jA, jB, err);
   }

@@ -319,9 +319,8 @@ pair_fp64_kernel(const double* __restrict__ x, const double* __restrict__ y, con
 //
 // Accumulation: as the FP32 kernels, in integers (associative, so the result does not
 // depend on the order of the warps), here in two words per sum: hi in units of 1 / scale and
-// the remainder in units of 2^-kLoBits / scale. |lo| stays below 2^39 per term, so 2^23 terms
-// fit; scale leaves 2^57 for the bound on |S_i|, so lo resolves 2^-97 of it.
-constexpr int kLoBits = 40;
+// the remainder in units of 2^-kLoBits / scale (pair_sym.cuh). |lo| stays below 2^39 per term, so
+// 2^23 terms fit; scale leaves 2^57 for the bound on |S_i|, so lo resolves 2^-97 of it.
 constexpr int kThreads64 = 128;
 
 struct Fix64Acc {
@@ -345,9 +344,8 @@ __device__ __forceinline__ void fix64_add(const Fix64Acc& F, int c, int i, doubl
 static __global__ void fix64_sum_kernel(const unsigned long long* __restrict__ hi,
                                         const unsigned long long* __restrict__ lo, long long m, double inv_scale,
                                         double* __restrict__ out) {
-  const double inv_lo = inv_scale / (double)(1LL << kLoBits);
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x)
-    out[q] = fma((double)(long long)lo[q], inv_lo, (double)(long long)hi[q] * inv_scale);
+    out[q] = fix_sum(hi[q], lo + q, inv_scale);
 }
 
 __host__ __device__ __forceinline__ long long row_step64(int b, int NB) { return 16LL * b * (2LL * NB - b); }

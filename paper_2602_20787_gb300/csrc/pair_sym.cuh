@@ -30,7 +30,8 @@
 // so the result does not depend on the order in which CTAs finish: the force
 // evaluation stays deterministic and bit-reproducible. 2^S is chosen on the host
 // from a bound on |S_i| (total mass times the largest softened force); a value
-// beyond 2^62 / 2^S sets an error bit instead of wrapping.
+// beyond 2^62 / 2^S sets an error bit instead of wrapping. The R^3 force and the FP64 form
+// (pair_fp64.cuh) take two words per sum: see "scale and spread" below.
 #pragma once
 #include <cstdint>
 
@@ -101,7 +102,34 @@ struct FixAcc {
   float scale_f;  // the scale when it is a normal float, else 0
   int* err;
   int world, base, extra, chunk;
+  unsigned long long* lo = nullptr;  // low words [3][n] of two-word sums (unsharded)
 };
+
+// Scale and spread. With B a bound on any |S_i| the scale is 2^57 / B, so one unit is 2^-57 B,
+// and how that compares with the sums themselves is a matter of the load: B holds the force at
+// the smallest softening, a typical sum the force at the distances between the particles. A
+// sum of two words (hi in units of 1 / scale, lo the remainder in units of 2^-kLoBits / scale)
+// resolves 2^-97 B. The spread is B over an estimate from below of a typical sum: the mass
+// beside the heaviest particle at the load's largest separation D (units of L), in R^3 over D^2
+// and in the cylinder over the line's D sqrt(N^2 + D^2) / (2 N), N = n_cut. It has no units: it is the
+// same for any total mass and, in R^3, any unit of length. Up to kMaxSpread the unit is 2^-69 of a
+// typical sum, below FP64's rounding also when a load spreads a hundredfold between two looks at it. Beyond
+// (softenings of some 1e-4 of the load's size: these loads had the row kernels before) the row kernels
+// take the pairs.
+constexpr int kLoBits = 40;
+constexpr double kMaxSpread = 0x1p28;
+
+// B: one image's softened force is at most 4 / hh^2 <= (L / h_min)^2 = q^2 (the peak of the
+// spline of eq. Force_spline_kernel with hh >= 2 h_min), the other images of the window add at
+// most 2 sum_k 1 / (k - 1/2)^2 < 10 (none in R^3), and the masses add up to M.
+__host__ __device__ __forceinline__ double fix_bound(double M, double q, bool images) {
+  return M * (q * q + (images ? 10.0 : 0.0));
+}
+// n_cut = 0: R^3.
+__host__ __device__ __forceinline__ double fix_spread(double B, double M, double m_max, double D, int n_cut) {
+  const double N = n_cut;
+  return B / (M - m_max) * (n_cut > 0 ? D * sqrt(fma(D, D, N * N)) / (2.0 * N) : D * D);
+}
 
 __device__ __forceinline__ long long fix_index(const FixAcc& F, int c, int i) {
   if (F.world == 0) return (long long)c * F.n + i;
@@ -111,34 +139,56 @@ __device__ __forceinline__ long long fix_index(const FixAcc& F, int c, int i) {
   return ((long long)r * 3 + c) * F.chunk + (i - first);
 }
 
-// value * scale as a 64-bit integer; one beyond 2^62 (or not finite) sets the error bit
-// and gives 0, so that nothing ever wraps. The scale is a power of two: where it is a
-// normal float (F.scale_f, else 0) the product is exact in FP32 and the conversion keeps
+// value * scale as a 64-bit integer (and, TWO, the remainder); one beyond 2^62 (or not finite)
+// sets the error bit and gives 0, so that nothing ever wraps. The scale is a power of two: where it
+// is a normal float (F.scale_f, else 0) the product is exact in FP32 and the conversion keeps
 // off the FP64 pipe, whose 2 lanes per SM and clock took 10 of the 40 us of an R^3
 // force at N = 5,000 (three or four FP64 operations per sum).
-__device__ __forceinline__ long long fix_value(const FixAcc& F, float v) {
+struct FixValue {
+  long long hi, lo;
+  __device__ __forceinline__ void add(const FixValue& v) {
+    hi += v.hi;
+    lo += v.lo;
+  }
+  __device__ __forceinline__ void sub(const FixValue& v) {
+    hi -= v.hi;
+    lo -= v.lo;
+  }
+};
+template <bool TWO>
+__device__ __forceinline__ FixValue fix_value(const FixAcc& F, float v) {
   if (F.scale_f > 0.0f) {
     const float q = v * F.scale_f;
-    if (fabsf(q) < 4.0e18f) return __float2ll_rn(q);
+    if (fabsf(q) < 4.0e18f)
+      return {__float2ll_rn(q), TWO ? __float2ll_rn((q - rintf(q)) * (float)(1LL << kLoBits)) : 0};
   } else {
     const double q = (double)v * F.scale;
-    if (fabs(q) < 4.0e18) return __double2ll_rn(q);
+    if (fabs(q) < 4.0e18)
+      return {__double2ll_rn(q), TWO ? __double2ll_rn((q - rint(q)) * (double)(1LL << kLoBits)) : 0};
   }
   atomicOr(F.err, kErrFixRange);
-  return 0;
+  return {0, 0};
 }
-__device__ __forceinline__ void fix_add(const FixAcc& F, int c, int i, long long q) {
+template <bool TWO>
+__device__ __forceinline__ void fix_add(const FixAcc& F, int c, int i, const FixValue& q) {
   const long long size = F.world == 0 ? 3LL * F.n : 3LL * F.world * F.chunk;
-  atomicAdd(F.acc + checked_index(fix_index(F, c, i), size), (unsigned long long)q);
+  const long long o = checked_index(fix_index(F, c, i), size);
+  atomicAdd(F.acc + o, (unsigned long long)q.hi);
+  if (TWO) atomicAdd(F.lo + o, (unsigned long long)q.lo);
 }
 // The sums of rows i0 and i1 (packed s, compensation k) into component c.
-template <bool KAHAN>
+template <bool KAHAN, bool TWO>
 __device__ __forceinline__ void fix_add_rows(const FixAcc& F, int c, int i0, int i1, u64 s, u64 k) {
   float s0, s1, k0, k1;
   upk(s, s0, s1);
   upk(k, k0, k1);
-  if (i0 < F.n) fix_add(F, c, i0, fix_value(F, s0) - (KAHAN ? fix_value(F, k0) : 0));
-  if (i1 < F.n) fix_add(F, c, i1, fix_value(F, s1) - (KAHAN ? fix_value(F, k1) : 0));
+  FixValue v0 = fix_value<TWO>(F, s0), v1 = fix_value<TWO>(F, s1);
+  if (KAHAN) {
+    v0.sub(fix_value<TWO>(F, k0));
+    v1.sub(fix_value<TWO>(F, k1));
+  }
+  if (i0 < F.n) fix_add<TWO>(F, c, i0, v0);
+  if (i1 < F.n) fix_add<TWO>(F, c, i1, v1);
 }
 
 // Offset of row b of the upper triangle (units t = b .. NB - 1 per row).
@@ -481,10 +531,10 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
           if (j < n) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-              long long f = 0;
+              FixValue f{0, 0};
 #pragma unroll
-              for (int w = 0; w < kSymThreads / 32; ++w) f -= fix_value(F, sh.J[w * kJRow + 3 * s + q]);
-              fix_add(F, q, j, f);
+              for (int w = 0; w < kSymThreads / 32; ++w) f.sub(fix_value<false>(F, sh.J[w * kJRow + 3 * s + q]));
+              fix_add<false>(F, q, j, f);
             }
           }
         }
@@ -492,7 +542,7 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
     }
     const u64 S[3] = {sx, sy, sz}, K[3] = {cx, cy, cz};
 #pragma unroll
-    for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN>(F, q, i0, i1, S[q], K[q]);
+    for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN, false>(F, q, i0, i1, S[q], K[q]);
     u += v1 - v0;
   }
 }
@@ -639,7 +689,12 @@ pair_sym_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
           const int j = t * jt + s;
           if (j < n) {
 #pragma unroll
-            for (int q = 0; q < 3; ++q) fix_add(F, q, j, -fix_value(F, row[3 * s + q]) - fix_value(F, row[kJRow + 3 * s + q]));
+            for (int q = 0; q < 3; ++q) {
+              FixValue f{0, 0};
+              f.sub(fix_value<true>(F, row[3 * s + q]));
+              f.sub(fix_value<true>(F, row[kJRow + 3 * s + q]));
+              fix_add<true>(F, q, j, f);
+            }
           }
         }
       }
@@ -648,7 +703,7 @@ pair_sym_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
     for (int s = 0; s < NS; ++s) {
       const int i0 = b * kBI + 64 * s + lane;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN>(F, q, i0, i0 + 32, S[s][q], K[s][q]);
+      for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN, true>(F, q, i0, i0 + 32, S[s][q], K[s][q]);
     }
     u += t1 - t0;
   }

@@ -251,7 +251,7 @@ struct steps_cyl_ctx {
   std::vector<int> perm_h;  // host copy of perm, when perm_h_ok (see host_perm)
   bool perm_h_ok = false;
   unsigned* mhist = nullptr;            // digit counts and offsets of the Morton sort, 2 x 256 per sort tile
-  unsigned long long* mbox = nullptr;   // its bounding box: min x, min y, max x, max y (ordered words)
+  unsigned long long* mbox = nullptr;   // its bounding box: min x, min y, max x, max y (ordered words); extent
   int64_t* idx = nullptr;   // subset indices (grown on demand)
   int idx_cap = 0;
   double* sub = nullptr;    // subset sums (3 * idx_cap)
@@ -268,10 +268,15 @@ struct steps_cyl_ctx {
   int Ccap = 0, SCcap = 0, TCcap = 0;
   // symmetric (Newton's third law) evaluation into fixed-point accumulators
   unsigned long long* facc = nullptr;  // [3][n]
-  unsigned long long* facc_lo = nullptr;  // [3][n], the FP64 form's low words (allocated when it first runs)
-  double fix_scale = 0.0;              // 2^S
+  // [3][n], the low words: R^3, right behind facc; else the FP64 form's, allocated when it first runs
+  unsigned long long* facc_lo = nullptr;
+  double fix_scale = 0.0;              // 2^S, 0: none
+  double fix_B = 0.0, fix_M = 0.0, m_max = 0.0;  // bound on a sum, total mass, the largest one
   double h_max = 0.0;                  // the largest softening (set with fix_scale)
-  bool fix_ready = false, fix_ok = false;
+  bool fix_ready = false, fix_ok = false;  // fix_ok: of the S1xR2 FP32 sums (one word)
+  double extent = 0.0;                 // largest distance from the axis (R^3: the origin), where ext_ok
+  bool ext_ok = false;
+  int steps_since_extent = 0;
   long long Usym = 0;
   int tpb = 1;                         // j-tiles per block of 128 rows of the symmetric kernels
   int sp = 1;                          // units a quarter tile's steps are split over
@@ -458,11 +463,14 @@ __global__ void positions_changed_kernel(const double* __restrict__ x, const dou
   }
 }
 
-__global__ void max_rho_kernel(const double* __restrict__ x, const double* __restrict__ y, int n,
-                               unsigned long long* __restrict__ out) {
+// Largest distance from the axis, or (z not null) from the origin.
+__global__ void max_rho_kernel(const double* __restrict__ x, const double* __restrict__ y,
+                               const double* __restrict__ z, int n, unsigned long long* __restrict__ out) {
   double r = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    r = fmax(r, sqrt(x[i] * x[i] + y[i] * y[i]));
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double w = z ? z[i] : 0.0;
+    r = fmax(r, sqrt(x[i] * x[i] + y[i] * y[i] + w * w));
+  }
   // non-negative doubles order like their bit patterns
   atomicMax(out, (unsigned long long)__double_as_longlong(r));
 }
@@ -760,7 +768,7 @@ int build_background(steps_cyl_ctx* c) {
   unsigned long long* dmax = nullptr;
   CK(cudaMallocAsync(&dmax, sizeof(unsigned long long), c->st));
   CK(cudaMemsetAsync(dmax, 0, sizeof(unsigned long long), c->st));
-  max_rho_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(c->x, c->y, c->n, dmax);
+  max_rho_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(c->x, c->y, nullptr, c->n, dmax);
   CKLAUNCH("max_rho");
   unsigned long long hb = 0;
   CK(cudaMemcpyAsync(&hb, dmax, sizeof hb, cudaMemcpyDeviceToHost, c->st));
@@ -1166,47 +1174,68 @@ RadialCorr radial_corr(const steps_cyl_ctx* c) {
   return r;
 }
 
-// Scale of the fixed-point accumulators of the symmetric kernels, from a bound
-// on any particle's pair sum |sum_j m_j v_ij| (positions in units of L): one
-// image's softened force is at most 4 / hh^2 <= (L / h_min)^2 (the peak of the
-// spline of eq. Force_spline_kernel with hh >= 2 h_min), the other images of
-// the window add at most 2 sum_k 1 / (k - 1/2)^2 < 10, and the masses add up
-// to M. With a factor 16 to spare, 2^S = 2^61 / (16 B) rounded down to a power
-// of two. Below 2^40 (a softening so small that the unit 2^-S would not be far
-// below FP32 rounding of typical sums) the row kernels are used instead.
+// Scale of the fixed-point accumulators of the symmetric kernels, from the bound B on any
+// particle's pair sum (pair_sym.cuh): with a factor 16 to spare, 2^S = 2^61 / (16 B) rounded
+// down to a power of two. The S1xR2 FP32 sums, of one word, take the row kernels where it is
+// below 2^40 (a softening so small that the unit 2^-S would not be far below FP32 rounding of
+// typical sums of a total mass of order one); the two-word sums go by the spread (use_sym).
 int fix_scale(steps_cyl_ctx* c) {
   std::vector<double> hm(c->n), hh(c->n);
   CK(cudaMemcpyAsync(hm.data(), c->m, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
   CK(cudaMemcpyAsync(hh.data(), c->h, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
-  double M = 0.0, hmin = INFINITY, hmax = 0.0;
+  double M = 0.0, mmax = 0.0, hmin = INFINITY, hmax = 0.0;
   for (int k = 0; k < c->n; ++k) {
     M += std::fabs(hm[k]);
+    mmax = std::max(mmax, std::fabs(hm[k]));
     hmin = std::min(hmin, hh[k]);
     hmax = std::max(hmax, hh[k]);
   }
   c->h_max = hmax;
-  const double q = c->p.L / hmin;
-  const double B = M * (q * q + 10.0);
-  const int S = (int)std::floor(57.0 - std::log2(B));
-  c->fix_ok = std::isfinite(B) && B > 0 && S >= 40 && S <= 1000;
-  c->fix_scale = c->fix_ok ? std::ldexp(1.0, S) : 0.0;
+  c->fix_M = M;
+  c->m_max = mmax;
+  const double B = c->fix_B = fix_bound(M, c->p.L / hmin, !is_r3(c));
+  const int S = std::isfinite(B) && B > 0 ? (int)std::floor(57.0 - std::log2(B)) : -2000;
+  c->fix_scale = S >= -900 && S <= 1000 ? std::ldexp(1.0, S) : 0.0;
+  c->fix_ok = S >= 40 && S <= 1000;
   c->fix_ready = true;
   return STEPS_OK;
 }
 
+// Whether the next force evaluation's sums have two words.
+bool two_words(const steps_cyl_ctx* c) { return !is_tree(c) && (is_r3(c) || c->p.precision == STEPS_FP64); }
+
+// The extent of the load, which the spread of two-word sums depends on: taken with the state and at the end
+// of each KDK call, and every kExtentEvery steps of one (the host waits for it).
+constexpr int kExtentEvery = 32;
+int launch_extent(steps_cyl_ctx* c) {
+  CK(cudaMemsetAsync(c->mbox + 4, 0, sizeof(unsigned long long), c->st));
+  max_rho_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(c->x, c->y, is_r3(c) ? c->z : nullptr, c->n, c->mbox + 4);
+  CKLAUNCH("extent");
+  c->ext_ok = false;
+  c->steps_since_extent = 0;
+  CK(cudaMemcpyAsync(&c->extent, c->mbox + 4, sizeof(double), cudaMemcpyDeviceToHost, c->st));
+  return STEPS_OK;
+}
+
 float fix_scale_f(const steps_cyl_ctx* c) {
-  return c->fix_scale <= std::ldexp(1.0, kMaxFixExpF) ? (float)c->fix_scale : 0.0f;
+  return c->fix_scale <= std::ldexp(1.0, kMaxFixExpF) && c->fix_scale >= std::ldexp(1.0, -kMaxFixExpF)
+             ? (float)c->fix_scale
+             : 0.0f;
 }
 
 #ifndef STEPS_SYMMETRIC
 #define STEPS_SYMMETRIC 1  // evaluate each unordered pair once (build-time switch)
 #endif
 
-// The FP32 direct forms take the symmetric kernels, unless the context's rows are
-// shared with other ranks (a rank has no j side for rows it does not own).
+// The direct forms take the symmetric kernels, unless the context's rows are shared with
+// other ranks (a rank has no j side for rows it does not own) or the sums' unit is too coarse.
 bool use_sym(const steps_cyl_ctx* c) {
-  return STEPS_SYMMETRIC && (!c->shard || c->shard_world == 1) && c->fix_ok;
+  if (!STEPS_SYMMETRIC || (c->shard && c->shard_world != 1)) return false;
+  if (!two_words(c)) return c->fix_ok;
+  const double D = 2.0 * c->extent * c->invL;
+  return c->fix_scale > 0.0 && c->ext_ok &&
+         fix_spread(c->fix_B, c->fix_M, c->m_max, D, is_r3(c) ? 0 : c->p.n_cut) <= kMaxSpread;
 }
 
 // The pair form of the next force evaluation: FP64, the selected modelled tail
@@ -1370,9 +1399,11 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     if (rc) return rc;
   }
   if (form != Form::FP64 && use_sym(c)) {
-    if (!cleared) CK(cudaMemsetAsync(c->facc, 0, sizeof(unsigned long long) * 3 * (size_t)c->n, c->st));
+    unsigned long long* lo = is_r3(c) ? c->facc_lo : nullptr;
+    if (!cleared) CK(cudaMemsetAsync(c->facc, 0, sizeof(unsigned long long) * (lo ? 6 : 3) * (size_t)c->n, c->st));
     CK(cudaEventRecord(c->e0, c->st));
-    int rc = launch_sym(c, form, 0, c->Usym, FixAcc{c->facc, c->n, c->fix_scale, fix_scale_f(c), c->err, 0, 0, 0, 0});
+    int rc = launch_sym(c, form, 0, c->Usym,
+                        FixAcc{c->facc, c->n, c->fix_scale, fix_scale_f(c), c->err, 0, 0, 0, 0, lo});
     if (rc) return rc;
     CK(cudaEventRecord(c->e1, c->st));
     c->timed = true;
@@ -1381,13 +1412,13 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     c->last_sym = true;
     if (next) {
       finalize_fix_drift_kernel<<<(c->n + ft - 1) / ft, ft, 0, c->st>>>(
-          c->facc, c->n, 1.0 / c->fix_scale, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K, c->px,
+          c->facc, lo, c->n, 1.0 / c->fix_scale, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K, c->px,
           c->py, c->pz, c->m, c->h, *next, c->jA, c->jB, c->err);
       CKLAUNCH("finalize_fix_drift");
       return STEPS_OK;
     }
     finalize_fix_kernel<<<(c->n + ft - 1) / ft, ft, 0, c->st>>>(
-        c->facc, c->n, 0, c->n, 1.0 / c->fix_scale, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz,
+        c->facc, lo, c->n, 0, c->n, 1.0 / c->fix_scale, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz,
         K, kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, out, c->err);
     CKLAUNCH("finalize_fix");
     return STEPS_OK;
@@ -1500,9 +1531,11 @@ int validate_state(steps_cyl_ctx* c) {
   validate_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(c->x, c->y, c->z, c->px, c->py, c->pz, c->m, c->h, c->n,
                                                            is_r3(c) ? 0.0 : c->p.L, c->err);
   CKLAUNCH("validate");
-  int bad = 0;
-  int rc = read_and_clear_err(c, &bad);
-  if (rc) return rc;
+  int bad = 0, rc;
+  c->ext_ok = false;
+  if (two_words(c) && (rc = launch_extent(c))) return rc;
+  if ((rc = read_and_clear_err(c, &bad))) return rc;
+  c->ext_ok = two_words(c);
   if (bad & 1) return fail(STEPS_EINVAL, "non-finite position or velocity");
   if (bad & 2) return fail(STEPS_EINVAL, "masses must be finite and > 0");
   if (bad & 4) return fail(STEPS_EINVAL, "softenings must be finite and > 0");
@@ -1570,7 +1603,7 @@ void release(steps_cyl_ctx* c) {
   cudaFree(c->chk);
   cudaFree(c->shard_off);
   cudaFree(c->facc);
-  cudaFree(c->facc_lo);
+  if (!is_r3(c)) cudaFree(c->facc_lo);
   {
     auto& T = c->tr;
     void* ptrs[] = {T.key[0], T.key[1], T.val[0], T.val[1], T.hist, T.offs, T.u4, T.u4s, T.zt, T.sA, T.sB,
@@ -2411,7 +2444,7 @@ int allocate_context(steps_cyl_ctx* c) {
   CKA(cudaMalloc(&c->iperm, sizeof(int) * nb));
   CKA(cudaMalloc(&c->ord, sizeof(int) * nb));
   CKA(cudaMalloc(&c->mhist, sizeof(unsigned) * 512 * ((nb + kSortTile - 1) / kSortTile)));
-  CKA(cudaMalloc(&c->mbox, sizeof(unsigned long long) * 4));
+  CKA(cudaMalloc(&c->mbox, sizeof(unsigned long long) * 5));
   CKA(cudaMalloc(&c->err, sizeof(int)));
   CKA(cudaMemsetAsync(c->err, 0, sizeof(int), c->st));
 
@@ -2442,7 +2475,8 @@ int allocate_context(steps_cyl_ctx* c) {
   c->SYC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(yocc, 1) * STEPS_CTA_MULT);
   c->SYSC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(ysocc, 1) * STEPS_CTA_MULT);
   c->SYTC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(ytocc, 1) * STEPS_CTA_MULT);
-  CKA(cudaMalloc(&c->facc, sizeof(unsigned long long) * nb * 3));
+  CKA(cudaMalloc(&c->facc, sizeof(unsigned long long) * nb * (is_r3(c) ? 6 : 3)));
+  if (is_r3(c)) c->facc_lo = c->facc + 3 * nb;
   c->part_elems = std::max((size_t)(c->NB + std::max({c->C, c->SC, c->TC})) * 3 * kBI, nb * 3);
   CKA(cudaMalloc(&c->part, sizeof(double) * c->part_elems));
 
@@ -2670,7 +2704,8 @@ int steps_cyl_kdk_step(steps_cyl_ctx* c, double dt, int32_t nsteps) {
       const int kt = particle_threads(c->n);
       kick_drift_pack_kernel<<<grid_for(c->n, kt), kt, 0, c->st>>>(c->x, c->y, c->z, c->px, c->py, c->pz, c->gx, c->gy,
                                                                    c->gz, c->m, c->h, c->n, drift_step(c, f), c->jA,
-                                                                   c->jB, c->err, c->facc);
+                                                                   c->jB, c->err, c->facc,
+                                                                   is_r3(c) ? c->facc_lo : nullptr);
       CKLAUNCH("kick_drift_pack");
     }
     // the next step's kick and drift go with this step's finalize when nothing stands between them
@@ -2687,6 +2722,12 @@ int steps_cyl_kdk_step(steps_cyl_ctx* c, double dt, int32_t nsteps) {
     c->t += dt;
     if (c->p.reorder_every > 0 && ++c->steps_since_order >= c->p.reorder_every) {
       if ((rc = reorder(c))) return rc;
+    }
+    c->ext_ok = c->ext_ok && two_words(c);
+    if (two_words(c) && ++c->steps_since_extent >= kExtentEvery && s + 1 < nsteps) {
+      if ((rc = launch_extent(c))) return rc;
+      CK(cudaStreamSynchronize(c->st));
+      c->ext_ok = true;
     }
     // modelled tail: periodic comparison with the plain image sum
     const bool surr = c->p.tail == STEPS_TAIL_SURROGATE && c->surr_ok;
@@ -2709,7 +2750,10 @@ int steps_cyl_kdk_step(steps_cyl_ctx* c, double dt, int32_t nsteps) {
     }
   }
   int e = 0;
+  const bool ext = two_words(c) && nsteps > 0;
+  if (ext && (rc = launch_extent(c))) return rc;
   if ((rc = read_and_clear_err(c, &e))) return rc;
+  c->ext_ok = c->ext_ok || ext;
   if (e) return device_error(e);
   if (rejected) return fail(STEPS_ESURROGATE_REJECTED, "%s", reject_msg);
   return STEPS_OK;
@@ -2774,6 +2818,14 @@ int steps_cyl_set_precision(steps_cyl_ctx* c, int32_t precision) {
   c->p.precision = precision;
   if (precision == STEPS_FP64) c->p.tail = STEPS_TAIL_FULL;
   c->forces_stale = true;  // refreshed by the next force evaluation or KDK step
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(c->st, &cap));
+  if (two_words(c) && !c->ext_ok && cap == cudaStreamCaptureStatusNone) {
+    int rc;
+    if ((rc = launch_extent(c))) return rc;
+    CK(cudaStreamSynchronize(c->st));
+    c->ext_ok = true;
+  }
   return STEPS_OK;
 }
 
@@ -2866,7 +2918,7 @@ int steps_cyl_shard_drift(steps_cyl_ctx* c, double dt, float* send) {
   const int k0 = c->k0, rows = c->k1 - c->k0;
   kick_drift_pack_kernel<<<grid_for(rows, 256), 256, 0, c->st>>>(
       c->x + k0, c->y + k0, c->z + k0, c->px + k0, c->py + k0, c->pz + k0, c->gx + k0, c->gy + k0, c->gz + k0,
-      c->m + k0, c->h + k0, rows, drift_step(c, f), c->jA + k0, c->jB + k0, c->err, nullptr);
+      c->m + k0, c->h + k0, rows, drift_step(c, f), c->jA + k0, c->jB + k0, c->err, nullptr, nullptr);
   CKLAUNCH("kick_drift_pack");
   shard_send_kernel<<<grid_for(c->chunk, 256), 256, 0, c->st>>>(c->jA, c->jB, k0, rows, c->chunk,
                                                                  reinterpret_cast<float4*>(send));
@@ -2896,7 +2948,10 @@ int steps_cyl_shard_kick(steps_cyl_ctx* c, const float* recv) {
   c->t += c->pend_dt;
   c->drifted = false;
   int e = 0;
+  const bool ext = two_words(c) && c->shard_world == 1;  // the rows of other ranks are not held here
+  if (ext && (rc = launch_extent(c))) return rc;
   if ((rc = read_and_clear_err(c, &e))) return rc;
+  c->ext_ok = ext;
   if (e) return device_error(e);
   return STEPS_OK;
 }
@@ -2967,7 +3022,7 @@ int steps_cyl_shard_finish(steps_cyl_ctx* c, const int64_t* own) {
   const int rows = c->k1 - c->k0;
   const int ft = particle_threads(rows);
   finalize_fix_kernel<<<(rows + ft - 1) / ft, ft, 0, c->st>>>(
-      reinterpret_cast<const unsigned long long*>(own), c->k1, c->k0, c->chunk, 1.0 / c->fix_scale,
+      reinterpret_cast<const unsigned long long*>(own), nullptr, c->k1, c->k0, c->chunk, 1.0 / c->fix_scale,
       -c->p.G * c->invL * c->invL, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, c->pend_K2, c->px, c->py,
       c->pz, AccelOut{}, c->err);
   CKLAUNCH("finalize_fix");
