@@ -15,22 +15,36 @@ constexpr int kErrZRange = 4;        // z left [0, L) by more than rounding
 constexpr int kErrTreeRange = 8;     // a particle lies outside the octree's root cube
 constexpr int kErrTreeStack = 16;    // an octree walk outgrew its stack
 
+// The farthest from the axis, in units of L, that a finite window's packed words go: beyond dR of some
+// 1e15 the products of a pair vanish in FP32, so nothing changes by it, but dR^2 stays finite, which the
+// closed form of the image line relies on. (The infinite window's pair falls as 1 / dR^2 and the closed form is
+// finite at any dR; R^3 has none: no cap.) Words that are not finite stay so.
+constexpr float kPackCap = 6e18f;
+
 // FP64 positions -> FP32 hi/lo words in units of L (see pair_fp32.cuh).
-__device__ __forceinline__ void pack_one(double x, double y, double z, double m, double h, int i, double invL,
+__device__ __forceinline__ void pack_one(double x, double y, double z, double m, double h, int i, double invL, float cap,
                                          float4* __restrict__ jA, float4* __restrict__ jB) {
-  const double xu = x * invL, yu = y * invL, zu = z * invL;
-  const float xh = (float)xu, yh = (float)yu, zh = (float)zu;
-  const float xl = (float)(xu - (double)xh), yl = (float)(yu - (double)yh), zl = (float)(zu - (double)zh);
-  jA[i] = make_float4(xh, yh, zh, (float)m);
-  jB[i] = make_float4(xl, yl, zl, (float)(h * invL));
+  const double u[3] = {x * invL, y * invL, z * invL};
+  float hi[3], lo[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    hi[c] = (float)u[c];
+    lo[c] = (float)(u[c] - (double)hi[c]);
+    if (c < 2 && fabsf(hi[c]) > cap && isfinite(hi[c])) {
+      hi[c] = copysignf(cap, hi[c]);
+      lo[c] = 0.0f;
+    }
+  }
+  jA[i] = make_float4(hi[0], hi[1], hi[2], (float)m);
+  jB[i] = make_float4(lo[0], lo[1], lo[2], (float)(h * invL));
 }
 
 static __global__ void pack_kernel(const double* __restrict__ x, const double* __restrict__ y,
                             const double* __restrict__ z, const double* __restrict__ m,
-                            const double* __restrict__ h, int n, double invL, float4* __restrict__ jA,
+                            const double* __restrict__ h, int n, double invL, float cap, float4* __restrict__ jA,
                             float4* __restrict__ jB) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    pack_one(x[i], y[i], z[i], m[i], h[i], i, invL, jA, jB);
+    pack_one(x[i], y[i], z[i], m[i], h[i], i, invL, cap, jA, jB);
 }
 
 // Background of eq. ComovingEquationsOfMotionCylindrical: returns F_h(rho) (< 0
@@ -212,6 +226,7 @@ static __global__ void finalize_kernel(const double* __restrict__ part, int n, i
 // bits do not depend on the kernel that takes it.
 struct DriftStep {
   double K1, D, L, invL;
+  float cap;  // of the packed words
   int wrap;
 };
 __device__ __forceinline__ void kick_drift_one(int i, double g0, double g1, double g2, const DriftStep& S, double* x,
@@ -229,7 +244,7 @@ __device__ __forceinline__ void kick_drift_one(int i, double g0, double g1, doub
   }
   if (!isfinite(nx) || !isfinite(ny) || !isfinite(nz)) atomicOr(err, kErrNonFinite);
   x[i] = nx; y[i] = ny; z[i] = nz;
-  pack_one(nx, ny, nz, m[i], h[i], i, S.invL, jA, jB);
+  pack_one(nx, ny, nz, m[i], h[i], i, S.invL, S.cap, jA, jB);
 }
 
 // A fixed-point sum as a double: hi in units of inv_scale, *lo (null: none) in units of 2^-40 of it.

@@ -402,7 +402,7 @@ static __global__ void tree_pack_kernel(int nn, const double4_32a* __restrict__ 
     const double4_32a c = mom[id];
     double zc = c.w / c.x - zeta;
     if (periodic && zc < 0.0) zc += L;
-    pack_one(c.y / c.x, c.z / c.x, zc, c.x, hmax[id], id, invL, nA, nB);
+    pack_one(c.y / c.x, c.z / c.x, zc, c.x, hmax[id], id, invL, __int_as_float(0x7f800000), nA, nB);
   }
 }
 

@@ -364,19 +364,23 @@ __device__ __forceinline__ u64 base_poly_z(u64 Q, u64 D2) {
 
 // The far ends: s and e at N, and what they add to the sums to infinity (the integral
 // of f ends at N). e e_N / (s + s_N): the product of the two squares leaves FP32's normal range
-// from dR = 3e9 on. WIDE takes the reciprocal between them, so that no product does before the
-// sum itself: the row kernels, whose sums are in floating point. In the symmetric kernels all pairs
-// so far apart add up to a few units of the fixed-point sums at most, and they keep the order with the
-// shorter chain (N = 65,536, N_cut = 16, literal law: 13.35 ms, the other order 13.46). kFarFloor
-// keeps the reciprocals finite where dR^2 is infinite, and is below the rounding of what it is added to elsewhere.
-constexpr float kFarFloor = 1e-30f;
+// from dR = 3e9 on. WIDE multiplies it and the sum by 2^60, so that it does not before the image
+// sum itself, at no rounding: the row kernels, whose sums are in floating point. In the symmetric kernels all
+// pairs so far apart add up to a few units of the fixed-point sums at most. (The reciprocal between the squares does
+// it as well, and takes 0.9% longer in the symmetric kernels: 13.46 ms against 13.35 at N = 65,536, N_cut = 16,
+// literal law.) dR^2 is finite: kPackCap.
+constexpr float kFarUp = 0x1p60f;
+template <bool WIDE>
+__device__ __forceinline__ u64 far_rcp2(u64 x) {
+  return rcp2(WIDE ? mul2(x, dup(kFarUp)) : x);
+}
 struct FarEnd2 {
   u64 IH, SN, EN, R, Z;
 };
 __device__ __forceinline__ FarEnd2 far_end2(u64 DR2, u64 ADZ, float N) {
   FarEnd2 f;
   f.IH = rsq2(add2(DR2, dup(N * N)));
-  f.SN = fma2(f.IH, dup(N), dup(kFarFloor));
+  f.SN = mul2(f.IH, dup(N));
   f.EN = mul2(f.IH, f.IH);
   const u64 D = sub2(ADZ, dup(0.5f)), D2 = mul2(D, D);
   const u64 G = mul2(f.SN, f.EN);
@@ -418,8 +422,9 @@ __device__ __forceinline__ void line_far2(u64 DR2, u64 ADZ, float N, u64& SR, u6
     I = mul2(mul2(E, dup(2.0f)), rcp2(add2(S, dup(1.0f))));
   } else {
     const FarEnd2 f = far_end2(DR2, ADZ, N);
-    const u64 EC = mul2(E, dup(2.0f * (N * N - kPolyA * kPolyA))), V = rcp2(add2(S, f.SN));
-    I = WIDE ? fma2(EC, mul2(f.EN, V), f.R) : fma2(mul2(EC, f.EN), V, f.R);
+    constexpr float UP = WIDE ? kFarUp : 1.0f;
+    const u64 EE = mul2(mul2(E, dup(2.0f * UP * (N * N - kPolyA * kPolyA))), f.EN);
+    I = fma2(EE, far_rcp2<WIDE>(add2(S, f.SN)), f.R);
     SZ = add2(SZ, f.Z);
   }
   SR = add2(SR, fma2(mul2(G, E), T, I));
@@ -437,8 +442,8 @@ template <bool WIDE>
 __device__ __forceinline__ LineSide2 line_side2(u64 LO, u64 DR2, const FarEnd2& f, float N2) {
   const u64 IL = rsq2(fma2(LO, LO, DR2));
   const u64 S = mul2(LO, IL), E = mul2(IL, IL);
-  const u64 NN = fma2(LO, LO, dup(-N2)), V = rcp2(add2(S, f.SN));
-  const u64 NI = WIDE ? mul2(mul2(NN, E), mul2(f.EN, V)) : mul2(mul2(NN, mul2(E, f.EN)), V);
+  const u64 EE = mul2(WIDE ? mul2(E, dup(kFarUp)) : E, f.EN);
+  const u64 NI = mul2(mul2(fma2(LO, LO, dup(-N2)), EE), far_rcp2<WIDE>(add2(S, f.SN)));
   const u64 Q = mul2(S, S), W = mul2(E, Q);
   u64 PR = fma2(W, dup(0.238131417f), fma2(E, dup(-0.168406769f), dup(-0.127495596f)));
   PR = fma2(W, PR, fma2(E, dup(0.0547808694f), dup(0.125f)));
@@ -481,8 +486,8 @@ __device__ __forceinline__ void window_walk2(u64 DR2, u64 HH, u64 R2C, u64 ADZ, 
   SR = add2(SR, sub2(f.R, add2(a.NR, b.NR)));
   // the integrals of z f, IL_a - IL_b, without cancellation at large dR
   const u64 P = mul2(a.IL, b.IL);
-  const u64 AD = mul2(ADZ, dup(-4.0f * A)), V = rcp2(add2(add2(a.IL, dup(kFarFloor)), b.IL));
-  const u64 IZ = WIDE ? mul2(mul2(P, AD), mul2(P, V)) : mul2(mul2(mul2(P, P), AD), V);
+  const u64 PP = mul2(WIDE ? mul2(P, dup(kFarUp)) : P, P);
+  const u64 IZ = mul2(mul2(PP, mul2(ADZ, dup(-4.0f * A))), far_rcp2<WIDE>(add2(a.IL, b.IL)));
   SZ = add2(SZ, add2(add2(IZ, sub2(a.Z, b.Z)), f.Z));
   fix_dz0<true>(ADZ, DR2, fnc, SR, SZ);
 }

@@ -1359,8 +1359,9 @@ int launch_sym(steps_cyl_ctx* c, Form form, long long Ua, long long U, const Fix
   return STEPS_OK;
 }
 
+float pack_cap(const steps_cyl_ctx* c) { return is_r3(c) || is_inf(c) ? INFINITY : kPackCap; }
 DriftStep drift_step(const steps_cyl_ctx* c, const Factors& f) {
-  return DriftStep{f.K1, f.D, c->p.L, c->invL, is_r3(c) ? 0 : 1};
+  return DriftStep{f.K1, f.D, c->p.L, c->invL, pack_cap(c), is_r3(c) ? 0 : 1};
 }
 // Whether the next force evaluation ends in the finalize that can take a kick and drift along.
 bool takes_drift(const steps_cyl_ctx* c) {
@@ -1545,7 +1546,8 @@ int validate_state(steps_cyl_ctx* c) {
 
 int pack_positions(steps_cyl_ctx* c) {
   Range range("steps_cyl.pack");
-  pack_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(c->x, c->y, c->z, c->m, c->h, c->n, c->invL, c->jA, c->jB);
+  pack_kernel<<<grid_for(c->n, 256), 256, 0, c->st>>>(c->x, c->y, c->z, c->m, c->h, c->n, c->invL, pack_cap(c), c->jA,
+                                                        c->jB);
   CKLAUNCH("pack");
   return STEPS_OK;
 }

@@ -69,7 +69,7 @@ noalloc_pack_kernel(const double* __restrict__ x, const double* __restrict__ y, 
   double s = 0.0;
   unsigned long long hb = ~0ull;
   if (i < n) {
-    pack_one(x[i], y[i], z[i], m[i], h[i], i, invL, jA, jB);
+    pack_one(x[i], y[i], z[i], m[i], h[i], i, invL, kPackCap, jA, jB);
     acc[i] = acc[(size_t)n + i] = acc[2 * (size_t)n + i] = 0;
     s = fabs(m[i]);
     hb = h[i] > 0.0 ? (unsigned long long)__double_as_longlong(h[i]) : 0ull;
