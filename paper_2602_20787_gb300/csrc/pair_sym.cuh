@@ -30,8 +30,8 @@
 // so the result does not depend on the order in which CTAs finish: the force
 // evaluation stays deterministic and bit-reproducible. 2^S is chosen on the host
 // from a bound on |S_i| (total mass times the largest softened force); a value
-// beyond 2^62 / 2^S sets an error bit instead of wrapping. The R^3 force and the FP64 form
-// (pair_fp64.cuh) take two words per sum: see "scale and spread" below.
+// beyond 2^62 / 2^S sets an error bit instead of wrapping. The R^3 force, the allocation-free
+// call and the FP64 form (pair_fp64.cuh) take two words per sum: see "Scale and spread" below.
 #pragma once
 #include <cstdint>
 
@@ -125,10 +125,11 @@ constexpr double kMaxSpread = 0x1p28;
 __host__ __device__ __forceinline__ double fix_bound(double M, double q, bool images) {
   return M * (q * q + (images ? 10.0 : 0.0));
 }
-// n_cut = 0: R^3.
-__host__ __device__ __forceinline__ double fix_spread(double B, double M, double m_max, double D, int n_cut) {
-  const double N = n_cut;
-  return B / (M - m_max) * (n_cut > 0 ? D * sqrt(fma(D, D, N * N)) / (2.0 * N) : D * D);
+// Whether the spread is at most kMaxSpread (n_cut = 0: R^3), without a division or a root: sqrt(N^2 + D^2)
+// is taken as N + D.
+__host__ __device__ __forceinline__ bool fix_resolves(double B, double M, double m_max, double D, int n_cut) {
+  const double N = n_cut, T = kMaxSpread * (M - m_max);
+  return n_cut > 0 ? B * D * (N + D) <= 2.0 * N * T : B * D * D <= T;
 }
 
 __device__ __forceinline__ long long fix_index(const FixAcc& F, int c, int i) {
@@ -475,7 +476,7 @@ struct SymShared {
   float J[kSymThreads / 32 * kJRow];
 };
 
-template <bool KAHAN, class Form>
+template <bool KAHAN, bool TWO = false, class Form>
 __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, const float4* __restrict__ jB, int n,
                                              int NB, int tpb, int sp, long long Ua, long long U, int C, SymShared& sh,
                                              const FixAcc& F, const Form& form) {
@@ -533,8 +534,8 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
             for (int q = 0; q < 3; ++q) {
               FixValue f{0, 0};
 #pragma unroll
-              for (int w = 0; w < kSymThreads / 32; ++w) f.sub(fix_value<false>(F, sh.J[w * kJRow + 3 * s + q]));
-              fix_add<false>(F, q, j, f);
+              for (int w = 0; w < kSymThreads / 32; ++w) f.sub(fix_value<TWO>(F, sh.J[w * kJRow + 3 * s + q]));
+              fix_add<TWO>(F, q, j, f);
             }
           }
         }
@@ -542,7 +543,7 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
     }
     const u64 S[3] = {sx, sy, sz}, K[3] = {cx, cy, cz};
 #pragma unroll
-    for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN, false>(F, q, i0, i1, S[q], K[q]);
+    for (int q = 0; q < 3; ++q) fix_add_rows<KAHAN, TWO>(F, q, i0, i1, S[q], K[q]);
     u += v1 - v0;
   }
 }

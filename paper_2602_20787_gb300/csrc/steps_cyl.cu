@@ -1235,7 +1235,7 @@ bool use_sym(const steps_cyl_ctx* c) {
   if (!two_words(c)) return c->fix_ok;
   const double D = 2.0 * c->extent * c->invL;
   return c->fix_scale > 0.0 && c->ext_ok &&
-         fix_spread(c->fix_B, c->fix_M, c->m_max, D, is_r3(c) ? 0 : c->p.n_cut) <= kMaxSpread;
+         fix_resolves(c->fix_B, c->fix_M, c->m_max, D, is_r3(c) ? 0 : c->p.n_cut);
 }
 
 // The pair form of the next force evaluation: FP64, the selected modelled tail

@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <mutex>
 
 #include "steps_cyl.h"
@@ -40,23 +41,25 @@ static_assert(kScratchBytes == STEPS_NOALLOC_SCRATCH_BYTES, "scratch size must m
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-// Each unordered pair is evaluated once where the fixed-point sums that this takes (pair_sym.cuh)
-// have a scale. Their bound needs the total mass and the smallest softening, which the
-// host cannot look at without waiting: the pack kernel reduces them on the device, the symmetric
-// kernel derives the scale, or leaves the pairs to the row kernel, whose CTAs otherwise
-// return at once. (N = 10,007, N_cut = 16, literal softening law: rows alone 730 us.)
+// Each unordered pair is evaluated once where the fixed-point sums that this takes (two words,
+// pair_sym.cuh) resolve the load. That needs the total mass and the largest one, the smallest softening and
+// the extent, which the host cannot look at without waiting: the pack kernel reduces them on the
+// device, the symmetric kernel derives the scale, or leaves the pairs to the row kernel, whose CTAs
+// otherwise return at once. (N = 10,007, N_cut = 16, literal softening law: rows alone 730 us.)
 // The record lies in the partials' last slot, which the row kernel's split never reaches.
 constexpr int kPackThreads = 256;
 constexpr int kPackParts = (kNoallocMaxN + kPackThreads - 1) / kPackThreads;
 struct NoallocHead {
   unsigned long long hmin;  // bits of the smallest h; 0 when some h is not > 0
+  unsigned long long rmax;  // bits of the largest (|x| + |y|) / L, no less than the distance from the axis
+  unsigned long long mmax;  // bits of the largest |m|
   int err, sym;             // error bits of the symmetric kernel; whether it has taken the pairs
   double scale;             // its sums' scale
   double mass[kPackParts];  // sums of |m| over each CTA of the pack kernel
 };
 constexpr size_t kHeadOffset = kScratchBytes - sizeof(double) * 3 * kBI;
 static_assert(sizeof(NoallocHead) <= sizeof(double) * 3 * kBI, "the record takes one partial-sum slot");
-static_assert(sizeof(unsigned long long) * 3 * kNoallocMaxN <= kPartBytes - sizeof(double) * 3 * kBI,
+static_assert(sizeof(unsigned long long) * 6 * kNoallocMaxN <= kPartBytes - sizeof(double) * 3 * kBI,
               "the fixed-point sums take the partials' place");
 
 __global__ void __launch_bounds__(kPackThreads)
@@ -67,20 +70,26 @@ noalloc_pack_kernel(const double* __restrict__ x, const double* __restrict__ y, 
   __shared__ double warp[kPackThreads / 32];
   const int i = blockIdx.x * kPackThreads + threadIdx.x;
   double s = 0.0;
-  unsigned long long hb = ~0ull;
+  unsigned long long hb = ~0ull, rb = 0, mb = 0;  // non-negative doubles order like their bits, NaN above all
   if (i < n) {
     pack_one(x[i], y[i], z[i], m[i], h[i], i, invL, kPackCap, jA, jB);
-    acc[i] = acc[(size_t)n + i] = acc[2 * (size_t)n + i] = 0;
+    for (int c = 0; c < 6; ++c) acc[c * (size_t)n + i] = 0;
     s = fabs(m[i]);
     hb = h[i] > 0.0 ? (unsigned long long)__double_as_longlong(h[i]) : 0ull;
+    rb = (unsigned long long)__double_as_longlong((fabs(x[i]) + fabs(y[i])) * invL);
+    mb = (unsigned long long)__double_as_longlong(s);
   }
   for (int o = 16; o > 0; o >>= 1) {
     s += __shfl_down_sync(0xffffffffu, s, o);
     hb = min(hb, __shfl_down_sync(0xffffffffu, hb, o));
+    rb = max(rb, __shfl_down_sync(0xffffffffu, rb, o));
+    mb = max(mb, __shfl_down_sync(0xffffffffu, mb, o));
   }
   if ((threadIdx.x & 31) == 0) {
     warp[threadIdx.x >> 5] = s;
     atomicMin(&head->hmin, hb);
+    atomicMax(&head->rmax, rb);
+    atomicMax(&head->mmax, mb);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -90,15 +99,18 @@ noalloc_pack_kernel(const double* __restrict__ x, const double* __restrict__ y, 
   }
 }
 
-// The scale as the contexts choose it (2^57 over the bound on |S_i|, at least 2^40), 0: none. By a whole warp.
-__device__ __forceinline__ double noalloc_scale(const NoallocHead* head, int parts, double L) {
+// The scale as the contexts choose it (2^57 over the bound on |S_i|), 0: none. By a whole warp.
+__device__ __forceinline__ double noalloc_scale(const NoallocHead* head, int parts, double L, int n_cut) {
   double M = 0.0;
   for (int k = threadIdx.x & 31; k < parts; k += 32) M += head->mass[k];
   for (int o = 16; o > 0; o >>= 1) M += __shfl_xor_sync(0xffffffffu, M, o);
-  const double q = L / __longlong_as_double((long long)head->hmin), B = M * (q * q + 10.0);
-  if (!(B >= 1e-290 && B < 1e290)) return 0.0;
-  const int S = 57 - (((__double2hiint(B) >> 20) & 0x7ff) - 1022);  // B < 2^(exponent + 1)
-  return S >= 40 && S <= 1000 ? __hiloint2double((S + 1023) << 20, 0) : 0.0;
+  const double B = fix_bound(M, L / __longlong_as_double((long long)head->hmin), true);
+  if (!(B >= 1e-290 && B < 1e270)) return 0.0;
+  if (!fix_resolves(B, M, __longlong_as_double((long long)head->mmax),
+                    2.0 * __longlong_as_double((long long)head->rmax), n_cut))
+    return 0.0;
+  const int S = 57 - (((__double2hiint(B) >> 20) & 0x7ff) - 1022);  // B < 2^(exponent + 1); |S| < 1,023
+  return __hiloint2double((S + 1023) << 20, 0);
 }
 
 template <bool KAHAN, bool LINE>
@@ -107,15 +119,16 @@ noalloc_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
                    int sp, long long U, int C, unsigned long long* __restrict__ acc, NoallocHead* __restrict__ head,
                    int parts, double L) {
   __shared__ SymShared sh;
-  const double scale = noalloc_scale(head, parts, L);
+  const double scale = noalloc_scale(head, parts, L, n_cut);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     head->sym = scale > 0.0;
     head->scale = scale;
   }
   if (!(scale > 0.0)) return;
-  const float f = scale <= ldexp(1.0, kMaxFixExpF) ? (float)scale : 0.0f;
-  sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, sp, 0, U, C, sh, FixAcc{acc, n, scale, f, &head->err, 0, 0, 0, 0},
-                      PlainForm<LINE, false>{n_cut, (float)n_cut});
+  const float f = scale <= ldexp(1.0, kMaxFixExpF) && scale >= ldexp(1.0, -kMaxFixExpF) ? (float)scale : 0.0f;
+  sym_stream_k<KAHAN, true>(jA, jB, n, NB, tpb, sp, 0, U, C, sh,
+                            FixAcc{acc, n, scale, f, &head->err, 0, 0, 0, 0, acc + 3 * (size_t)n},
+                            PlainForm<LINE, false>{n_cut, (float)n_cut});
 }
 
 // Accelerations from either kernel's sums. A sum beyond the fixed-point range can only come from a
@@ -129,8 +142,10 @@ __global__ void noalloc_finalize_kernel(const unsigned long long* __restrict__ a
   double s[3] = {0.0, 0.0, 0.0};
   if (head->sym) {
     const double inv = 1.0 / head->scale;
-    for (int q = 0; q < 3; ++q)
-      s[q] = head->err ? __longlong_as_double(0x7ff8000000000000LL) : (double)(long long)acc[(size_t)q * n + i] * inv;
+    for (int q = 0; q < 3; ++q) {
+      const size_t o = (size_t)q * n + i;
+      s[q] = head->err ? __longlong_as_double(0x7ff8000000000000LL) : fix_sum(acc[o], acc + 3 * (size_t)n + o, inv);
+    }
   } else {
     row_sums(part, i, NT, U, C, s[0], s[1], s[2]);
   }
@@ -240,7 +255,7 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(part);
   const int parts = (nn + kPackThreads - 1) / kPackThreads;
   cudaMemsetAsync(&head->hmin, 0xff, sizeof head->hmin, st);
-  cudaMemsetAsync(&head->err, 0, 2 * sizeof(int), st);
+  cudaMemsetAsync(&head->rmax, 0, offsetof(NoallocHead, scale) - offsetof(NoallocHead, rmax), st);
   noalloc_pack_kernel<<<parts, kPackThreads, 0, st>>>(x, y, z, m, h, nn, invL, jA, jB, acc, head);
   const bool kahan = precision == STEPS_FP32_KAHAN;
   int tpb, sp;

@@ -1,4 +1,4 @@
-"""Which loads the two-word fixed-point sums take (fix_bound, fix_spread and their limit in
+"""Which loads the two-word fixed-point sums take (fix_bound, fix_resolves in
 pair_sym.cuh, built from the source for the CPU), and that the sums they accept lose nothing: the
 kernels' terms (one FP32 sum per particle and block of 128) are rounded to the accumulator's unit and
 added up, for total masses from 1e-12 to 1e12, radii from 1 to 1e8 of the unit of length, and a
@@ -12,7 +12,7 @@ import device_source as ds
 
 WRAP = """
 extern "C" double bound(double M, double q, int images) { return fix_bound(M, q, images != 0); }
-extern "C" double spread(double B, double M, double m, double D, int n) { return fix_spread(B, M, m, D, n); }
+extern "C" int resolves(double B, double M, double m, double D, int n) { return fix_resolves(B, M, m, D, n); }
 extern "C" double limit() { return kMaxSpread; }
 extern "C" int bits() { return kLoBits; }
 """
@@ -21,10 +21,10 @@ extern "C" int bits() { return kLoBits; }
 @pytest.fixture(scope="module")
 def rule(tmp_path_factory):
     lib = ds.compile_host(tmp_path_factory.mktemp("fix"), ds.constants("pair_sym.cuh", "kLoBits", "kMaxSpread"),
-                          ds.function("pair_sym.cuh", "fix_bound"), ds.function("pair_sym.cuh", "fix_spread"), WRAP)
+                          ds.function("pair_sym.cuh", "fix_bound"), ds.function("pair_sym.cuh", "fix_resolves"), WRAP)
     d = ctypes.c_double
-    for f, a in ((lib.bound, [d, d, ctypes.c_int]), (lib.spread, [d, d, d, d, ctypes.c_int]), (lib.limit, [])):
-        f.argtypes, f.restype = a, d
+    lib.bound.argtypes, lib.bound.restype, lib.limit.restype = [d, d, ctypes.c_int], d, d
+    lib.resolves.argtypes = [d, d, d, d, ctypes.c_int]
     return lib
 
 
@@ -73,23 +73,30 @@ def test_accepted_sums_lose_nothing(rule, n_cut, M, R, soft, heavy):
     exact = t.sum(1)
     assert abs(exact).max() <= 16 * B  # 2^57 / B leaves no sum beyond 2^62
     D = 2 * np.sqrt((pos[:, :2 if n_cut else 3] ** 2).sum(1)).max()
-    spread = rule.spread(B, m.sum(), m.max(), D, n_cut)
+    spread = B / (m.sum() - m.max()) * (D * np.hypot(D, n_cut) / (2 * n_cut) if n_cut else D * D)
+    taken = rule.resolves(B, m.sum(), m.max(), D, n_cut)
+    assert not taken or spread <= rule.limit()
     got = two_word(t, np.longdouble(2) ** np.floor(57 - np.log2(B)), rule.bits())
     err = np.linalg.norm(got - exact, axis=1) / np.linalg.norm(exact, axis=1)
     # one unit is at most 2^-96 B (a power of two below 2^57 / B); a particle's sum rounds once per
     # term, half a unit each, in three components
     unit = 2.0 ** -96 * spread * 2 * np.sqrt(3 * t.shape[1])
-    if spread <= rule.limit():  # FP64's rounding of a sum is 1.1e-16
+    if taken:  # FP64's rounding of a sum is 1.1e-16
         assert np.median(err) <= unit and err[0] <= 30 * unit and unit <= 1e-17
     # what does not depend on the units: a load with an ordinary softening is accepted
     if soft >= 1e-3 and not heavy and (n_cut == 0 or R == 1.0):
-        assert spread <= rule.limit()
+        assert taken
 
 
-def test_spread_has_no_units(rule):
+def test_the_rule_has_no_units(rule):
+    def largest(n_cut, M, length):  # the largest L / h that is taken
+        lo, hi = 1.0, 1e12
+        for _ in range(80):
+            q = np.sqrt(lo * hi)
+            ok = rule.resolves(rule.bound(M, q / length, int(n_cut > 0)), M, 0.25 * M, 3.0 * length, n_cut)
+            lo, hi = (q, hi) if ok else (lo, q)
+        return lo
     for n_cut in (0, 16):
-        a = rule.spread(rule.bound(1.0, 50.0, int(n_cut > 0)), 1.0, 0.25, 3.0, n_cut)
-        b = rule.spread(rule.bound(1e-9, 50.0, int(n_cut > 0)), 1e-9, 0.25e-9, 3.0, n_cut)
-        assert abs(a - b) <= 1e-12 * a
-    c = rule.spread(rule.bound(1.0, 50.0 / 1e6, 0), 1.0, 0.25, 3.0e6, 0)
-    assert abs(c - rule.spread(rule.bound(1.0, 50.0, 0), 1.0, 0.25, 3.0, 0)) <= 1e-12 * c
+        a = largest(n_cut, 1.0, 1.0)
+        assert a > 1e3 and abs(largest(n_cut, 1e-9, 1.0) - a) <= 1e-9 * a
+    assert abs(largest(0, 1.0, 1e6) - largest(0, 1.0, 1.0)) <= 1e-9 * a

@@ -38,7 +38,7 @@ def r3(sc, precision, R):
                                                 (1.0, 1.0, 0.05, 1e4, 1), (1.0, 1.0, 0.05, 1e9, 0),
                                                 (1.0, 1.0, 1e-8, 0, 0)])
 def test_r3(sc, R, M, soft, heavy, sym):
-    n = 500
+    n = 160
     pos, m, h = ball(n, R, M, soft, heavy)
     ref, mag = image_sums(pos, m, h, 1, r3=True)
     for pre in (sc.STEPS_FP32_KAHAN, sc.STEPS_FP32_PLAIN, sc.STEPS_FP64):
@@ -57,7 +57,7 @@ def test_r3(sc, R, M, soft, heavy, sym):
 def test_r3_spreads_in_a_run(sc):
     # outward velocities carry the particles from R = 1 to 1e6 within one call, beyond what the sums'
     # unit was looked at for
-    n, steps = 300, 80
+    n, steps = 160, 80
     pos, m, h = ball(n, 1.0, 1.0, 0.05)
     v = pos * (1e6 / (steps * 1e-2))
     for split in (1, steps):
