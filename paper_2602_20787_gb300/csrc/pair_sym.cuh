@@ -219,23 +219,32 @@ __device__ __forceinline__ int jslot(int k) {
 // After each group of STEPS_KAHAN_GROUP steps the sums (of 2 x 8 terms) are added
 // to the slots' sums in the warp's shared row, so that no FP32 running sum is
 // longer than those groups.
-// COMP: the rounding of each sum of groups is kept beside it (exactly, by the two-sum), in the second half
-// of a row of 2 kJRow floats, so that only the groups themselves round. The R^3 force takes it: there
-// four rows per lane make a group of 64 terms, and its 2-norm error against FP64 at N = 20,000 was 3.38e-7 without,
-// 3.27e-7 with it (as with sums of 16 terms), for 1.5% of its time.
+// COMP: after every kCompGroup steps, and the rounding of each sum of groups is kept beside it (exactly, by
+// the two-sum), in the second half of a row of 2 kJRow floats, so that only the groups themselves round, as on the
+// i side. The R^3 force and the allocation-free call under Kahan summation take it, whose rows had a
+// compensated sum over every j before: 2-norm error against FP64 over ten loads, rows / without it / with it, R^3 at
+// N = 20,000 3.37e-7 / 3.38e-7 / 3.34e-7 (2.3% of its time beside groups of 8 steps), the call at N = 10,007, N_cut = 16
+// 3.944e-8 / 3.989e-8 / 3.942e-8 (4% of its time).
+constexpr int kCompGroup = 4;
 template <bool COMP>
 struct JRing {
   float a[3] = {0.f, 0.f, 0.f};
-  // a += m_i v of both pairs: X = m_i sr (packed), Z = m_i sz
-  __device__ __forceinline__ void take(u64 DX, u64 DY, u64 X, u64 Z, bool shift_on) {
+  // a += m_i v of both pairs: M = m_i, X = m_i sr (packed); COMP: z fused, as on the i side
+  __device__ __forceinline__ void take(u64 DX, u64 DY, u64 M, u64 X, u64 SZ, bool shift_on) {
     float x0, x1, d0, d1, z0, z1;
     upk(X, x0, x1);
     upk(DX, d0, d1);
     a[0] = fmaf(d1, x1, fmaf(d0, x0, a[0]));
     upk(DY, d0, d1);
     a[1] = fmaf(d1, x1, fmaf(d0, x0, a[1]));
-    upk(Z, z0, z1);
-    a[2] += z0 + z1;
+    if (COMP) {
+      upk(M, d0, d1);
+      upk(SZ, z0, z1);
+      a[2] = fmaf(d1, z1, fmaf(d0, z0, a[2]));
+    } else {
+      upk(mul2(M, SZ), z0, z1);
+      a[2] += z0 + z1;
+    }
     if (shift_on) shift();
   }
   // a += both halves of V
@@ -271,7 +280,7 @@ struct JRing {
     }
   }
 };
-static_assert(32 % STEPS_KAHAN_GROUP == 0, "a round of 32 slots holds whole groups");
+static_assert(32 % STEPS_KAHAN_GROUP == 0 && STEPS_KAHAN_GROUP % kCompGroup == 0, "a round of 32 slots holds whole groups");
 
 // ---- pair forms ------------------------------------------------------------------
 // A form gives the image sums (SR, SZ) of a thread's two pairs.
@@ -471,21 +480,23 @@ inline void sym_split(int NB, int sms, bool steps, int& tpb, int& sp) {
     sp *= 2;
 }
 
+template <bool COMP>
 struct SymShared {
   JTile2 T;
-  float J[kSymThreads / 32 * kJRow];
+  float J[kSymThreads / 32 * (COMP ? 2 : 1) * kJRow];
 };
 
-template <bool KAHAN, bool TWO = false, class Form>
+template <bool KAHAN, bool TWO = false, bool COMP = false, class Form>
 __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, const float4* __restrict__ jB, int n,
-                                             int NB, int tpb, int sp, long long Ua, long long U, int C, SymShared& sh,
+                                             int NB, int tpb, int sp, long long Ua, long long U, int C, SymShared<COMP>& sh,
                                              const FixAcc& F, const Form& form) {
   // the units [Ua, Ua + U) (all of them, or a rank's share), split over C CTAs
   const int c = blockIdx.x;
   const long long u0 = Ua + (long long)c * U / C;
   const long long u1 = Ua + (long long)(c + 1) * U / C;
   const int jt = kBJ / tpb, upb = tpb * sp, ks = jt / sp;  // units per block, steps per unit
-  float* row = sh.J + (threadIdx.x >> 5) * kJRow;
+  constexpr int kRow = (COMP ? 2 : 1) * kJRow;
+  float* row = sh.J + (threadIdx.x >> 5) * kRow;
   long long u = u0;
   while (u < u1) {
     const int b = (int)checked_index(tri_row(u / upb, NB), NB);
@@ -500,7 +511,8 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
       load_tile2<kSymThreads>(jA, jB, n, t, jt, sh.T);
       __syncthreads();
       const bool sym = t / tpb != b;
-      JRing<false> ring;
+      JRing<COMP> ring;
+      constexpr int kGroup = COMP ? kCompGroup : STEPS_KAHAN_GROUP;  // a power of two that divides a unit's steps
 #pragma unroll 1
       for (int k0 = kb; k0 < kb + ks; k0 += STEPS_KAHAN_GROUP) {
         u64 gx = 0, gy = 0, gz = 0;
@@ -517,10 +529,12 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
           gy = fma2(P.dy, MS, gy);
           gz = fma2(m, SZ, gz);
           if (sym) {
-            ring.take(P.dx, P.dy, mul2(I.m, SR), mul2(I.m, SZ), k + 1 != k0 + STEPS_KAHAN_GROUP);
+            const bool full = ((k + 1) & (kGroup - 1)) == 0;  // the group's last step: its sums stay where they are
+            ring.take(P.dx, P.dy, I.m, mul2(I.m, SR), SZ, !full);
+            if (COMP && full) ring.flush(row, k, k < kb + kGroup || (k & 31) < kGroup);
           }
         }
-        if (sym) ring.flush(row, k0 + STEPS_KAHAN_GROUP - 1, k0 == kb || (k0 & 31) == 0);
+        if (!COMP && sym) ring.flush(row, k0 + STEPS_KAHAN_GROUP - 1, k0 == kb || (k0 & 31) == 0);
         acc2<KAHAN>(sx, cx, gx);
         acc2<KAHAN>(sy, cy, gy);
         acc2<KAHAN>(sz, cz, gz);
@@ -534,7 +548,10 @@ __device__ __forceinline__ void sym_stream_k(const float4* __restrict__ jA, cons
             for (int q = 0; q < 3; ++q) {
               FixValue f{0, 0};
 #pragma unroll
-              for (int w = 0; w < kSymThreads / 32; ++w) f.sub(fix_value<TWO>(F, sh.J[w * kJRow + 3 * s + q]));
+              for (int w = 0; w < kSymThreads / 32; ++w) {
+                f.sub(fix_value<TWO>(F, sh.J[w * kRow + 3 * s + q]));
+                if (COMP) f.sub(fix_value<TWO>(F, sh.J[w * kRow + kJRow + 3 * s + q]));
+              }
               fix_add<TWO>(F, q, j, f);
             }
           }
@@ -553,7 +570,7 @@ template <bool KAHAN, bool LINE, bool FAR>
 __global__ void __launch_bounds__(kSymThreads, FAR ? STEPS_SYM_FAR_MIN_BLOCKS : STEPS_SYM_MIN_BLOCKS)
 pair_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb, int sp,
                 long long Ua, long long U, int C, FixAcc F) {
-  __shared__ SymShared sh;
+  __shared__ SymShared<false> sh;
   sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, sp, Ua, U, C, sh, F, PlainForm<LINE, FAR>{n_cut, (float)n_cut});
 }
 
@@ -561,7 +578,7 @@ template <bool KAHAN, int MODEL, bool FAR>
 __global__ void __launch_bounds__(kSymThreads, STEPS_SYM_SURR_MIN_BLOCKS)
 pair_sym_surr_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb, int sp,
                      long long Ua, long long U, int C, const SurrLane* __restrict__ wl, SurrConst S, FixAcc F) {
-  __shared__ SymShared sh;
+  __shared__ SymShared<false> sh;
   __shared__ __align__(16) uint32_t sWT[32 * kSurrStride];
   __shared__ __align__(16) uint32_t sIn[kSymThreads / 32][2 * kInWords];
   uint32_t* ibuf = sIn[threadIdx.x >> 5];
@@ -575,7 +592,7 @@ template <bool KAHAN, int MODEL, int READ, bool FAR>
 __global__ void __launch_bounds__(kSymThreads, STEPS_SYM_TABLE_MIN_BLOCKS)
 pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb, int sp,
                       long long Ua, long long U, int C, TableTail T, SurrConst S, FixAcc F) {
-  __shared__ SymShared sh;
+  __shared__ SymShared<false> sh;
   sym_stream_k<KAHAN>(jA, jB, n, NB, tpb, sp, Ua, U, C, sh, F, TableForm<MODEL, READ, FAR>{n_cut, S, T});
 }
 
@@ -675,10 +692,12 @@ pair_sym_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
               for (int s = 1; s < NS; ++s) V[a] = fma2(D[s][a], X[s], V[a]);
             }
             ring.add(V);
-            if (k + 1 != k0 + STEPS_KAHAN_GROUP) ring.shift();
+            if ((k + 1) % kCompGroup == 0)
+              ring.flush(row, k, (k & 31) < kCompGroup);
+            else
+              ring.shift();
           }
         }
-        if (sym) ring.flush(row, k0 + STEPS_KAHAN_GROUP - 1, (k0 & 31) == 0);
 #pragma unroll
         for (int s = 0; s < NS; ++s)
 #pragma unroll

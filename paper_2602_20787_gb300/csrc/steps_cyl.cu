@@ -1466,7 +1466,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     CKLAUNCH("pair_fp32_r3");
   } else {
     const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
-    auto kernel = line_form(c->p.n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
+    auto kernel = line_form_rows(c->p.n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
                                         : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
     kernel<<<c->C, kPairThreads, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, c->U, c->NT, c->C, c->part, c->b0, nullptr);
     CKLAUNCH("pair_row");

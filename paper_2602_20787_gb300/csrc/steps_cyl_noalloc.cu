@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kSymThreads, STEPS_SYM_MIN_BLOCKS)
 noalloc_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
                    int sp, long long U, int C, unsigned long long* __restrict__ acc, NoallocHead* __restrict__ head,
                    int parts, double L) {
-  __shared__ SymShared sh;
+  __shared__ SymShared<KAHAN> sh;
   const double scale = noalloc_scale(head, parts, L, n_cut);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     head->sym = scale > 0.0;
@@ -126,7 +126,7 @@ noalloc_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB,
   }
   if (!(scale > 0.0)) return;
   const float f = scale <= ldexp(1.0, kMaxFixExpF) && scale >= ldexp(1.0, -kMaxFixExpF) ? (float)scale : 0.0f;
-  sym_stream_k<KAHAN, true>(jA, jB, n, NB, tpb, sp, 0, U, C, sh,
+  sym_stream_k<KAHAN, true, KAHAN>(jA, jB, n, NB, tpb, sp, 0, U, C, sh,
                             FixAcc{acc, n, scale, f, &head->err, 0, 0, 0, 0, acc + 3 * (size_t)n},
                             PlainForm<LINE, false>{n_cut, (float)n_cut});
 }
@@ -262,10 +262,10 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   sym_split(NB, d->sms, true, tpb, sp);
   const long long SU = (long long)NB * (NB + 1) / 2 * tpb * sp;
   const int SC = (int)std::min<long long>(SU, 32LL * d->sym_ctas);
-  auto sym = line_form(n_cut) ? (kahan ? noalloc_sym_kernel<true, true> : noalloc_sym_kernel<false, true>)
+  auto sym = line_form_rows(n_cut) ? (kahan ? noalloc_sym_kernel<true, true> : noalloc_sym_kernel<false, true>)
                               : (kahan ? noalloc_sym_kernel<true, false> : noalloc_sym_kernel<false, false>);
   sym<<<SC, kSymThreads, 0, st>>>(jA, jB, nn, n_cut, NB, tpb, sp, SU, SC, acc, head, parts, L);
-  auto kernel = line_form(n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
+  auto kernel = line_form_rows(n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
                                  : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
   kernel<<<C, kPairThreads, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part, 0, &head->sym);
   const int ft = particle_threads(nn);

@@ -59,3 +59,15 @@ def test_far_particles(sc, n_cut):
         # beyond some n_cut periods all images pull alike: 2 n_cut (one fewer at equal z) of them
         want = -((m[:-1] * 2 * n_cut / ((D ** 2).sum(1) + n_cut ** 2 / 3) ** 1.5)[:, None] * D).sum(0)
         assert np.linalg.norm(a[-1, :2] - want) <= 1e-5 * np.linalg.norm(want), (f, a[-1], want)
+
+
+@pytest.mark.parametrize("n_cut", [5, 16])
+@pytest.mark.parametrize("half", [128, 512, 2048])
+def test_both_sides_are_summed_alike(sc, n_cut, half):
+    # two points with as many equal particles each: every pair across them has the same terms, the
+    # first half adds them up as rows and the other as j sides, in groups of eight either way, and the groups
+    # exactly but for Kahan's second order: the accelerations are opposite
+    pos = np.repeat([[0.0, 0.0, 0.1], [0.37, 0.21, 0.43]], half, axis=0)
+    a = accel(sc, pos, np.full(2 * half, 1.0 / 3.0), np.full(2 * half, 0.05), n_cut, sc.STEPS_FP32_KAHAN)
+    assert np.all(a[:half] == a[0]) and np.all(a[half:] == a[half])
+    assert np.all(abs(a[0] + a[half]) <= 1e-11 * abs(a[0])), (a[0], a[half])
