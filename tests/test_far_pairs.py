@@ -40,7 +40,7 @@ def sums(tmp_path_factory):
         ds.constants("pair2.cuh", "kPolyA"),
         *[ds.constants("pair2.cuh", k) for k in ("kFarFloor", "kFarUp") if k in src], *[ds.function("pair2.cuh", f) for f in f2],
         ds.function("pair_fp32.cuh", "spline_outer_value"), ds.function("pair_fp32.cuh", "spline_value_r2"),
-        *[ds.function("pair2.cuh", f) for f in ("spline2", "soft_bound2", "spline_k2", "spline_centre2", "near_soft_walk2",
+        *[ds.function("pair2.cuh", f) for f in ("spline2", "soft_bound2", "spline_one2", "spline_centre2", "near_soft_walk2",
                                                 "near_newton2", "line_poly_r", "line_poly_z", "base_poly_r", "base_poly_z",
                                                 *(["far_rcp2"] if "far_rcp2" in src else []), "far_end2", "fix_dz0", "line_far2", "line_side2", "window_walk2")], WRAP)
     lib.run.argtypes = [ctypes.c_int, ctypes.c_float, ctypes.c_float, ctypes.c_int, ctypes.c_void_p]
