@@ -51,7 +51,8 @@ extern "C" {
 #define STEPS_FP32_KAHAN 1  /* FP32 pair math on hi/lo split positions, Kahan-compensated j sum */
 #define STEPS_FP32_PLAIN 2  /* FP32 pair math on hi/lo split positions, plain j sum */
 
-#define STEPS_TAIL_FULL 0       /* every image of the window: one by one for n_cut < 12 (FP64: < 14); else the near
+#define STEPS_TAIL_FULL 0       /* every image of the window: one by one for n_cut < 12 (FP64, and where
+                                 * every FP32 sum is compensated: < 16); else the near
                                  * images (and the softened ones) one by one and the others, a smooth function of
                                  * the image number, in closed form to below the precision's rounding */
 #define STEPS_TAIL_SURROGATE 1  /* images |k| <= n0 direct, far tail from the learned surrogate */

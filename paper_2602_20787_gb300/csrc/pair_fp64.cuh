@@ -5,13 +5,15 @@
 // holds it for 16 cycles), while loads, shuffles, integer and FP32 instructions are free
 // beside it. So the kernels spend other instructions wherever one of FP64 is saved:
 //   - each unordered pair once (pair_sym_fp64_kernel), added to both particles;
-//   - of the window's 2 n_cut images the 2 x 7 + 1 near ones, and both ends of the rest by
+//   - of the window's 2 n_cut images the 2 x 8 + 1 near ones, and both ends of the rest by
 //     the midpoint rule's Euler-Maclaurin series: its first three terms (near ends, two at
-//     the far ones) in FP64 and the others, together below 4e-10 of the sum, in FP32, where
-//     they round at 4e-16 of the sum at most and 6e-17 in the mean;
+//     the far ones) in FP64 and the others, together below 2e-10 of the sum, in FP32 from
+//     rounded inputs. A pair's force is then closer to the exact one than the walk's for any
+//     window that takes this form (rms error in 2^-52, closed form / walk, at dR = 1 .. 4 and
+//     4 .. 16: n_cut = 16 0.74 / 1.22 and 0.80 / 0.95, n_cut = 64 0.73 / 2.4 and 0.72 / 2.2);
 //   - 1 / r^3 straight from the hardware's 20-bit 1 / r by a two-term series;
 //   - comparisons, signs, conversions and the period's wrap on the integer pipe.
-// That leaves about 280 FP64 instructions per pair for any n_cut.
+// That leaves about 300 FP64 instructions per pair for any n_cut.
 #pragma once
 #include <cstdint>
 
@@ -30,6 +32,10 @@ __device__ __forceinline__ float float_trunc(double x) {
   if (hi < 0x38100000u) return 0.0f;
   if (hi >= 0x47f00000u) return __uint_as_float(0x7f800000u);
   return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
+}
+// The same, rounded (half up).
+__device__ __forceinline__ float float_rn(double x) {
+  return float_trunc(__longlong_as_double(__double_as_longlong(x) + (1LL << 28)));
 }
 // A float as a double; subnormals become 0.
 __device__ __forceinline__ double double_of(float x) {
@@ -85,7 +91,7 @@ __device__ __forceinline__ double image64(double r2, bool soft, const Soft64& h)
 // plus s e^(p+1) C_p(q) and i e^p D_p(q), p = 1, 2, ..., the polynomials from the
 // derivatives of f and z f and the midpoint rule's coefficients 1/24, -7/5760, 31/967680, ...
 // line_rest: the terms from p = 4 on over s e^5 and i e^4, in t = 1 - q (in which
-// they cancel least): p = 4 and 5 exact, the rest fitted over x >= 7.
+// they cancel least): p = 4 and 5 exact, the rest fitted over x >= 7 (the ends lie at 8 and beyond).
 __device__ __forceinline__ void line_rest(float t, float e, float& R, float& Z) {
   const float r0 = fmaf(t, fmaf(t, fmaf(t, -1.66268921f, 2.66030273f), -1.22783203f), 0.148828125f);
   const float r1 = fmaf(t, fmaf(t, fmaf(t, fmaf(t, -13.6419233f, 28.7198385f), -20.2728271f), 5.40608724f), -0.415852865f);
@@ -106,7 +112,7 @@ __device__ __forceinline__ void line_rest(float t, float e, float& R, float& Z) 
 
 // An end at x: i, s, e, and the images beyond it without the integral of f: FP64 terms R
 // and Z (with z f's integral i), FP32 terms fr and fz. NEAR: p <= 3 in FP64, else p <= 2 (for
-// x >= 13, where the third is below 4e-10 of the sum).
+// x >= 15, where the third is below 2e-10 of the sum).
 struct End64 {
   double s, e, R, Z;
   float fr, fz;
@@ -118,7 +124,9 @@ __device__ __forceinline__ End64 line_end64(double x, double dR2, float R2f) {
   E.s = x * i;
   E.e = i * i;
   const double q = E.s * E.s, e = E.e;
-  const float fi = float_trunc(i), fe = fi * fi, fs = float_trunc(E.s), ft = R2f * fe, fe2 = fe * fe;
+  // rounded, and each from FP64: the terms are up to tenth powers of their inputs, and inputs cut
+  // off at 23 bits left 0.9 of 2^-52 of the sum
+  const float fi = float_rn(i), fe = float_rn(e), fs = float_rn(E.s), ft = R2f * fe, fe2 = fe * fe;
   float gr, gz;
   line_rest(ft, fe, gr, gz);
   double c = fma(q, 49.0 / 384.0, -7.0 / 128.0);
@@ -140,13 +148,13 @@ __device__ __forceinline__ End64 line_end64(double x, double dR2, float R2f) {
 }
 
 // ---- the window ------------------------------------------------------------------------
-// Near images of the closed form, and the n_cut it is taken from. Seven is the fewest for
-// which the FP32 terms stay at FP64's rounding (six: 1.2e-15 of the sum). The walk of a
-// window of 14 images takes as many FP64 instructions as the closed form; from there on the far ends lie at 13
-// or beyond. Beyond dR = 16 the window is walked: there the sums' integrals, of order
-// 1 / dR^2 and 1 / dR, would cancel for a short window.
-constexpr int kNear64 = 7;
-constexpr int kLineMin64 = 14;
+// Near images of the closed form, and the n_cut it is taken from. Eight is the fewest for
+// which a pair's error is no larger than the walk's from dR = 4 on as well (seven: 0.98 against 0.95 of 2^-52,
+// n_cut = 16). The walk of a window of 15 images takes as many FP64 instructions as the closed form; from
+// n_cut = 16 on the far ends lie at 15 or beyond. Beyond dR = 16 the window is walked: there the sums'
+// integrals, of order 1 / dR^2 and 1 / dR, would cancel for a short window.
+constexpr int kNear64 = 8;
+constexpr int kLineMin64 = 16;
 constexpr double kLineMaxR2 = 256.0;
 __host__ __device__ __forceinline__ bool line_form64(int n_cut) { return n_cut >= kLineMin64; }
 
@@ -169,7 +177,7 @@ __device__ __forceinline__ void window64(double dR2, double dz, double hh, int n
   int m = KIND == kPair64Line ? kNear64 : n_cut - 1;
   float R2f = 0.0f;
   if (KIND == kPair64Line) {
-    R2f = float_trunc(dR2);
+    R2f = float_rn(dR2);
     if (!less_pos(dR2, kLineMaxR2)) m = n_cut - 1;
   }
   if (soft) {

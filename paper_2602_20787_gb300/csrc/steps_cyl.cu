@@ -829,7 +829,7 @@ int launch_fp64_sym(steps_cyl_ctx* c, double* out) {
   const int NB = (c->n + 31) / 32, nc = n_cut_eff(c);
   const long long W = row_step64(NB, NB);
   // One wave of 16 warps per SM (what 128 registers allow) shares the steps evenly and so keeps every SM
-  // busy to the end: 155 / 1,253 us at N = 600 / 2,048 (N_cut = 64), 182 / 1,256 with two waves. From 128 steps a
+  // busy to the end: 155 / 1,253 us at N = 600 / 2,048 (N_cut = 64, with seven near images), 182 / 1,256 with two waves. From 128 steps a
   // warp on two waves make up for the steps' unequal work: N = 6,000, N_cut = 30 10.39 -> 10.28 ms.
   const long long wave = 16LL * sms;
   const long long warps = std::max(1LL, std::min(W / 2, W / wave < 128 ? wave : 2 * wave));
