@@ -276,14 +276,9 @@ static __global__ void finalize_fix_drift_kernel(unsigned long long* __restrict_
     acc[o] = 0;
     if (lo) lo[o] = 0;
   }
-  double g0 = pair_scale * s[0], g1 = pair_scale * s[1], g2 = pair_scale * s[2];
-  add_background(bg, x[i], y[i], z[i], g0, g1, g2, err);
-  if (!isfinite(g0) || !isfinite(g1) || !isfinite(g2)) atomicOr(err, kErrNonFinite);
-  gx[i] = g0; gy[i] = g1; gz[i] = g2;
-  px[i] = fma(g0, K, px[i]);
-  py[i] = fma(g1, K, py[i]);
-  pz[i] = fma(g2, K, pz[i]);
-  kick_drift_one(i, g0, g1, g2, S, x, y, z, px, py, pz, m, h, jA, jB, err);
+  finish_particle(i, s[0], s[1], s[2], pair_scale, bg, x, y, z, gx, gy, gz, K, px, py, pz, AccelOut{}, err,
+                  RadialCorr{nullptr, 0, 0.0, 0});
+  kick_drift_one(i, gx[i], gy[i], gz[i], S, x, y, z, px, py, pz, m, h, jA, jB, err);
 }
 
 // Finalize from the fixed-point accumulators of the symmetric pair kernels
