@@ -471,6 +471,9 @@ struct TableForm {
 #ifndef STEPS_SYM_MAX_STEP_SPLIT
 #define STEPS_SYM_MAX_STEP_SPLIT 4
 #endif
+static_assert(STEPS_SYM_MAX_STEP_SPLIT >= 1 && 32 % STEPS_SYM_MAX_STEP_SPLIT == 0 &&
+                  (32 / STEPS_SYM_MAX_STEP_SPLIT) % STEPS_KAHAN_GROUP == 0,
+              "a unit's steps are whole Kahan groups");
 inline void sym_split(int NB, int sms, bool steps, int& tpb, int& sp) {
   const long long blocks = (long long)NB * (NB + 1) / 2;
   tpb = blocks < STEPS_SYM_SPLIT * (long long)sms ? 4 : 1;
