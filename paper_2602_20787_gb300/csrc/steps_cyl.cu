@@ -2309,6 +2309,19 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
     return order;
   };
   std::vector<std::future<std::vector<int>>> orders(ahead);
+  // The GPU may still read an epoch's order and corrections when the copies have returned (pageable memory
+  // that it can address needs no staging): both are kept until the event behind them, and to the stream's
+  // end on every way out.
+  std::vector<int> order;
+  struct Sent {
+    cudaStream_t st;
+    cudaEvent_t copies = nullptr;
+    ~Sent() {
+      cudaStreamSynchronize(st);
+      if (copies) cudaEventDestroy(copies);
+    }
+  } sent{c->st};
+  CK(cudaEventCreateWithFlags(&sent.copies, cudaEventDisableTiming));
   auto draw = [&](int ep) {
     SplitMix g = rng;
     g.skip((uint64_t)ep * (uint64_t)(ntrain - 1));
@@ -2323,8 +2336,10 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
   float last_loss = 0.f;
   int64_t last_count = 1;
   for (int ep = 0; ep < cfg->epochs; ++ep) {
-    const std::vector<int> order = orders[ep % ahead].get();
+    std::vector<int> next = orders[ep % ahead].get();
     if (ep + ahead < cfg->epochs) draw(ep + ahead);
+    if (ep > 0) CK(cudaEventSynchronize(sent.copies));
+    order.swap(next);
     CK(cudaMemcpyAsync(B.order, order.data(), sizeof(int) * ntrain, cudaMemcpyHostToDevice, c->st));
     adam.lr = (float)(cfg->lr * 0.5 * (1.0 + std::cos(M_PI * ep / cfg->epochs)));
     for (int64_t k = 0; k < nsteps; ++k) {
@@ -2335,6 +2350,7 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
     last_count = ntrain - (nsteps - 1) * cfg->batch;
     if (whole) {
       CK(cudaMemcpyAsync(B.corr, corr.data(), sizeof(float2) * nsteps, cudaMemcpyHostToDevice, c->st));
+      CK(cudaEventRecord(sent.copies, c->st));
       CK(cudaMemsetAsync(B.bar, 0, sizeof(unsigned), c->st));  // the arrivals; bar[1] stays
       int64_t nt = ntrain;
       int batch = cfg->batch;
@@ -2346,6 +2362,7 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
                                      c->st));
       continue;
     }
+    CK(cudaEventRecord(sent.copies, c->st));
     for (int64_t first = 0; first < ntrain; first += cfg->batch) {
       const int64_t count = std::min<int64_t>(cfg->batch, ntrain - first);
       const int nblk = (int)((count + kTrainThreads - 1) / kTrainThreads);
