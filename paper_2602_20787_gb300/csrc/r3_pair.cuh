@@ -11,7 +11,7 @@
 // lane of the warp has one of its two j inside the softening support (the
 // three-branch select of spline_value_r2); the self pair (r = 0) always takes it
 // and gives the finite centre. The stream-K split and the partial layout are
-// those of pair_fp32_kernel.
+// those of pair_row_kernel (pair2.cuh).
 #pragma once
 #include <cstdint>
 
@@ -98,7 +98,7 @@ __device__ __forceinline__ void pair_tile_r3(const IParticle& I, const R3Tile& T
   }
 }
 
-// part layout: [slot][3][kBI] doubles, slot = i-block + CTA (as pair_fp32_kernel).
+// part layout: [slot][3][kBI] doubles, slot = i-block + CTA (as pair_row_kernel).
 template <bool KAHAN>
 __global__ void __launch_bounds__(kBI, 8)
 pair_r3_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, long long U, int NT, int C,

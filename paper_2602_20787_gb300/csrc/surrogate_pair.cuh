@@ -465,7 +465,7 @@ __device__ __forceinline__ void pair_tile(const IParticle& I, const float4* sA, 
 }
 
 // Stream-K kernel with the surrogate tail (same work split and partial layout
-// as pair_fp32_kernel).
+// as pair_row_kernel, pair2.cuh).
 #ifndef STEPS_SURR_MIN_BLOCKS
 #define STEPS_SURR_MIN_BLOCKS 4  // co-resident CTAs per SM asked of the register allocator
 #endif

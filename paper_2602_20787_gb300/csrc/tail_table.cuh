@@ -284,7 +284,7 @@ __device__ __forceinline__ void pair_tile_table(const IParticle& I, const float4
 #endif
 
 // Stream-K kernel with the table tail (work split and partial layout of
-// pair_fp32_kernel).
+// pair_row_kernel, pair2.cuh).
 template <bool KAHAN, bool INF = false>
 __global__ void __launch_bounds__(kBI, STEPS_TABLE_MIN_BLOCKS)
 pair_fp32_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, long long U,
