@@ -214,7 +214,9 @@ __device__ __forceinline__ u64 spline_centre2(u64 R2C, u64 H2, const Soft2& s) {
 
 // The near images of a step with softened pairs: the full spline up to k1, the outer
 // shell up to kw, Newtonian beyond. Every image value is the same function of (r^2, h)
-// in each tier, so a pair's bits do not depend on the other lanes of its warp. M fixed
+// in each tier, so a pair's bits do not depend on the other lanes of its warp (in the closed
+// form up to kw = kPolyMaxSoft: a step that is softened farther out takes window_walk2 for all its pairs,
+// whose near range is the step's). M fixed
 // (unrolled; one warp-uniform branch per k), or m at run time.
 template <int M>
 __device__ __forceinline__ void near_soft2(u64 DR2, const Soft2& s, u64 ADZ, int kw, int k1, u64& SR, u64& SZ) {
