@@ -447,8 +447,9 @@ mlp_reduce_adam_kernel(const float* __restrict__ gpart, int nblocks, float inv_b
 // ---------------------------------------------------------------------------
 constexpr unsigned kBarrierSpins = 1u << 22;  // polls (of some 0.5 us) before a barrier gives up
 
-// Every CTA of the grid arrives (target: arrivals once all have). A wait that runs out sets *fail, and
-// later waits end at once.
+// Every CTA of the grid arrives (target: arrivals once all have). A wait that runs out sets *fail; the
+// waits after it in the same epoch end after 1,024 polls, half a millisecond each (the flag is not
+// looked at before: that would cost every barrier a round trip), and later epochs do nothing.
 __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, int* fail) {
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -474,6 +475,7 @@ mlp_epoch_kernel(float* w, const float* __restrict__ u, const float* __restrict_
   float* red = &sh.s_a1[0][0];
   unsigned target = 0;
   int step = 0;
+  if (*static_cast<volatile int*>(fail) != 0) return;  // a barrier of an earlier epoch ran out
   TrainSample in = load_sample(u, t, order, 0, min((int64_t)batch, ntrain), blockIdx.x);
   for (int64_t first = 0; first < ntrain; first += batch, ++step) {
     const int64_t count = min((int64_t)batch, ntrain - first), rest = ntrain - first - count;
