@@ -574,16 +574,39 @@ __device__ __forceinline__ void window2(const Sep2& P, int n_cut, float fnc, u64
 }
 
 // ---- the row kernel of the plain window -----------------------------------------
-// Rows against every j (shards' row step and the allocation-free call): the work split
-// and partial layout of the row kernels, [slot][3][kBI] doubles, slot = i-block + CTA. The
-// units cover the i-blocks [b0, b0 + U / NT), and slots count i-blocks from b0.
+// Rows against every j (shards' row step, loads whose sums fixed point does not resolve): the
+// work split and partial layout of the row kernels, [slot][3][kBI] doubles, slot = i-block + CTA. The
+// units cover the i-blocks [b0, b0 + U / NT), and slots count i-blocks from b0. A unit's j-tile has jt slots, 128
+// or fewer where that lets the places for CTAs share the units more evenly: the time goes as the largest number of units
+// of a place times jt and some 14 more for the tile's staging (N = 10,000, N_cut = 8 .. 16: 507 / 557 us whole / in
+// quarters; N = 2,000, N_cut = 8: 75 / 56).
 #ifndef STEPS_ROW_MIN_BLOCKS
 #define STEPS_ROW_MIN_BLOCKS 10  // resident CTAs per SM the kernel is compiled for (registers)
 #endif
+struct RowSplit {
+  long long U;
+  int NT, jt, C;
+};
+inline RowSplit row_split(int blocks, int n, int ctas) {
+  const int places = ctas < 152 * STEPS_ROW_MIN_BLOCKS ? ctas : 152 * STEPS_ROW_MIN_BLOCKS;
+  RowSplit best{0, 0, 0, 0};
+  long long cost = 0;
+  for (int jt = kBJ; jt >= 32; jt /= 2) {
+    const int NT = (n + jt - 1) / jt;
+    const long long U = (long long)blocks * NT;
+    const int C = (int)(U < ctas ? U : ctas);
+    const long long t = (U + places - 1) / places * (jt + 14);
+    if (best.jt == 0 || t < cost) {
+      best = RowSplit{U, NT, jt, C};
+      cost = t;
+    }
+  }
+  return best;
+}
 template <bool KAHAN, bool LINE>
 __global__ void __launch_bounds__(kPairThreads, STEPS_ROW_MIN_BLOCKS)
 pair_row_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, long long U, int NT,
-                int C, double* __restrict__ part, int b0, const int* __restrict__ skip = nullptr) {
+                int jt, int C, double* __restrict__ part, int b0, const int* __restrict__ skip = nullptr) {
   __shared__ JTile2 T;
   if (skip && *skip) return;  // the symmetric kernel has taken the pairs
   const int c = blockIdx.x;
@@ -599,10 +622,10 @@ pair_row_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, in
     u64 sx = 0, sy = 0, sz = 0, cx = 0, cy = 0, cz = 0;
     for (int t = t0; t < t1; ++t) {
       __syncthreads();
-      load_tile2<kPairThreads>(jA, jB, n, t, kBJ, T);
+      load_tile2<kPairThreads>(jA, jB, n, t, jt, T);
       __syncthreads();
 #pragma unroll 1
-      for (int k0 = 0; k0 < kBJ; k0 += STEPS_KAHAN_GROUP) {
+      for (int k0 = 0; k0 < jt; k0 += STEPS_KAHAN_GROUP) {
         u64 gx = 0, gy = 0, gz = 0;
 #pragma unroll 1
         for (int k = k0; k < k0 + STEPS_KAHAN_GROUP; ++k) {

@@ -113,11 +113,12 @@ struct FixAcc {
 // beside the heaviest particle at the load's largest separation D (units of L), in R^3 over D^2
 // and in the cylinder over the line's D sqrt(N^2 + D^2) / (2 N), N = n_cut. It has no units: it is the
 // same for any total mass and, in R^3, any unit of length. Up to kMaxSpread the unit is 2^-69 of a
-// typical sum, below FP64's rounding also when a load spreads a hundredfold between two looks at it. Beyond
-// (softenings of some 1e-4 of the load's size: these loads had the row kernels before) the row kernels
-// take the pairs.
+// typical sum, below FP64's rounding also when a load spreads a hundredfold between two looks at it: for
+// contexts (a softening of some 1e-4 of the load's size; their row kernels are as fast in R^3). The
+// allocation-free call looks at every load and adds FP32 sums: up to kMaxSpreadF, 2^-45 (1e-8 of the size).
+// Beyond, the row kernels take the pairs.
 constexpr int kLoBits = 40;
-constexpr double kMaxSpread = 0x1p28;
+constexpr double kMaxSpread = 0x1p28, kMaxSpreadF = 0x1p52;
 
 // B: one image's softened force is at most 4 / hh^2 <= (L / h_min)^2 = q^2 (the peak of the
 // spline of eq. Force_spline_kernel with hh >= 2 h_min), the other images of the window add at
@@ -125,10 +126,10 @@ constexpr double kMaxSpread = 0x1p28;
 __host__ __device__ __forceinline__ double fix_bound(double M, double q, bool images) {
   return M * (q * q + (images ? 10.0 : 0.0));
 }
-// Whether the spread is at most kMaxSpread (n_cut = 0: R^3), without a division or a root: sqrt(N^2 + D^2)
+// Whether the spread is at most `most` (n_cut = 0: R^3), without a division or a root: sqrt(N^2 + D^2)
 // is taken as N + D.
-__host__ __device__ __forceinline__ bool fix_resolves(double B, double M, double m_max, double D, int n_cut) {
-  const double N = n_cut, T = kMaxSpread * (M - m_max);
+__host__ __device__ __forceinline__ bool fix_resolves(double B, double M, double m_max, double D, int n_cut, double most) {
+  const double N = n_cut, T = most * (M - m_max);
   return n_cut > 0 ? B * D * (N + D) <= 2.0 * N * T : B * D * D <= T;
 }
 

@@ -1235,7 +1235,7 @@ bool use_sym(const steps_cyl_ctx* c) {
   if (!two_words(c)) return c->fix_ok;
   const double D = 2.0 * c->extent * c->invL;
   return c->fix_scale > 0.0 && c->ext_ok &&
-         fix_resolves(c->fix_B, c->fix_M, c->m_max, D, is_r3(c) ? 0 : c->p.n_cut);
+         fix_resolves(c->fix_B, c->fix_M, c->m_max, D, is_r3(c) ? 0 : c->p.n_cut, kMaxSpread);
 }
 
 // The pair form of the next force evaluation: FP64, the selected modelled tail
@@ -1425,6 +1425,7 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     return STEPS_OK;
   }
   CK(cudaEventRecord(c->e0, c->st));
+  RowSplit row{c->U, c->NT, kBJ, c->C};
   if (form == Form::FP64) {
     int rc = use_sym(c) ? launch_fp64_sym(c, c->part) : launch_fp64(c, nullptr, c->n, c->part);  // never sharded
     if (rc) return rc;
@@ -1468,7 +1469,9 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
     const bool kahan = c->p.precision == STEPS_FP32_KAHAN;
     auto kernel = line_form_rows(c->p.n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
                                         : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
-    kernel<<<c->C, kPairThreads, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, c->U, c->NT, c->C, c->part, c->b0, nullptr);
+    row = row_split(c->nbo, c->n, c->Ccap);
+    kernel<<<row.C, kPairThreads, 0, c->st>>>(c->jA, c->jB, c->n, c->p.n_cut, row.U, row.NT, row.jt, row.C, c->part, c->b0,
+                                             nullptr);
     CKLAUNCH("pair_row");
   }
   CK(cudaEventRecord(c->e1, c->st));
@@ -1477,11 +1480,13 @@ int eval_forces(steps_cyl_ctx* c, bool kick, double K, const AccelOut& out = Acc
   c->last_sym = form == Form::FP64 && use_sym(c);
   c->last_straight = false;
   c->last_pairs = (double)(c->k1 - c->k0) * (double)(c->n - 1) * (c->last_sym ? 0.5 : 1.0);
-  const int NT = form == Form::FP64 ? 0 : c->NT;
-  const int ctas = form == Form::FP64 ? 1 : form == Form::SURROGATE ? c->SC : form == Form::TABLE ? c->TC : c->C;
+  if (form == Form::FP64)
+    row = RowSplit{c->U, 0, kBJ, 1};
+  else if (form != Form::PLAIN)
+    row.C = form == Form::SURROGATE ? c->SC : c->TC;
   // rows [k0, k1): every row, or the rows this context owns when they are sharded
   finalize_kernel<<<(c->k1 - c->k0 + ft - 1) / ft, ft, 0, c->st>>>(
-      c->part, c->k1, NT, c->U, ctas, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K,
+      c->part, c->k1, row.NT, row.U, row.C, pair_scale, bg_params(c), c->x, c->y, c->z, c->gx, c->gy, c->gz, K,
       kick ? c->px : nullptr, kick ? c->py : nullptr, kick ? c->pz : nullptr, out, c->err,
       RadialCorr{nullptr, 0, 0.0, 0}, c->k0);
   CKLAUNCH("finalize");
@@ -2496,7 +2501,7 @@ int allocate_context(steps_cyl_ctx* c) {
   c->SYTC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(ytocc, 1) * STEPS_CTA_MULT);
   CKA(cudaMalloc(&c->facc, sizeof(unsigned long long) * nb * (is_r3(c) ? 6 : 3)));
   if (is_r3(c)) c->facc_lo = c->facc + 3 * nb;
-  c->part_elems = std::max((size_t)(c->NB + std::max({c->C, c->SC, c->TC})) * 3 * kBI, nb * 3);
+  c->part_elems = std::max((size_t)(c->NB + std::max({row_split(c->NB, c->n, c->Ccap).C, c->C, c->SC, c->TC})) * 3 * kBI, nb * 3);
   CKA(cudaMalloc(&c->part, sizeof(double) * c->part_elems));
 
 #undef CKA

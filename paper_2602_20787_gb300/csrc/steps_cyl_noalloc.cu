@@ -44,8 +44,9 @@ __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 // Each unordered pair is evaluated once where the fixed-point sums that this takes (two words,
 // pair_sym.cuh) resolve the load. That needs the total mass and the largest one, the smallest softening and
 // the extent, which the host cannot look at without waiting: the pack kernel reduces them on the
-// device, the symmetric kernel derives the scale, or leaves the pairs to the row kernel, whose CTAs
-// otherwise return at once. (N = 10,007, N_cut = 16, literal softening law: rows alone 730 us.)
+// device, its last CTA derives the scale, and the symmetric kernel or the row kernel takes the pairs; the
+// other's CTAs return at once. (Derived by every CTA of the symmetric kernel, the scale cost the row route 20 us
+// at N = 500, where its launch alone remains. N = 10,007, N_cut = 16, literal softening law: rows alone 730 us.)
 // The record lies in the partials' last slot, which the row kernel's split never reaches.
 constexpr int kPackThreads = 256;
 constexpr int kPackParts = (kNoallocMaxN + kPackThreads - 1) / kPackThreads;
@@ -53,8 +54,10 @@ struct NoallocHead {
   unsigned long long hmin;  // bits of the smallest h; 0 when some h is not > 0
   unsigned long long rmax;  // bits of the largest (|x| + |y|) / L, no less than the distance from the axis
   unsigned long long mmax;  // bits of the largest |m|
-  int err, sym;             // error bits of the symmetric kernel; whether it has taken the pairs
-  double scale;             // its sums' scale
+  int err, sym;             // error bits of the symmetric kernel; whether it takes the pairs
+  unsigned done;            // CTAs of the pack kernel that have finished
+  unsigned massive;         // particles whose mass is not zero
+  double scale;             // the sums' scale
   double mass[kPackParts];  // sums of |m| over each CTA of the pack kernel
 };
 constexpr size_t kHeadOffset = kScratchBytes - sizeof(double) * 3 * kBI;
@@ -62,12 +65,29 @@ static_assert(sizeof(NoallocHead) <= sizeof(double) * 3 * kBI, "the record takes
 static_assert(sizeof(unsigned long long) * 6 * kNoallocMaxN <= kPartBytes - sizeof(double) * 3 * kBI,
               "the fixed-point sums take the partials' place");
 
+// The scale as the contexts choose it (2^57 over the bound on |S_i|), 0: none. By a whole warp, once
+// every CTA's share is in the record (volatile: other CTAs wrote it).
+__device__ __forceinline__ double noalloc_scale(const volatile NoallocHead* head, int parts, double L, int n_cut) {
+  double M = 0.0;
+  for (int k = threadIdx.x & 31; k < parts; k += 32) M += head->mass[k];
+  for (int o = 16; o > 0; o >>= 1) M += __shfl_xor_sync(0xffffffffu, M, o);
+  const double B = fix_bound(M, L / __longlong_as_double((long long)head->hmin), true);
+  if (!(B >= 1e-290 && B < 1e270)) return 0.0;
+  // one mass among massless particles has no sum of its own to resolve
+  if (!fix_resolves(B, M, head->massive > 1 ? __longlong_as_double((long long)head->mmax) : 0.0,
+                    2.0 * __longlong_as_double((long long)head->rmax), n_cut, kMaxSpreadF))
+    return 0.0;
+  const int S = 57 - (((__double2hiint(B) >> 20) & 0x7ff) - 1022);  // B < 2^(exponent + 1); |S| < 1,023
+  return __hiloint2double((S + 1023) << 20, 0);
+}
+
 __global__ void __launch_bounds__(kPackThreads)
 noalloc_pack_kernel(const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
-                    const double* __restrict__ m, const double* __restrict__ h, int n, double invL,
+                    const double* __restrict__ m, const double* __restrict__ h, int n, double L, double invL, int n_cut,
                     float4* __restrict__ jA, float4* __restrict__ jB, unsigned long long* __restrict__ acc,
-                    NoallocHead* __restrict__ head) {
+                    NoallocHead* head) {
   __shared__ double warp[kPackThreads / 32];
+  __shared__ bool last;
   const int i = blockIdx.x * kPackThreads + threadIdx.x;
   double s = 0.0;
   unsigned long long hb = ~0ull, rb = 0, mb = 0;  // non-negative doubles order like their bits, NaN above all
@@ -79,6 +99,7 @@ noalloc_pack_kernel(const double* __restrict__ x, const double* __restrict__ y, 
     rb = (unsigned long long)__double_as_longlong((fabs(x[i]) + fabs(y[i])) * invL);
     mb = (unsigned long long)__double_as_longlong(s);
   }
+  const unsigned massive = __popc(__ballot_sync(0xffffffffu, mb != 0));
   for (int o = 16; o > 0; o >>= 1) {
     s += __shfl_down_sync(0xffffffffu, s, o);
     hb = min(hb, __shfl_down_sync(0xffffffffu, hb, o));
@@ -90,40 +111,34 @@ noalloc_pack_kernel(const double* __restrict__ x, const double* __restrict__ y, 
     atomicMin(&head->hmin, hb);
     atomicMax(&head->rmax, rb);
     atomicMax(&head->mmax, mb);
+    atomicAdd(&head->massive, massive);
+    __threadfence();
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < kPackThreads / 32; ++w) t += warp[w];
     head->mass[blockIdx.x] = t;
+    __threadfence();
+    last = atomicAdd(&head->done, 1u) == gridDim.x - 1;
   }
-}
-
-// The scale as the contexts choose it (2^57 over the bound on |S_i|), 0: none. By a whole warp.
-__device__ __forceinline__ double noalloc_scale(const NoallocHead* head, int parts, double L, int n_cut) {
-  double M = 0.0;
-  for (int k = threadIdx.x & 31; k < parts; k += 32) M += head->mass[k];
-  for (int o = 16; o > 0; o >>= 1) M += __shfl_xor_sync(0xffffffffu, M, o);
-  const double B = fix_bound(M, L / __longlong_as_double((long long)head->hmin), true);
-  if (!(B >= 1e-290 && B < 1e270)) return 0.0;
-  if (!fix_resolves(B, M, __longlong_as_double((long long)head->mmax),
-                    2.0 * __longlong_as_double((long long)head->rmax), n_cut))
-    return 0.0;
-  const int S = 57 - (((__double2hiint(B) >> 20) & 0x7ff) - 1022);  // B < 2^(exponent + 1); |S| < 1,023
-  return __hiloint2double((S + 1023) << 20, 0);
+  __syncthreads();
+  if (last && threadIdx.x < 32) {
+    __threadfence();
+    const double scale = noalloc_scale(head, gridDim.x, L, n_cut);
+    if (threadIdx.x == 0) {
+      head->scale = scale;
+      head->sym = scale > 0.0;
+    }
+  }
 }
 
 template <bool KAHAN, bool LINE>
 __global__ void __launch_bounds__(kSymThreads, STEPS_SYM_MIN_BLOCKS)
 noalloc_sym_kernel(const float4* __restrict__ jA, const float4* __restrict__ jB, int n, int n_cut, int NB, int tpb,
-                   int sp, long long U, int C, unsigned long long* __restrict__ acc, NoallocHead* __restrict__ head,
-                   int parts, double L) {
+                   int sp, long long U, int C, unsigned long long* __restrict__ acc, NoallocHead* __restrict__ head) {
   __shared__ SymShared<KAHAN> sh;
-  const double scale = noalloc_scale(head, parts, L, n_cut);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    head->sym = scale > 0.0;
-    head->scale = scale;
-  }
+  const double scale = head->scale;
   if (!(scale > 0.0)) return;
   const float f = scale <= ldexp(1.0, kMaxFixExpF) && scale >= ldexp(1.0, -kMaxFixExpF) ? (float)scale : 0.0f;
   sym_stream_k<KAHAN, true, KAHAN>(jA, jB, n, NB, tpb, sp, 0, U, C, sh,
@@ -243,9 +258,8 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   float4* jA = reinterpret_cast<float4*>(d->base);
   float4* jB = reinterpret_cast<float4*>(d->base + kPackBytes);
   double* part = reinterpret_cast<double*>(d->base + 2 * kPackBytes);
-  const int NB = (nn + kBI - 1) / kBI, NT = (nn + kBJ - 1) / kBJ;
-  const long long U = (long long)NB * NT;
-  const int C = (int)std::min<long long>(U, d->ctas);
+  const int NB = (nn + kBI - 1) / kBI;
+  const RowSplit row = row_split(NB, nn, d->ctas);
   const double invL = 1.0 / L;
 
   // every byte of the scratch array this call reads, it writes first: the record, the packed
@@ -256,7 +270,7 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   const int parts = (nn + kPackThreads - 1) / kPackThreads;
   cudaMemsetAsync(&head->hmin, 0xff, sizeof head->hmin, st);
   cudaMemsetAsync(&head->rmax, 0, offsetof(NoallocHead, scale) - offsetof(NoallocHead, rmax), st);
-  noalloc_pack_kernel<<<parts, kPackThreads, 0, st>>>(x, y, z, m, h, nn, invL, jA, jB, acc, head);
+  noalloc_pack_kernel<<<parts, kPackThreads, 0, st>>>(x, y, z, m, h, nn, L, invL, n_cut, jA, jB, acc, head);
   const bool kahan = precision == STEPS_FP32_KAHAN;
   int tpb, sp;
   sym_split(NB, d->sms, true, tpb, sp);
@@ -264,12 +278,12 @@ extern "C" int steps_cyl_pair_accel_noalloc(int64_t n, const double* x, const do
   const int SC = (int)std::min<long long>(SU, 32LL * d->sym_ctas);
   auto sym = line_form_rows(n_cut) ? (kahan ? noalloc_sym_kernel<true, true> : noalloc_sym_kernel<false, true>)
                               : (kahan ? noalloc_sym_kernel<true, false> : noalloc_sym_kernel<false, false>);
-  sym<<<SC, kSymThreads, 0, st>>>(jA, jB, nn, n_cut, NB, tpb, sp, SU, SC, acc, head, parts, L);
+  sym<<<SC, kSymThreads, 0, st>>>(jA, jB, nn, n_cut, NB, tpb, sp, SU, SC, acc, head);
   auto kernel = line_form_rows(n_cut) ? (kahan ? pair_row_kernel<true, true> : pair_row_kernel<false, true>)
                                  : (kahan ? pair_row_kernel<true, false> : pair_row_kernel<false, false>);
-  kernel<<<C, kPairThreads, 0, st>>>(jA, jB, nn, n_cut, U, NT, C, part, 0, &head->sym);
+  kernel<<<row.C, kPairThreads, 0, st>>>(jA, jB, nn, n_cut, row.U, row.NT, row.jt, row.C, part, 0, &head->sym);
   const int ft = particle_threads(nn);
-  noalloc_finalize_kernel<<<(nn + ft - 1) / ft, ft, 0, st>>>(acc, part, head, nn, NT, U, C, -G * invL * invL, ax, ay,
+  noalloc_finalize_kernel<<<(nn + ft - 1) / ft, ft, 0, st>>>(acc, part, head, nn, row.NT, row.U, row.C, -G * invL * invL, ax, ay,
                                                              az);
   // a launch failure replaces the thread's last error; one equal to the error
   // pending before the call is taken as the caller's, which stays in place

@@ -12,8 +12,8 @@ import device_source as ds
 
 WRAP = """
 extern "C" double bound(double M, double q, int images) { return fix_bound(M, q, images != 0); }
-extern "C" int resolves(double B, double M, double m, double D, int n) { return fix_resolves(B, M, m, D, n); }
-extern "C" double limit() { return kMaxSpread; }
+extern "C" int resolves(double B, double M, double m, double D, int n, double most) { return fix_resolves(B, M, m, D, n, most); }
+extern "C" double limit(int fp32) { return fp32 ? kMaxSpreadF : kMaxSpread; }
 extern "C" int bits() { return kLoBits; }
 """
 
@@ -24,7 +24,7 @@ def rule(tmp_path_factory):
                           ds.function("pair_sym.cuh", "fix_bound"), ds.function("pair_sym.cuh", "fix_resolves"), WRAP)
     d = ctypes.c_double
     lib.bound.argtypes, lib.bound.restype, lib.limit.restype = [d, d, ctypes.c_int], d, d
-    lib.resolves.argtypes = [d, d, d, d, ctypes.c_int]
+    lib.resolves.argtypes = [d, d, d, d, ctypes.c_int, d]
     return lib
 
 
@@ -74,18 +74,20 @@ def test_accepted_sums_lose_nothing(rule, n_cut, M, R, soft, heavy):
     assert abs(exact).max() <= 16 * B  # 2^57 / B leaves no sum beyond 2^62
     D = 2 * np.sqrt((pos[:, :2 if n_cut else 3] ** 2).sum(1)).max()
     spread = B / (m.sum() - m.max()) * (D * np.hypot(D, n_cut) / (2 * n_cut) if n_cut else D * D)
-    taken = rule.resolves(B, m.sum(), m.max(), D, n_cut)
-    assert not taken or spread <= rule.limit()
     got = two_word(t, np.longdouble(2) ** np.floor(57 - np.log2(B)), rule.bits())
     err = np.linalg.norm(got - exact, axis=1) / np.linalg.norm(exact, axis=1)
     # one unit is at most 2^-96 B (a power of two below 2^57 / B); a particle's sum rounds once per
     # term, half a unit each, in three components
     unit = 2.0 ** -96 * spread * 2 * np.sqrt(3 * t.shape[1])
-    if taken:  # FP64's rounding of a sum is 1.1e-16
-        assert np.median(err) <= unit and err[0] <= 30 * unit and unit <= 1e-17
-    # what does not depend on the units: a load with an ordinary softening is accepted
-    if soft >= 1e-3 and not heavy and (n_cut == 0 or R == 1.0):
-        assert taken
+    for fp32 in (0, 1):
+        most = rule.limit(fp32)
+        taken = rule.resolves(B, m.sum(), m.max(), D, n_cut, most)
+        assert not taken or spread <= most
+        if taken:  # FP64's rounding of a sum is 1.1e-16, FP32's 6e-8
+            assert np.median(err) <= unit and err[0] <= 30 * unit and unit <= (1e-12 if fp32 else 1e-17)
+        # what does not depend on the units: a load with an ordinary softening is accepted
+        if soft >= (1e-7 if fp32 else 1e-3) and not heavy and (n_cut == 0 or R == 1.0):
+            assert taken
 
 
 def test_the_rule_has_no_units(rule):
@@ -93,7 +95,7 @@ def test_the_rule_has_no_units(rule):
         lo, hi = 1.0, 1e12
         for _ in range(80):
             q = np.sqrt(lo * hi)
-            ok = rule.resolves(rule.bound(M, q / length, int(n_cut > 0)), M, 0.25 * M, 3.0 * length, n_cut)
+            ok = rule.resolves(rule.bound(M, q / length, int(n_cut > 0)), M, 0.25 * M, 3.0 * length, n_cut, rule.limit(0))
             lo, hi = (q, hi) if ok else (lo, q)
         return lo
     for n_cut in (0, 16):

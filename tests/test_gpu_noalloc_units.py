@@ -71,3 +71,17 @@ def test_both_sides_are_summed_alike(sc, n_cut, half):
     a = accel(sc, pos, np.full(2 * half, 1.0 / 3.0), np.full(2 * half, 0.05), n_cut, sc.STEPS_FP32_KAHAN)
     assert np.all(a[:half] == a[0]) and np.all(a[half:] == a[half])
     assert np.all(abs(a[0] + a[half]) <= 1e-11 * abs(a[0])), (a[0], a[half])
+
+
+@pytest.mark.parametrize("n_cut", [5, 16])
+def test_one_mass_among_massless_particles(sc, n_cut):
+    d = ics.particle_load(300, 9, 1.0)
+    m = np.zeros(300)
+    m[7] = 2.5
+    h = np.full(300, 1e-3)
+    a = accel(sc, d["pos"], m, h, n_cut, sc.STEPS_FP32_KAHAN)
+    ref = oracle.pair_field(d["pos"], m, h, 1.0, 1.0, n_cut)
+    assert np.all(a[7] == 0.0) and np.array_equal(ref[7], np.zeros(3))
+    k = np.arange(300) != 7
+    err = np.linalg.norm(a[k] - ref[k], axis=1) / np.linalg.norm(ref[k], axis=1)
+    assert np.median(err) <= 1e-6 and err.max() <= 1e-4
