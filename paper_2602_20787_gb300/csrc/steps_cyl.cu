@@ -1205,8 +1205,9 @@ int fix_scale(steps_cyl_ctx* c) {
 // Whether the next force evaluation's sums have two words.
 bool two_words(const steps_cyl_ctx* c) { return !is_tree(c) && (is_r3(c) || c->p.precision == STEPS_FP64); }
 
-// The extent of the load, which the spread of two-word sums depends on: taken with the state and at the end
-// of each KDK call, and every kExtentEvery steps of one (the host waits for it).
+// The extent of the load, which the spread of two-word sums depends on: taken with the state and every
+// kExtentEvery KDK steps, however these are split into calls (the host waits for it: 10 us, which each call
+// of one step would feel).
 constexpr int kExtentEvery = 32;
 int launch_extent(steps_cyl_ctx* c) {
   CK(cudaMemsetAsync(c->mbox + 4, 0, sizeof(unsigned long long), c->st));
@@ -2748,7 +2749,7 @@ int steps_cyl_kdk_step(steps_cyl_ctx* c, double dt, int32_t nsteps) {
       if ((rc = reorder(c))) return rc;
     }
     c->ext_ok = c->ext_ok && two_words(c);
-    if (two_words(c) && ++c->steps_since_extent >= kExtentEvery && s + 1 < nsteps) {
+    if (two_words(c) && ++c->steps_since_extent >= kExtentEvery) {
       if ((rc = launch_extent(c))) return rc;
       CK(cudaStreamSynchronize(c->st));
       c->ext_ok = true;
@@ -2774,10 +2775,7 @@ int steps_cyl_kdk_step(steps_cyl_ctx* c, double dt, int32_t nsteps) {
     }
   }
   int e = 0;
-  const bool ext = two_words(c) && nsteps > 0;
-  if (ext && (rc = launch_extent(c))) return rc;
   if ((rc = read_and_clear_err(c, &e))) return rc;
-  c->ext_ok = c->ext_ok || ext;
   if (e) return device_error(e);
   if (rejected) return fail(STEPS_ESURROGATE_REJECTED, "%s", reject_msg);
   return STEPS_OK;
@@ -2972,10 +2970,11 @@ int steps_cyl_shard_kick(steps_cyl_ctx* c, const float* recv) {
   c->t += c->pend_dt;
   c->drifted = false;
   int e = 0;
-  const bool ext = two_words(c) && c->shard_world == 1;  // the rows of other ranks are not held here
+  // (the rows of other ranks are not held here: they take the row kernels)
+  const bool ext = two_words(c) && c->shard_world == 1 && ++c->steps_since_extent >= kExtentEvery;
   if (ext && (rc = launch_extent(c))) return rc;
   if ((rc = read_and_clear_err(c, &e))) return rc;
-  c->ext_ok = ext;
+  c->ext_ok = ext || (c->ext_ok && two_words(c) && c->shard_world == 1);
   if (e) return device_error(e);
   return STEPS_OK;
 }
