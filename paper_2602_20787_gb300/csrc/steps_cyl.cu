@@ -2294,11 +2294,13 @@ int train_surrogate(steps_cyl_ctx* c, const steps_cyl_train_cfg* cfg, double* re
   AdamCfg adam{0.f, 0.9f, 0.999f, 1e-8f};
   // one cooperative launch per epoch where all blocks of a step fit the GPU at once
   const int64_t nsteps = (ntrain + cfg->batch - 1) / cfg->batch;
-  const int grid = (int)((std::min<int64_t>(cfg->batch, ntrain) + kTrainThreads - 1) / kTrainThreads);
+  int grid = (int)((std::min<int64_t>(cfg->batch, ntrain) + kTrainThreads - 1) / kTrainThreads);
   int sms = 0, per_sm = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_epoch_kernel, kTrainCta, 0));
   const bool whole = grid <= sms * per_sm;
+  // the update's 32 weights per CTA: with fewer blocks of samples than that, CTAs without any share it
+  grid = std::max(grid, std::min((kNW + 31) / 32, sms * per_sm));
   CK(cudaMallocAsync(&B.corr, sizeof(float2) * nsteps, c->st));
   CK(cudaMallocAsync(&B.bar, sizeof(unsigned) * 2, c->st));
   CK(cudaMemsetAsync(B.bar, 0, sizeof(unsigned) * 2, c->st));
