@@ -587,6 +587,11 @@ struct RowSplit {
   long long U;
   int NT, jt, C;
 };
+// The most CTAs that row_split gives any number of blocks up to `blocks` (partials are allocated for them).
+inline int row_ctas(int blocks, int n, int ctas) {
+  const long long U = (long long)blocks * ((n + 31) / 32);
+  return (int)(U < ctas ? U : ctas);
+}
 inline RowSplit row_split(int blocks, int n, int ctas) {
   const int places = ctas < 152 * STEPS_ROW_MIN_BLOCKS ? ctas : 152 * STEPS_ROW_MIN_BLOCKS;
   RowSplit best{0, 0, 0, 0};

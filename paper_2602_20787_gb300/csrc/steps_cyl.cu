@@ -2504,7 +2504,7 @@ int allocate_context(steps_cyl_ctx* c) {
   c->SYTC = (int)std::min<long long>(c->Usym, (long long)sms * std::max(ytocc, 1) * STEPS_CTA_MULT);
   CKA(cudaMalloc(&c->facc, sizeof(unsigned long long) * nb * (is_r3(c) ? 6 : 3)));
   if (is_r3(c)) c->facc_lo = c->facc + 3 * nb;
-  c->part_elems = std::max((size_t)(c->NB + std::max({row_split(c->NB, c->n, c->Ccap).C, c->C, c->SC, c->TC})) * 3 * kBI, nb * 3);
+  c->part_elems = std::max((size_t)(c->NB + std::max({row_ctas(c->NB, c->n, c->Ccap), c->SC, c->TC})) * 3 * kBI, nb * 3);
   CKA(cudaMalloc(&c->part, sizeof(double) * c->part_elems));
 
 #undef CKA
