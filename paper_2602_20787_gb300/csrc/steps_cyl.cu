@@ -2842,13 +2842,16 @@ int steps_cyl_set_precision(steps_cyl_ctx* c, int32_t precision) {
   c->p.precision = precision;
   if (precision == STEPS_FP64) c->p.tail = STEPS_TAIL_FULL;
   c->forces_stale = true;  // refreshed by the next force evaluation or KDK step
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  CK(cudaStreamIsCapturing(c->st, &cap));
-  if (two_words(c) && !c->ext_ok && cap == cudaStreamCaptureStatusNone) {
-    int rc;
-    if ((rc = launch_extent(c))) return rc;
-    CK(cudaStreamSynchronize(c->st));
-    c->ext_ok = true;
+  if (two_words(c) && !c->ext_ok) {  // without a look (a capture in progress) the row kernels run
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) {
+      cudaGetLastError();
+    } else if (cap == cudaStreamCaptureStatusNone) {
+      int rc;
+      if ((rc = launch_extent(c))) return rc;
+      CK(cudaStreamSynchronize(c->st));
+      c->ext_ok = true;
+    }
   }
   return STEPS_OK;
 }
