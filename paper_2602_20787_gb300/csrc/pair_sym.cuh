@@ -607,7 +607,8 @@ pair_sym_table_kernel(const float4* __restrict__ jA, const float4* __restrict__ 
 // ring's three shuffles and the loop serve four pairs, and one warp is a CTA. With two
 // rows per lane the duplicated j words alone would keep the shared-memory pipe busier
 // than the FP32 one. The row kernel (r3_pair.cuh) evaluates every ordered pair in 31 issue
-// slots per 32 pairs: 3.39 ms per force at N = 65,536 against 2.85 here.
+// slots per 32 pairs: 3.39 ms per force at N = 65,536 against 2.97 here (2.85 with one-word sums and j-side
+// groups of eight steps, which lost sums or digits that the row kernel kept).
 #ifndef STEPS_SYM_R3_MIN_BLOCKS
 #define STEPS_SYM_R3_MIN_BLOCKS 16  // resident CTAs (warps) per SM the kernel is compiled for
 #endif
