@@ -54,7 +54,9 @@ extern "C" {
 #define STEPS_TAIL_FULL 0       /* every image of the window: one by one for n_cut < 12 (FP64, and where
                                  * every FP32 sum is compensated: < 16); else the near
                                  * images (and the softened ones) one by one and the others, a smooth function of
-                                 * the image number, in closed form to below the precision's rounding */
+                                 * the image number, in closed form to below the precision's rounding (FP64: the
+                                 * form's last terms, below 2e-10 of the sum, in FP32; the pair's error stays below
+                                 * that of the images one by one) */
 #define STEPS_TAIL_SURROGATE 1  /* images |k| <= n0 direct, far tail from the learned surrogate */
 #define STEPS_TAIL_TABLE 2      /* images |k| <= n0 direct, far tail from the correction table */
 
